@@ -133,29 +133,27 @@ template <> __device__ __forceinline__ void store_split<bf16>(bf16 *p, long long
   if (lo_delta) p[lo_delta] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// Output of a GEMM: rows are cut into chunks of (1 << chunk_shift) rows, one launch each,
-// chunk_stride floats apart.  Inside a chunk the stream-K tensor-core kernel leaves up to
-// ceil(kb / upc) + 1 partial sums per 256-column tile, stacked in slots of slot_stride floats; the
-// SIMT kernel leaves one (upc == 0).
+// Output of a GEMM: [rows][ld].  The stream-K tensor-core kernel leaves up to ceil(kb / upc) + 1 partial
+// sums per 256-column tile, stacked in slots of slot_stride floats; the SIMT kernel leaves one
+// (upc == 0).
 struct GemmOut {
   const float *base;
   long long slot_stride;   // floats between consecutive slots
-  long long chunk_stride;  // floats between consecutive row chunks
-  int chunk_shift;         // log2 of the rows per chunk
   int ld;                  // floats between consecutive rows (tokens)
   int kb;                  // k-panels per tile
-  int upc;                 // work units (tile, k-panel) per CTA; 0 = single slot
+  int upc;                 // work units (tile, k-panel) per worker; 0 = single slot
 };
 
+__device__ __forceinline__ int gemm_extra_slots(const GemmOut &g, int c) {
+  if (!g.upc) return 0;
+  unsigned u0 = (unsigned)(c >> 8) * (unsigned)g.kb;
+  return (int)((u0 + (unsigned)g.kb - 1u) / (unsigned)g.upc) - (int)(u0 / (unsigned)g.upc);
+}
 __device__ __forceinline__ float gemm_val(const GemmOut &g, int r, int c) {
-  int ch = r >> g.chunk_shift;
-  const float *p = g.base + (long long)ch * g.chunk_stride + (long long)(r - (ch << g.chunk_shift)) * g.ld + c;
+  const float *p = g.base + (long long)r * g.ld + c;
   float s = *p;
-  if (g.upc) {
-    unsigned u0 = (unsigned)(c >> 8) * (unsigned)g.kb;
-    int extra = (int)((u0 + (unsigned)g.kb - 1u) / (unsigned)g.upc) - (int)(u0 / (unsigned)g.upc);
-    for (int i = 1; i <= extra; ++i) s += p[(long long)i * g.slot_stride];
-  }
+  const int extra = gemm_extra_slots(g, c);
+  for (int i = 1; i <= extra; ++i) s += p[(long long)i * g.slot_stride];
   return s;
 }
 
@@ -163,15 +161,8 @@ __device__ __forceinline__ float gemm_val(const GemmOut &g, int r, int c) {
 // The slots are added in slot order, but fetched four at a time so that a value made of many
 // partial sums costs a few memory round trips instead of one per slot.
 __device__ __forceinline__ void add4(float4 &s, const float4 &t) { s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w; }
-__device__ __forceinline__ int gemm_extra_slots(const GemmOut &g, int c) {
-  if (!g.upc) return 0;
-  unsigned u0 = (unsigned)(c >> 8) * (unsigned)g.kb;
-  return (int)((u0 + (unsigned)g.kb - 1u) / (unsigned)g.upc) - (int)(u0 / (unsigned)g.upc);
-}
 __device__ __forceinline__ float4 gemm_val4(const GemmOut &g, int r, int c) {
-  int ch = r >> g.chunk_shift;
-  const float4 *p = reinterpret_cast<const float4 *>(g.base + (long long)ch * g.chunk_stride +
-                                                     (long long)(r - (ch << g.chunk_shift)) * g.ld + c);
+  const float4 *p = reinterpret_cast<const float4 *>(g.base + (long long)r * g.ld + c);
   float4 s = *p;
   const int extra = gemm_extra_slots(g, c);
   const long long st4 = g.slot_stride >> 2;
@@ -193,9 +184,7 @@ __device__ __forceinline__ float4 gemm_val4(const GemmOut &g, int r, int c) {
 // read values made of many partial sums, such as the outputs of the narrow projections).
 template <int MAXS>
 __device__ __forceinline__ float4 gemm_val4_wide(const GemmOut &g, int r, int c) {
-  int ch = r >> g.chunk_shift;
-  const float4 *p = reinterpret_cast<const float4 *>(g.base + (long long)ch * g.chunk_stride +
-                                                     (long long)(r - (ch << g.chunk_shift)) * g.ld + c);
+  const float4 *p = reinterpret_cast<const float4 *>(g.base + (long long)r * g.ld + c);
   float4 s = *p;
   const int extra = gemm_extra_slots(g, c);
   const long long st4 = g.slot_stride >> 2;

@@ -38,7 +38,6 @@ struct dream_ctx {
   int use_tc, use_pdl, gemm_failed;
   cudaError_t launch_err;              // first refused kernel launch of the call being enqueued
   const char *launch_err_name;
-  int chunk;                           // prompt rows per pass of the prefill loop
   double *rope_inv;                    // [head_dim / 2] rotary inverse frequencies
   float2 *rope_tab;                    // [ROW_CHUNK][head_dim / 2] rotary (cos, sin) of the rows of the call being enqueued
   std::vector<const void *> ln1, wqkv, wo, ln2, wgu, wd;
@@ -281,7 +280,6 @@ static void derive(dream_ctx *c) {
   c->cap_rows = f.max_seq + c->ts.NI;
   c->pps = (f.max_seq + f.page_tokens - 1) / f.page_tokens;
   c->n_pages = c->pps * f.max_batch;
-  c->chunk = f.dtype == DREAM_BF16 ? TC_ROWS_SPLIT_1MMA : ROW_CHUNK;
   c->RM = (imax(ROW_CHUNK, f.max_prompt) + 15) & ~15;
   c->XR = c->RM;
   c->three = f.draft_blocks == 3;
@@ -341,23 +339,16 @@ static size_t carve(dream_ctx *c, char *base) {
   c->act = a.take_bytes((size_t)planes * ROW_CHUNK * f.d_ff * e);
   int lm_rows = ((imax(MB * T, MB * imax(c->ts.D + 2, f.tree_beam)) + 15) / 16) * 16;
   c->gemm_rows_lm = lm_rows;
-  // GEMM output: the widest of every projection's footprint.  fp32: rows x N.  bf16: one region
-  // per 64-row chunk, each with room for the stream-K partial-sum slots (bound for <= 192 SMs).
+  // GEMM output: the widest of every projection's footprint.  fp32: rows x N.  bf16: room for the
+  // stream-K partial-sum slots (bound for <= 192 SMs).
   {
     const int shapes[8][2] = {{c->qkvN, d}, {d, c->Hhd}, {2 * f.d_ff, d}, {d, f.d_ff}, {c->Hhd, d}, {c->kvN, d}, {f.vocab, d}, {0, 0}};
     size_t need = 0;
     for (int i = 0; shapes[i][0]; ++i) {
       int N = shapes[i][0], K = shapes[i][1];
       size_t fl;
-      if (f.dtype == DREAM_BF16) {
-        long long per = (gemm_tc_out_floats(192, TC_ROWS_SPLIT_1MMA, N, K) + 63) & ~63LL;
-        long long per2 = (gemm_tc_out_floats(192, TC_ROWS_MAX, N, K) + 63) & ~63LL;
-        fl = (size_t)imax(1, ROW_CHUNK / TC_ROWS_SPLIT_1MMA) * per;
-        size_t fl2 = (size_t)imax(1, ROW_CHUNK / TC_ROWS_MAX) * per2;
-        if (fl2 > fl) fl = fl2;
-        size_t fl3 = (size_t)((gemm_tc_out_floats(192, ROW_CHUNK, N, K) + 63) & ~63LL);
-        if (fl3 > fl) fl = fl3;
-      } else fl = (size_t)ROW_CHUNK * N;
+      if (f.dtype == DREAM_BF16) fl = (size_t)((gemm_tc_out_floats(192, ROW_CHUNK, N, K) + 63) & ~63LL);
+      else fl = (size_t)ROW_CHUNK * N;
       if (fl > need) need = fl;
     }
     c->gout_floats = need;
@@ -412,52 +403,35 @@ extern "C" dream_status dream_arena_bytes(const dream_config *cfg, size_t *bytes
 
 // ------------------------------------------------------------------------------------- GEMM dispatch
 
-// How the rows of a bf16 GEMM input buffer are laid out for a launch set of R rows: up to 64 rows
-// high and low rows alternate; more rows use two planes (high parts first, low parts lo_rows rows
-// further on); up to 256 rows go through a GEMM in one launch (two token tiles per weight panel).
+// How the rows of a GEMM input buffer are laid out: bf16 configurations keep two planes (high parts,
+// then low parts lo_rows rows further on).
 struct XMode { int mode, lo_rows; };
-static XMode xmode(const dream_ctx *c, int R) {
-  if (c->cfg.dtype != DREAM_BF16) return XMode{TC_X_PLAIN, 0};
-  if (R <= TC_ROWS_SPLIT_1MMA) return XMode{TC_X_INTERLEAVED, 0};
-  return XMode{TC_X_PLANAR, R <= TC_ROWS_MAX ? TC_ROWS_MAX : ROW_CHUNK};
+static XMode xmode(const dream_ctx *c) {
+  return c->cfg.dtype == DREAM_BF16 ? XMode{TC_X_PLANAR, ROW_CHUNK} : XMode{TC_X_PLAIN, 0};
 }
 static XLayout xlay(XMode m, long long width) {
-  if (m.mode == TC_X_INTERLEAVED) return XLayout{2 * width, width};
-  if (m.mode == TC_X_PLANAR) return XLayout{width, (long long)m.lo_rows * width};
-  return XLayout{width, 0};
+  return XLayout{width, m.mode == TC_X_PLANAR ? (long long)m.lo_rows * width : 0};
 }
 
-// out[r][c] = sum_k X[r][k] W[c][k] for r < rows, c < N; X holds the rows in layout m.
+// out[r][c] = sum_k X[r][k] W[c][k] for r < rows <= ROW_CHUNK, c < N; X holds the rows in layout m.
 // Returns the descriptor consumers read the result through.
 template <typename T>
 static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int rows, int N, int K) {
   GemmOut g;
   if (sizeof(T) == 2) {
-    // rows per launch: 64 (interleaved), 128 (two planes), 256 (two planes with room for two token tiles)
-    int chunk = m.mode == TC_X_INTERLEAVED ? TC_ROWS_SPLIT_1MMA : (m.mode == TC_X_PLANAR && m.lo_rows >= 2 * TC_ROWS_MAX ? 2 * TC_ROWS_MAX : TC_ROWS_MAX);
-    int nch = (rows + chunk - 1) / chunk;
-    int slot_rows = nch > 1 ? chunk : rows;
-    long long per = (gemm_tc_out_floats(c->tc.n_sms, slot_rows, N, K) + 63) & ~63LL;
-    XLayout lay = xlay(m, K);
-    for (int ch = 0; ch < nch; ++ch) {
-      int rows_c = imin(chunk, rows - ch * chunk);
-      const bf16 *Xc = (const bf16 *)X + (long long)ch * chunk * lay.row_stride;
-      bool timed = c->prof_on && 2 * (c->prof_n + 1) <= (int)c->prof_ev.size();
-      if (timed) cudaEventRecord(c->prof_ev[2 * c->prof_n], c->stream);
-      if (!gemm_tc_launch(&c->tc, c->stream, W, Xc, m.mode, m.lo_rows, rows_c, slot_rows, N, K, c->gout + (long long)ch * per,
-                          (long long)c->gout_floats - (long long)ch * per, &g))
-        c->gemm_failed = 1;
-      if (timed) { cudaEventRecord(c->prof_ev[2 * c->prof_n + 1], c->stream); c->prof_n++; c->prof_bytes += 2.0 * N * K; }
-      c->launches++;
-      c->tc_launches++;
-    }
-    g.base = c->gout; g.chunk_stride = per; g.chunk_shift = chunk == 64 ? 6 : (chunk == 128 ? 7 : 8);
+    bool timed = c->prof_on && 2 * (c->prof_n + 1) <= (int)c->prof_ev.size();
+    if (timed) cudaEventRecord(c->prof_ev[2 * c->prof_n], c->stream);
+    if (!gemm_tc_launch(&c->tc, c->stream, W, X, m.mode, m.lo_rows, rows, N, K, c->gout, (long long)c->gout_floats, &g))
+      c->gemm_failed = 1;
+    if (timed) { cudaEventRecord(c->prof_ev[2 * c->prof_n + 1], c->stream); c->prof_n++; c->prof_bytes += 2.0 * N * K; }
+    c->launches++;
+    c->tc_launches++;
     return g;
   }
   c->simt_launches++;
   dim3 grid((N + SG_BN - 1) / SG_BN, (rows + SG_BM - 1) / SG_BM);
   LAUNCH(c, (k_gemm_simt<T>), grid, 256, 0, (const T *)X, (const T *)W, c->gout, rows, N, K, N);
-  g.base = c->gout; g.slot_stride = 0; g.chunk_stride = 0; g.chunk_shift = 30; g.ld = N; g.kb = 0; g.upc = 0;
+  g.base = c->gout; g.slot_stride = 0; g.ld = N; g.kb = 0; g.upc = 0;
   return g;
 }
 
@@ -479,7 +453,7 @@ static FlatKV flat(dream_ctx *c, float *base) {
   kv.split = c->cfg.dtype == DREAM_BF16 ? 1 : 0;
   return kv;
 }
-static const GemmOut NO_GEMM = {nullptr, 0, 0, 30, 0, 0, 0};
+static const GemmOut NO_GEMM = {nullptr, 0, 0, 0, 0};
 
 // ------------------------------------------------------------------------------------- prefix bounds
 
@@ -701,7 +675,7 @@ template <typename T, int HD> struct AttnLaunch {
       // walks all keys up to its last row; row log-sum-exp and entropy (Eq. 2) come out of the same pass
       AttnTcArgs a = {};
       a.mode = AT_PREFILL;
-      a.n_keys = n; a.lay = xlay(xmode(c, ROW_CHUNK), c->Hhd);
+      a.n_keys = n; a.lay = xlay(xmode(c), c->Hhd);
       a.out_chunk_rows = ROW_CHUNK; a.out_chunk_stride = prefill_chunk_stride(c);
       a.lse = c->lse_pre; a.ent = c->ent_pre;
       c->cur_seq[0] = seq;
@@ -709,7 +683,7 @@ template <typename T, int HD> struct AttnLaunch {
       return;
     }
     dim3 grid((n + ATT_WARPS * ATT_PF_ROWS - 1) / (ATT_WARPS * ATT_PF_ROWS), c->cfg.n_heads);
-    const XMode m = xmode(c, ROW_CHUNK);
+    const XMode m = xmode(c);
     LAUNCH(c, (k_attn_prefill<T, HD>), grid, ATT_WARPS * 32, 0, c->qbuf, paged(c, layer), seq, n, c->cfg.n_heads,
            1.f / sqrtf((float)HD), (T *)c->attn_out, xlay(m, c->Hhd), ROW_CHUNK, prefill_chunk_stride(c), c->lse_pre, c->ent_pre);
   }
@@ -898,8 +872,7 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
   LAUNCH(c, k_iota_rows, (n + 255) / 256, 256, 0, c->rm[0], seq, n);
   LAUNCH(c, (k_build_prompt<T>), n, 256, 0, (const T *)c->embed, (const T *)visual, ids, vis_start, v, c->x, c->x0,
          d, f.vocab, c->status);
-  const XMode mp = xmode(c, CH);           // the layout of a full chunk of rows
-  const XMode m1 = xmode(c, 1);
+  const XMode mp = xmode(c);
   const long long att_chunk = prefill_chunk_stride(c);
   for (int l = 0; l < L; ++l) {
     for (int r0 = 0; r0 < n; r0 += CH) {
@@ -926,8 +899,8 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
     }
   }
   // first token: LM head on the last prompt row
-  norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, m1);
-  GemmOut g = gemm<T>(c, c->lm_head, c->xn, m1, 1, f.vocab, d);
+  norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
+  GemmOut g = gemm<T>(c, c->lm_head, c->xn, mp, 1, f.vocab, d);
   TOPK_LAUNCH(c, dim3(1, c->tk_nsplit), g, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
   LAUNCH(c, k_first_token, 1, 32, 0, c->top_id, c->top_val, first_token, first_margin);
   LAUNCH(c, k_set_seq, 1, 32, 0, c->sd, seq, n, c->top_id, -1, -1);
@@ -1024,12 +997,12 @@ static GemmOut draft_rows(dream_ctx *c, const RowMeta &rm, int R, XMode xm, int 
 template <typename T>
 static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *forced, int *kept, float *scores) {
   const dream_config &f = c->cfg;
-  int v = c->pf_v, q = c->pf_q, n = v + q, d = f.d_model, nc = q + k, CH = c->chunk;
+  int v = c->pf_v, q = c->pf_q, n = v + q, d = f.d_model, nc = q + k, CH = ROW_CHUNK;
   LAUNCH(c, k_select_visual, 1, 1024, 0, c->scores_all, (long long)imax(f.max_visual, 1), c->sd.tap + seq, c->tap_lo_eff,
          v, k, c->pf_vis_start, n, forced, kept, scores, c->ctx_pos, c->flags);
   // draft self-attention K/V of the compressed context, from the input embeddings
   const char *wkv = (const char *)c->dw.wqkv + (size_t)c->Hhd * d * c->esz;
-  const XMode m1 = xmode(c, 1);
+  const XMode m1 = xmode(c);
   for (int r0 = 0; r0 < nc && !c->three; r0 += CH) {
     int rows = imin(CH, nc - r0);
     LAUNCH(c, k_ctx_rows, (rows + 255) / 256, 256, 0, c->ctx_pos + r0, rows, 0, seq, c->rm[0], c->gather_idx, r0, 0);
@@ -1058,7 +1031,7 @@ static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *force
     c->cur_seq[0] = seq;
     for (int r0 = 0; r0 < nc; r0 += CH) {
       int rows = imin(CH, nc - r0);
-      const XMode xm = xmode(c, rows);
+      const XMode xm = xmode(c);
       LAUNCH(c, k_ctx_rows, (rows + 255) / 256, 256, 0, c->ctx_pos + r0, rows, 0, seq, c->rm[0], c->gather_idx, r0, f.xattn_full_memory);
       LAUNCH(c, (k_gather_rows<float>), rows, 256, 0, c->x0, c->gather_idx, c->x, d, (const int *)nullptr, 0, 0LL, XLayout{d, 0});
       draft_rows<T>(c, c->rm[0], rows, xm, 1, rows, imax(nc, nm), true, false, true, (const float2 *)nullptr);
@@ -1121,7 +1094,7 @@ static dream_status draft_impl(dream_ctx *c, const TreeBatch &tb, int B) {
   for (int p = 1; p <= ts.D; ++p) {
     int m = p == 1 ? ts.D + 2 : ts.beam[p - 1];
     int R = B * m;
-    const XMode xm = xmode(c, R);
+    const XMode xm = xmode(c);
     RowMeta &rm = c->rm[cur], &rn = c->rm[cur ^ 1];
     if (p == 1) LAUNCH(c, k_draft_begin, 1, 32, 0, tb, B, c->sd, c->dt, ts, rm, m, c->cap_rows, c->status);
     LAUNCH(c, (k_embed<T>), dim3(R, (d + 1023) / 1024), 256, 0, (const T *)c->embed, rm.tok, c->x, d, f.vocab, c->status,
@@ -1165,7 +1138,7 @@ template <typename T>
 static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *argmax, float *margin, float *logits) {
   const dream_config &f = c->cfg;
   int d = f.d_model, L = f.n_layers, R = B * c->T;
-  const XMode xm = xmode(c, R);
+  const XMode xm = xmode(c);
   RowMeta &rm = c->rm[0];
   int key_ub = 0;
   for (int b = 0; b < B; ++b) { key_ub = imax(key_ub, c->p_ub[tb.seq[b]] + c->T); c->cur_seq[b] = tb.seq[b]; }
@@ -1237,7 +1210,7 @@ static dream_status accept_impl(dream_ctx *c, const TreeBatch &tb, int B, const 
   LAUNCH(c, (k_compact_kv<T>), dim3(f.n_layers * 2, B), 256, 0, tb, c->sd, c->kv_pool, c->layer_stride, c->kv_stride, paged(c, 0));
   if (c->ent_sum) LAUNCH(c, k_accept_entropy, B, 64, 0, tb, c->T, f.n_layers, f.n_heads, ROW_CHUNK, c->sd, (const float *)c->row_ent, c->ent_sum);
   LAUNCH(c, k_accept_rows, 1, 32, 0, tb, B, c->T, D, c->sd, c->gather_idx, rm, c->cap_rows - c->ts.NI, c->status);
-  const XMode xm = xmode(c, R);
+  const XMode xm = xmode(c);
   LAUNCH(c, (k_gather_rows<T>), R, 256, 0, c->tapbuf, c->gather_idx, (T *)c->raw, d, (const int *)nullptr, 0, 0LL, xlay(xm, d));
   GemmOut g = gemm<T>(c, c->dw.xkv, c->raw, xm, R, c->kvN, d);
   LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, (const int *)nullptr, (const int *)nullptr, 0, flat(c, c->dmem));
@@ -1412,13 +1385,11 @@ extern "C" dream_status dream_debug_gemm(dream_ctx *c, const void *W, const floa
   else return fail(c, DREAM_E_ARG, "K exceeds the context's widest GEMM input");
   if (rows < 1 || rows > ROW_CHUNK) return fail(c, DREAM_E_ARG, "rows out of range");
   if (bf && (K % 64 || N % 8)) return fail(c, DREAM_E_ARG, "K must be a multiple of 64 and N of 8");
-  XMode xm = xmode(c, rows);
+  XMode xm = xmode(c);
   if (bf && !split) {                     // single bf16 row per token
-    if (rows > TC_ROWS_MAX) return fail(c, DREAM_E_ARG, "unsplit inputs take at most 128 rows");
+    if (rows > 128) return fail(c, DREAM_E_ARG, "unsplit inputs take at most 128 rows");
     xm = XMode{TC_X_PLAIN, 0};
   }
-  size_t need_out = (size_t)rows * N;
-  (void)need_out;
   LAUNCH(c, k_split_rows, rows, 256, 0, X, buf, K, xlay(xm, K), bf ? 1 : 0);
   GemmOut g = bf ? gemm<bf16>(c, W, buf, xm, rows, N, K) : gemm<float>(c, W, buf, xm, rows, N, K);
   LAUNCH(c, k_gemm_collect, dim3((N + 255) / 256, rows), 256, 0, g, out, N);
@@ -1475,7 +1446,7 @@ extern "C" dream_status dream_topk_lse_static(const float *logits, int32_t rows,
   TopkScratch ts;
   ts.pv = sc->pv; ts.pi = sc->pi; ts.pm = sc->pm; ts.pz = sc->pz; ts.counter = sc->counter;
   GemmOut g;                                   // a plain [rows][vocab] matrix: one slot, one chunk
-  g.base = logits; g.slot_stride = 0; g.chunk_stride = 0; g.chunk_shift = 30; g.ld = vocab; g.kb = 0; g.upc = 0;
+  g.base = logits; g.slot_stride = 0; g.ld = vocab; g.kb = 0; g.upc = 0;
   int nsplit = (vocab + TOPK_COLS - 1) / TOPK_COLS;
   k_topk_lse<TOPK_COLS / TOPK_THREADS><<<dim3(rows, nsplit), TOPK_THREADS, 0, stream>>>(g, vocab, ktop, nsplit, ts, top_val, top_id, lse, (float *)nullptr);
   e = cudaGetLastError();

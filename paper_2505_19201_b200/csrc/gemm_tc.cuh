@@ -1,28 +1,36 @@
-// Weight-streaming small-M GEMM for sm_100a:  out[t][c] = sum_k X[t][k] * W[c][k].
+// Weight-streaming GEMM on pairs of SMs for sm_100a:  out[t][c] = sum_k X[t][k] * W[c][k].
 //
-// The token count is tiny (<= 128 rows) and the weight matrix is large, so the kernel is bound
-// by streaming W from HBM once.  Design:
-//   * tokens are the MMA's M (the 128 TMEM lanes) and 256 weight rows are its N (TMEM columns):
-//     one tcgen05.mma (cta_group::1, kind::f16, bf16 x bf16 -> fp32) covers 128 x 256 x 16, so a
-//     32 KB weight panel costs four instructions and the issuing thread never limits the stream;
-//   * activations carry ~16 mantissa bits as two bf16 rows per token (high and low part):
-//       - up to 64 tokens: the rows are interleaved (row 2t = high, row 2t+1 = low), one A tile
-//         holds both, and the epilogue adds neighbouring TMEM lanes with one shuffle;
-//       - 65..128 tokens: high and low parts are two A tiles and two MMAs per k-step accumulate
-//         into the same TMEM columns;
-//   * two independent shared-memory rings fed by TMA (cp.async.bulk.tensor.2d, 128-byte swizzle,
-//     no multicast): one for W panels (256 rows x 64 k, evict-first) and one for X panels
-//     (128 rows x 64 k, served by L2, evict-last);
-//   * persistent stream-K: the (tile, panel) units are dealt out in equal contiguous ranges to one
-//     CTA per SM; a CTA that covers part of a tile writes a partial sum to its own slot and the
-//     consumer adds the slots in a fixed order;
+// A decode call has few tokens (1..256 rows), so this is a stream of W from HBM.  Design:
+//   * a cluster of two CTAs on neighbouring SMs works on one tile: 256 weight rows are the MMA's M
+//     (tcgen05.mma.cta_group::2, 128 rows and 128 TMEM lanes per CTA) and up to 256 token rows its N, of
+//     which each CTA stages one half.  Half as many workers as SMs also means half as many partial
+//     sums per tile for the consumers to add;
+//   * activations carry ~16 mantissa bits as two bf16 rows per token, kept as two planes (high parts,
+//     then low parts lo_rows further on):
+//       - up to 128 tokens (TC_X_CONCAT): both planes side by side are one N = 2 x tokens operand (the
+//         first CTA stages the high plane, the second the low plane), the epilogue adds column t and
+//         column tokens + t.  The weight panel is read from shared memory once;
+//       - more tokens (TC_X_TWO): two MMAs per k-step, high then low, into the same columns;
+//   * the tensor core adds into its accumulator with truncation, about half a unit in the last place
+//     per MMA and always towards zero, so chains of MMAs into one accumulator are kept short: CONCAT deals
+//     its k-steps out to as many accumulators as fit, TWO changes the accumulator every TC_CHAIN panels
+//     and the epilogue warps carry the sums in registers;
+//   * two shared-memory rings fed by TMA (cp.async.bulk.tensor.2d, 128-byte swizzle, no multicast), wp
+//     panels of 64 k per stage: W (128 rows, 16 KB a panel) and X.  W gets all the room X leaves: it is
+//     what a CTA can fetch before its grid dependency resolves.  One commit per stage frees both: the X
+//     producer waits on the W stage that went with the X stage it reuses;
+//   * persistent stream-K: the (tile, panel) units are dealt out in equal contiguous ranges to the
+//     pairs; a pair that covers part of a tile writes a partial sum to its own slot and the consumer
+//     adds the slots in a fixed order;
 //   * programmatic dependent launch: W never changes, so its ring fills before the grid
 //     dependency resolves; only the X producer and the epilogue wait for the previous kernel;
-//   * warp roles: 0 = W producer, 1 = MMA issuer and TMEM owner, 6 = X producer, 2..5 and 7..10 =
-//     epilogue (tcgen05.ld -> 128-bit stores; the first set drains accumulator columns 0..127, the
-//     second 128..255, loads software-pipelined, each chunk turned in shared memory so that a
-//     store covers whole 128-byte runs of a row); two TMEM accumulators alternate so that the
-//     epilogue of one segment overlaps the MMAs of the next;
+//   * the MMA issuer and the producers are whole warps that run their loops together and elect a lane for
+//     the asynchronous instructions.  Run by one lane of a diverged warp, their operands are moved to uniform
+//     registers one by one: measured 180..380 cycles of issue per MMA against 48..128 (its own time) so;
+//   * warp roles: 0 = W producer, 1 = MMA issuer (first CTA of the pair) and TMEM owner, 2 = X producer,
+//     4..11 = epilogue.  A TMEM lane is an output column c, so a warp's store of one token covers 128
+//     contiguous bytes without a transpose; two TMEM accumulators alternate so that the epilogue of
+//     one segment overlaps the MMAs of the next;
 //   * every mbarrier wait is bounded: on expiry the kernel raises the status word and leaves.
 #pragma once
 #include <cuda.h>
@@ -34,26 +42,29 @@
 
 #include "common.cuh"
 
-#define TC_BN 256               // weight rows per tile (MMA N)
+#define TC_BN 256               // weight rows per tile (MMA M, both CTAs)
 #define TC_BK 64                // k elements per panel (128 bytes: one swizzle row)
-#define TC_THREADS 352          // 11 warps, see the roles above
+#define TC_THREADS 384          // 12 warps, see the roles above
 #define TC_SPIN_LIMIT (1u << 24)
-#define TC_WPANEL (TC_BN * TC_BK * 2)
-#define TC_STG_LD 36            // floats per row of an epilogue staging tile (32 + padding)
-#define TC_STG_BYTES (8 * 16 * TC_STG_LD * 4)
-#define TC_XTILE (128 * TC_BK * 2)
+#define TC_WPANEL (128 * TC_BK * 2)          // one CTA's half of a weight panel
+#define TC_MAX_STAGES 12
+#define TC_CHAIN 8              // panels per accumulator in the two-MMA form (64 MMAs)
 
-enum { TC_X_PLAIN = 0, TC_X_INTERLEAVED = 1, TC_X_PLANAR = 2 };
+// How the token rows lie in the X buffer.  PLAIN: one bf16 row per token.  PLANAR: high parts, then
+// the low parts lo_rows rows further on.
+enum { TC_X_PLAIN = 0, TC_X_PLANAR = 1 };
+// How the MMA takes them (see above).
+enum { TC_X_ONE = 0, TC_X_CONCAT = 1, TC_X_TWO = 2 };
 
 struct TcParams {
   float *out;
   long long slot_stride;        // floats between partial-sum slots
-  int N, K, KB, n_tiles, total_units, upc;
+  int N, KB, total_units, upc;  // output columns, k panels, units = tiles x panels, units per pair
+  int tile_t, mma_n;            // tokens per tile, N of an MMA
+  int n_sub;                    // CONCAT / ONE: accumulators the k-steps of a segment are dealt out to (1, 2 or 4)
   int n_tok;                    // real token rows
-  int x_mode;                   // TC_X_*
-  int lo_rows;                  // TC_X_PLANAR: row of the first low part in the X tensor map
-  int m_tiles;                  // token tiles of 128 rows per launch: 1, or 2 (TC_X_PLANAR, 129..256 tokens)
-  int wp, w_stages, x_stages;   // panels per ring stage, ring depths
+  int lo_rows;                  // row of the first low part in the X tensor map
+  int wp, w_stages, x_stages;   // panels per stage, ring depths
   int *status;
 };
 
@@ -129,249 +140,300 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr) : "memory");
+}
 
+// One lane of a converged warp (always the same one).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+  return p != 0;
+}
+// The bounded wait made by a whole warp, which stays together whatever its lanes see.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+
+// ---- pairs of CTAs (cluster of two; the even rank leads)
+__device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r)); return r; }
+// Address of this shared-memory location in the CTA of the given rank.
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// A load into this CTA's shared memory that completes on the pair leader's barrier.
+__device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, uint32_t leader_bar, int x, int y, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(leader_bar), "r"(x), "r"(y), "l"(policy) : "memory");
+}
+__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
+}
+// Arrives on the barrier at this offset in both CTAs once the MMAs issued so far are done.
+__device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+               ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
 
 // ------------------------------------------------------------------------------------------ kernel
-// Dynamic shared memory (1024-byte aligned): W ring [w_stages][wp][32 KB], X ring
-// [x_stages][wp][16 KB, or 32 KB = high tile | low tile when planar], then the barriers.
-__global__ void __launch_bounds__(TC_THREADS, 1)
+// Dynamic shared memory (1024-byte aligned): W ring [w_stages][wp][16 KB], X ring [x_stages][wp][panel], barriers.
+template <int FORM>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  const bool planar = p.x_mode == TC_X_PLANAR;
-  const uint32_t wstage_bytes = (uint32_t)p.wp * TC_WPANEL;
-  const uint32_t xpanel_bytes = planar ? 2u * TC_XTILE * (uint32_t)p.m_tiles : (uint32_t)TC_XTILE;   // per token tile: high | low
-  const int n_buf = p.m_tiles == 2 ? 1 : 2;                // two token tiles fill all 512 TMEM columns: one accumulator set
-  const uint32_t xstage_bytes = (uint32_t)p.wp * xpanel_bytes;
+  // bytes of token rows one CTA stages per k panel
+  const uint32_t xtile_bytes = (uint32_t)(FORM == TC_X_CONCAT ? p.tile_t : p.mma_n >> 1) * 128u;
+  const uint32_t xpanel_bytes = FORM == TC_X_TWO ? 2u * xtile_bytes : xtile_bytes;
+  const uint32_t wstage_bytes = (uint32_t)p.wp * TC_WPANEL, xstage_bytes = (uint32_t)p.wp * xpanel_bytes;
   uint8_t *wring = smem, *xring = smem + (size_t)p.w_stages * wstage_bytes;
   uint64_t *bars = (uint64_t *)(xring + (size_t)p.x_stages * xstage_bytes);
-  uint64_t *full_w = bars, *empty_w = full_w + p.w_stages, *full_x = empty_w + p.w_stages, *empty_x = full_x + p.x_stages;
-  uint64_t *acc_full = empty_x + p.x_stages, *acc_empty = acc_full + 2;
+  uint64_t *full_w = bars, *empty_w = full_w + TC_MAX_STAGES, *full_x = empty_w + TC_MAX_STAGES;
+  uint64_t *acc_full = full_x + TC_MAX_STAGES, *acc_empty = acc_full + 2;
   uint32_t *tmem_base_p = (uint32_t *)(acc_empty + 2);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
-  float *stage_tiles = (float *)(bars + 64);               // 8 warps x [16][TC_STG_LD] floats, 512 bytes behind the barriers' start
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1;
   if (blockIdx.x == 0 && threadIdx.x == 0) trace_stamp(TR_none);     // CTA start, before any dependency
-  if (warp == 0) {      // one barrier pair per lane: the set-up is a few instructions deep instead of a loop
-    if (lane < p.w_stages) { mbar_init(full_w + lane, 1); mbar_init(empty_w + lane, 1); }
-    else if (lane >= 8 && lane < 8 + p.x_stages) { mbar_init(full_x + lane - 8, 1); mbar_init(empty_x + lane - 8, 1); }
-    else if (lane >= 16 && lane < 18) { mbar_init(acc_full + lane - 16, 1); mbar_init(acc_empty + lane - 16, 8); }
+  if (warp == 0) {      // a lane per barrier: the set-up is a few instructions deep instead of a loop
+    if (lane < TC_MAX_STAGES) { mbar_init(full_w + lane, 1); mbar_init(empty_w + lane, 1); }
+    else if (lane < 2 * TC_MAX_STAGES) mbar_init(full_x + lane - TC_MAX_STAGES, 1);
+    else if (lane < 2 * TC_MAX_STAGES + 2) { mbar_init(acc_full + lane - 2 * TC_MAX_STAGES, 1); mbar_init(acc_empty + lane - 2 * TC_MAX_STAGES, 16); }
     else if (lane == 31) *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) {      // all 512 TMEM columns (two accumulators of 256), allocated by one full warp
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_p)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  if (warp == 1) {      // all 512 TMEM columns (two accumulators of 256), allocated by one full warp of each CTA
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_p)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();                            // the peer's barriers are initialised
   tc_fence_after();
   pdl_trigger();
   const uint32_t tmem_base = *tmem_base_p;
-  const int u_begin = blockIdx.x * p.upc, u_end = min(u_begin + p.upc, p.total_units);
+  const int u_begin = pair * p.upc, u_end = min(u_begin + p.upc, p.total_units);
+  auto give_up = [&]() { if (lane == 0) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ W producer: weights are
     // constant, so nothing here waits for anything but ring space
-    if (lane == 0) {
-      const uint64_t pol = policy_evict_first();
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
-      int s = 0, u = u_begin;
-      uint32_t ph = 0;
-      bool wrapped = false;
-      while (u < u_end) {
-        int tile = u / p.KB, kb = u - tile * p.KB;
-        int np = min(p.wp, min(p.KB - kb, u_end - u));
-        if (wrapped && !mbar_wait(empty_w + s, ph ^ 1)) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; break; }
-        if (*abort_flag) break;
+    const uint64_t pol = policy_evict_first();
+    if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
+    __syncwarp();
+    const uint32_t bar0 = mapa(smem_u32(full_w), 0);
+    int s = 0;
+    uint32_t ph = 1;
+    for (int u = u_begin; u < u_end;) {
+      const int tile = u / p.KB, kb = u - tile * p.KB, np = min(p.wp, min(p.KB - kb, u_end - u));
+      const int y = tile * TC_BN + (int)rank * 128;
+      if (!mbar_wait_warp(empty_w + s, ph)) { give_up(); break; }
+      if (__any_sync(0xffffffffu, *abort_flag)) break;
+      if (elect_one()) {
+        if (rank == 0) mbar_expect_tx(full_w + s, 2u * (uint32_t)np * TC_WPANEL);
         uint8_t *dst = wring + (size_t)s * wstage_bytes;
-        mbar_expect_tx(full_w + s, (uint32_t)np * TC_WPANEL);
-        for (int q = 0; q < np; ++q) tma_load_2d(dst + (size_t)q * TC_WPANEL, &map_w, full_w + s, (kb + q) * TC_BK, tile * TC_BN, pol);
-        u += np;
-        if (++s == p.w_stages) { s = 0; ph ^= 1; wrapped = true; }
+        for (int i = 0; i < np; ++i) tma_load_2d_pair(dst + (size_t)i * TC_WPANEL, &map_w, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
       }
+      __syncwarp();
+      u += np;
+      if (++s == p.w_stages) { s = 0; ph ^= 1; }
     }
-  } else if (warp == 6) {
+  } else if (warp == 2) {
     // ------------------------------------------------------------------ X producer: waits until the
     // input exists (previous kernel), then feeds one X stage per W stage
-    if (lane == 0) {
-      const uint64_t pol = policy_evict_last();
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
-      pdl_wait();
-      if (blockIdx.x == 0) trace_stamp(TR_k_gemm_tc);
-      int s = 0, u = u_begin;
-      uint32_t ph = 0;
-      bool wrapped = false;
-      while (u < u_end) {
-        int tile = u / p.KB, kb = u - tile * p.KB;
-        int np = min(p.wp, min(p.KB - kb, u_end - u));
-        if (wrapped && !mbar_wait(empty_x + s, ph ^ 1)) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; break; }
-        if (*abort_flag) break;
-        uint8_t *dst = xring + (size_t)s * xstage_bytes;
-        mbar_expect_tx(full_x + s, (uint32_t)np * xpanel_bytes);
-        for (int q = 0; q < np; ++q) {
-          if (!planar) tma_load_2d(dst + (size_t)q * xpanel_bytes, &map_x, full_x + s, (kb + q) * TC_BK, 0, pol);
-          else
-            for (int mt = 0; mt < p.m_tiles; ++mt) {
-              uint8_t *dt = dst + (size_t)q * xpanel_bytes + (size_t)mt * 2 * TC_XTILE;
-              tma_load_2d(dt, &map_x, full_x + s, (kb + q) * TC_BK, mt * 128, pol);
-              tma_load_2d(dt + TC_XTILE, &map_x, full_x + s, (kb + q) * TC_BK, p.lo_rows + mt * 128, pol);
-            }
-        }
-        u += np;
-        if (++s == p.x_stages) { s = 0; ph ^= 1; wrapped = true; }
+    const uint64_t pol = policy_evict_last();
+    if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
+    __syncwarp();
+    pdl_wait();
+    if (blockIdx.x == 0 && lane == 0) trace_stamp(TR_k_gemm_tc);
+    __syncwarp();
+    const uint32_t bar0 = mapa(smem_u32(full_x), 0);
+    const int y = FORM == TC_X_CONCAT ? (int)rank * p.lo_rows : (int)rank * (p.mma_n >> 1);   // first token row this CTA stages
+    int s = 0, n_free = p.x_stages, ws = 0;      // unused X stages left; W stage that went with the X stage to reuse
+    uint32_t wph = 0;
+    for (int u = u_begin; u < u_end;) {
+      const int tile = u / p.KB, kb = u - tile * p.KB, np = min(p.wp, min(p.KB - kb, u_end - u));
+      if (n_free > 0) --n_free;
+      else {
+        if (!mbar_wait_warp(empty_w + ws, wph)) { give_up(); break; }
+        if (++ws == p.w_stages) { ws = 0; wph ^= 1; }
       }
+      if (__any_sync(0xffffffffu, *abort_flag)) break;
+      if (elect_one()) {
+        if (rank == 0) mbar_expect_tx(full_x + s, 2u * (uint32_t)np * xpanel_bytes);
+        for (int i = 0; i < np; ++i) {
+          uint8_t *dst = xring + (size_t)s * xstage_bytes + (size_t)i * xpanel_bytes;
+          tma_load_2d_pair(dst, &map_x, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
+          if (FORM == TC_X_TWO) tma_load_2d_pair(dst + xtile_bytes, &map_x, bar0 + 8u * s, (kb + i) * TC_BK, p.lo_rows + y, pol);
+        }
+      }
+      __syncwarp();
+      u += np;
+      if (++s == p.x_stages) s = 0;
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      // instruction descriptor: fp32 accumulate, bf16 A and B, both K-major, N = 256, M = 128
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TC_BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    // ------------------------------------------------------------------ MMA issuer (the pair's first CTA)
+    if (rank == 0) {
+      // instruction descriptor: fp32 accumulate, bf16 A and B, both K-major, M = 256
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.mma_n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+      const uint64_t wdesc = smem_desc(smem_u32(wring)), xdesc = smem_desc(smem_u32(xring));
+      const int w_stages = p.w_stages, x_stages = p.x_stages, wp = p.wp;
+      const uint32_t sub_n = (uint32_t)p.mma_n, sub_mask = (uint32_t)p.n_sub - 1u;
       int ws = 0, xs = 0, u = u_begin;
-      uint32_t wph = 0, xph = 0, seg = 0;
+      uint32_t wph = 0, xph = 0, fill = 0;                            // fill counts accumulator fills
       bool ok = true;
       while (u < u_end && ok) {
-        int tile = u / p.KB;
-        int seg_end = min((tile + 1) * p.KB, u_end);
-        const int buf = (int)seg % n_buf, use = (int)seg / n_buf;       // use: earlier segments in this accumulator set
-        if (use >= 1 && !mbar_wait(acc_empty + buf, (uint32_t)(use - 1) & 1u)) { ok = false; break; }
+        const int seg_end = min((u / p.KB + 1) * p.KB, u_end);
+        const int fill_end = FORM == TC_X_TWO ? min(seg_end, u + TC_CHAIN) : seg_end;
+        const uint32_t buf = fill & 1u, use = fill >> 1;              // use: earlier fills of this accumulator
+        ++fill;
+        if (!mbar_wait_warp(acc_empty + buf, (use & 1u) ^ 1u)) { ok = false; break; }
         tc_fence_after();
-        uint32_t d_addr = tmem_base + (uint32_t)buf * TC_BN;
-        uint32_t accum = 0u;
-        while (u < seg_end) {
-          int np = min(p.wp, seg_end - u);
-          if (!mbar_wait(full_w + ws, wph) || !mbar_wait(full_x + xs, xph)) { ok = false; break; }
+        const uint32_t d_addr = tmem_base + buf * 256u;
+        uint32_t begun = 0u;                                          // 0: the first MMA of an accumulator overwrites it
+        while (u < fill_end) {
+          const int np = min(wp, fill_end - u);
+          if (!__all_sync(0xffffffffu, mbar_wait(full_w + ws, wph) && mbar_wait(full_x + xs, xph))) { ok = false; break; }
           tc_fence_after();
-          uint32_t sw0 = smem_u32(wring + (size_t)ws * wstage_bytes), sx0 = smem_u32(xring + (size_t)xs * xstage_bytes);
-          for (int q = 0; q < np; ++q) {
-            uint64_t bd = smem_desc(sw0 + (uint32_t)q * TC_WPANEL);
-            for (int mt = 0; mt < p.m_tiles; ++mt) {
-              const uint32_t xa = sx0 + (uint32_t)q * xpanel_bytes + (uint32_t)mt * 2u * TC_XTILE;
-              const uint64_t ad = smem_desc(xa), al = smem_desc(xa + TC_XTILE);
-              const uint32_t dm = d_addr + (uint32_t)mt * TC_BN;
-              uint32_t acc = accum;
+          for (int i = 0; i < np; ++i) {
+            const uint64_t ad = wdesc + (uint64_t)((ws * wp + i) * (TC_WPANEL >> 4));
+            const uint64_t bd = xdesc + (uint64_t)((uint32_t)(xs * wp + i) * (xpanel_bytes >> 4));
+            if (elect_one()) {
 #pragma unroll
               for (int k = 0; k < TC_BK / 16; ++k) {
-                mma_bf16(dm, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, acc);
-                acc = 1u;
-                if (planar) mma_bf16(dm, al + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, 1u);
+                if (FORM == TC_X_TWO) {
+                  mma_bf16_pair(d_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, k ? 1u : begun);
+                  mma_bf16_pair(d_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)((xtile_bytes >> 4) + k * 2), idesc, 1u);
+                } else {
+                  const uint32_t sub = (uint32_t)k & sub_mask;
+                  mma_bf16_pair(d_addr + sub * sub_n, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, (uint32_t)k > sub_mask ? 1u : begun);
+                }
               }
             }
-            accum = 1u;
+            begun = 1u;
           }
-          mma_commit(empty_x + xs);           // frees both stages once these MMAs have read them
-          mma_commit(empty_w + ws);
+          if (elect_one()) mma_commit_pair(empty_w + ws);             // frees both stages in both CTAs once these MMAs have read them
           u += np;
-          if (++ws == p.w_stages) { ws = 0; wph ^= 1; }
-          if (++xs == p.x_stages) { xs = 0; xph ^= 1; }
+          if (++ws == w_stages) { ws = 0; wph ^= 1; }
+          if (++xs == x_stages) { xs = 0; xph ^= 1; }
         }
-        if (!ok) break;
-        mma_commit(acc_full + buf);           // accumulator complete
-        ++seg;
+        if (ok && elect_one()) mma_commit_pair(acc_full + buf);       // accumulator complete
+        __syncwarp();
       }
-      if (!ok) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
+      if (!ok) give_up();
     }
-  } else {
-    // ------------------------------------------------------------------ warps 2..5, 7..10: epilogue
-    // of the CTA's segments (partial sums to this CTA's slot)
-    const int q = warp & 3;                   // TMEM lane quarter this warp may read
-    const int half = warp >= 7 ? 1 : 0;       // which 128 accumulator columns this warp drains
-    const int pwarp = warp < 7 ? warp - 2 : warp - 3;                   // 0..7 among these warps
-    float *stg = stage_tiles + pwarp * (16 * TC_STG_LD);                // this warp's staging tile
+  } else if (warp >= 4) {
+    // ------------------------------------------------------------------ epilogue: this CTA's 128 output
+    // columns of every segment, one per TMEM lane; warps 4..7 and 8..11 take token groups in turn
+    const int q = warp & 3, half = warp >= 8 ? 1 : 0;       // TMEM lane quarter this warp may read; its token groups
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    const uint32_t done_bar = mapa(smem_u32(acc_empty), 0);
     pdl_wait();                               // the output buffer belongs to earlier kernels
-    const bool inter = p.x_mode == TC_X_INTERLEAVED;
-    const int part = inter ? lane & 1 : 0;
-    uint32_t seg = 0;
+    uint32_t fill = 0;
     int u = u_begin;
-    while (u < u_end) {
-      int tile = u / p.KB;
-      int seg_end = min((tile + 1) * p.KB, u_end);
-      const int buf = (int)seg % n_buf, use = (int)seg / n_buf;
-      int ok = 1;
-      if (lane == 0) ok = mbar_wait(acc_full + buf, (uint32_t)use & 1u) ? 1 : 0;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok || *abort_flag) { if (lane == 0) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } break; }
+    bool ok = true;
+    auto wait_full = [&](uint32_t buf, uint32_t use) {
+      int w = 1;
+      if (lane == 0) w = mbar_wait(acc_full + buf, use & 1u) ? 1 : 0;
+      w = __shfl_sync(0xffffffffu, w, 0);
+      if (!w || __any_sync(0xffffffffu, *abort_flag)) { give_up(); ok = false; }
       tc_fence_after();
-      int first_cta = (tile * p.KB) / p.upc;
-      int slot = (int)blockIdx.x - first_cta;
-      float *dst0 = p.out + (long long)slot * p.slot_stride + tile * TC_BN;       // row 0 of this CTA's slot, first column of the tile
-      for (int mt = 0; mt < p.m_tiles; ++mt) {      // token tiles: rows mt * 128 .. of the output, accumulator columns mt * 256 ..
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf + mt) * TC_BN;
-      // four chunks of 32 columns; the TMEM load of chunk i+1 is in flight while chunk i is stored.
-      // A lane holds values of one row, but a store instruction is cheapest when the lanes of a
-      // warp cover whole 128-byte runs of a row: the chunk goes through a [16][32] tile in shared
-      // memory (rows padded to 36 floats) and leaves as 4 stores of 4 rows x 128 bytes.
-      uint32_t ra[32], rb[32];
-      tmem_ld32(taddr + (uint32_t)half * 128u, ra);
+    };
+    while (u < u_end && ok) {
+      const int tile = u / p.KB, seg_end = min((tile + 1) * p.KB, u_end);
+      const int slot = pair - (tile * p.KB) / p.upc, nt = p.n_tok;
+      const int c = tile * TC_BN + (int)rank * 128 + q * 32 + lane;
+      float *dst = p.out + (long long)slot * p.slot_stride + c;
+      if (FORM == TC_X_TWO) {
+        // token groups of 16: half 0 takes groups 0, 2, .., half 1 groups 1, 3, ..
+        float run[128];
 #pragma unroll
-      for (int ci = 0; ci < 4; ++ci) {
-        const int col0 = half * 128 + ci * 32;
-        uint32_t (&r)[32] = (ci & 1) ? rb : ra;
-        tmem_ld_wait();
-        if (ci + 1 < 4) tmem_ld32(taddr + (uint32_t)(col0 + 32), (ci & 1) ? ra : rb);
-        const int c4 = (lane & 7) * 4;
-        const bool col_ok = tile * TC_BN + col0 + c4 < p.N;
-        if (inter) {
-          // lanes 2t and 2t+1 hold the products of token t's high and low parts.  The even lane
-          // keeps columns 0..15 of the chunk and the odd lane 16..31: each sends the partner
-          // the 16 values it needs and adds what it receives to its own.
-          float4 *srow = reinterpret_cast<float4 *>(stg + (lane >> 1) * TC_STG_LD + part * 16);
+        for (int j = 0; j < 128; ++j) run[j] = 0.f;
+        for (; u < seg_end; u += min(TC_CHAIN, seg_end - u)) {
+          const uint32_t buf = fill & 1u;
+          wait_full(buf, fill >> 1);
+          ++fill;
+          if (!ok) break;
+          const uint32_t taddr = lane_addr + buf * 256u + (uint32_t)(half * 16);
 #pragma unroll
-          for (int j4 = 0; j4 < 4; ++j4) {
-            float v[4];
+          for (int g = 0; g < 8; ++g)
+            if ((2 * g + half) * 16 < nt) {
+              uint32_t r[16];
+              tmem_ld16(taddr + (uint32_t)(g * 32), r);
+              tmem_ld_wait();
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int j = j4 * 4 + e;
-              float send = __uint_as_float(part ? r[j] : r[16 + j]);
-              float mine = __uint_as_float(part ? r[16 + j] : r[j]);
-              v[e] = mine + __shfl_xor_sync(0xffffffffu, send, 1);
+              for (int j = 0; j < 16; ++j) run[g * 16 + j] += __uint_as_float(r[j]);
             }
-            srow[j4] = make_float4(v[0], v[1], v[2], v[3]);
-          }
+          tc_fence_before();
           __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(done_bar + 8u * buf);
+        }
+        if (ok && c < p.N) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int tl = i * 4 + (lane >> 3), tok = q * 16 + tl;
-            float4 val = *reinterpret_cast<const float4 *>(stg + tl * TC_STG_LD + c4);
-            if (tok < p.n_tok && col_ok) *reinterpret_cast<float4 *>(dst0 + (long long)tok * p.N + col0 + c4) = val;
+          for (int g = 0; g < 8; ++g)
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int t = (2 * g + half) * 16 + j;
+              if (t < nt) dst[(long long)t * p.N] = run[g * 16 + j];
+            }
+        }
+      } else {
+        const uint32_t buf = fill & 1u;
+        wait_full(buf, fill >> 1);
+        ++fill;
+        if (!ok) break;
+        const uint32_t taddr = lane_addr + buf * 256u;
+        // the parts of a sum: accumulators, and within each (CONCAT) the high and the low plane's columns
+        const int n_part = p.n_sub * (FORM == TC_X_CONCAT ? 2 : 1), part_n = FORM == TC_X_CONCAT ? p.tile_t : p.mma_n;
+#pragma unroll 1
+        for (int t0 = half * 32; t0 < nt; t0 += 64) {
+          float v[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = 0.f;
+#pragma unroll 1
+          for (int i = 0; i < n_part; ++i) {
+            uint32_t r[32];
+            tmem_ld32(taddr + (uint32_t)(i * part_n + t0), r);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
           }
-          __syncwarp();
-        } else {
-          // one row per lane: two halves of 16 rows through the same tile
+          if (c < p.N) {
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if ((lane >> 4) == h) {
-              float4 *srow = reinterpret_cast<float4 *>(stg + (lane & 15) * TC_STG_LD);
-#pragma unroll
-              for (int j4 = 0; j4 < 8; ++j4)
-                srow[j4] = make_float4(__uint_as_float(r[j4 * 4]), __uint_as_float(r[j4 * 4 + 1]), __uint_as_float(r[j4 * 4 + 2]),
-                                       __uint_as_float(r[j4 * 4 + 3]));
-            }
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int tl = i * 4 + (lane >> 3), tok = mt * 128 + q * 32 + h * 16 + tl;
-              float4 val = *reinterpret_cast<const float4 *>(stg + tl * TC_STG_LD + c4);
-              if (tok < p.n_tok && col_ok) *reinterpret_cast<float4 *>(dst0 + (long long)tok * p.N + col0 + c4) = val;
-            }
-            __syncwarp();
+            for (int j = 0; j < 32; ++j)
+              if (t0 + j < nt) dst[(long long)(t0 + j) * p.N] = v[j];
           }
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(done_bar + 8u * buf);
+        u = seg_end;
       }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty + buf);
-      u = seg_end;
-      ++seg;
     }
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();                          // neither CTA leaves while its peer may still signal it or read its operands
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
 }
 
@@ -396,16 +458,17 @@ static inline const char *gemm_tc_plan_init(GemmTcPlan *pl, int *status, int use
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&pl->n_sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&pl->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_gemm_tc<TC_X_ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_gemm_tc<TC_X_CONCAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_gemm_tc<TC_X_TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess)
     return "cannot raise the dynamic shared memory limit";
   pl->status = status;
   pl->use_pdl = use_pdl;
   return nullptr;
 }
 
-// Largest token count one launch takes: 64 with interleaved high/low rows, 128 otherwise.
-#define TC_ROWS_SPLIT_1MMA 64
-#define TC_ROWS_MAX 128
+// Most token rows of one launch.
+#define TC_ROWS_MAX 256
 
 static inline bool gemm_tc_supported(int N, int K) {
   return K % TC_BK == 0 && K >= TC_BK && N % 8 == 0 && N >= 8;
@@ -433,67 +496,69 @@ static inline bool tc_map(GemmTcPlan *pl, const void *ptr, int rows, int K, int 
   return true;
 }
 
+// Units of (256-row tile, k panel) a pair takes.
+static inline int gemm_tc_units_per_pair(int n_sms, long long total) {
+  long long pairs = n_sms / 2 > 0 ? n_sms / 2 : 1;
+  if (pairs > total) pairs = total;
+  return (int)((total + pairs - 1) / pairs);
+}
+
 // Floats one launch may write when its slots hold slot_rows x N: a tile is shared by at most
-// ceil(KB / upc) + 1 CTAs.  n_sms <= 0 gives the bound that holds for any SM count.
+// ceil(KB / upc) + 1 pairs.
 static inline long long gemm_tc_out_floats(int n_sms, int slot_rows, int N, int K) {
   int KB = K / TC_BK, n_tiles = (N + TC_BN - 1) / TC_BN;
-  long long total = (long long)n_tiles * KB;
-  long long slots;
-  if (n_sms <= 0) slots = KB + 1;
-  else {
-    long long grid = n_sms < total ? n_sms : total;
-    long long upc = (total + grid - 1) / grid;
-    slots = (KB + upc - 1) / upc + 1;
-  }
+  long long upc = gemm_tc_units_per_pair(n_sms, (long long)n_tiles * KB);
+  long long slots = (KB + upc - 1) / upc + 1;
   return slots * (long long)slot_rows * N;
 }
 
-// Enqueue one GEMM.
-//   X: bf16, row-major, K columns.  TC_X_PLAIN: row t = token t.  TC_X_INTERLEAVED: row 2t = high
-//   part of token t, row 2t+1 = low part.  TC_X_PLANAR: row t = high part, row lo_rows + t = low part.
-//   rows <= 64 when interleaved, <= 128 otherwise, except that TC_X_PLANAR with lo_rows >= 256 takes
-//   up to 256 rows as two token tiles that share every weight panel (the weights stream once;
-//   both accumulators fill the TMEM, so epilogues no longer overlap the next segment's MMAs).
-//   slot_rows >= rows: rows of a partial-sum slot.
+// Enqueue one GEMM of up to TC_ROWS_MAX token rows.
+//   X: bf16, row-major, K columns.  TC_X_PLAIN: row t = token t.  TC_X_PLANAR: row t = high part, row
+//   lo_rows + t = low part.
 // *g receives the descriptor consumers read the result through.  Returns false if the launch could
 // not be made.
 static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const void *W, const void *X, int x_mode, int lo_rows,
-                                  int rows, int slot_rows, int N, int K, float *out, long long out_floats, GemmOut *g) {
+                                  int rows, int N, int K, float *out, long long out_floats, GemmOut *g) {
+  if (rows < 1 || rows > TC_ROWS_MAX) return false;
   TcParams p;
-  p.n_tok = rows; p.x_mode = x_mode; p.lo_rows = lo_rows;
-  p.m_tiles = rows > TC_ROWS_MAX ? 2 : 1;
-  if (rows > 2 * TC_ROWS_MAX || (p.m_tiles == 2 && (x_mode != TC_X_PLANAR || lo_rows < 2 * TC_ROWS_MAX))) return false;
-  p.N = N; p.K = K; p.KB = K / TC_BK;
-  p.n_tiles = (N + TC_BN - 1) / TC_BN;
-  p.total_units = p.n_tiles * p.KB;
-  // W stages of two panels (256-byte runs per weight row) unless the X ring needs the room
-  p.wp = (x_mode == TC_X_PLANAR || p.KB < 2) ? 1 : 2;
-  int grid = pl->n_sms < p.total_units ? pl->n_sms : p.total_units;
-  p.upc = (p.total_units + grid - 1) / grid;
-  if (p.KB % p.wp == 0) p.upc = (p.upc + p.wp - 1) / p.wp * p.wp;       // CTA ranges cover whole ring stages
-  grid = (p.total_units + p.upc - 1) / p.upc;
+  p.n_tok = rows; p.lo_rows = lo_rows;
+  p.N = N; p.KB = K / TC_BK;
+  p.total_units = (N + TC_BN - 1) / TC_BN * p.KB;
+  // N of an MMA is a multiple of 16 and each CTA stages half of it (8-row groups)
+  int form;
+  if (x_mode == TC_X_PLAIN) { form = TC_X_ONE; p.tile_t = p.mma_n = (rows + 15) & ~15; }
+  else if (rows <= 128) { form = TC_X_CONCAT; p.tile_t = (rows + 7) & ~7; p.mma_n = 2 * p.tile_t; }
+  else { form = TC_X_TWO; p.tile_t = p.mma_n = (rows + 15) & ~15; }
+  p.n_sub = p.mma_n <= 64 ? 4 : p.mma_n <= 128 ? 2 : 1;
+  p.upc = gemm_tc_units_per_pair(pl->n_sms, p.total_units);
+  const int n_pairs = (p.total_units + p.upc - 1) / p.upc;
   p.out = out;
-  p.slot_stride = (long long)slot_rows * N;
-  long long max_slots = (p.KB + p.upc - 1) / p.upc + 1;
-  if (p.slot_stride * max_slots > out_floats) return false;
-  int x_rows = x_mode == TC_X_INTERLEAVED ? 2 * rows : (x_mode == TC_X_PLANAR ? lo_rows + rows : rows);
+  p.slot_stride = (long long)rows * N;
+  if (gemm_tc_out_floats(pl->n_sms, rows, N, K) > out_floats) return false;
   CUtensorMap mw, mx;
-  if (!tc_map(pl, W, N, K, TC_BN, &mw) || !tc_map(pl, X, x_rows, K, 128, &mx)) return false;
-  g->base = p.out; g->slot_stride = p.slot_stride; g->chunk_stride = 0; g->chunk_shift = 30; g->ld = N; g->kb = p.KB; g->upc = p.upc;
-  int xstage = p.wp * (x_mode == TC_X_PLANAR ? 2 * TC_XTILE * p.m_tiles : TC_XTILE);
-  p.x_stages = 2;
-  int budget = pl->max_smem - 2048 - TC_STG_BYTES - p.x_stages * xstage;
-  p.w_stages = budget / (p.wp * TC_WPANEL);
-  if (p.w_stages > 8) p.w_stages = 8;
-  if (p.w_stages < 2) return false;
-  if (budget - p.w_stages * p.wp * TC_WPANEL >= xstage) p.x_stages = 3;   // room left over: a third X stage
+  const int x_rows = x_mode == TC_X_PLANAR ? lo_rows + rows : rows;
+  const int x_box = form == TC_X_CONCAT ? p.tile_t : p.mma_n / 2;
+  if (!tc_map(pl, W, N, K, 128, &mw) || !tc_map(pl, X, x_rows, K, x_box, &mx)) return false;
+  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = N; g->kb = p.KB; g->upc = p.upc;
+  // Stages of two panels halve the waits and commits per panel (61 rows, 12288 x 4096: 22.2 -> 20.9 us) as
+  // long as five fit; where a token panel is larger than a weight panel (244 rows: 38.3 against 39.4 us) the
+  // rings are deeper with one
+  const int xpanel = x_box * 128 * (form == TC_X_TWO ? 2 : 1);
+  p.wp = xpanel <= TC_WPANEL / 2 ? 2 : 1;
+  const int xstage = p.wp * xpanel, wstage = p.wp * TC_WPANEL;
+  const int room = pl->max_smem - 2048;
+  p.x_stages = xpanel < TC_WPANEL ? 6 / p.wp : xpanel == TC_WPANEL ? 4 : room / (xstage + wstage);
+  p.w_stages = (room - p.x_stages * xstage) / wstage;
+  if (p.w_stages > TC_MAX_STAGES) p.w_stages = TC_MAX_STAGES;
+  if (p.w_stages < 2 || p.x_stages < 2) return false;
   p.status = pl->status;
-  size_t smem = (size_t)p.w_stages * p.wp * TC_WPANEL + (size_t)p.x_stages * xstage + 1024 + 512 + TC_STG_BYTES;
+  size_t smem = (size_t)p.w_stages * wstage + (size_t)p.x_stages * xstage + 2048;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.gridDim = dim3(2 * n_pairs); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = pl->use_pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_gemm_tc, mw, mx, p) == cudaSuccess;
+  auto *kernel = form == TC_X_CONCAT ? k_gemm_tc<TC_X_CONCAT> : form == TC_X_TWO ? k_gemm_tc<TC_X_TWO> : k_gemm_tc<TC_X_ONE>;
+  return cudaLaunchKernelEx(&cfg, kernel, mw, mx, p) == cudaSuccess;
 }
