@@ -418,7 +418,7 @@ static XLayout xlay(XMode m, long long width) {
 template <typename T>
 static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int rows, int N, int K) {
   GemmOut g;
-  if (sizeof(T) == 2) {
+  if constexpr (sizeof(T) == 2) {
     bool timed = c->prof_on && 2 * (c->prof_n + 1) <= (int)c->prof_ev.size();
     if (timed) cudaEventRecord(c->prof_ev[2 * c->prof_n], c->stream);
     if (!gemm_tc_launch(&c->tc, c->stream, W, X, m.mode, m.lo_rows, rows, N, K, c->gout, (long long)c->gout_floats, &g))
@@ -426,12 +426,20 @@ static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int row
     if (timed) { cudaEventRecord(c->prof_ev[2 * c->prof_n + 1], c->stream); c->prof_n++; c->prof_bytes += 2.0 * N * K; }
     c->launches++;
     c->tc_launches++;
-    return g;
+  } else {
+    c->simt_launches++;
+    // as many k-slices as there are steps, up to the warps of a block: the chain of dependent loads is then
+    // one step long up to K = 1024; four rows per warp only where the rows are that few
+    int ks = 1;
+    while (ks < SG_WARPS && ks * SG_STEP < K) ks *= 2;
+    const bool vec = K % 4 == 0 && ((uintptr_t)W & 15) == 0 && ((uintptr_t)X & 15) == 0;
+    const int tr = rows <= 4 ? 4 : 8;
+    auto *kernel = tr == 4 ? (vec ? k_gemm_simt<4, true> : k_gemm_simt<4, false>) : (vec ? k_gemm_simt<8, true> : k_gemm_simt<8, false>);
+    const int cols = SG_TC * (SG_WARPS / ks);
+    launch_k(c, "k_gemm_simt", kernel, dim3((N + cols - 1) / cols, (rows + tr - 1) / tr), dim3(SG_WARPS * 32), 0,
+             (const float *)X, (const float *)W, c->gout, rows, N, K, N, ks);
+    g.base = c->gout; g.slot_stride = 0; g.ld = N; g.kb = 0; g.upc = 0;
   }
-  c->simt_launches++;
-  dim3 grid((N + SG_BN - 1) / SG_BN, (rows + SG_BM - 1) / SG_BM);
-  LAUNCH(c, (k_gemm_simt<T>), grid, 256, 0, (const T *)X, (const T *)W, c->gout, rows, N, K, N);
-  g.base = c->gout; g.slot_stride = 0; g.ld = N; g.kb = 0; g.upc = 0;
   return g;
 }
 
@@ -670,7 +678,7 @@ static long long prefill_chunk_stride(const dream_ctx *c) {
 template <typename T, int HD> struct AttnLaunch {
   // The output rows are laid out per prefill chunk of ROW_CHUNK rows (the O projection's input).
   static void prefill(dream_ctx *c, int layer, int seq, int n) {
-    if (sizeof(T) == 2) {
+    if constexpr (sizeof(T) == 2) {
       // causal attention of the n prompt rows on the tensor cores: one CTA per (KV head, 64 entries)
       // walks all keys up to its last row; row log-sum-exp and entropy (Eq. 2) come out of the same pass
       AttnTcArgs a = {};
@@ -680,18 +688,17 @@ template <typename T, int HD> struct AttnLaunch {
       a.lse = c->lse_pre; a.ent = c->ent_pre;
       c->cur_seq[0] = seq;
       tc(c, a, layer, nullptr, 1, n, 0, nullptr);
-      return;
+    } else {
+      dim3 grid((n + ATT_WARPS * ATT_PF_ROWS - 1) / (ATT_WARPS * ATT_PF_ROWS), c->cfg.n_heads);
+      LAUNCH(c, (k_attn_prefill<HD>), grid, ATT_WARPS * 32, 0, (const float *)c->qbuf, paged(c, layer), seq, n, c->cfg.n_heads,
+             1.f / sqrtf((float)HD), (float *)c->attn_out, c->lse_pre, c->ent_pre);
     }
-    dim3 grid((n + ATT_WARPS * ATT_PF_ROWS - 1) / (ATT_WARPS * ATT_PF_ROWS), c->cfg.n_heads);
-    const XMode m = xmode(c);
-    LAUNCH(c, (k_attn_prefill<T, HD>), grid, ATT_WARPS * 32, 0, c->qbuf, paged(c, layer), seq, n, c->cfg.n_heads,
-           1.f / sqrtf((float)HD), (T *)c->attn_out, xlay(m, c->Hhd), ROW_CHUNK, prefill_chunk_stride(c), c->lse_pre, c->ent_pre);
   }
   static void colsum(dream_ctx *c, int layer, int seq, int n, int vis_start, int v, float *score) {
     if (v == 0) return;
     // the per-head sums land in the entropy buffer, which is idle between this layer's entropy mean
     // and the next layer's attention ([H][n] floats, v <= n)
-    if (sizeof(T) == 2) {
+    if constexpr (sizeof(T) == 2) {
       // tensor cores: 128 keys of one head per CTA, the query rows stream past (colsum_tc.cuh)
       const dream_config &f = c->cfg;
       ColsumTcArgs a = {};
@@ -722,11 +729,10 @@ template <typename T, int HD> struct AttnLaunch {
       cudaError_t e = colsum_tc_launch<HD>(c->stream, c->use_pdl, mq, mk, a, n_tiles);
       if (e != cudaSuccess && c->launch_err == cudaSuccess) { c->launch_err = e; c->launch_err_name = "k_colsum_tc"; }
       c->launches++;
-      LAUNCH(c, k_colsum_heads, (v + 255) / 256, 256, 0, (const float *)c->ent_pre, c->cfg.n_heads, v, score);
-      return;
+    } else {
+      LAUNCH(c, (k_colsum<HD>), dim3((v + ATT_WARPS - 1) / ATT_WARPS, c->cfg.n_heads), ATT_WARPS * 32, 0, (const float *)c->qbuf, paged(c, layer), seq, n,
+             c->cfg.n_heads, 1.f / sqrtf((float)HD), c->lse_pre, vis_start, v, c->cfg.score_include_self, c->ent_pre);
     }
-    LAUNCH(c, (k_colsum<T, HD>), dim3((v + ATT_WARPS - 1) / ATT_WARPS, c->cfg.n_heads), ATT_WARPS * 32, 0, c->qbuf, paged(c, layer), seq, n,
-           c->cfg.n_heads, 1.f / sqrtf((float)HD), c->lse_pre, vis_start, v, c->cfg.score_include_self, c->ent_pre);
     LAUNCH(c, k_colsum_heads, (v + 255) / 256, 256, 0, (const float *)c->ent_pre, c->cfg.n_heads, v, score);
   }
   // The tcgen05 attention (bf16 configurations): split-K plan, tensor maps, launch, merge of the chunks.
@@ -792,39 +798,34 @@ template <typename T, int HD> struct AttnLaunch {
     }
   }
   static void tree(dream_ctx *c, int layer, int R, XMode m, int B, int key_ub) {
-    if (sizeof(T) == 2) {
+    float *ent = c->row_ent ? c->row_ent + (size_t)layer * ROW_CHUNK * c->cfg.n_heads : nullptr;
+    if constexpr (sizeof(T) == 2) {
       AttnTcArgs a = {};
       a.mode = AT_VERIFY;
       a.next_w.ptr = (const char *)c->wo[layer]; a.next_w.bytes = (unsigned long long)c->cfg.d_model * c->Hhd * 2;
       a.prefix_len = c->sd.P; a.mask = c->vmask; a.tail_len = c->T; a.lay = xlay(m, c->Hhd);
-      if (c->row_ent) { a.row_ent = c->row_ent + (size_t)layer * ROW_CHUNK * c->cfg.n_heads; a.part_u = c->am_part_u; }
+      if (ent) { a.row_ent = ent; a.part_u = c->am_part_u; }
       tc(c, a, layer, nullptr, B, c->T, key_ub, nullptr);
-      return;
+    } else {
+      auto *kernel = ent ? k_attn_tree<HD, true> : k_attn_tree<HD, false>;
+      launch_k(c, "k_attn_tree", kernel, dim3(R, c->cfg.n_heads), dim3(ATT_WARPS * 32), 0, (const float *)c->qbuf, paged(c, layer), c->rm[0].seq,
+               c->sd.P, c->vmask, c->T, c->cfg.n_heads, 1.f / sqrtf((float)HD), (float *)c->attn_out, ent);
     }
-    dim3 grid((R + ATT_WARPS - 1) / ATT_WARPS, c->cfg.n_heads);
-    if (c->row_ent)
-      LAUNCH(c, (k_attn_tree<T, HD, true>), grid, ATT_WARPS * 32, 0, c->qbuf, paged(c, layer), c->rm[0].seq, c->rm[0].in,
-             c->sd.P, c->vmask, R, c->T, c->cfg.n_heads, 1.f / sqrtf((float)HD), (T *)c->attn_out, xlay(m, c->Hhd),
-             c->row_ent + (size_t)layer * ROW_CHUNK * c->cfg.n_heads);
-    else
-      LAUNCH(c, (k_attn_tree<T, HD, false>), grid, ATT_WARPS * 32, 0, c->qbuf, paged(c, layer), c->rm[0].seq, c->rm[0].in,
-             c->sd.P, c->vmask, R, c->T, c->cfg.n_heads, 1.f / sqrtf((float)HD), (T *)c->attn_out, xlay(m, c->Hhd), (float *)nullptr);
   }
   // row_vis: null, or per row the number of leading cache rows a permanent row sees (RowMeta::vis_d / vis_m).
   // tail: false when no row of the launch reads the tree region (the draft's run over the context).
   static void draft(dream_ctx *c, const RowMeta &rm, float *cache, const int *nperm, int strict, int R, XMode m, int B,
                     int rows_per_seq, int key_ub, const int *row_vis = nullptr, bool tail = true) {
-    if (sizeof(T) == 2) {
+    if constexpr (sizeof(T) == 2) {
       AttnTcArgs a = {};
       a.mode = AT_DRAFT;
       a.prefix_len = nperm; a.anc = c->dt.in_anc; a.anc_stride = c->ts.NI; a.strict = strict; a.tail_len = tail ? c->ts.NI : 0;
       a.lay = xlay(m, c->Hhd);
       tc(c, a, 0, cache, B, rows_per_seq, key_ub, rm.in, row_vis);
-      return;
+    } else {
+      LAUNCH(c, (k_attn_draft<HD>), dim3(R, c->cfg.n_heads), ATT_WARPS * 32, 0, (const float *)c->qbuf, flat(c, cache), rm.seq, rm.in, row_vis, nperm,
+             c->dt.in_anc, c->ts.NI, strict, c->cfg.n_heads, 1.f / sqrtf((float)HD), (float *)c->attn_out);
     }
-    dim3 grid((R + ATT_WARPS - 1) / ATT_WARPS, c->cfg.n_heads);
-    LAUNCH(c, (k_attn_draft<T, HD>), grid, ATT_WARPS * 32, 0, c->qbuf, flat(c, cache), rm.seq, rm.in, row_vis, nperm,
-           c->dt.in_anc, c->ts.NI, strict, R, c->cfg.n_heads, 1.f / sqrtf((float)HD), (T *)c->attn_out, xlay(m, c->Hhd));
   }
 };
 
