@@ -142,7 +142,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   uint32_t *tmem_base_p = (uint32_t *)(o_done + 1);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   const int chunk = blockIdx.x, kvh = blockIdx.y / a.n_rt, rt = blockIdx.y - kvh * a.n_rt, slot = blockIdx.z;
   const int seq = a.slot_seq[slot];
   if (warp == 0) {      // a lane per ring stage: the set-up is a few instructions deep instead of a loop
@@ -184,42 +184,47 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   const int b0 = chunk * a.blocks_per_chunk, b1 = min(nb, b0 + a.blocks_per_chunk);
   const int n_blk = max(0, b1 - b0);
 
-  // K and V of the chunk's block `it` into ring stage it % GROUP (producer thread only)
+  // K and V of the chunk's block `it` into ring stage it % GROUP (the whole producer warp)
   const uint64_t pol_kv = policy_evict_first();
   auto issue_kv = [&](int it) {
     const int st = it % GROUP, j0 = (b0 + it) * AT_KBLK;
     // K: [plane][panel][stage][64 keys], so the blocks of a group form one operand of 64 x blocks keys
     uint8_t *kd = k_s + st * AT_KVTILE, *vd = v_s + st * Sh::KV_STAGE;
     constexpr int KSTEP = GROUP * AT_KVTILE;                 // bytes between consecutive (plane, panel) of K
-    mbar_expect_tx(k_full + st, (uint32_t)Sh::KV_STAGE);
-    mbar_expect_tx(v_full + st, (uint32_t)Sh::KV_STAGE);
+    if (elect_one()) { mbar_expect_tx(k_full + st, (uint32_t)Sh::KV_STAGE); mbar_expect_tx(v_full + st, (uint32_t)Sh::KV_STAGE); }
     if (FLAT) {
       // rows of the map: (sequence, K | V, KV head, key); the second coordinate selects the plane
       const long long rk = (((long long)seq * 2 + 0) * a.hkv + kvh) * a.flat_rows_per_head + j0;
       const long long rv = (((long long)seq * 2 + 1) * a.hkv + kvh) * a.flat_rows_per_head + j0;
-      for (int pl = 0; pl < PLANES; ++pl)
-        for (int kp = 0; kp < KP; ++kp) {
-          tma_load_3d(kd + (pl * KP + kp) * KSTEP, &map_k, k_full + st, kp * 64, pl, (int)rk, pol_kv);
-          tma_load_3d(vd + (pl * KP + kp) * AT_KVTILE, &map_v, v_full + st, kp * 64, pl, (int)rv, pol_kv);
-        }
+      if (elect_one())
+        for (int pl = 0; pl < PLANES; ++pl)
+          for (int kp = 0; kp < KP; ++kp) {
+            tma_load_3d(kd + (pl * KP + kp) * KSTEP, &map_k, k_full + st, kp * 64, pl, (int)rk, pol_kv);
+            tma_load_3d(vd + (pl * KP + kp) * AT_KVTILE, &map_v, v_full + st, kp * 64, pl, (int)rv, pol_kv);
+          }
     } else {
       const int sub_rows = min(64, a.page_tokens), n_sub = 64 / sub_rows;
       for (int sb = 0; sb < n_sub; ++sb) {
         const int j = min(j0 + sb * sub_rows, a.pages_per_seq * a.page_tokens - 1);
         const int pg = a.page_table[seq * a.pages_per_seq + (j >> a.page_shift)];
         const int row = (pg * a.hkv + kvh) * a.page_tokens + (j & (a.page_tokens - 1));
-        for (int kp = 0; kp < KP; ++kp) {
-          tma_load_2d(kd + kp * KSTEP + sb * sub_rows * 128, &map_k, k_full + st, kp * 64, row, pol_kv);
-          tma_load_2d(vd + kp * AT_KVTILE + sb * sub_rows * 128, &map_v, v_full + st, kp * 64, row, pol_kv);
-        }
+        if (elect_one())
+          for (int kp = 0; kp < KP; ++kp) {
+            tma_load_2d(kd + kp * KSTEP + sb * sub_rows * 128, &map_k, k_full + st, kp * 64, row, pol_kv);
+            tma_load_2d(vd + kp * AT_KVTILE + sb * sub_rows * 128, &map_v, v_full + st, kp * 64, row, pol_kv);
+          }
       }
     }
+    __syncwarp();
   };
   int n_pre = 0;                                            // blocks of the first group already under way
   if (early) {
-    if (threadIdx.x == 0 && n_blk > 0) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
+    if (warp == 0 && n_blk > 0) {
+      if (lane == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
+      }
+      __syncwarp();
       while (n_pre < min(n_blk, GROUP) && (b0 + n_pre + 1) * AT_KBLK <= P) { issue_kv(n_pre); ++n_pre; }
     }
     pdl_wait();
@@ -228,36 +233,43 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0 && n_blk > 0) {
+    if (n_blk > 0) {
       const uint64_t pol_q = policy_evict_last();
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
+      if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
+      __syncwarp();
       // queries: box (64 columns, high | low, G heads, 64 / G rows) -> row 2 e + part of the tile
-      mbar_expect_tx(q_full, (uint32_t)Sh::Q_BYTES);
       const int node0 = slot * a.rows_per_seq + e_base / a.G;
-      for (int kp = 0; kp < KP; ++kp) tma_load_4d(q_s + kp * AT_QTILE, &map_q, q_full, kp * 64, 0, kvh * a.G, node0, pol_q);
+      if (elect_one()) {
+        mbar_expect_tx(q_full, (uint32_t)Sh::Q_BYTES);
+        for (int kp = 0; kp < KP; ++kp) tma_load_4d(q_s + kp * AT_QTILE, &map_q, q_full, kp * 64, 0, kvh * a.G, node0, pol_q);
+      }
+      __syncwarp();
       for (int it = n_pre; it < n_blk; ++it) {
         const int st = it % GROUP, use = it / GROUP;
-        if (use >= 1 && (!mbar_wait(k_empty + st, (uint32_t)(use - 1) & 1u) || !mbar_wait(v_empty + st, (uint32_t)(use - 1) & 1u))) {
-          atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; break;
+        if (use >= 1 && !__all_sync(0xffffffffu, mbar_wait(k_empty + st, (uint32_t)(use - 1) & 1u) && mbar_wait(v_empty + st, (uint32_t)(use - 1) & 1u))) {
+          if (lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
+          break;
         }
-        if (*abort_flag) break;
+        if (__any_sync(0xffffffffu, *abort_flag)) break;
         issue_kv(it);
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && n_blk > 0) {
+    // ------------------------------------------------------------------ MMA issuer: the whole warp, an elected
+    // lane for the tcgen05 instructions (as in the GEMM)
+    if (n_blk > 0) {
       // fp32 accumulate, bf16 operands, M = 128; S: N = 64, both K-major; O: N = head_dim, B MN-major
       const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t o_addr = tmem_base, s_addr0 = tmem_base + HD;
-      bool ok = mbar_wait(q_full, 0);
+      bool ok = mbar_wait_warp(q_full, 0);
+      const uint64_t qd = smem_desc(smem_u32(q_s)), kd = smem_desc(smem_u32(k_s)), pd = smem_desc(smem_u32(p_s)), vd = smem_desc_mn(smem_u32(v_s), AT_KVTILE);
       const int n_groups = (n_blk + GROUP - 1) / GROUP;
       for (int gi = 0; gi < n_groups && ok; ++gi) {
         const int gb = gi * GROUP, ge = min(n_blk, gb + GROUP);
         // S = Q K^T for all keys of the group at once: N = 64 x blocks
         for (int it = gb; it < ge && ok; ++it) {
           const int st = it % GROUP;
-          if (!mbar_wait(k_full + st, (uint32_t)gi & 1u) || (gi >= 1 && !mbar_wait(s_free + st, (uint32_t)(gi - 1) & 1u))) ok = false;
+          if (!__all_sync(0xffffffffu, mbar_wait(k_full + st, (uint32_t)gi & 1u) && (gi < 1 || mbar_wait(s_free + st, (uint32_t)(gi - 1) & 1u)))) ok = false;
         }
         if (!ok) break;
         tc_fence_after();
@@ -268,30 +280,39 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           uint32_t acc = 0u;
           for (int pl = 0; pl < PLANES; ++pl)
             for (int kp = 0; kp < KP; ++kp) {
-              const uint64_t ad = smem_desc(smem_u32(q_s + kp * AT_QTILE));
-              const uint64_t bd = smem_desc(smem_u32(k_s + ((pl * KP + kp) * GROUP + b0) * AT_KVTILE));
+              const uint64_t ad = qd + (uint64_t)(kp * (AT_QTILE >> 4));
+              const uint64_t bd = kd + (uint64_t)(((pl * KP + kp) * GROUP + b0) * (AT_KVTILE >> 4));
+              if (elect_one()) {
 #pragma unroll
-              for (int k = 0; k < 4; ++k) { mma_bf16(s_addr0 + (uint32_t)(b0 * 64), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc_s, acc); acc = 1u; }
+                for (int k = 0; k < 4; ++k) mma_bf16(s_addr0 + (uint32_t)(b0 * 64), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc_s, k ? 1u : acc);
+              }
+              acc = 1u;
             }
         }
-        for (int it = gb; it < ge; ++it) { mma_commit(k_empty + it % GROUP); mma_commit(s_full + it % GROUP); }
+        if (elect_one())
+          for (int it = gb; it < ge; ++it) { mma_commit(k_empty + it % GROUP); mma_commit(s_full + it % GROUP); }
+        __syncwarp();
         for (int it = gb; it < ge && ok; ++it) {                       // O += P_b V_b
           const int st = it % GROUP, pb = it & 1;
-          if (!mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u) || !mbar_wait(v_full + st, (uint32_t)gi & 1u)) { ok = false; break; }
+          if (!__all_sync(0xffffffffu, mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u) && mbar_wait(v_full + st, (uint32_t)gi & 1u))) { ok = false; break; }
           tc_fence_after();
-          const uint64_t ad = smem_desc(smem_u32(p_s + pb * AT_PTILE));
-          for (int pl = 0; pl < PLANES; ++pl) {
-            const uint64_t bd = smem_desc_mn(smem_u32(v_s + st * Sh::KV_STAGE + pl * KP * AT_KVTILE), AT_KVTILE);
+          const uint64_t ad = pd + (uint64_t)(pb * (AT_PTILE >> 4));
+          if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)                                 // 16 keys = two groups of 8 K-rows = 2048 bytes
-              mma_bf16(o_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc_o, (it > 0 || pl > 0 || k > 0) ? 1u : 0u);
+            for (int pl = 0; pl < PLANES; ++pl) {
+              const uint64_t bd = vd + (uint64_t)((st * Sh::KV_STAGE + pl * KP * AT_KVTILE) >> 4);
+#pragma unroll
+              for (int k = 0; k < 4; ++k)                               // 16 keys = two groups of 8 K-rows = 2048 bytes
+                mma_bf16(o_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc_o, (it > 0 || pl > 0 || k > 0) ? 1u : 0u);
+            }
+            mma_commit(p_empty + pb);
+            mma_commit(v_empty + st);
+            if (it == ge - 1) mma_commit(o_done);
           }
-          mma_commit(p_empty + pb);
-          mma_commit(v_empty + st);
-          if (it == ge - 1) mma_commit(o_done);
+          __syncwarp();
         }
       }
-      if (!ok) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
+      if (!ok && lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else {
     // ------------------------------------------------------------------ softmax and epilogue: one row per thread

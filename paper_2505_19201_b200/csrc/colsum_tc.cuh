@@ -50,7 +50,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   uint32_t *tmem_base_p = (uint32_t *)(s_free + 2);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   const int tile = blockIdx.x, h = blockIdx.y, kvh = h / a.G;
   if (threadIdx.x == 0) {
     mbar_init(k_full, 1);
@@ -75,50 +75,64 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0 && n_steps > 0) {
+    if (n_steps > 0) {
       const uint64_t pol = policy_evict_first();
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
-      mbar_expect_tx(k_full, (uint32_t)Sh::K_BYTES);
+      if (lane == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_k) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
+      }
+      __syncwarp();
+      if (elect_one()) mbar_expect_tx(k_full, (uint32_t)Sh::K_BYTES);
+      __syncwarp();
       const int sub_rows = min(64, a.page_tokens), n_sub = CS_KEYS / sub_rows;
       for (int sb = 0; sb < n_sub; ++sb) {
         const int j = min(j0 + sb * sub_rows, a.pages_per_seq * a.page_tokens - sub_rows);
         const int pg = a.page_table[a.seq * a.pages_per_seq + (j >> a.page_shift)];
         const int row = (pg * a.hkv + kvh) * a.page_tokens + (j & (a.page_tokens - 1));
-        for (int kp = 0; kp < KP; ++kp)
-          tma_load_2d(k_s + kp * (CS_KEYS * 128) + sb * sub_rows * 128, &map_k, k_full, kp * 64, row, pol);
+        if (elect_one())
+          for (int kp = 0; kp < KP; ++kp)
+            tma_load_2d(k_s + kp * (CS_KEYS * 128) + sb * sub_rows * 128, &map_k, k_full, kp * 64, row, pol);
+        __syncwarp();
       }
       for (int t = 0; t < n_steps; ++t) {
         const int st = t & 1, use = t >> 1;
-        if (use >= 1 && !mbar_wait(q_empty + st, (uint32_t)(use - 1) & 1u)) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; break; }
-        if (*abort_flag) break;
-        mbar_expect_tx(q_full + st, (uint32_t)Sh::Q_STAGE);
-        for (int pl = 0; pl < 2; ++pl)
-          for (int kp = 0; kp < KP; ++kp)
-            tma_load_4d(q_s + st * Sh::Q_STAGE + (pl * KP + kp) * (NQ * 128), &map_q, q_full + st, kp * 64, pl, h, j0 + t * NQ, pol);
+        if (use >= 1 && !mbar_wait_warp(q_empty + st, (uint32_t)(use - 1) & 1u)) { if (lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } break; }
+        if (__any_sync(0xffffffffu, *abort_flag)) break;
+        if (elect_one()) {
+          mbar_expect_tx(q_full + st, (uint32_t)Sh::Q_STAGE);
+          for (int pl = 0; pl < 2; ++pl)
+            for (int kp = 0; kp < KP; ++kp)
+              tma_load_4d(q_s + st * Sh::Q_STAGE + (pl * KP + kp) * (NQ * 128), &map_q, q_full + st, kp * 64, pl, h, j0 + t * NQ, pol);
+        }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: S^T = K Q_hi^T + K Q_lo^T
-    if (lane == 0 && n_steps > 0) {
+    // (the whole warp, an elected lane for the tcgen05 instructions, as in the GEMM)
+    if (n_steps > 0) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NQ >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-      bool ok = mbar_wait(k_full, 0);
+      const uint64_t kd = smem_desc(smem_u32(k_s)), qd = smem_desc(smem_u32(q_s));
+      bool ok = mbar_wait_warp(k_full, 0);
       for (int t = 0; t < n_steps && ok; ++t) {
         const int st = t & 1, use = t >> 1;
-        if (!mbar_wait(q_full + st, (uint32_t)use & 1u) || (use >= 1 && !mbar_wait(s_free + st, (uint32_t)(use - 1) & 1u))) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(q_full + st, (uint32_t)use & 1u) && (use < 1 || mbar_wait(s_free + st, (uint32_t)(use - 1) & 1u)))) { ok = false; break; }
         tc_fence_after();
         uint32_t acc = 0u;
         for (int pl = 0; pl < 2; ++pl)
           for (int kp = 0; kp < KP; ++kp) {
-            const uint64_t ad = smem_desc(smem_u32(k_s + kp * (CS_KEYS * 128)));
-            const uint64_t bd = smem_desc(smem_u32(q_s + st * Sh::Q_STAGE + (pl * KP + kp) * (NQ * 128)));
+            const uint64_t ad = kd + (uint64_t)(kp * ((CS_KEYS * 128) >> 4));
+            const uint64_t bd = qd + (uint64_t)((st * Sh::Q_STAGE + (pl * KP + kp) * (NQ * 128)) >> 4);
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) { mma_bf16(tmem_base + (uint32_t)(st * NQ), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, acc); acc = 1u; }
+              for (int k = 0; k < 4; ++k) mma_bf16(tmem_base + (uint32_t)(st * NQ), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, k ? 1u : acc);
+            }
+            acc = 1u;
           }
-        mma_commit(q_empty + st);
-        mma_commit(s_full + st);
+        if (elect_one()) { mma_commit(q_empty + st); mma_commit(s_full + st); }
+        __syncwarp();
       }
-      if (!ok) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
+      if (!ok && lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else {
     // ------------------------------------------------------------------ one key (column of the attention matrix) per thread
