@@ -133,26 +133,30 @@ template <> __device__ __forceinline__ void store_split<bf16>(bf16 *p, long long
   if (lo_delta) p[lo_delta] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// Output of a GEMM: [rows][ld].  The stream-K tensor-core kernel leaves up to ceil(kb / upc) + 1 partial
-// sums per 256-column tile, stacked in slots of slot_stride floats; the SIMT kernel leaves one
-// (upc == 0).
+// Output of a GEMM: [rows][ld].  The stream-K part of the tensor-core kernel (tiles n_full and up) leaves
+// up to ceil(kb / units per worker) + 1 partial sums per tile, stacked in slots of slot_stride floats; its full waves and
+// the SIMT kernel leave one.
 struct GemmOut {
   const float *base;
   long long slot_stride;   // floats between consecutive slots
   int ld;                  // floats between consecutive rows (tokens)
   int kb;                  // k-panels per tile
-  int upc;                 // work units (tile, k-panel) per worker; 0 = single slot
+  int n_full, n_tt;        // tiles with a single slot; token tiles per 256 columns
+  float inv_upc, inv_tile; // 1 / work units (tile, k-panel) per worker (0: nothing has more slots); 1 / tokens per tile (0: one token tile)
 };
+// a / b of small non-negative integers (below 2^21) from 1 / b: the half keeps the product a half of 1 / b away from
+// the next integer, which its rounding does not bridge.  An integer division is thirty instructions of code that
+// every launch fetches anew.
+__device__ __forceinline__ int div_small(int a, float inv_b) { return (int)(((float)a + 0.5f) * inv_b); }
 
-__device__ __forceinline__ int gemm_extra_slots(const GemmOut &g, int c) {
-  if (!g.upc) return 0;
-  unsigned u0 = (unsigned)(c >> 8) * (unsigned)g.kb;
-  return (int)((u0 + (unsigned)g.kb - 1u) / (unsigned)g.upc) - (int)(u0 / (unsigned)g.upc);
+__device__ __forceinline__ int gemm_extra_slots(const GemmOut &g, int r, int c) {
+  const int tile = (c >> 8) * g.n_tt + div_small(r, g.inv_tile) - g.n_full, u0 = max(tile, 0) * g.kb;
+  return tile < 0 ? 0 : div_small(u0 + g.kb - 1, g.inv_upc) - div_small(u0, g.inv_upc);
 }
 __device__ __forceinline__ float gemm_val(const GemmOut &g, int r, int c) {
   const float *p = g.base + (long long)r * g.ld + c;
   float s = *p;
-  const int extra = gemm_extra_slots(g, c);
+  const int extra = gemm_extra_slots(g, r, c);
   for (int i = 1; i <= extra; ++i) s += p[(long long)i * g.slot_stride];
   return s;
 }
@@ -164,7 +168,7 @@ __device__ __forceinline__ void add4(float4 &s, const float4 &t) { s.x += t.x; s
 __device__ __forceinline__ float4 gemm_val4(const GemmOut &g, int r, int c) {
   const float4 *p = reinterpret_cast<const float4 *>(g.base + (long long)r * g.ld + c);
   float4 s = *p;
-  const int extra = gemm_extra_slots(g, c);
+  const int extra = gemm_extra_slots(g, r, c);
   const long long st4 = g.slot_stride >> 2;
   int i = 1;
   for (; i + 3 <= extra; i += 4) {
@@ -186,7 +190,7 @@ template <int MAXS>
 __device__ __forceinline__ float4 gemm_val4_wide(const GemmOut &g, int r, int c) {
   const float4 *p = reinterpret_cast<const float4 *>(g.base + (long long)r * g.ld + c);
   float4 s = *p;
-  const int extra = gemm_extra_slots(g, c);
+  const int extra = gemm_extra_slots(g, r, c);
   const long long st4 = g.slot_stride >> 2;
   for (int i = 1; i <= extra; i += MAXS) {
     float4 t[MAXS];

@@ -22,7 +22,10 @@
 #include "tree.cuh"
 
 #define AM_MAX_CHUNKS 32        // most key chunks the split-K attention cuts a sequence into
-#define ROW_CHUNK 256          // most rows any launch set holds (max_batch * tree nodes, a prefill chunk)
+#define ROW_CHUNK 256          // most rows a decode call holds (max_batch * tree nodes)
+// Most prompt rows per pass of the set-up.  The weights stream once per pass and a GEMM's output of this
+// many rows still stays in L2 for the row kernel behind it at the widths met (1152 x 16384 floats: 75 MB).
+#define PROMPT_ROWS 1280
 
 #define SNAP_SLOTS 4
 
@@ -34,7 +37,7 @@ struct dream_ctx {
   dream_config cfg;
   cudaStream_t stream;
   TreeShape ts;
-  int T, esz, qkvN, Hhd, kvN, n_cand, tap_lo_eff, cap_rows, pps, n_pages, RM, XR, gemm_rows_lm;
+  int T, esz, qkvN, Hhd, kvN, n_cand, tap_lo_eff, cap_rows, pps, n_pages, RM, XR, PR, gemm_rows_lm;
   int use_tc, use_pdl, gemm_failed;
   cudaError_t launch_err;              // first refused kernel launch of the call being enqueued
   const char *launch_err_name;
@@ -282,6 +285,7 @@ static void derive(dream_ctx *c) {
   c->n_pages = c->pps * f.max_batch;
   c->RM = (imax(ROW_CHUNK, f.max_prompt) + 15) & ~15;
   c->XR = c->RM;
+  c->PR = imax(ROW_CHUNK, imin(PROMPT_ROWS, (f.max_prompt + 15) & ~15));   // rows of a GEMM input buffer
   c->three = f.draft_blocks == 3;
 }
 
@@ -332,11 +336,11 @@ static size_t carve(dream_ctx *c, char *base) {
   c->x0 = a.take<float>((size_t)f.max_prompt * d);
   c->qbuf = a.take<float>((size_t)c->XR * c->Hhd);
   int planes = f.dtype == DREAM_BF16 ? 2 : 1;      // bf16 GEMM inputs: a high and a low row per token
-  // attention outputs: whole prefill chunks of ROW_CHUNK rows
-  c->attn_out = a.take_bytes((size_t)planes * ((c->XR + ROW_CHUNK - 1) / ROW_CHUNK * ROW_CHUNK) * c->Hhd * e);
-  c->xn = a.take_bytes((size_t)planes * ROW_CHUNK * d * e);
-  c->raw = a.take_bytes((size_t)planes * ROW_CHUNK * d * e);
-  c->act = a.take_bytes((size_t)planes * ROW_CHUNK * f.d_ff * e);
+  // attention outputs: whole passes over the prompt of PR rows
+  c->attn_out = a.take_bytes((size_t)planes * ((c->XR + c->PR - 1) / c->PR * c->PR) * c->Hhd * e);
+  c->xn = a.take_bytes((size_t)planes * c->PR * d * e);
+  c->raw = a.take_bytes((size_t)planes * c->PR * d * e);
+  c->act = a.take_bytes((size_t)planes * c->PR * f.d_ff * e);
   int lm_rows = ((imax(MB * T, MB * imax(c->ts.D + 2, f.tree_beam)) + 15) / 16) * 16;
   c->gemm_rows_lm = lm_rows;
   // GEMM output: the widest of every projection's footprint.  fp32: rows x N.  bf16: room for the
@@ -345,11 +349,14 @@ static size_t carve(dream_ctx *c, char *base) {
     const int shapes[8][2] = {{c->qkvN, d}, {d, c->Hhd}, {2 * f.d_ff, d}, {d, f.d_ff}, {c->Hhd, d}, {c->kvN, d}, {f.vocab, d}, {0, 0}};
     size_t need = 0;
     for (int i = 0; shapes[i][0]; ++i) {
-      int N = shapes[i][0], K = shapes[i][1];
-      size_t fl;
-      if (f.dtype == DREAM_BF16) fl = (size_t)((gemm_tc_out_floats(192, ROW_CHUNK, N, K) + 63) & ~63LL);
-      else fl = (size_t)ROW_CHUNK * N;
-      if (fl > need) need = fl;
+      const int N = shapes[i][0], K = shapes[i][1], most = N == f.vocab && K == d ? ROW_CHUNK : c->PR;
+      if (f.dtype == DREAM_BF16) {
+        // more workers mean more slots (never fewer than two); fewer rows mean fewer tiles, so more slots per tile
+        for (int rows = 16; rows <= most; rows += 16) {
+          const size_t fl = (size_t)imax(2, gemm_tc_split(192, rows, N, K).slots) * rows * N;
+          if (fl > need) need = fl;
+        }
+      } else if ((size_t)most * N > need) need = (size_t)most * N;
     }
     c->gout_floats = need;
   }
@@ -407,13 +414,13 @@ extern "C" dream_status dream_arena_bytes(const dream_config *cfg, size_t *bytes
 // then low parts lo_rows rows further on).
 struct XMode { int mode, lo_rows; };
 static XMode xmode(const dream_ctx *c) {
-  return c->cfg.dtype == DREAM_BF16 ? XMode{TC_X_PLANAR, ROW_CHUNK} : XMode{TC_X_PLAIN, 0};
+  return c->cfg.dtype == DREAM_BF16 ? XMode{TC_X_PLANAR, c->PR} : XMode{TC_X_PLAIN, 0};
 }
 static XLayout xlay(XMode m, long long width) {
   return XLayout{width, m.mode == TC_X_PLANAR ? (long long)m.lo_rows * width : 0};
 }
 
-// out[r][c] = sum_k X[r][k] W[c][k] for r < rows <= ROW_CHUNK, c < N; X holds the rows in layout m.
+// out[r][c] = sum_k X[r][k] W[c][k] for r < rows <= PR, c < N; X holds the rows in layout m.
 // Returns the descriptor consumers read the result through.
 template <typename T>
 static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int rows, int N, int K) {
@@ -438,7 +445,7 @@ static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int row
     const int cols = SG_TC * (SG_WARPS / ks);
     launch_k(c, "k_gemm_simt", kernel, dim3((N + cols - 1) / cols, (rows + tr - 1) / tr), dim3(SG_WARPS * 32), 0,
              (const float *)X, (const float *)W, c->gout, rows, N, K, N, ks);
-    g.base = c->gout; g.slot_stride = 0; g.ld = N; g.kb = 0; g.upc = 0;
+    g.base = c->gout; g.slot_stride = 0; g.ld = N; g.kb = 0; g.n_full = 0; g.n_tt = 1; g.inv_upc = g.inv_tile = 0.f;
   }
   return g;
 }
@@ -461,7 +468,7 @@ static FlatKV flat(dream_ctx *c, float *base) {
   kv.split = c->cfg.dtype == DREAM_BF16 ? 1 : 0;
   return kv;
 }
-static const GemmOut NO_GEMM = {nullptr, 0, 0, 0, 0};
+static const GemmOut NO_GEMM = {nullptr, 0, 0, 0, 0, 1, 0.f, 0.f};
 
 // ------------------------------------------------------------------------------------- prefix bounds
 
@@ -670,13 +677,18 @@ __global__ void k_read_row(const T *src, long long head_stride, float *dst, int 
     dst[(long long)blockIdx.x * n + i] = to_f(s[i]) + (split ? to_f(s[n + i]) : 0.f);
 }
 
-// Elements between the attention outputs of consecutive prefill chunks (ROW_CHUNK rows each; bf16
-// configurations keep a plane of high and a plane of low rows per chunk).
-static long long prefill_chunk_stride(const dream_ctx *c) {
-  return (long long)(c->cfg.dtype == DREAM_BF16 ? 2 : 1) * ROW_CHUNK * c->Hhd;
+// Rows per pass over a prompt of n rows: equal passes of at most PR rows.
+static int prompt_pass_rows(const dream_ctx *c, int n) {
+  const int passes = (n + c->PR - 1) / c->PR;
+  return imin(c->PR, ((n + passes - 1) / passes + 15) & ~15);
+}
+// Elements between the attention outputs of consecutive passes (bf16 configurations keep a plane of
+// high and a plane of low rows per pass).
+static long long prefill_chunk_stride(const dream_ctx *c, int pass_rows) {
+  return (long long)(c->cfg.dtype == DREAM_BF16 ? 2 * c->PR : pass_rows) * c->Hhd;
 }
 template <typename T, int HD> struct AttnLaunch {
-  // The output rows are laid out per prefill chunk of ROW_CHUNK rows (the O projection's input).
+  // The output rows are laid out per pass over the prompt (the O projection's input).
   static void prefill(dream_ctx *c, int layer, int seq, int n) {
     if constexpr (sizeof(T) == 2) {
       // causal attention of the n prompt rows on the tensor cores: one CTA per (KV head, 64 entries)
@@ -684,7 +696,7 @@ template <typename T, int HD> struct AttnLaunch {
       AttnTcArgs a = {};
       a.mode = AT_PREFILL;
       a.n_keys = n; a.lay = xlay(xmode(c), c->Hhd);
-      a.out_chunk_rows = ROW_CHUNK; a.out_chunk_stride = prefill_chunk_stride(c);
+      a.out_chunk_rows = prompt_pass_rows(c, n); a.out_chunk_stride = prefill_chunk_stride(c, a.out_chunk_rows);
       a.lse = c->lse_pre; a.ent = c->ent_pre;
       c->cur_seq[0] = seq;
       tc(c, a, layer, nullptr, 1, n, 0, nullptr);
@@ -867,14 +879,13 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
                                  const int *ids, int q, int *first_token, float *first_margin,
                                  float *layer_entropy, int *tap_layer) {
   const dream_config &f = c->cfg;
-  // The prompt goes through the projections ROW_CHUNK rows at a time: the weights stream once per
-  // chunk (bf16: two token tiles of 128 rows share every weight panel).
-  int n = q + v, d = f.d_model, L = f.n_layers, CH = ROW_CHUNK;
+  // The prompt goes through the projections in passes of CH rows: the weights stream once per pass.
+  int n = q + v, d = f.d_model, L = f.n_layers, CH = prompt_pass_rows(c, n);
   LAUNCH(c, k_iota_rows, (n + 255) / 256, 256, 0, c->rm[0], seq, n);
   LAUNCH(c, (k_build_prompt<T>), n, 256, 0, (const T *)c->embed, (const T *)visual, ids, vis_start, v, c->x, c->x0,
          d, f.vocab, c->status);
   const XMode mp = xmode(c);
-  const long long att_chunk = prefill_chunk_stride(c);
+  const long long att_chunk = prefill_chunk_stride(c, CH);
   for (int l = 0; l < L; ++l) {
     for (int r0 = 0; r0 < n; r0 += CH) {
       int rows = imin(CH, n - r0);
@@ -998,7 +1009,7 @@ static GemmOut draft_rows(dream_ctx *c, const RowMeta &rm, int R, XMode xm, int 
 template <typename T>
 static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *forced, int *kept, float *scores) {
   const dream_config &f = c->cfg;
-  int v = c->pf_v, q = c->pf_q, n = v + q, d = f.d_model, nc = q + k, CH = ROW_CHUNK;
+  int v = c->pf_v, q = c->pf_q, n = v + q, d = f.d_model, nc = q + k, CH = c->PR;
   LAUNCH(c, k_select_visual, 1, 1024, 0, c->scores_all, (long long)imax(f.max_visual, 1), c->sd.tap + seq, c->tap_lo_eff,
          v, k, c->pf_vis_start, n, forced, kept, scores, c->ctx_pos, c->flags);
   // draft self-attention K/V of the compressed context, from the input embeddings
@@ -1447,7 +1458,7 @@ extern "C" dream_status dream_topk_lse_static(const float *logits, int32_t rows,
   TopkScratch ts;
   ts.pv = sc->pv; ts.pi = sc->pi; ts.pm = sc->pm; ts.pz = sc->pz; ts.counter = sc->counter;
   GemmOut g;                                   // a plain [rows][vocab] matrix: one slot, one chunk
-  g.base = logits; g.slot_stride = 0; g.ld = vocab; g.kb = 0; g.upc = 0;
+  g.base = logits; g.slot_stride = 0; g.ld = vocab; g.kb = 0; g.n_full = 0; g.n_tt = 1; g.inv_upc = g.inv_tile = 0.f;
   int nsplit = (vocab + TOPK_COLS - 1) / TOPK_COLS;
   k_topk_lse<TOPK_COLS / TOPK_THREADS><<<dim3(rows, nsplit), TOPK_THREADS, 0, stream>>>(g, vocab, ktop, nsplit, ts, top_val, top_id, lse, (float *)nullptr);
   e = cudaGetLastError();

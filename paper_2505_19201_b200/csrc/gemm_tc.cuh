@@ -1,6 +1,7 @@
 // Weight-streaming GEMM on pairs of SMs for sm_100a:  out[t][c] = sum_k X[t][k] * W[c][k].
 //
-// A decode call has few tokens (1..256 rows), so this is a stream of W from HBM.  Design:
+// A decode call has few tokens (1..256 rows), so this is a stream of W from HBM; a prompt has hundreds,
+// and the tensor cores bound it.  Design:
 //   * a cluster of two CTAs on neighbouring SMs works on one tile: 256 weight rows are the MMA's M
 //     (tcgen05.mma.cta_group::2, 128 rows and 128 TMEM lanes per CTA) and up to 256 token rows its N, of
 //     which each CTA stages one half.  Half as many workers as SMs also means half as many partial
@@ -19,9 +20,12 @@
 //     panels of 64 k per stage: W (128 rows, 16 KB a panel) and X.  W gets all the room X leaves: it is
 //     what a CTA can fetch before its grid dependency resolves.  One commit per stage frees both: the X
 //     producer waits on the W stage that went with the X stage it reuses;
-//   * persistent stream-K: the (tile, panel) units are dealt out in equal contiguous ranges to the
-//     pairs; a pair that covers part of a tile writes a partial sum to its own slot and the consumer
-//     adds the slots in a fixed order;
+//   * tiles are 256 weight rows x up to 256 tokens, the token tiles of one weight tile next to each other.
+//     With several token tiles, full waves of tiles come first, one tile per pair, so that neighbouring pairs read the same weight
+//     panels at the same time (one HBM read serves them all).  The rest, between one and two waves of tiles
+//     (or all of them when there are fewer than two), is stream-K: its (tile, panel) units are dealt
+//     out in equal contiguous ranges; a pair that covers part of a tile writes a partial sum to its own
+//     slot and the consumer adds the slots in a fixed order;
 //   * programmatic dependent launch: W never changes, so its ring fills before the grid
 //     dependency resolves; only the X producer and the epilogue wait for the previous kernel;
 //   * the MMA issuer and the producers are whole warps that run their loops together and elect a lane for
@@ -54,13 +58,18 @@
 // the low parts lo_rows rows further on.
 enum { TC_X_PLAIN = 0, TC_X_PLANAR = 1 };
 // How the MMA takes them (see above).
-enum { TC_X_ONE = 0, TC_X_CONCAT = 1, TC_X_TWO = 2 };
+// TILES: TWO over several token tiles, with full waves of tiles; a form of its own because the decode forms'
+// code is fetched anew at every launch and each division in it shows (one kernel for all: rounds 4 % slower).
+enum { TC_X_ONE = 0, TC_X_CONCAT = 1, TC_X_TWO = 2, TC_X_TILES = 3 };
 
 struct TcParams {
   float *out;
   long long slot_stride;        // floats between partial-sum slots
-  int N, KB, total_units, upc;  // output columns, k panels, units = tiles x panels, units per pair
-  int tile_t, mma_n;            // tokens per tile, N of an MMA
+  int N, KB;                    // output columns, k panels
+  int n_pairs, n_waves, n_full; // pairs, full waves, tiles in them (n_pairs * n_waves)
+  int sk_units, upc;            // stream-K part: units = tiles x panels, units per pair
+  float inv_kb, inv_upc;        // their reciprocals, for div_small
+  int n_tt, tile_t, mma_n;      // token tiles, tokens per tile, N of an MMA
   int n_sub;                    // CONCAT / ONE: accumulators the k-steps of a segment are dealt out to (1, 2 or 4)
   int n_tok;                    // real token rows
   int lo_rows;                  // row of the first low part in the X tensor map
@@ -105,6 +114,11 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 __device__ __forceinline__ uint64_t policy_evict_last() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ uint64_t policy_evict_normal() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -190,6 +204,20 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t *bar) {
                ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
 }
 
+// The segments (tile, panels [k0, k1)) of one pair, in order.  TILES: full waves first.
+template <bool TILES> struct TcWalk {
+  int pair, w, u, u_end;
+  __device__ __forceinline__ TcWalk(const TcParams &p, int pair_) : pair(pair_), w(0) { u = pair * p.upc; u_end = min(u + p.upc, p.sk_units); }
+  __device__ __forceinline__ bool next(const TcParams &p, int &tile, int &k0, int &k1) {
+    if (TILES && w < p.n_waves) { tile = w * p.n_pairs + pair; k0 = 0; k1 = p.KB; ++w; return true; }
+    if (u >= u_end) return false;
+    tile = div_small(u, p.inv_kb); k0 = u - tile * p.KB; k1 = min(p.KB, k0 + u_end - u);
+    u += k1 - k0;
+    if (TILES) tile += p.n_full;
+    return true;
+  }
+};
+
 // ------------------------------------------------------------------------------------------ kernel
 // Dynamic shared memory (1024-byte aligned): W ring [w_stages][wp][16 KB], X ring [x_stages][wp][panel], barriers.
 template <int FORM>
@@ -199,7 +227,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   // bytes of token rows one CTA stages per k panel
   const uint32_t xtile_bytes = (uint32_t)(FORM == TC_X_CONCAT ? p.tile_t : p.mma_n >> 1) * 128u;
-  const uint32_t xpanel_bytes = FORM == TC_X_TWO ? 2u * xtile_bytes : xtile_bytes;
+  const uint32_t xpanel_bytes = FORM >= TC_X_TWO ? 2u * xtile_bytes : xtile_bytes;
   const uint32_t wstage_bytes = (uint32_t)p.wp * TC_WPANEL, xstage_bytes = (uint32_t)p.wp * xpanel_bytes;
   uint8_t *wring = smem, *xring = smem + (size_t)p.w_stages * wstage_bytes;
   uint64_t *bars = (uint64_t *)(xring + (size_t)p.x_stages * xstage_bytes);
@@ -229,31 +257,35 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   tc_fence_after();
   pdl_trigger();
   const uint32_t tmem_base = *tmem_base_p;
-  const int u_begin = pair * p.upc, u_end = min(u_begin + p.upc, p.total_units);
+  int tile, k0, k1;
+  constexpr bool TILES = FORM == TC_X_TILES;
+  TcWalk<TILES> walk(p, pair);
   auto give_up = [&]() { if (lane == 0) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } };
 
   if (warp == 0) {
     // ------------------------------------------------------------------ W producer: weights are
     // constant, so nothing here waits for anything but ring space
-    const uint64_t pol = policy_evict_first();
+    const uint64_t pol = TILES ? policy_evict_normal() : policy_evict_first();     // several token tiles read a weight panel
     if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
     __syncwarp();
     const uint32_t bar0 = mapa(smem_u32(full_w), 0);
     int s = 0;
     uint32_t ph = 1;
-    for (int u = u_begin; u < u_end;) {
-      const int tile = u / p.KB, kb = u - tile * p.KB, np = min(p.wp, min(p.KB - kb, u_end - u));
-      const int y = tile * TC_BN + (int)rank * 128;
-      if (!mbar_wait_warp(empty_w + s, ph)) { give_up(); break; }
-      if (__any_sync(0xffffffffu, *abort_flag)) break;
-      if (elect_one()) {
-        if (rank == 0) mbar_expect_tx(full_w + s, 2u * (uint32_t)np * TC_WPANEL);
-        uint8_t *dst = wring + (size_t)s * wstage_bytes;
-        for (int i = 0; i < np; ++i) tma_load_2d_pair(dst + (size_t)i * TC_WPANEL, &map_w, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
+    bool ok = true;
+    while (ok && walk.next(p, tile, k0, k1)) {
+      const int y = (TILES ? tile / p.n_tt : tile) * TC_BN + (int)rank * 128;
+      for (int kb = k0; kb < k1; kb += p.wp) {
+        const int np = min(p.wp, k1 - kb);
+        if (!mbar_wait_warp(empty_w + s, ph)) { give_up(); ok = false; break; }
+        if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(full_w + s, 2u * (uint32_t)np * TC_WPANEL);
+          uint8_t *dst = wring + (size_t)s * wstage_bytes;
+          for (int i = 0; i < np; ++i) tma_load_2d_pair(dst + (size_t)i * TC_WPANEL, &map_w, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
+        }
+        __syncwarp();
+        if (++s == p.w_stages) { s = 0; ph ^= 1; }
       }
-      __syncwarp();
-      u += np;
-      if (++s == p.w_stages) { s = 0; ph ^= 1; }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ X producer: waits until the
@@ -261,32 +293,36 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const uint64_t pol = policy_evict_last();
     if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
     __syncwarp();
+    bool more = walk.next(p, tile, k0, k1);
     pdl_wait();
     if (blockIdx.x == 0 && lane == 0) trace_stamp(TR_k_gemm_tc);
     __syncwarp();
     const uint32_t bar0 = mapa(smem_u32(full_x), 0);
-    const int y = FORM == TC_X_CONCAT ? (int)rank * p.lo_rows : (int)rank * (p.mma_n >> 1);   // first token row this CTA stages
+    const int y_off = FORM == TC_X_CONCAT ? (int)rank * p.lo_rows : (int)rank * (p.mma_n >> 1);   // first token row this CTA stages, from the tile's
     int s = 0, n_free = p.x_stages, ws = 0;      // unused X stages left; W stage that went with the X stage to reuse
     uint32_t wph = 0;
-    for (int u = u_begin; u < u_end;) {
-      const int tile = u / p.KB, kb = u - tile * p.KB, np = min(p.wp, min(p.KB - kb, u_end - u));
-      if (n_free > 0) --n_free;
-      else {
-        if (!mbar_wait_warp(empty_w + ws, wph)) { give_up(); break; }
-        if (++ws == p.w_stages) { ws = 0; wph ^= 1; }
-      }
-      if (__any_sync(0xffffffffu, *abort_flag)) break;
-      if (elect_one()) {
-        if (rank == 0) mbar_expect_tx(full_x + s, 2u * (uint32_t)np * xpanel_bytes);
-        for (int i = 0; i < np; ++i) {
-          uint8_t *dst = xring + (size_t)s * xstage_bytes + (size_t)i * xpanel_bytes;
-          tma_load_2d_pair(dst, &map_x, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
-          if (FORM == TC_X_TWO) tma_load_2d_pair(dst + xtile_bytes, &map_x, bar0 + 8u * s, (kb + i) * TC_BK, p.lo_rows + y, pol);
+    bool ok = true;
+    for (; ok && more; more = walk.next(p, tile, k0, k1)) {
+      const int y = (TILES ? tile % p.n_tt * p.tile_t : 0) + y_off;
+      for (int kb = k0; kb < k1; kb += p.wp) {
+        const int np = min(p.wp, k1 - kb);
+        if (n_free > 0) --n_free;
+        else {
+          if (!mbar_wait_warp(empty_w + ws, wph)) { give_up(); ok = false; break; }
+          if (++ws == p.w_stages) { ws = 0; wph ^= 1; }
         }
+        if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
+        if (elect_one()) {
+          if (rank == 0) mbar_expect_tx(full_x + s, 2u * (uint32_t)np * xpanel_bytes);
+          for (int i = 0; i < np; ++i) {
+            uint8_t *dst = xring + (size_t)s * xstage_bytes + (size_t)i * xpanel_bytes;
+            tma_load_2d_pair(dst, &map_x, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
+            if (FORM >= TC_X_TWO) tma_load_2d_pair(dst + xtile_bytes, &map_x, bar0 + 8u * s, (kb + i) * TC_BK, p.lo_rows + y, pol);
+          }
+        }
+        __syncwarp();
+        if (++s == p.x_stages) s = 0;
       }
-      __syncwarp();
-      u += np;
-      if (++s == p.x_stages) s = 0;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (the pair's first CTA)
@@ -296,20 +332,20 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       const uint64_t wdesc = smem_desc(smem_u32(wring)), xdesc = smem_desc(smem_u32(xring));
       const int w_stages = p.w_stages, x_stages = p.x_stages, wp = p.wp;
       const uint32_t sub_n = (uint32_t)p.mma_n, sub_mask = (uint32_t)p.n_sub - 1u;
-      int ws = 0, xs = 0, u = u_begin;
+      int ws = 0, xs = 0;
       uint32_t wph = 0, xph = 0, fill = 0;                            // fill counts accumulator fills
       bool ok = true;
-      while (u < u_end && ok) {
-        const int seg_end = min((u / p.KB + 1) * p.KB, u_end);
-        const int fill_end = FORM == TC_X_TWO ? min(seg_end, u + TC_CHAIN) : seg_end;
+      k0 = k1 = 0;
+      while (ok && (k0 < k1 || walk.next(p, tile, k0, k1))) {
+        const int fill_end = FORM >= TC_X_TWO ? min(k1, k0 + TC_CHAIN) : k1;
         const uint32_t buf = fill & 1u, use = fill >> 1;              // use: earlier fills of this accumulator
         ++fill;
         if (!mbar_wait_warp(acc_empty + buf, (use & 1u) ^ 1u)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_addr = tmem_base + buf * 256u;
         uint32_t begun = 0u;                                          // 0: the first MMA of an accumulator overwrites it
-        while (u < fill_end) {
-          const int np = min(wp, fill_end - u);
+        while (k0 < fill_end) {
+          const int np = min(wp, fill_end - k0);
           if (!__all_sync(0xffffffffu, mbar_wait(full_w + ws, wph) && mbar_wait(full_x + xs, xph))) { ok = false; break; }
           tc_fence_after();
           for (int i = 0; i < np; ++i) {
@@ -318,7 +354,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
             if (elect_one()) {
 #pragma unroll
               for (int k = 0; k < TC_BK / 16; ++k) {
-                if (FORM == TC_X_TWO) {
+                if (FORM >= TC_X_TWO) {
                   mma_bf16_pair(d_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, k ? 1u : begun);
                   mma_bf16_pair(d_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)((xtile_bytes >> 4) + k * 2), idesc, 1u);
                 } else {
@@ -330,7 +366,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
             begun = 1u;
           }
           if (elect_one()) mma_commit_pair(empty_w + ws);             // frees both stages in both CTAs once these MMAs have read them
-          u += np;
+          k0 += np;
           if (++ws == w_stages) { ws = 0; wph ^= 1; }
           if (++xs == x_stages) { xs = 0; xph ^= 1; }
         }
@@ -347,7 +383,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const uint32_t done_bar = mapa(smem_u32(acc_empty), 0);
     pdl_wait();                               // the output buffer belongs to earlier kernels
     uint32_t fill = 0;
-    int u = u_begin;
     bool ok = true;
     auto wait_full = [&](uint32_t buf, uint32_t use) {
       int w = 1;
@@ -356,17 +391,17 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       if (!w || __any_sync(0xffffffffu, *abort_flag)) { give_up(); ok = false; }
       tc_fence_after();
     };
-    while (u < u_end && ok) {
-      const int tile = u / p.KB, seg_end = min((tile + 1) * p.KB, u_end);
-      const int slot = pair - (tile * p.KB) / p.upc, nt = p.n_tok;
-      const int c = tile * TC_BN + (int)rank * 128 + q * 32 + lane;
-      float *dst = p.out + (long long)slot * p.slot_stride + c;
-      if (FORM == TC_X_TWO) {
+    while (ok && walk.next(p, tile, k0, k1)) {
+      const int sk_tile = TILES ? tile - p.n_full : tile, slot = TILES && sk_tile < 0 ? 0 : pair - div_small(sk_tile * p.KB, p.inv_upc);
+      const int ct = TILES ? tile / p.n_tt : tile, tok0 = TILES ? (tile - ct * p.n_tt) * p.tile_t : 0, nt = min(p.tile_t, p.n_tok - tok0);
+      const int c = ct * TC_BN + (int)rank * 128 + q * 32 + lane;
+      float *dst = p.out + (long long)slot * p.slot_stride + (long long)tok0 * p.N + c;
+      if (FORM >= TC_X_TWO) {
         // token groups of 16: half 0 takes groups 0, 2, .., half 1 groups 1, 3, ..
         float run[128];
 #pragma unroll
         for (int j = 0; j < 128; ++j) run[j] = 0.f;
-        for (; u < seg_end; u += min(TC_CHAIN, seg_end - u)) {
+        for (; k0 < k1; k0 += TC_CHAIN) {
           const uint32_t buf = fill & 1u;
           wait_full(buf, fill >> 1);
           ++fill;
@@ -424,7 +459,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(done_bar + 8u * buf);
-        u = seg_end;
       }
     }
   }
@@ -460,15 +494,15 @@ static inline const char *gemm_tc_plan_init(GemmTcPlan *pl, int *status, int use
   cudaDeviceGetAttribute(&pl->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (cudaFuncSetAttribute(k_gemm_tc<TC_X_ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
       cudaFuncSetAttribute(k_gemm_tc<TC_X_CONCAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_gemm_tc<TC_X_TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess)
+      cudaFuncSetAttribute(k_gemm_tc<TC_X_TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
+      cudaFuncSetAttribute(k_gemm_tc<TC_X_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess)
     return "cannot raise the dynamic shared memory limit";
   pl->status = status;
   pl->use_pdl = use_pdl;
   return nullptr;
 }
 
-// Most token rows of one launch.
-#define TC_ROWS_MAX 256
+#define TC_TOKENS 256           // most tokens of a tile
 
 static inline bool gemm_tc_supported(int N, int K) {
   return K % TC_BK == 0 && K >= TC_BK && N % 8 == 0 && N >= 8;
@@ -496,54 +530,62 @@ static inline bool tc_map(GemmTcPlan *pl, const void *ptr, int rows, int K, int 
   return true;
 }
 
-// Units of (256-row tile, k panel) a pair takes.
-static inline int gemm_tc_units_per_pair(int n_sms, long long total) {
-  long long pairs = n_sms / 2 > 0 ? n_sms / 2 : 1;
-  if (pairs > total) pairs = total;
-  return (int)((total + pairs - 1) / pairs);
+// How a launch of `rows` token rows is cut (see the head of the file).
+struct TcSplit { int n_tt, tile_t, n_pairs, n_waves, sk_units, upc, slots; };
+static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
+  TcSplit t;
+  const int KB = K / TC_BK;
+  t.n_tt = (rows + TC_TOKENS - 1) / TC_TOKENS;
+  // tokens in 16s (the N of an MMA over both CTAs); up to 128 rows both planes share an MMA, so 8s do
+  t.tile_t = t.n_tt > 1 || rows > 128 ? ((rows + t.n_tt - 1) / t.n_tt + 15) & ~15 : (rows + 7) & ~7;
+  const int pairs = n_sms / 2 > 0 ? n_sms / 2 : 1, tiles = (N + TC_BN - 1) / TC_BN * t.n_tt;
+  t.n_waves = t.n_tt > 1 && tiles / pairs > 1 ? tiles / pairs - (tiles % pairs ? 1 : 0) : 0;
+  t.sk_units = (tiles - t.n_waves * pairs) * KB;
+  t.upc = t.sk_units ? (t.sk_units + pairs - 1) / pairs : 1;
+  t.n_pairs = t.n_waves ? pairs : (t.sk_units + t.upc - 1) / t.upc;
+  t.slots = t.sk_units ? (KB + t.upc - 1) / t.upc + 1 : 1;      // a tile is shared by at most as many pairs
+  return t;
+}
+// Floats one launch may write.
+static inline long long gemm_tc_out_floats(int n_sms, int rows, int N, int K) {
+  return gemm_tc_split(n_sms, rows, N, K).slots * (long long)rows * N;
 }
 
-// Floats one launch may write when its slots hold slot_rows x N: a tile is shared by at most
-// ceil(KB / upc) + 1 pairs.
-static inline long long gemm_tc_out_floats(int n_sms, int slot_rows, int N, int K) {
-  int KB = K / TC_BK, n_tiles = (N + TC_BN - 1) / TC_BN;
-  long long upc = gemm_tc_units_per_pair(n_sms, (long long)n_tiles * KB);
-  long long slots = (KB + upc - 1) / upc + 1;
-  return slots * (long long)slot_rows * N;
-}
-
-// Enqueue one GEMM of up to TC_ROWS_MAX token rows.
-//   X: bf16, row-major, K columns.  TC_X_PLAIN: row t = token t.  TC_X_PLANAR: row t = high part, row
-//   lo_rows + t = low part.
+// Enqueue one GEMM of `rows` token rows.
+//   X: bf16, row-major, K columns.  TC_X_PLAIN (up to 128 rows): row t = token t.  TC_X_PLANAR: row t =
+//   high part, row lo_rows + t = low part.
 // *g receives the descriptor consumers read the result through.  Returns false if the launch could
 // not be made.
 static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const void *W, const void *X, int x_mode, int lo_rows,
                                   int rows, int N, int K, float *out, long long out_floats, GemmOut *g) {
-  if (rows < 1 || rows > TC_ROWS_MAX) return false;
+  if (rows < 1 || (x_mode == TC_X_PLAIN && rows > 128)) return false;
+  const TcSplit t = gemm_tc_split(pl->n_sms, rows, N, K);
+  if (t.sk_units + K / TC_BK >= 1 << 21) return false;          // div_small
   TcParams p;
   p.n_tok = rows; p.lo_rows = lo_rows;
   p.N = N; p.KB = K / TC_BK;
-  p.total_units = (N + TC_BN - 1) / TC_BN * p.KB;
+  p.n_pairs = t.n_pairs; p.n_waves = t.n_waves; p.n_full = t.n_pairs * t.n_waves; p.sk_units = t.sk_units; p.upc = t.upc;
+  p.n_tt = t.n_tt; p.tile_t = t.tile_t;
+  p.inv_kb = 1.f / (float)p.KB; p.inv_upc = 1.f / (float)p.upc;
   // N of an MMA is a multiple of 16 and each CTA stages half of it (8-row groups)
   int form;
   if (x_mode == TC_X_PLAIN) { form = TC_X_ONE; p.tile_t = p.mma_n = (rows + 15) & ~15; }
-  else if (rows <= 128) { form = TC_X_CONCAT; p.tile_t = (rows + 7) & ~7; p.mma_n = 2 * p.tile_t; }
-  else { form = TC_X_TWO; p.tile_t = p.mma_n = (rows + 15) & ~15; }
+  else if (rows <= 128) { form = TC_X_CONCAT; p.mma_n = 2 * p.tile_t; }
+  else { form = p.n_tt > 1 ? TC_X_TILES : TC_X_TWO; p.mma_n = p.tile_t; }
   p.n_sub = p.mma_n <= 64 ? 4 : p.mma_n <= 128 ? 2 : 1;
-  p.upc = gemm_tc_units_per_pair(pl->n_sms, p.total_units);
-  const int n_pairs = (p.total_units + p.upc - 1) / p.upc;
   p.out = out;
   p.slot_stride = (long long)rows * N;
-  if (gemm_tc_out_floats(pl->n_sms, rows, N, K) > out_floats) return false;
+  if (t.slots * p.slot_stride > out_floats) return false;
   CUtensorMap mw, mx;
   const int x_rows = x_mode == TC_X_PLANAR ? lo_rows + rows : rows;
   const int x_box = form == TC_X_CONCAT ? p.tile_t : p.mma_n / 2;
   if (!tc_map(pl, W, N, K, 128, &mw) || !tc_map(pl, X, x_rows, K, x_box, &mx)) return false;
-  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = N; g->kb = p.KB; g->upc = p.upc;
+  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = N; g->kb = p.KB; g->n_full = p.n_full; g->n_tt = p.n_tt;
+  g->inv_upc = p.inv_upc; g->inv_tile = p.n_tt > 1 ? 1.f / (float)p.tile_t : 0.f;
   // Stages of two panels halve the waits and commits per panel (61 rows, 12288 x 4096: 22.2 -> 20.9 us) as
   // long as five fit; where a token panel is larger than a weight panel (244 rows: 38.3 against 39.4 us) the
   // rings are deeper with one
-  const int xpanel = x_box * 128 * (form == TC_X_TWO ? 2 : 1);
+  const int xpanel = x_box * 128 * (form >= TC_X_TWO ? 2 : 1);
   p.wp = xpanel <= TC_WPANEL / 2 ? 2 : 1;
   const int xstage = p.wp * xpanel, wstage = p.wp * TC_WPANEL;
   const int room = pl->max_smem - 2048;
@@ -554,11 +596,11 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   p.status = pl->status;
   size_t smem = (size_t)p.w_stages * wstage + (size_t)p.x_stages * xstage + 2048;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * n_pairs); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.gridDim = dim3(2 * p.n_pairs); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = pl->use_pdl ? 1 : 0;
-  auto *kernel = form == TC_X_CONCAT ? k_gemm_tc<TC_X_CONCAT> : form == TC_X_TWO ? k_gemm_tc<TC_X_TWO> : k_gemm_tc<TC_X_ONE>;
+  auto *kernel = form == TC_X_CONCAT ? k_gemm_tc<TC_X_CONCAT> : form == TC_X_TWO ? k_gemm_tc<TC_X_TWO> : form == TC_X_TILES ? k_gemm_tc<TC_X_TILES> : k_gemm_tc<TC_X_ONE>;
   return cudaLaunchKernelEx(&cfg, kernel, mw, mx, p) == cudaSuccess;
 }
