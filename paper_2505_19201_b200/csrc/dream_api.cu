@@ -62,6 +62,7 @@ struct dream_ctx {
   int *gather_idx, *ctx_pos, *flags;
   uint32_t *vmask;
   void *qbuf;                          // query rows, 4 bytes per element (see q_store4)
+  float *ssq;                          // [PR][SSQ_LD] sums of squares of the rows in xn (k_resid)
   float *x, *x0, *gout, *lse_pre, *ent_pre, *ae, *scores_all, *taps_store, *tapbuf;
   void *xn, *raw, *act, *attn_out;
   float *top_val, *lse_rows, *margin_i;
@@ -361,6 +362,7 @@ static size_t carve(dream_ctx *c, char *base) {
     c->gout_floats = need;
   }
   c->gout = a.take<float>(c->gout_floats);
+  c->ssq = a.take<float>((size_t)c->PR * SSQ_LD);
   c->rope_inv = a.take<double>(f.head_dim / 2);
   c->rope_tab = a.take<float2>((size_t)ROW_CHUNK * (f.head_dim / 2));
   c->lse_pre = a.take<float>((size_t)f.n_heads * f.max_prompt);
@@ -848,27 +850,24 @@ template <typename T, int HD> struct AttnLaunch {
     else AttnLaunch<T, 256>::call;                                \
   } while (0)
 
-// x (+= GEMM output) -> RMSNorm -> GEMM input rows in c->xn; see k_resid_norm for the side outputs.
+// x (+= GEMM output) -> x * gain, GEMM input rows in c->xn; see k_resid for the side outputs.  The consumer of the
+// GEMM that reads them scales its rows by what this returns.
 template <typename T>
-static void norm_rows(dream_ctx *c, float *x, const GemmOut &gin, bool has_in, const void *gain, int rows, XMode m,
-                      float *copy = nullptr, const int *row_seq = nullptr, const int *tap = nullptr, int layer = 0,
-                      bool want_raw = false) {
-  const int d4 = c->cfg.d_model / 4;
-  int nv = 1;
-  while ((d4 + nv - 1) / nv > 1024) nv *= 2;                 // d_model <= 16384 by check_config
-  const int threads = ((d4 + nv - 1) / nv + 31) & ~31;
-  if (nv == 1) LAUNCH(c, (k_resid_norm<T, 1>), rows, threads, 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, c->cfg.d_model,
-         (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, c->cfg.d_model));
-  else if (nv == 2) LAUNCH(c, (k_resid_norm<T, 2>), rows, threads, 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, c->cfg.d_model,
-         (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, c->cfg.d_model));
-  else LAUNCH(c, (k_resid_norm<T, 4>), rows, threads, 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, c->cfg.d_model,
-         (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, c->cfg.d_model));
+static RowScale norm_rows(dream_ctx *c, float *x, const GemmOut &gin, bool has_in, const void *gain, int rows, XMode m,
+                          float *copy = nullptr, const int *row_seq = nullptr, const int *tap = nullptr, int layer = 0,
+                          bool want_raw = false) {
+  const int d = c->cfg.d_model;
+  LAUNCH(c, (k_resid<T>), dim3((d + 1023) / 1024, rows), 256, 0, x, gin, has_in ? 1 : 0, (const T *)gain, d,
+         (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, d), c->ssq);
+  return RowScale{c->ssq, (d + 127) / 128, 1.f / (float)d, c->cfg.rms_eps};
 }
+static const RowScale NO_NORM = {nullptr, 0, 0.f, 0.f};
+// norm: of the rows in c->xn.
 template <typename T>
-static GemmOut mlp_rows(dream_ctx *c, const void *wgu, const void *wd, int rows, XMode m) {
+static GemmOut mlp_rows(dream_ctx *c, const RowScale &norm, const void *wgu, const void *wd, int rows, XMode m) {
   const dream_config &f = c->cfg;
   GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model);
-  LAUNCH(c, (k_silu_mul<T>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, (T *)c->act, f.d_ff, xlay(m, f.d_ff));
+  LAUNCH(c, (k_silu_mul<T>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, norm, (T *)c->act, f.d_ff, xlay(m, f.d_ff));
   return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
 }
 
@@ -886,34 +885,39 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
          d, f.vocab, c->status);
   const XMode mp = xmode(c);
   const long long att_chunk = prefill_chunk_stride(c, CH);
+  // projections of layer l for the rows of one pass, whose normalised input sits in c->xn
+  auto qkv = [&](int l, int r0, int rows, const RowScale &norm) {
+    GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d);
+    LAUNCH(c, (k_qkv_post_target<T>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].pos, c->rm[0].slot, r0, c->qbuf,
+           paged(c, l), f.n_heads, c->rope_inv, (const float2 *)nullptr);
+  };
+  for (int r0 = 0; r0 < n; r0 += CH) {
+    const int rows = imin(CH, n - r0);
+    qkv(0, r0, rows, norm_rows<T>(c, c->x + (size_t)r0 * d, NO_GEMM, false, c->ln1[0], rows, mp));
+  }
   for (int l = 0; l < L; ++l) {
-    for (int r0 = 0; r0 < n; r0 += CH) {
-      int rows = imin(CH, n - r0);
-      norm_rows<T>(c, c->x + (size_t)r0 * d, NO_GEMM, false, c->ln1[l], rows, mp);
-      GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d);
-      LAUNCH(c, (k_qkv_post_target<T>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, c->rm[0].seq, c->rm[0].pos, c->rm[0].slot, r0, c->qbuf,
-             paged(c, l), f.n_heads, c->rope_inv, (const float2 *)nullptr);
-    }
     HD_DISPATCH(c, T, prefill(c, l, seq, n));
     LAUNCH(c, k_entropy_mean, 1, 1024, 0, c->ent_pre, f.n_heads * n, c->ae + l,
            c->ent_sum ? c->ent_sum + (size_t)seq * L + l : (float *)nullptr);
     int cand = l + 1 - c->tap_lo_eff;
     bool is_cand = cand >= 0 && cand < c->n_cand;
     if (is_cand) HD_DISPATCH(c, T, colsum(c, l, seq, n, vis_start, v, c->scores_all + (size_t)cand * imax(f.max_visual, 1)));
+    // the rest of the layer and the next layer's projections, pass by pass (the queries of layer l are done with)
     for (int r0 = 0; r0 < n; r0 += CH) {
       int rows = imin(CH, n - r0);
       float *xr = c->x + (size_t)r0 * d;
       GemmOut g = gemm<T>(c, c->wo[l], (const T *)c->attn_out + (long long)(r0 / CH) * att_chunk, mp, rows, d, c->Hhd);
-      norm_rows<T>(c, xr, g, true, c->ln2[l], rows, mp);
-      g = mlp_rows<T>(c, c->wgu[l], c->wd[l], rows, mp);
+      RowScale norm = norm_rows<T>(c, xr, g, true, c->ln2[l], rows, mp);
+      g = mlp_rows<T>(c, norm, c->wgu[l], c->wd[l], rows, mp);
       float *copy = is_cand ? c->taps_store + ((size_t)cand * f.max_prompt + r0) * d : nullptr;
-      LAUNCH(c, k_resid_add, dim3(rows, (d + 1023) / 1024), 256, 0, xr, g, d, copy);
+      norm = norm_rows<T>(c, xr, g, true, l + 1 < L ? c->ln1[l + 1] : c->ln_f, rows, mp, copy);
+      if (l + 1 < L) qkv(l + 1, r0, rows, norm);
     }
   }
   // first token: LM head on the last prompt row
-  norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
+  const RowScale last = norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
   GemmOut g = gemm<T>(c, c->lm_head, c->xn, mp, 1, f.vocab, d);
-  TOPK_LAUNCH(c, dim3(1, c->tk_nsplit), g, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
+  TOPK_LAUNCH(c, dim3(1, c->tk_nsplit), g, last, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
   LAUNCH(c, k_first_token, 1, 32, 0, c->top_id, c->top_val, first_token, first_margin);
   LAUNCH(c, k_set_seq, 1, 32, 0, c->sd, seq, n, c->top_id, -1, -1);
   LAUNCH(c, k_select_tap, 1, 32, 0, c->ae, f.tap_mode, f.tap_layer, f.tap_lo, f.tap_hi, c->sd.tap + seq, tap_layer);
@@ -977,31 +981,31 @@ static GemmOut draft_rows(dream_ctx *c, const RowMeta &rm, int R, XMode xm, int 
   const dream_draft_weights &w = c->dw;
   const int *vd = vis ? rm.vis_d : nullptr, *vm = vis ? rm.vis_m : nullptr;
   GemmOut g;
-  norm_rows<T>(c, c->x, NO_GEMM, false, w.ln1, R, xm);
+  RowScale norm = norm_rows<T>(c, c->x, NO_GEMM, false, w.ln1, R, xm);
   g = gemm<T>(c, w.wqkv, c->xn, xm, R, c->qkvN, d);
-  LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, rm.seq, rm.pos, rm.dst, 0, 1, c->qbuf, flat(c, c->dself), f.n_heads, c->rope_inv, rope_tab);
+  LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself), f.n_heads, c->rope_inv, rope_tab);
   HD_DISPATCH(c, T, draft(c, rm, c->dself, c->sd.nperm_d, 0, R, xm, B, m, key_ub, vd, tail));
   g = gemm<T>(c, w.wo, c->attn_out, xm, R, d, c->Hhd);
   if (c->three) {
-    norm_rows<T>(c, c->x, g, true, w.i_ln2, R, xm);
-    g = mlp_rows<T>(c, w.i_wgu, w.i_wd, R, xm);
+    norm = norm_rows<T>(c, c->x, g, true, w.i_ln2, R, xm);
+    g = mlp_rows<T>(c, norm, w.i_wgu, w.i_wd, R, xm);
   }
-  norm_rows<T>(c, c->x, g, true, w.lnx, R, xm);
+  norm = norm_rows<T>(c, c->x, g, true, w.lnx, R, xm);
   g = gemm<T>(c, w.xq, c->xn, xm, R, c->Hhd, d);
-  LAUNCH(c, k_gemm_to_q, dim3(R, (c->Hhd + 1023) / 1024), 256, 0, g, c->qbuf, f.n_heads, f.head_dim, sizeof(T) == 2 ? 1 : 0);
+  LAUNCH(c, k_gemm_to_q, dim3(R, (c->Hhd + 1023) / 1024), 256, 0, g, norm, c->qbuf, f.n_heads, f.head_dim, sizeof(T) == 2 ? 1 : 0);
   HD_DISPATCH(c, T, draft(c, rm, c->dmem, c->sd.nperm_m, 1, R, xm, B, m, key_ub, vm, tail));
   g = gemm<T>(c, w.xo, c->attn_out, xm, R, d, c->Hhd);
-  norm_rows<T>(c, c->x, g, true, w.ln2, R, xm);
-  g = mlp_rows<T>(c, w.wgu, w.wd, R, xm);
+  norm = norm_rows<T>(c, c->x, g, true, w.ln2, R, xm);
+  g = mlp_rows<T>(c, norm, w.wgu, w.wd, R, xm);
   if (c->three) {
-    norm_rows<T>(c, c->x, g, true, w.f_ln1, R, xm);
+    norm = norm_rows<T>(c, c->x, g, true, w.f_ln1, R, xm);
     g = gemm<T>(c, w.f_wqkv, c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, rm.seq, rm.pos, rm.dst, 0, 1, c->qbuf, flat(c, c->dself2), f.n_heads, c->rope_inv, rope_tab);
+    LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself2), f.n_heads, c->rope_inv, rope_tab);
     if (context) return g;
     HD_DISPATCH(c, T, draft(c, rm, c->dself2, c->sd.nperm_d, 0, R, xm, B, m, key_ub, vd, tail));
     g = gemm<T>(c, w.f_wo, c->attn_out, xm, R, d, c->Hhd);
-    norm_rows<T>(c, c->x, g, true, w.f_ln2, R, xm);
-    g = mlp_rows<T>(c, w.f_wgu, w.f_wd, R, xm);
+    norm = norm_rows<T>(c, c->x, g, true, w.f_ln2, R, xm);
+    g = mlp_rows<T>(c, norm, w.f_wgu, w.f_wd, R, xm);
   }
   return g;
 }
@@ -1019,9 +1023,9 @@ static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *force
     int rows = imin(CH, nc - r0);
     LAUNCH(c, k_ctx_rows, (rows + 255) / 256, 256, 0, c->ctx_pos + r0, rows, 0, seq, c->rm[0], c->gather_idx, r0, 0);
     LAUNCH(c, (k_gather_rows<float>), rows, 256, 0, c->x0, c->gather_idx, c->x, d, (const int *)nullptr, 0, 0LL, XLayout{d, 0});
-    norm_rows<T>(c, c->x, NO_GEMM, false, c->dw.ln1, rows, m1);
+    const RowScale norm = norm_rows<T>(c, c->x, NO_GEMM, false, c->dw.ln1, rows, m1);
     GemmOut g = gemm<T>(c, wkv, c->xn, m1, rows, c->kvN, d);
-    LAUNCH(c, k_qkv_post_draft, dim3(rows, (c->kvN / 8 + 255) / 256), 256, 0, g, c->rm[0].seq, c->rm[0].pos, c->rm[0].dst, 0, 0, (float *)nullptr,
+    LAUNCH(c, k_qkv_post_draft, dim3(rows, (c->kvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].pos, c->rm[0].dst, 0, (float *)nullptr,
            flat(c, c->dself), f.n_heads, c->rope_inv, (const float2 *)nullptr);
   }
   // cross-attention memory: tapped features at the context positions, projected (Eq. 1)
@@ -1032,7 +1036,7 @@ static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *force
     LAUNCH(c, (k_gather_rows<T>), rows, 256, 0, c->taps_store, c->gather_idx, (T *)c->raw, d, c->sd.tap + seq, c->tap_lo_eff,
            (long long)f.max_prompt * d, xlay(m1, d));
     GemmOut g = gemm<T>(c, c->dw.xkv, c->raw, m1, rows, c->kvN, d);
-    LAUNCH(c, k_mem_append, dim3(rows, (c->kvN + 1023) / 1024), 256, 0, g, c->rm[0].seq, c->rm[0].dst, (const int *)nullptr, (const int *)nullptr, 0, flat(c, c->dmem));
+    LAUNCH(c, k_mem_append, dim3(rows, (c->kvN + 1023) / 1024), 256, 0, g, c->rm[0].seq, c->rm[0].dst, (const int *)nullptr, (const int *)nullptr, flat(c, c->dmem));
   }
   LAUNCH(c, k_set_seq, 1, 32, 0, c->sd, seq, -1, (const int *)nullptr, nc, nm);
   if (c->three) {
@@ -1114,13 +1118,13 @@ static dream_status draft_impl(dream_ctx *c, const TreeBatch &tb, int B) {
     // pass 1 of the three-block draft carries the catch-up rows through every block
     GemmOut g = draft_rows<T>(c, rm, R, xm, B, m, key_ub, c->three && p == 1, true, false, (const float2 *)c->rope_tab);
     // e^M = x: the raw copy feeds the memory projection, the normalised copy the LM head
-    norm_rows<T>(c, c->x, g, true, c->ln_f, R, xm, nullptr, nullptr, nullptr, 0, true);
+    const RowScale norm = norm_rows<T>(c, c->x, g, true, c->ln_f, R, xm, nullptr, nullptr, nullptr, 0, true);
     if (p < ts.D) {     // the last pass's features have no descendants to attend to them
       g = gemm<T>(c, c->dw.xkv, c->raw, xm, R, c->kvN, d);
-      LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, rm.in, c->sd.nperm_m, 0, flat(c, c->dmem));
+      LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, rm.in, c->sd.nperm_m, flat(c, c->dmem));
     }
     g = gemm<T>(c, c->lm_head, c->xn, xm, R, f.vocab, d);
-    TOPK_LAUNCH(c, dim3(R, c->tk_nsplit), g, f.vocab, ts.K, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
+    TOPK_LAUNCH(c, dim3(R, c->tk_nsplit), g, norm, f.vocab, ts.K, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
     int next_m = p < ts.D ? ts.beam[p] : 1;
     LAUNCH(c, k_tree_expand, B, 128, 0, tb, c->sd, c->dt, ts, p, m, c->top_val, c->top_id, c->lse_rows, rn, next_m);
     cur ^= 1;
@@ -1160,17 +1164,17 @@ static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *a
   GemmOut gd = NO_GEMM, g;
   for (int l = 0; l < L; ++l) {
     // the first norm completes S^l (for l >= 1) and captures it where a sequence taps layer l
-    norm_rows<T>(c, c->x, gd, l > 0, c->ln1[l], R, xm, l > 0 ? c->tapbuf : nullptr, rm.seq, c->sd.tap, l);
+    RowScale norm = norm_rows<T>(c, c->x, gd, l > 0, c->ln1[l], R, xm, l > 0 ? c->tapbuf : nullptr, rm.seq, c->sd.tap, l);
     g = gemm<T>(c, c->wqkv[l], c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, rm.seq, rm.pos, rm.slot, 0, c->qbuf, paged(c, l), f.n_heads, c->rope_inv, (const float2 *)c->rope_tab);
+    LAUNCH(c, (k_qkv_post_target<T>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.slot, 0, c->qbuf, paged(c, l), f.n_heads, c->rope_inv, (const float2 *)c->rope_tab);
     HD_DISPATCH(c, T, tree(c, l, R, xm, B, key_ub));
     g = gemm<T>(c, c->wo[l], c->attn_out, xm, R, d, c->Hhd);
-    norm_rows<T>(c, c->x, g, true, c->ln2[l], R, xm);
-    gd = mlp_rows<T>(c, c->wgu[l], c->wd[l], R, xm);
+    norm = norm_rows<T>(c, c->x, g, true, c->ln2[l], R, xm);
+    gd = mlp_rows<T>(c, norm, c->wgu[l], c->wd[l], R, xm);
   }
-  norm_rows<T>(c, c->x, gd, true, c->ln_f, R, xm, c->tapbuf, rm.seq, c->sd.tap, L);
+  const RowScale norm = norm_rows<T>(c, c->x, gd, true, c->ln_f, R, xm, c->tapbuf, rm.seq, c->sd.tap, L);
   g = gemm<T>(c, c->lm_head, c->xn, xm, R, f.vocab, d);
-  TOPK_LAUNCH(c, dim3(R, c->tk_nsplit), g, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, logits);
+  TOPK_LAUNCH(c, dim3(R, c->tk_nsplit), g, norm, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, logits);
   LAUNCH(c, k_argmax_out, (R + 127) / 128, 128, 0, c->top_id, c->top_val, R, argmax, margin,
          argmax == c->argmax_i ? (int *)nullptr : c->argmax_i);
   return DREAM_OK;
@@ -1225,7 +1229,7 @@ static dream_status accept_impl(dream_ctx *c, const TreeBatch &tb, int B, const 
   const XMode xm = xmode(c);
   LAUNCH(c, (k_gather_rows<T>), R, 256, 0, c->tapbuf, c->gather_idx, (T *)c->raw, d, (const int *)nullptr, 0, 0LL, xlay(xm, d));
   GemmOut g = gemm<T>(c, c->dw.xkv, c->raw, xm, R, c->kvN, d);
-  LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, (const int *)nullptr, (const int *)nullptr, 0, flat(c, c->dmem));
+  LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, (const int *)nullptr, (const int *)nullptr, flat(c, c->dmem));
   return DREAM_OK;
 }
 
@@ -1460,7 +1464,7 @@ extern "C" dream_status dream_topk_lse_static(const float *logits, int32_t rows,
   GemmOut g;                                   // a plain [rows][vocab] matrix: one slot, one chunk
   g.base = logits; g.slot_stride = 0; g.ld = vocab; g.kb = 0; g.n_full = 0; g.n_tt = 1; g.inv_upc = g.inv_tile = 0.f;
   int nsplit = (vocab + TOPK_COLS - 1) / TOPK_COLS;
-  k_topk_lse<TOPK_COLS / TOPK_THREADS><<<dim3(rows, nsplit), TOPK_THREADS, 0, stream>>>(g, vocab, ktop, nsplit, ts, top_val, top_id, lse, (float *)nullptr);
+  k_topk_lse<TOPK_COLS / TOPK_THREADS><<<dim3(rows, nsplit), TOPK_THREADS, 0, stream>>>(g, NO_NORM, vocab, ktop, nsplit, ts, top_val, top_id, lse, (float *)nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(nullptr, DREAM_E_CUDA, "k_topk_lse launch: %s", cudaGetErrorString(e));
   return DREAM_OK;

@@ -184,8 +184,13 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
 }
+// Releases nothing: what it hands over is TMEM, ordered by the tcgen05 fences.  (An arrive with release at cluster
+// scope waits until the thread's stores to global memory have been performed, 1.5 us behind an epilogue.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ void cluster_sync_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed;\n barrier.cluster.wait;" ::: "memory");
 }
 // A load into this CTA's shared memory that completes on the pair leader's barrier.
 __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, uint32_t leader_bar, int x, int y, uint64_t policy) {
@@ -220,8 +225,10 @@ template <bool TILES> struct TcWalk {
 
 // ------------------------------------------------------------------------------------------ kernel
 // Dynamic shared memory (1024-byte aligned): W ring [w_stages][wp][16 KB], X ring [x_stages][wp][panel], barriers.
+// Registers: the decode forms are held to 64, so that the row kernel that waits for this launch is resident beside
+// it as a whole (its blocks have started, hence the next GEMM's CTAs can start as soon as these leave).
 template <int FORM>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, FORM >= TC_X_TWO ? 1 : 2)
 k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -438,22 +445,25 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         // the parts of a sum: accumulators, and within each (CONCAT) the high and the low plane's columns
         const int n_part = p.n_sub * (FORM == TC_X_CONCAT ? 2 : 1), part_n = FORM == TC_X_CONCAT ? p.tile_t : p.mma_n;
 #pragma unroll 1
-        for (int t0 = half * 32; t0 < nt; t0 += 64) {
-          float v[32];
+        for (int t0 = half * 16; t0 < nt; t0 += 32) {
+          float v[16];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = 0.f;
+          for (int j = 0; j < 16; ++j) v[j] = 0.f;
 #pragma unroll 1
           for (int i = 0; i < n_part; ++i) {
-            uint32_t r[32];
-            tmem_ld32(taddr + (uint32_t)(i * part_n + t0), r);
+            uint32_t r[16];
+            tmem_ld16(taddr + (uint32_t)(i * part_n + t0), r);
             tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] += __uint_as_float(r[j]);
+            for (int j = 0; j < 16; ++j) v[j] += __uint_as_float(r[j]);
           }
           if (c < p.N) {
+            float *d = dst + (long long)t0 * p.N;
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (t0 + j < nt) dst[(long long)(t0 + j) * p.N] = v[j];
+            for (int j = 0; j < 16; ++j) {
+              if (t0 + j < nt) *d = v[j];
+              d += p.N;
+            }
           }
         }
         tc_fence_before();
@@ -464,7 +474,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   }
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();                          // neither CTA leaves while its peer may still signal it or read its operands
+  cluster_sync_relaxed();                      // neither CTA leaves while its peer may still signal it or read its operands
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
@@ -588,7 +598,8 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   const int xpanel = x_box * 128 * (form >= TC_X_TWO ? 2 : 1);
   p.wp = xpanel <= TC_WPANEL / 2 ? 2 : 1;
   const int xstage = p.wp * xpanel, wstage = p.wp * TC_WPANEL;
-  const int room = pl->max_smem - 2048;
+  // a few KB stay free for the blocks of the row kernel that waits beside this launch (1 KB each)
+  const int room = pl->max_smem - 2048 - 4096;
   p.x_stages = xpanel < TC_WPANEL ? 6 / p.wp : xpanel == TC_WPANEL ? 4 : room / (xstage + wstage);
   p.w_stages = (room - p.x_stages * xstage) / wstage;
   if (p.w_stages > TC_MAX_STAGES) p.w_stages = TC_MAX_STAGES;

@@ -52,66 +52,58 @@ __global__ void k_build_prompt(const T *__restrict__ embed, const T *__restrict_
 }
 
 // ---------------------------------------------------------------------------------------
-// Per row: x += (GEMM output, if any); xn = RMSNorm(x) * gain as the next GEMM's input.
+// RMSNorm in two halves.  k_resid writes x * gain as the next GEMM's input and leaves, per row, the sums
+// of squares of its 128-column pieces; the factor 1 / rms is common to a row, so it commutes with the
+// projection and the GEMM's consumer applies it (row_inv_rms).  No kernel has to wait for a whole row.
+#define SSQ_LD 128                       // pieces per row, d_model <= 16384
+struct RowScale {
+  const float *ssq;                      // [rows][SSQ_LD], or null: the rows are not normalised
+  int parts;
+  float inv_d, eps;
+};
+// Every lane of the warp must take part; the pieces are added in a fixed order.
+__device__ __forceinline__ float row_inv_rms(const RowScale &n, int r, bool on) {
+  float s = 0.f;
+  int i = threadIdx.x & 31;
+  do {
+    s += on && n.ssq && i < n.parts ? n.ssq[(long long)r * SSQ_LD + i] : 0.f;
+    i += 32;
+  } while (i < n.parts);
+  s = warp_sum(s);
+  return n.ssq ? rsqrtf(s * n.inv_d + n.eps) : 1.f;
+}
+
+// Per row: x += (GEMM output, if any); xn = x * gain as the next GEMM's input, ssq as above.
 // Optional side outputs of the updated residual: `copy` (fp32; when tap_state is given the
 // row is copied only if its sequence's tap layer equals `layer`) and `raw` (element type,
 // unnormalised: the memory side of Eq. 1 takes features without a norm).
-// Block size: ceil(d / 4 / NV) threads rounded up to a warp (at most 1024); a thread keeps NV
-// groups of four elements, so rows of up to 4096 * NV elements fit.  The partial-sum slots of a
-// value are all fetched at once (up to 12 per round trip).
-template <typename T, int NV>
-__global__ void __launch_bounds__(1024)
-k_resid_norm(float *x, GemmOut gin, int has_in, const T *__restrict__ gain,
-             float eps, int d, T *xn, float *copy, const int *row_seq,
-             const int *tap_state, int layer, T *raw, XLayout lay) {
-  __shared__ float sh[33];
-  const int r = blockIdx.x, d4 = d >> 2, nt = blockDim.x;
+// grid (ceil(d / 1024), rows), a thread per four columns.  Blocks of 256 threads and 56 registers without
+// shared memory, so that they are resident beside a GEMM's CTA before it ends and the next GEMM's CTAs start
+// filling their rings when it does; a block of 1024 threads per row kept those out until the norm was done.
+template <typename T>
+__global__ void __launch_bounds__(256, 5)
+k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, int d, T *xn, float *copy, const int *row_seq,
+        const int *tap_state, int layer, T *raw, XLayout lay, float *ssq) {
+  pdl_trigger();
+  const int r = blockIdx.y, i = (blockIdx.x * 256 + threadIdx.x) * 4;
   // the gains are weights: they can be fetched before the predecessor has finished
-  float4 gq[NV];
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    int i = threadIdx.x + j * nt;
-    gq[j] = (xn && i < d4) ? ld_f4(gain + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  kernel_entry(TR_k_resid_norm);
-  float *xr = x + (long long)r * d;
-  float4 v[NV];
-  float ss = 0.f;
-  // every load of the row is issued before the first use
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    int i = threadIdx.x + j * nt;
-    v[j] = i < d4 ? ld_f4(xr + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  if (has_in) {
-    float4 gv[NV];
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      int i = threadIdx.x + j * nt;
-      gv[j] = i < d4 ? gemm_val4_wide<12 / NV>(gin, r, 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 g = xn && i < d ? ld_f4(gain + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 *xr = reinterpret_cast<float4 *>(x + (long long)r * d + i);
+#pragma unroll 1
+  for (int pass = warm_first(); pass < 2; ++pass) {
+    const bool on = warm_pass(pass, TR_k_resid) && i < d;
+    float4 v = on ? *xr : make_float4(0.f, 0.f, 0.f, 0.f);
+    bool do_copy = copy != nullptr && on;
+    if (tap_state && do_copy) do_copy = tap_state[row_seq[r]] == layer;
+    if (has_in) {
+      add4(v, gemm_val4<5>(gin, r, i, on));
+      if (on) *xr = v;
     }
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      int i = threadIdx.x + j * nt;
-      v[j].x += gv[j].x; v[j].y += gv[j].y; v[j].z += gv[j].z; v[j].w += gv[j].w;
-      if (i < d4) *reinterpret_cast<float4 *>(xr + 4 * i) = v[j];
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < NV; ++j) ss += v[j].x * v[j].x + v[j].y * v[j].y + v[j].z * v[j].z + v[j].w * v[j].w;
-  float tot = block_sum(ss, sh);
-  float inv = rsqrtf(tot / (float)d + eps);
-  bool do_copy = copy != nullptr && (tap_state == nullptr || tap_state[row_seq[r]] == layer);
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    int i = threadIdx.x + j * nt;
-    if (i >= d4) continue;
-    float4 t = v[j];
-    if (do_copy) *reinterpret_cast<float4 *>(copy + (long long)r * d + 4 * i) = t;
-    if (raw) store_split4<T>(raw + r * lay.row_stride + 4 * i, lay.lo_delta, t);
-    if (xn)
-      store_split4<T>(xn + r * lay.row_stride + 4 * i, lay.lo_delta,
-                      make_float4(t.x * inv * gq[j].x, t.y * inv * gq[j].y, t.z * inv * gq[j].z, t.w * inv * gq[j].w));
+    const float ss = warp_sum(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
+    if (on && (threadIdx.x & 31) == 0) ssq[(long long)r * SSQ_LD + (i >> 7)] = ss;
+    if (do_copy) *reinterpret_cast<float4 *>(copy + (long long)r * d + i) = v;
+    if (on && raw) store_split4<T>(raw + r * lay.row_stride + i, lay.lo_delta, v);
+    if (on && xn) store_split4<T>(xn + r * lay.row_stride + i, lay.lo_delta, make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
   }
 }
 
@@ -155,42 +147,47 @@ struct PagedKV {
   }
 };
 
+// Rotary on four neighbouring pairs (a: columns i.., b: columns i + half..).
+__device__ __forceinline__ void rotate4(float4 &a, float4 &b, const float4 &cs01, const float4 &cs23) {
+  const float c0 = cs01.x, s0 = cs01.y, c1 = cs01.z, s1 = cs01.w, c2 = cs23.x, s2 = cs23.y, c3 = cs23.z, s3 = cs23.w;
+  const float4 ra = make_float4(a.x * c0 - b.x * s0, a.y * c1 - b.y * s1, a.z * c2 - b.z * s2, a.w * c3 - b.w * s3);
+  b = make_float4(b.x * c0 + a.x * s0, b.y * c1 + a.y * s1, b.z * c2 + a.z * s2, b.w * c3 + a.w * s3);
+  a = ra;
+}
+
 // After the QKV GEMM of target rows: rotary on q and k at row_pos, q -> qbuf (fp32),
 // k, v -> the paged cache at (row_seq, row_slot).  grid (rows, ceil(items / 256)); a work item
 // is four neighbouring rotary pairs of one head, read and written as 128-bit words.
 template <typename T>
-__global__ void k_qkv_post_target(GemmOut g, const int *__restrict__ row_seq,
-                                  const int *__restrict__ row_pos, const int *__restrict__ row_slot,
-                                  int row0, void *qbuf, PagedKV kv, int H, const double *__restrict__ inv_freq,
-                                  const float2 *__restrict__ rope_tab) {
-  kernel_entry(TR_k_qkv_post_target);
-  int r = blockIdx.x + row0, lr = blockIdx.x;
-  int hd = kv.hd, half = hd >> 1, q4 = half >> 2, Hkv = kv.hkv;
-  int w = blockIdx.y * blockDim.x + threadIdx.x;
-  if (w >= (H + 2 * Hkv) * q4) return;
-  int hh = w / q4, i = (w - hh * q4) * 4;
-  int seq = row_seq[r], pos = row_pos[r], slot = row_slot[r];
-  if (hh >= H && slot < 0) return;                 // an idle row (malformed tree node) stores no K/V
-  T *Kp = (T *)kv.base, *Vp = (T *)kv.base + kv.kv_stride;
-  float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
-  if (hh < H + Hkv) rope_cs4(rope_tab, r, half, pos, inv_freq, i, cs01, cs23);      // fetched along with the slots
-  float4 a = gemm_val4_wide<4>(g, lr, hh * hd + i), b = gemm_val4_wide<4>(g, lr, hh * hd + i + half);
-  if (hh < H + Hkv) {
-    const float c0 = cs01.x, s0 = cs01.y, c1 = cs01.z, s1 = cs01.w, c2 = cs23.x, s2 = cs23.y, c3 = cs23.z, s3 = cs23.w;
-    float4 ra = make_float4(a.x * c0 - b.x * s0, a.y * c1 - b.y * s1, a.z * c2 - b.z * s2, a.w * c3 - b.w * s3);
-    float4 rb = make_float4(b.x * c0 + a.x * s0, b.y * c1 + a.y * s1, b.z * c2 + a.z * s2, b.w * c3 + a.w * s3);
+__global__ void __launch_bounds__(256)
+k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_slot,
+                  int row0, void *qbuf, PagedKV kv, int H, const double *__restrict__ inv_freq, const float2 *__restrict__ rope_tab) {
+  pdl_trigger();
+  const int r = blockIdx.x + row0, lr = blockIdx.x;
+  const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv;     // hd / 8 items per head
+  const int w = blockIdx.y * 256 + threadIdx.x, hh = w >> q4_log2, i = (w - (hh << q4_log2)) * 4;
+#pragma unroll 1
+  for (int pass = warm_first(); pass < 2; ++pass) {
+    const bool live = warm_pass(pass, TR_k_qkv_post_target);
+    bool on = live && hh < H + 2 * Hkv;
+    const int seq = on ? row_seq[r] : 0, pos = on ? row_pos[r] : 0, slot = on ? row_slot[r] : 0;
+    if (hh >= H && slot < 0) on = false;               // an idle row (malformed tree node) stores no K/V
+    float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
+    if (on && hh < H + Hkv) rope_cs4(rope_tab, r, half, pos, inv_freq, i, cs01, cs23);      // fetched along with the slots
+    const float inv = row_inv_rms(norm, lr, live);
+    float4 a = gemm_val4<3>(g, lr, hh * hd + i, on), b = gemm_val4<3>(g, lr, hh * hd + i + half, on);
+    scale4(a, inv); scale4(b, inv);
+    rotate4(a, b, cs01, cs23);
+    if (!on) continue;
     if (hh < H) {
-      q_store4(qbuf, sizeof(T) == 2, (long long)r * H + hh, hd, i, ra);
-      q_store4(qbuf, sizeof(T) == 2, (long long)r * H + hh, hd, i + half, rb);
+      q_store4(qbuf, sizeof(T) == 2, (long long)r * H + hh, hd, i, a);
+      q_store4(qbuf, sizeof(T) == 2, (long long)r * H + hh, hd, i + half, b);
     } else {
-      long long o = kv.off(seq, slot, hh - H);
-      store_split4<T>(Kp + o + i, 0, ra);
-      store_split4<T>(Kp + o + i + half, 0, rb);
+      const int v = hh >= H + Hkv ? 1 : 0;
+      T *dst = (T *)kv.base + (v ? kv.kv_stride : 0) + kv.off(seq, slot, hh - H - (v ? Hkv : 0)) + i;
+      store_split4<T>(dst, 0, a);
+      store_split4<T>(dst + half, 0, b);
     }
-  } else {
-    long long o = kv.off(seq, slot, hh - H - Hkv);
-    store_split4<T>(Vp + o + i, 0, a);
-    store_split4<T>(Vp + o + i + half, 0, b);
   }
 }
 
@@ -212,95 +209,93 @@ struct FlatKV {
 // After a draft QKV GEMM (has_q: the GEMM produced q columns first, then K, then V; otherwise
 // K then V only): rotary, q -> qbuf (when has_q), k/v -> draft self-attention cache row
 // row_dst[r] (skipped when < 0).  Work items and grid as in k_qkv_post_target.
-__global__ void k_qkv_post_draft(GemmOut g, const int *__restrict__ row_seq,
-                                 const int *__restrict__ row_pos, const int *__restrict__ row_dst,
-                                 int row0, int has_q, void *qbuf, FlatKV kv, int H, const double *__restrict__ inv_freq,
-                                 const float2 *__restrict__ rope_tab) {
-  kernel_entry(TR_k_qkv_post_draft);
-  int r = blockIdx.x + row0, lr = blockIdx.x;
-  int hd = kv.hd, half = hd >> 1, q4 = half >> 2, Hkv = kv.hkv;
-  int Hq = has_q ? H : 0;
-  int w = blockIdx.y * blockDim.x + threadIdx.x;
-  if (w >= (Hq + 2 * Hkv) * q4) return;
-  int hh = w / q4, i = (w - hh * q4) * 4;
-  int dst = row_dst[r], seq = row_seq[r], pos = row_pos[r];
-  if (hh >= Hq && dst < 0) return;
-  float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
-  if (hh < Hq + Hkv) rope_cs4(rope_tab, r, half, pos, inv_freq, i, cs01, cs23);
-  float4 a = gemm_val4_wide<4>(g, lr, hh * hd + i), b = gemm_val4_wide<4>(g, lr, hh * hd + i + half);
-  if (hh < Hq + Hkv) {
-    const float c0 = cs01.x, s0 = cs01.y, c1 = cs01.z, s1 = cs01.w, c2 = cs23.x, s2 = cs23.y, c3 = cs23.z, s3 = cs23.w;
-    float4 ra = make_float4(a.x * c0 - b.x * s0, a.y * c1 - b.y * s1, a.z * c2 - b.z * s2, a.w * c3 - b.w * s3);
-    float4 rb = make_float4(b.x * c0 + a.x * s0, b.y * c1 + a.y * s1, b.z * c2 + a.z * s2, b.w * c3 + a.w * s3);
+__global__ void __launch_bounds__(256)
+k_qkv_post_draft(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_dst,
+                 int has_q, void *qbuf, FlatKV kv, int H, const double *__restrict__ inv_freq, const float2 *__restrict__ rope_tab) {
+  pdl_trigger();
+  const int r = blockIdx.x;
+  const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv, Hq = has_q ? H : 0;
+  const int w = blockIdx.y * 256 + threadIdx.x, hh = w >> q4_log2, i = (w - (hh << q4_log2)) * 4;
+#pragma unroll 1
+  for (int pass = warm_first(); pass < 2; ++pass) {
+    const bool live = warm_pass(pass, TR_k_qkv_post_draft);
+    bool on = live && hh < Hq + 2 * Hkv;
+    const int dst = on ? row_dst[r] : 0, seq = on ? row_seq[r] : 0, pos = on ? row_pos[r] : 0;
+    if (hh >= Hq && dst < 0) on = false;
+    float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
+    if (on && hh < Hq + Hkv) rope_cs4(rope_tab, r, half, pos, inv_freq, i, cs01, cs23);
+    const float inv = row_inv_rms(norm, r, live);
+    float4 a = gemm_val4<3>(g, r, hh * hd + i, on), b = gemm_val4<3>(g, r, hh * hd + i + half, on);
+    scale4(a, inv); scale4(b, inv);
+    rotate4(a, b, cs01, cs23);
+    if (!on) continue;
     if (hh < Hq) {
-      q_store4(qbuf, kv.split, (long long)r * H + hh, hd, i, ra);
-      q_store4(qbuf, kv.split, (long long)r * H + hh, hd, i + half, rb);
+      q_store4(qbuf, kv.split, (long long)r * H + hh, hd, i, a);
+      q_store4(qbuf, kv.split, (long long)r * H + hh, hd, i + half, b);
     } else {
-      long long o = kv.off(seq, 0, hh - Hq, dst);
-      kv.store4(o, i, ra);
-      kv.store4(o, i + half, rb);
+      const int v = hh >= Hq + Hkv ? 1 : 0;
+      const long long o = kv.off(seq, v, hh - Hq - (v ? Hkv : 0), dst);
+      kv.store4(o, i, a);
+      kv.store4(o, i + half, b);
     }
-  } else {
-    long long o = kv.off(seq, 1, hh - Hq - Hkv, dst);
-    kv.store4(o, i, a);
-    kv.store4(o, i + half, b);
   }
 }
 
 // A GEMM output [rows][H * hd] becomes the query rows of the cross-attention (no rotary).
 // grid (rows, ceil(H * hd / 1024)).
-__global__ void k_gemm_to_q(GemmOut g, void *qbuf, int H, int hd, int split) {
-  kernel_entry(TR_k_gemm_to_q);
-  int r = blockIdx.x, i = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
-  if (i >= H * hd) return;
-  int h = i / hd;
-  q_store4(qbuf, split, (long long)r * H + h, hd, i - h * hd, gemm_val4(g, r, i));
+__global__ void __launch_bounds__(256)
+k_gemm_to_q(GemmOut g, RowScale norm, void *qbuf, int H, int hd, int split) {
+  pdl_trigger();
+  const int r = blockIdx.x, i = (blockIdx.y * 256 + threadIdx.x) * 4, hd_log2 = 31 - __clz(hd), h = i >> hd_log2;
+#pragma unroll 1
+  for (int pass = warm_first(); pass < 2; ++pass) {
+    const bool live = warm_pass(pass, TR_k_gemm_to_q), on = live && h < H;
+    const float inv = row_inv_rms(norm, r, live);
+    float4 v = gemm_val4<6>(g, r, i, on);
+    scale4(v, inv);
+    if (on) q_store4(qbuf, split, (long long)r * H + h, hd, i - (h << hd_log2), v);
+  }
 }
 
 // Cross-attention memory rows (Eq. 1: K = S W_K, V = S W_V): GEMM output [rows][2 H_kv hd]
 // -> memory cache row of sequence row_seq[r]: row_dst[r] when nperm is null, else the
 // tree-region row nperm[seq] + row_in[r].  Negative indices skip the row.
 // grid (rows, ceil(2 H_kv hd / 1024)).
-__global__ void k_mem_append(GemmOut g, const int *__restrict__ row_seq,
-                             const int *__restrict__ row_dst, const int *__restrict__ row_in,
-                             const int *__restrict__ nperm, int row0, FlatKV kv) {
-  kernel_entry(TR_k_mem_append);
-  int r = blockIdx.x + row0, lr = blockIdx.x;
-  int seq = row_seq[r];
-  int dst = nperm ? (row_in[r] < 0 ? -1 : nperm[seq] + row_in[r]) : row_dst[r];
-  if (dst < 0) return;
-  int w = kv.hkv * kv.hd;
-  int i = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
-  if (i >= 2 * w) return;
-  int which = i >= w ? 1 : 0, j = i - which * w;
-  int h = j / kv.hd, e = j - h * kv.hd;
-  kv.store4(kv.off(seq, which, h, dst), e, gemm_val4(g, lr, i));
+__global__ void __launch_bounds__(256)
+k_mem_append(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__ row_dst, const int *__restrict__ row_in,
+             const int *__restrict__ nperm, FlatKV kv) {
+  pdl_trigger();
+  const int r = blockIdx.x, i = (blockIdx.y * 256 + threadIdx.x) * 4, hd_log2 = 31 - __clz(kv.hd), hh = i >> hd_log2;
+#pragma unroll 1
+  for (int pass = warm_first(); pass < 2; ++pass) {
+    bool on = warm_pass(pass, TR_k_mem_append) && hh < 2 * kv.hkv;
+    const int seq = on ? row_seq[r] : 0;
+    int dst = on ? (nperm ? row_in : row_dst)[r] : 0;
+    if (dst < 0) on = false;
+    if (nperm && on) dst += nperm[seq];
+    const float4 v = gemm_val4<6>(g, r, i, on);
+    const int which = hh >= kv.hkv ? 1 : 0;
+    if (on) kv.store4(kv.off(seq, which, hh - which * kv.hkv, dst), i - (hh << hd_log2), v);
+  }
 }
 
 // act = silu(gate) * up, from a GEMM output whose columns are [gate(ff) | up(ff)].
 // grid (ceil(ff / 1024), rows).
 template <typename T>
-__global__ void k_silu_mul(GemmOut g, T *act, int ff, XLayout lay) {
-  kernel_entry(TR_k_silu_mul);
-  int r = blockIdx.y;
-  int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (i >= ff) return;
-  float4 a = gemm_val4(g, r, i), b = gemm_val4(g, r, ff + i);
-  float4 o = make_float4(a.x / (1.f + __expf(-a.x)) * b.x, a.y / (1.f + __expf(-a.y)) * b.y,
-                         a.z / (1.f + __expf(-a.z)) * b.z, a.w / (1.f + __expf(-a.w)) * b.w);
-  store_split4<T>(act + r * lay.row_stride + i, lay.lo_delta, o);
-}
-
-// x += GEMM output; optional fp32 copy into a per-layer store (prefill tap candidates).
-// grid (rows, ceil(d / 1024)).
-__global__ void k_resid_add(float *x, GemmOut g, int d, float *copy) {
-  kernel_entry(TR_k_resid_add);
-  int r = blockIdx.x, i = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
-  if (i >= d) return;
-  float4 v = ld_f4(x + (long long)r * d + i), t = gemm_val4(g, r, i);
-  v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
-  *reinterpret_cast<float4 *>(x + (long long)r * d + i) = v;
-  if (copy) *reinterpret_cast<float4 *>(copy + (long long)r * d + i) = v;
+__global__ void __launch_bounds__(256, 8)
+k_silu_mul(GemmOut g, RowScale norm, T *act, int ff, XLayout lay) {
+  pdl_trigger();
+  const int r = blockIdx.y, i = (blockIdx.x * 256 + threadIdx.x) * 4;
+#pragma unroll 1
+  for (int pass = warm_first(); pass < 2; ++pass) {
+    const bool live = warm_pass(pass, TR_k_silu_mul), on = live && i < ff;
+    const float inv = row_inv_rms(norm, r, live);
+    float4 a = gemm_val4<2>(g, r, i, on), b = gemm_val4<2>(g, r, ff + i, on);
+    scale4(a, inv); scale4(b, inv);
+    const float4 o = make_float4(a.x / (1.f + __expf(-a.x)) * b.x, a.y / (1.f + __expf(-a.y)) * b.y,
+                                 a.z / (1.f + __expf(-a.z)) * b.z, a.w / (1.f + __expf(-a.w)) * b.w);
+    if (on) store_split4<T>(act + r * lay.row_stride + i, lay.lo_delta, o);
+  }
 }
 
 // Gather fp32 rows into element-type GEMM input rows: dst[r] = src[idx[r]] (idx < 0 -> zeros).
@@ -392,7 +387,7 @@ __device__ __forceinline__ void topk_rounds(const float (&v)[NV], const int (&id
 
 template <int NV>
 __global__ void __launch_bounds__(TOPK_THREADS)
-k_topk_lse(GemmOut g, int V, int ktop, int nsplit, TopkScratch ts, float *top_val, int *top_id, float *lse,
+k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts, float *top_val, int *top_id, float *lse,
            float *logits_out) {
   __shared__ float red[33];
   __shared__ float sh_v[TOPK_THREADS / 32 * TOPK_MAX];
@@ -403,12 +398,15 @@ k_topk_lse(GemmOut g, int V, int ktop, int nsplit, TopkScratch ts, float *top_va
   int c0 = sp * (NV * TOPK_THREADS);
   float v[NV];
   int id[NV];
+  const float inv = row_inv_rms(norm, r, true);
   if ((V & 3) == 0) {
     float4 q[NV / 4];
 #pragma unroll
     for (int j = 0; j < NV / 4; ++j) {
       int c = c0 + (j * TOPK_THREADS + tid) * 4;
-      q[j] = c < V ? gemm_val4(g, r, c) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      q[j] = gemm_val4<2>(g, r, c, c < V);
+      scale4(q[j], inv);
+      if (c >= V) q[j] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
     }
 #pragma unroll
     for (int j = 0; j < NV / 4; ++j) {
@@ -421,7 +419,7 @@ k_topk_lse(GemmOut g, int V, int ktop, int nsplit, TopkScratch ts, float *top_va
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       int c = c0 + j * TOPK_THREADS + tid;
-      v[j] = c < V ? gemm_val(g, r, c) : -INFINITY;
+      v[j] = c < V ? gemm_val(g, r, c) * inv : -INFINITY;
       id[j] = c;
       if (logits_out && c < V) logits_out[(long long)r * V + c] = v[j];
     }
