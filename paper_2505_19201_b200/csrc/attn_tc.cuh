@@ -5,25 +5,27 @@
 // A CTA owns one tile of 64 query entries (entry = (row, query head of one KV-head group)), one KV
 // head and one chunk of keys.  Queries carry ~16 mantissa bits as a high and a low bf16 row, so
 // the tile is the MMA's M = 128: row 2e = high part of entry e, row 2e + 1 = its low part; the two
-// accumulator lanes of an entry are added with one shuffle.  Keys are walked in blocks of 64,
-// GROUP blocks (one group) at a time:
-//   S = Q K^T            one chain of tcgen05.mma 128 x (64 x blocks) x 16 over head_dim for the whole
-//                        group, A = Q and B = K from shared memory (K-major, 128-byte swizzle,
-//                        TMA-fed; the group's K blocks are contiguous), fp32 accumulators in TMEM;
-//   softmax              four warps, one TMEM lane per thread; the two lanes of an entry split each
-//                        32-key piece between them.  A first pass over the group's S for the row
-//                        maximum, a second pass for P = 2^(s - m) (masked) and the row sum; P's high
-//                        bf16 part goes to the entry's even row and its low part to the odd row of a
-//                        shared-memory tile in the operand layout.  Between groups the O accumulator
-//                        is rescaled in TMEM (tcgen05.ld / tcgen05.st);
-//   O += P_b V_b         tcgen05.mma 128 x head_dim x 16 steps over each block's keys, A = P_b (K-major)
+// accumulator lanes of an entry are added with one shuffle.  Keys are walked in blocks of 64:
+//   S_b = Q K_b^T        tcgen05.mma 128 x 64 x 16 over head_dim, A = Q and B = K_b from shared memory
+//                        (K-major, 128-byte swizzle, TMA-fed), fp32 accumulators in a TMEM ring, up to
+//                        AHEAD blocks ahead of the softmax;
+//   softmax              eight warps, one TMEM lane per thread: two warps share a lane quarter and take 32 of
+//                        the block's keys each, the two lanes of an entry 16 each.  One pass: the block's row
+//                        maximum (the two warps exchange theirs through shared memory), then
+//                        P = 2^(s - m), its row sum, and P's high bf16 part to the entry's even row and its low
+//                        part to the odd row of a shared-memory tile in the operand layout.  m is any reference
+//                        near the maximum: it follows the maximum only when that has outgrown it by 2^8, so
+//                        the O accumulator is hardly ever rescaled (in TMEM, tcgen05.ld / tcgen05.st);
+//   O += P_b V_b         tcgen05.mma 128 x head_dim x 16 steps over the block's keys, A = P_b (K-major)
 //                        and B = V_b as stored ([key][head_dim]: an MN-major operand).
 // K/V blocks arrive through two TMA rings; during verification the blocks below the verified prefix
 // length are requested before the grid dependency resolves.  Flat draft caches carry a low plane
 // per key, which costs one more MMA per step.  A chunk leaves (m, l, O) partials for
 // k_attn_combine, or the finished rows (and, for the prefill, each row's log-sum-exp and entropy)
-// when it is the only chunk.  Warp roles: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..5 =
-// softmax and epilogue.  The softmax loops are kept compact on purpose: this kernel's code is
+// when it is the only chunk.  Warp roles: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..9 =
+// softmax and epilogue.  What bounds it is the softmax's instruction latency: with four warps (one per
+// scheduler) and two passes over S a block of 64 keys took 2.0 us of a LLaVA-7B-shaped verify launch.
+// The loops are kept compact on purpose: this kernel's code is
 // fetched anew at almost every launch (the weight stream between two launches pushes it out of the
 // caches), and straight-line code then costs its own fetch (a fully unrolled version of the same
 // loops ran four times slower).  Every mbarrier wait is bounded; on expiry the kernel raises the
@@ -37,7 +39,8 @@
 #include "gemm_tc.cuh"
 #include "rows.cuh"
 
-#define AT_THREADS 192
+#define AT_THREADS 320
+#define AT_RESCALE 8.f                 // the maximum may outgrow its reference by this power of two
 #define AT_KBLK 64
 #define AT_QTILE (128 * 64 * 2)        // one 64-column panel of the query tile (128 rows)
 #define AT_KVTILE (64 * 64 * 2)        // one 64-column panel of a 64-key block
@@ -45,21 +48,22 @@
 
 enum { AT_VERIFY = 0, AT_DRAFT = 1, AT_PREFILL = 2 };
 
-// Blocks per group: what the shared-memory rings (K and V blocks stay until their MMAs ran) and
-// the 512 TMEM columns (head_dim for O, 64 per S_b) hold.
+// Ring depths: what shared memory (K and V blocks stay until their MMAs ran) and the TMEM columns
+// (head_dim for O, 64 per S_b) hold.
 template <int HD, bool FLAT> struct AtShape {
   static constexpr int PLANES = FLAT ? 2 : 1;
   // head_dim 64 over the paged cache takes three blocks, so that O and S fit 256 TMEM columns and two
   // CTAs share an SM (98 KB of shared memory each): twice the key chunks in flight per layer
-  // head_dim 128 over the paged cache takes five (231 KB of the 227 KiB a CTA may hold, 448 TMEM columns):
-  // prefixes up to 1280 keys then stay one group per chunk when the sequence is cut four ways
-  static constexpr int GROUP = HD == 64 ? (FLAT ? 4 : 3) : (HD == 128 ? (FLAT ? 2 : 5) : (FLAT ? 1 : 2));
-  static constexpr int TMEM_COLS = HD + GROUP * 64 <= 256 ? 256 : 512;
+  static constexpr int STAGES = HD == 64 ? (FLAT ? 4 : 3) : (HD == 128 ? (FLAT ? 2 : 5) : (FLAT ? 1 : 2));   // K (and V) blocks
+  static constexpr int S_BUFS = HD == 64 ? 3 : 4;                    // S blocks in TMEM
+  // S blocks issued before the first O: with more than STAGES the K ring would wait for V blocks to be freed, which wait for O
+  static constexpr int AHEAD = S_BUFS < STAGES ? S_BUFS : STAGES;
+  static constexpr int TMEM_COLS = HD + S_BUFS * 64 <= 256 ? 256 : 512;
   static constexpr int CTAS_PER_SM = HD == 64 && !FLAT ? 2 : 1;
   static constexpr int KP = HD / 64;                                 // 64-column panels per row
   static constexpr int KV_STAGE = PLANES * KP * AT_KVTILE;           // one block of K (or of V)
   static constexpr int Q_BYTES = KP * AT_QTILE;
-  static constexpr size_t SMEM = 1024 + Q_BYTES + 2 * GROUP * KV_STAGE + 2 * AT_PTILE + 1024;
+  static constexpr size_t SMEM = 1024 + Q_BYTES + 2 * STAGES * KV_STAGE + 2 * AT_PTILE + 1024 + 384;
 };
 
 struct AttnTcArgs {
@@ -127,30 +131,38 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t saddr, uint32_t lbo_by
   return d;
 }
 
+// 2^x for x <= 8 or so, subnormal results as zero.
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ void bar_sync_pair(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+
 template <int HD, bool FLAT>
 __global__ void __launch_bounds__(AT_THREADS, (AtShape<HD, FLAT>::CTAS_PER_SM))
 k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
           const __grid_constant__ AttnTcArgs a) {
   using Sh = AtShape<HD, FLAT>;
-  constexpr int GROUP = Sh::GROUP, KP = Sh::KP, PLANES = Sh::PLANES;
+  constexpr int STAGES = Sh::STAGES, S_BUFS = Sh::S_BUFS, AHEAD = Sh::AHEAD, KP = Sh::KP, PLANES = Sh::PLANES;
   extern __shared__ uint8_t at_smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)at_smem_raw + 1023) & ~(uintptr_t)1023);
-  uint8_t *q_s = smem, *k_s = q_s + Sh::Q_BYTES, *v_s = k_s + GROUP * Sh::KV_STAGE, *p_s = v_s + GROUP * Sh::KV_STAGE;
-  uint64_t *bars = (uint64_t *)(p_s + 2 * AT_PTILE);
-  uint64_t *q_full = bars, *k_full = q_full + 1, *k_empty = k_full + 8, *v_full = k_empty + 8, *v_empty = v_full + 8;
-  uint64_t *s_full = v_empty + 8, *s_free = s_full + 8, *p_full = s_free + 8, *p_empty = p_full + 2, *o_done = p_empty + 2;
-  uint32_t *tmem_base_p = (uint32_t *)(o_done + 1);
+  uint8_t *q_s = smem, *k_s = q_s + Sh::Q_BYTES, *v_s = k_s + STAGES * Sh::KV_STAGE, *p_s = v_s + STAGES * Sh::KV_STAGE;
+  float *mx_s = (float *)(p_s + 2 * AT_PTILE);                // [2 buffers][2 halves][64 entries]: exchange between the two warps of a quarter
+  uint64_t *bars = (uint64_t *)(mx_s + 256);
+  uint64_t *q_full = bars, *k_full = q_full + 1, *k_empty = k_full + STAGES, *v_full = k_empty + STAGES, *v_empty = v_full + STAGES;
+  uint64_t *s_full = v_empty + STAGES, *s_free = s_full + S_BUFS, *p_full = s_free + S_BUFS, *p_empty = p_full + 2;
+  uint32_t *tmem_base_p = (uint32_t *)(p_empty + 2);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   const int chunk = blockIdx.x, kvh = blockIdx.y / a.n_rt, rt = blockIdx.y - kvh * a.n_rt, slot = blockIdx.z;
   const int seq = a.slot_seq[slot];
   if (warp == 0) {      // a lane per ring stage: the set-up is a few instructions deep instead of a loop
-    if (lane < GROUP) {
-      mbar_init(k_full + lane, 1); mbar_init(k_empty + lane, 1); mbar_init(v_full + lane, 1); mbar_init(v_empty + lane, 1);
-      mbar_init(s_full + lane, 1); mbar_init(s_free + lane, 4);
-    } else if (lane >= 8 && lane < 10) { mbar_init(p_full + lane - 8, 4); mbar_init(p_empty + lane - 8, 1); }
-    else if (lane == 16) { mbar_init(q_full, 1); mbar_init(o_done, 1); *abort_flag = 0; }
+    if (lane < STAGES) { mbar_init(k_full + lane, 1); mbar_init(k_empty + lane, 1); mbar_init(v_full + lane, 1); mbar_init(v_empty + lane, 1); }
+    else if (lane >= 8 && lane < 8 + S_BUFS) { mbar_init(s_full + lane - 8, 1); mbar_init(s_free + lane - 8, 8); }
+    else if (lane >= 16 && lane < 18) { mbar_init(p_full + lane - 16, 8); mbar_init(p_empty + lane - 16, 1); }
+    else if (lane == 24) { mbar_init(q_full, 1); *abort_flag = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -162,6 +174,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_p;
+  auto give_up = [&]() { if (lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } };
   // Verification reads the verified prefix and its length, which were written rounds ago (hundreds
   // of kernels back in the stream): its K/V blocks below the prefix length are fetched before the
   // grid dependency resolves.  Everything else is an output of the immediate predecessors.
@@ -184,40 +197,32 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   const int b0 = chunk * a.blocks_per_chunk, b1 = min(nb, b0 + a.blocks_per_chunk);
   const int n_blk = max(0, b1 - b0);
 
-  // K and V of the chunk's block `it` into ring stage it % GROUP (the whole producer warp)
+  // K (which = 0) or V (1) of the chunk's block `it` into ring stage `st` (the whole producer warp)
   const uint64_t pol_kv = policy_evict_first();
-  auto issue_kv = [&](int it) {
-    const int st = it % GROUP, j0 = (b0 + it) * AT_KBLK;
-    // K: [plane][panel][stage][64 keys], so the blocks of a group form one operand of 64 x blocks keys
-    uint8_t *kd = k_s + st * AT_KVTILE, *vd = v_s + st * Sh::KV_STAGE;
-    constexpr int KSTEP = GROUP * AT_KVTILE;                 // bytes between consecutive (plane, panel) of K
-    if (elect_one()) { mbar_expect_tx(k_full + st, (uint32_t)Sh::KV_STAGE); mbar_expect_tx(v_full + st, (uint32_t)Sh::KV_STAGE); }
+  auto issue = [&](int which, int it, int st) {
+    const int j0 = (b0 + it) * AT_KBLK;
+    uint8_t *dst = (which ? v_s : k_s) + st * Sh::KV_STAGE;
+    uint64_t *full = (which ? v_full : k_full) + st;
+    const CUtensorMap *map = which ? &map_v : &map_k;
+    if (elect_one()) mbar_expect_tx(full, (uint32_t)Sh::KV_STAGE);
     if (FLAT) {
       // rows of the map: (sequence, K | V, KV head, key); the second coordinate selects the plane
-      const long long rk = (((long long)seq * 2 + 0) * a.hkv + kvh) * a.flat_rows_per_head + j0;
-      const long long rv = (((long long)seq * 2 + 1) * a.hkv + kvh) * a.flat_rows_per_head + j0;
+      const long long rk = (((long long)seq * 2 + which) * a.hkv + kvh) * a.flat_rows_per_head + j0;
       if (elect_one())
-        for (int pl = 0; pl < PLANES; ++pl)
-          for (int kp = 0; kp < KP; ++kp) {
-            tma_load_3d(kd + (pl * KP + kp) * KSTEP, &map_k, k_full + st, kp * 64, pl, (int)rk, pol_kv);
-            tma_load_3d(vd + (pl * KP + kp) * AT_KVTILE, &map_v, v_full + st, kp * 64, pl, (int)rv, pol_kv);
-          }
+        for (int pp = 0; pp < PLANES * KP; ++pp) tma_load_3d(dst + pp * AT_KVTILE, map, full, (pp % KP) * 64, pp / KP, (int)rk, pol_kv);
     } else {
       const int sub_rows = min(64, a.page_tokens), n_sub = 64 / sub_rows;
-      for (int sb = 0; sb < n_sub; ++sb) {
-        const int j = min(j0 + sb * sub_rows, a.pages_per_seq * a.page_tokens - 1);
+      for (int sub = 0; sub < n_sub; ++sub) {
+        const int j = min(j0 + sub * sub_rows, a.pages_per_seq * a.page_tokens - 1);
         const int pg = a.page_table[seq * a.pages_per_seq + (j >> a.page_shift)];
         const int row = (pg * a.hkv + kvh) * a.page_tokens + (j & (a.page_tokens - 1));
         if (elect_one())
-          for (int kp = 0; kp < KP; ++kp) {
-            tma_load_2d(kd + kp * KSTEP + sb * sub_rows * 128, &map_k, k_full + st, kp * 64, row, pol_kv);
-            tma_load_2d(vd + kp * AT_KVTILE + sb * sub_rows * 128, &map_v, v_full + st, kp * 64, row, pol_kv);
-          }
+          for (int kp = 0; kp < KP; ++kp) tma_load_2d(dst + kp * AT_KVTILE + sub * sub_rows * 128, map, full, kp * 64, row, pol_kv);
       }
     }
     __syncwarp();
   };
-  int n_pre = 0;                                            // blocks of the first group already under way
+  int n_pre = 0;                                            // blocks of the first ring filling already under way
   if (early) {
     if (warp == 0 && n_blk > 0) {
       if (lane == 0) {
@@ -225,7 +230,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         asm volatile("prefetch.tensormap [%0];" ::"l"(&map_v) : "memory");
       }
       __syncwarp();
-      while (n_pre < min(n_blk, GROUP) && (b0 + n_pre + 1) * AT_KBLK <= P) { issue_kv(n_pre); ++n_pre; }
+      while (n_pre < min(n_blk, STAGES) && (b0 + n_pre + 1) * AT_KBLK <= P) { issue(0, n_pre, n_pre); issue(1, n_pre, n_pre); ++n_pre; }
     }
     pdl_wait();
   }
@@ -244,14 +249,22 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         for (int kp = 0; kp < KP; ++kp) tma_load_4d(q_s + kp * AT_QTILE, &map_q, q_full, kp * 64, 0, kvh * a.G, node0, pol_q);
       }
       __syncwarp();
-      for (int it = n_pre; it < n_blk; ++it) {
-        const int st = it % GROUP, use = it / GROUP;
-        if (use >= 1 && !__all_sync(0xffffffffu, mbar_wait(k_empty + st, (uint32_t)(use - 1) & 1u) && mbar_wait(v_empty + st, (uint32_t)(use - 1) & 1u))) {
-          if (lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
-          break;
+      // K runs one block ahead of V: its stage is free as soon as S was computed, V's only after O
+      int ks = n_pre % STAGES, vs = ks;
+      uint32_t kph = n_pre >= STAGES ? 0u : 1u, vph = kph;    // parity of the stage's last release (1: none needed yet)
+      for (int it = n_pre; it <= n_blk; ++it) {
+        if (it < n_blk) {
+          if (!mbar_wait_warp(k_empty + ks, kph)) { give_up(); break; }
+          if (__any_sync(0xffffffffu, *abort_flag)) break;
+          issue(0, it, ks);
+          if (++ks == STAGES) { ks = 0; kph ^= 1u; }
         }
-        if (__any_sync(0xffffffffu, *abort_flag)) break;
-        issue_kv(it);
+        if (it > n_pre) {
+          if (!mbar_wait_warp(v_empty + vs, vph)) { give_up(); break; }
+          if (__any_sync(0xffffffffu, *abort_flag)) break;
+          issue(1, it - 1, vs);
+          if (++vs == STAGES) { vs = 0; vph ^= 1u; }
+        }
       }
     }
   } else if (warp == 1) {
@@ -259,64 +272,60 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     // lane for the tcgen05 instructions (as in the GEMM)
     if (n_blk > 0) {
       // fp32 accumulate, bf16 operands, M = 128; S: N = 64, both K-major; O: N = head_dim, B MN-major
+      const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t o_addr = tmem_base, s_addr0 = tmem_base + HD;
-      bool ok = mbar_wait_warp(q_full, 0);
       const uint64_t qd = smem_desc(smem_u32(q_s)), kd = smem_desc(smem_u32(k_s)), pd = smem_desc(smem_u32(p_s)), vd = smem_desc_mn(smem_u32(v_s), AT_KVTILE);
-      const int n_groups = (n_blk + GROUP - 1) / GROUP;
-      for (int gi = 0; gi < n_groups && ok; ++gi) {
-        const int gb = gi * GROUP, ge = min(n_blk, gb + GROUP);
-        // S = Q K^T for all keys of the group at once: N = 64 x blocks
-        for (int it = gb; it < ge && ok; ++it) {
-          const int st = it % GROUP;
-          if (!__all_sync(0xffffffffu, mbar_wait(k_full + st, (uint32_t)gi & 1u) && (gi < 1 || mbar_wait(s_free + st, (uint32_t)(gi - 1) & 1u)))) ok = false;
-        }
-        if (!ok) break;
-        tc_fence_after();
-        // (an MMA's N ends at 256: a group of five blocks takes a chain of four blocks and one of one)
-        for (int b0 = 0; b0 < ge - gb; b0 += 4) {
-          const uint32_t n_keys_g = (uint32_t)min(4, ge - gb - b0) * 64u;
-          const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((n_keys_g >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-          uint32_t acc = 0u;
-          for (int pl = 0; pl < PLANES; ++pl)
-            for (int kp = 0; kp < KP; ++kp) {
-              const uint64_t ad = qd + (uint64_t)(kp * (AT_QTILE >> 4));
-              const uint64_t bd = kd + (uint64_t)(((pl * KP + kp) * GROUP + b0) * (AT_KVTILE >> 4));
-              if (elect_one()) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) mma_bf16(s_addr0 + (uint32_t)(b0 * 64), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc_s, k ? 1u : acc);
-              }
-              acc = 1u;
-            }
-        }
-        if (elect_one())
-          for (int it = gb; it < ge; ++it) { mma_commit(k_empty + it % GROUP); mma_commit(s_full + it % GROUP); }
-        __syncwarp();
-        for (int it = gb; it < ge && ok; ++it) {                       // O += P_b V_b
-          const int st = it % GROUP, pb = it & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u) && mbar_wait(v_full + st, (uint32_t)gi & 1u))) { ok = false; break; }
+      bool ok = mbar_wait_warp(q_full, 0);
+      int ks = 0, sb = 0, vs = 0;                            // ring positions of K, S and V
+      uint32_t kph = 0, sph = 1, vph = 0;
+      // step i issues S of block i and O of block i - AHEAD
+#pragma unroll 1
+      for (int i = 0; i < n_blk + AHEAD && ok; ++i) {
+        const int it = i - AHEAD;
+        if (it >= 0) {
+          const int pb = it & 1;
+          if (!__all_sync(0xffffffffu, mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u) && mbar_wait(v_full + vs, vph))) { ok = false; break; }
           tc_fence_after();
           const uint64_t ad = pd + (uint64_t)(pb * (AT_PTILE >> 4));
           if (elect_one()) {
 #pragma unroll
             for (int pl = 0; pl < PLANES; ++pl) {
-              const uint64_t bd = vd + (uint64_t)((st * Sh::KV_STAGE + pl * KP * AT_KVTILE) >> 4);
+              const uint64_t bd = vd + (uint64_t)((vs * Sh::KV_STAGE + pl * KP * AT_KVTILE) >> 4);
 #pragma unroll
-              for (int k = 0; k < 4; ++k)                               // 16 keys = two groups of 8 K-rows = 2048 bytes
+              for (int k = 0; k < 4; ++k)                                 // 16 keys = two groups of 8 K-rows = 2048 bytes
                 mma_bf16(o_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc_o, (it > 0 || pl > 0 || k > 0) ? 1u : 0u);
             }
             mma_commit(p_empty + pb);
-            mma_commit(v_empty + st);
-            if (it == ge - 1) mma_commit(o_done);
+            mma_commit(v_empty + vs);
           }
           __syncwarp();
+          if (++vs == STAGES) { vs = 0; vph ^= 1u; }
+        }
+        if (i < n_blk) {
+          if (!__all_sync(0xffffffffu, mbar_wait(k_full + ks, kph) && mbar_wait(s_free + sb, sph))) { ok = false; break; }
+          tc_fence_after();
+          if (elect_one()) {
+#pragma unroll 1
+            for (int pp = 0; pp < PLANES * KP; ++pp) {
+              const uint64_t ad = qd + (uint64_t)((pp % KP) * (AT_QTILE >> 4)), bd = kd + (uint64_t)((ks * Sh::KV_STAGE + pp * AT_KVTILE) >> 4);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) mma_bf16(s_addr0 + (uint32_t)(sb * 64), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc_s, (pp > 0 || k > 0) ? 1u : 0u);
+            }
+            mma_commit(k_empty + ks);
+            mma_commit(s_full + sb);
+          }
+          __syncwarp();
+          if (++ks == STAGES) { ks = 0; kph ^= 1u; }
+          if (++sb == S_BUFS) { sb = 0; sph ^= 1u; }
         }
       }
-      if (!ok && lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
+      if (!ok) give_up();
     }
   } else {
-    // ------------------------------------------------------------------ softmax and epilogue: one row per thread
-    const int q = warp & 3;                                   // TMEM lane quarter this warp may access
+    // ------------------------------------------------------------------ softmax and epilogue: one row per thread,
+    // warps 2..5 and 6..9 each cover the 128 rows; `half` is the half of every block's keys this warp takes
+    const int q = warp & 3, half = warp >= 6 ? 1 : 0;          // TMEM lane quarter this warp may access
     const int row = q * 32 + lane, e = e_base + (row >> 1), part = row & 1;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     // what this row sees: keys below `vis_end`, plus tail key j (key index tail0 + j) for the bits of mw
@@ -364,139 +373,119 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       }
       return m;
     };
-    float m_run = -INFINITY, l_run = 0.f, u_run = 0.f;       // exp2 domain; u = sum p (s - m) for the entropy
+    // A wait that runs out (or finds that another warp's did) clears ok.  The warp then walks on to the end, its waits
+    // skipped, because its partner meets it at a barrier in every block.
+    bool ok = true;
+    auto wait = [&](uint64_t *bar, uint32_t parity) {            // one lane polls for the warp
+      int w = 1;
+      if (lane == 0 && (*abort_flag || !mbar_wait(bar, parity))) w = 0;
+      if (!__shfl_sync(0xffffffffu, w, 0)) { if (ok) give_up(); ok = false; }
+    };
+    float m_ref = -INFINITY, l_run = 0.f, u_run = 0.f;       // exp2 domain; u = sum p (s - m) for the entropy
     const bool want_ent = a.ent != nullptr || a.row_ent != nullptr;
-    bool ok = n_blk > 0;
-    const int n_groups = (n_blk + GROUP - 1) / GROUP;
+    int sb = 0;
+    uint32_t sph = 0;
 #pragma unroll 1
-    for (int gi = 0; gi < n_groups && ok; ++gi) {
-      const int gb = gi * GROUP, ge = min(n_blk, gb + GROUP);
-      // ---- first pass: the row maximum over the group's keys
-      float gmax = m_run;
-#pragma unroll 1
-      for (int it = gb; it < ge && ok; ++it) {
-        const int st = it % GROUP, j0 = (b0 + it) * AT_KBLK;
-        int w_ok = 1;
-        if (lane == 0) w_ok = mbar_wait(s_full + st, (uint32_t)gi & 1u) ? 1 : 0;
-        w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-        if (!w_ok || *abort_flag) { ok = false; break; }
+    for (int it = 0; it < n_blk; ++it) {
+      const int pb = it & 1;
+      wait(s_full + sb, sph);
+      tc_fence_after();
+      uint32_t sr[32];
+      tmem_ld32(lane_addr + (uint32_t)(HD + sb * 64 + half * 32), sr);
+      const uint32_t vm = vis32((b0 + it) * AT_KBLK + half * 32) >> (part * 16);
+      tmem_ld_wait();
+      tc_fence_before();
+      if (lane == 0) mbar_arrive(s_free + sb);
+      if (++sb == S_BUFS) { sb = 0; sph ^= 1u; }
+      // lanes 2e and 2e+1 hold the products of entry e's high and low query parts: the even lane
+      // keeps keys 0..15 of the 32 and the odd lane 16..31, each sends the partner what it needs
+      float t[16], bm = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        const float send = __uint_as_float(part ? sr[c] : sr[16 + c]), mine = __uint_as_float(part ? sr[16 + c] : sr[c]);
+        t[c] = mine + __shfl_xor_sync(0xffffffffu, send, 1);
+        t[c] = ((vm >> c) & 1u) ? t[c] : -INFINITY;
+        bm = fmaxf(bm, t[c]);
+      }
+      bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
+      float *mx = mx_s + pb * 128;
+      mx[half * 64 + (row >> 1)] = bm;
+      bar_sync_pair(1 + q);
+      bm = fmaxf(bm, mx[(half ^ 1) * 64 + (row >> 1)]) * scale;     // the block's row maximum, the same in all four threads of the row
+      const bool grow = bm > m_ref + AT_RESCALE && m_ref != -INFINITY;
+      if (__any_sync(0xffffffffu, grow)) {
+        // ---- the accumulator takes the new reference (behind the O of every earlier block)
+        wait(p_empty + (pb ^ 1), (uint32_t)((it - 1) >> 1) & 1u);
         tc_fence_after();
+        const float corr = grow ? ex2(m_ref - bm) : 1.f;
 #pragma unroll 1
-        for (int ch = 0; ch < 2; ++ch) {
-          uint32_t sr[32];
-          tmem_ld32(lane_addr + (uint32_t)(HD + st * 64 + ch * 32), sr);
-          const uint32_t vm = vis32(j0 + ch * 32);
+        for (int c0 = half * (HD / 2); c0 < (half + 1) * (HD / 2); c0 += 32) {
+          uint32_t orr[32];
+          tmem_ld32(lane_addr + (uint32_t)c0, orr);
           tmem_ld_wait();
-          // lanes 2e and 2e+1 hold the products of entry e's high and low query parts: the even lane
-          // keeps keys 0..15 of the chunk and the odd lane 16..31, each sends the partner what it needs
-          const uint32_t vmh = vm >> (part * 16);
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            const float send = __uint_as_float(part ? sr[c] : sr[16 + c]);
-            const float mine = __uint_as_float(part ? sr[16 + c] : sr[c]);
-            const float t = (mine + __shfl_xor_sync(0xffffffffu, send, 1)) * scale;
-            gmax = fmaxf(gmax, ((vmh >> c) & 1u) ? t : -INFINITY);
-          }
+          for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * corr);
+          tmem_st32(lane_addr + (uint32_t)c0, orr);
         }
+        tmem_st_wait();
+        if (grow) { u_run = corr * (u_run - (bm - m_ref) * l_run); l_run *= corr; m_ref = bm; }
       }
-      gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, 1));
-      if (!ok) break;
-      const float base = gmax == -INFINITY ? 0.f : gmax;
-      const float corr = exp2f(m_run - base);                 // 0 when nothing was seen before
-      if (gi >= 1) {
-        // ---- the accumulator of the earlier groups takes the new maximum
-        int w_ok = 1;
-        if (lane == 0) w_ok = mbar_wait(o_done, (uint32_t)(gi - 1) & 1u) ? 1 : 0;
-        w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-        if (!w_ok) { ok = false; break; }
-        tc_fence_after();
-        if (__any_sync(0xffffffffu, corr != 1.f)) {
-#pragma unroll 1
-          for (int c0 = 0; c0 < HD; c0 += 32) {
-            uint32_t orr[32];
-            tmem_ld32(lane_addr + (uint32_t)c0, orr);
-            tmem_ld_wait();
+      if (m_ref == -INFINITY) m_ref = bm;
+      const float base = m_ref == -INFINITY ? 0.f : m_ref;
+      if (it >= 2) wait(p_empty + pb, (uint32_t)((it >> 1) - 1) & 1u);
+      // ---- probabilities, row sum, P's high and low parts into shared memory
+      uint32_t ph[8], pl2[8];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * corr);
-            tmem_st32(lane_addr + (uint32_t)c0, orr);
-          }
-          tmem_st_wait();
-        }
-        if (want_ent) u_run = l_run > 0.f ? corr * (u_run - (base - m_run) * l_run) : 0.f;
-        l_run *= corr;
+      for (int c = 0; c < 16; c += 2) {
+        const float d0 = fmaf(t[c], scale, -base), d1 = fmaf(t[c + 1], scale, -base);
+        const float p0 = ex2(d0), p1 = ex2(d1);               // a masked key: 2^-inf = 0
+        l_run += p0 + p1;
+        if (want_ent) u_run += (p0 > 0.f ? p0 * d0 : 0.f) + (p1 > 0.f ? p1 * d1 : 0.f);
+        split_pair(p0, p1, ph[c >> 1], pl2[c >> 1]);
       }
-      m_run = gmax;
-      // ---- second pass: probabilities, row sum, P's high or low part into shared memory
-#pragma unroll 1
-      for (int it = gb; it < ge && ok; ++it) {
-        const int st = it % GROUP, pb = it & 1, j0 = (b0 + it) * AT_KBLK;
-        if ((it >> 1) >= 1) {
-          int w_ok = 1;
-          if (lane == 0) w_ok = mbar_wait(p_empty + pb, (uint32_t)((it >> 1) - 1) & 1u) ? 1 : 0;
-          w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-          if (!w_ok || *abort_flag) { ok = false; break; }
-        }
-        uint8_t *prow0 = p_s + pb * AT_PTILE;
-#pragma unroll 1
-        for (int ch = 0; ch < 2; ++ch) {
-          uint32_t sr[32];
-          tmem_ld32(lane_addr + (uint32_t)(HD + st * 64 + ch * 32), sr);
-          const uint32_t vm = vis32(j0 + ch * 32);
-          tmem_ld_wait();
-          const uint32_t vmh = vm >> (part * 16);
-          uint32_t ph[8], pl2[8];
+      // this lane's 16 keys: high parts into the entry's even row, low parts into its odd row; 16-byte
+      // pieces swizzled like the MMA expects a K-major operand (piece ^ (row & 7))
+      uint8_t *row_hi = p_s + pb * AT_PTILE + (row & ~1) * 128, *row_lo = row_hi + 128;
 #pragma unroll
-          for (int c = 0; c < 16; c += 2) {
-            const float s0 = __uint_as_float(part ? sr[c] : sr[16 + c]), s1 = __uint_as_float(part ? sr[c + 1] : sr[17 + c]);
-            const float m0 = __uint_as_float(part ? sr[16 + c] : sr[c]), m1 = __uint_as_float(part ? sr[17 + c] : sr[c + 1]);
-            const float d0 = (m0 + __shfl_xor_sync(0xffffffffu, s0, 1)) * scale - base;
-            const float d1 = (m1 + __shfl_xor_sync(0xffffffffu, s1, 1)) * scale - base;
-            const float p0 = ((vmh >> c) & 1u) ? exp2f(d0) : 0.f, p1 = ((vmh >> (c + 1)) & 1u) ? exp2f(d1) : 0.f;
-            l_run += p0 + p1;
-            if (want_ent) u_run += (p0 > 0.f ? p0 * d0 : 0.f) + (p1 > 0.f ? p1 * d1 : 0.f);
-            split_pair(p0, p1, ph[c >> 1], pl2[c >> 1]);
-          }
-          // this lane's 16 keys: high parts into the entry's even row, low parts into its odd row; 16-byte
-          // pieces swizzled like the MMA expects a K-major operand (piece ^ (row & 7))
-          uint8_t *row_hi = prow0 + (row & ~1) * 128, *row_lo = row_hi + 128;
-#pragma unroll
-          for (int pc = 0; pc < 2; ++pc) {
-            const int piece = ch * 4 + part * 2 + pc;
-            *reinterpret_cast<uint4 *>(row_hi + ((piece ^ (row & 6)) << 4)) = make_uint4(ph[pc * 4], ph[pc * 4 + 1], ph[pc * 4 + 2], ph[pc * 4 + 3]);
-            *reinterpret_cast<uint4 *>(row_lo + ((piece ^ ((row & 6) | 1)) << 4)) = make_uint4(pl2[pc * 4], pl2[pc * 4 + 1], pl2[pc * 4 + 2], pl2[pc * 4 + 3]);
-          }
-        }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) { mbar_arrive(p_full + pb); mbar_arrive(s_free + st); }
+      for (int pc = 0; pc < 2; ++pc) {
+        const int piece = half * 4 + part * 2 + pc;
+        *reinterpret_cast<uint4 *>(row_hi + ((piece ^ (row & 6)) << 4)) = make_uint4(ph[pc * 4], ph[pc * 4 + 1], ph[pc * 4 + 2], ph[pc * 4 + 3]);
+        *reinterpret_cast<uint4 *>(row_lo + ((piece ^ ((row & 6) | 1)) << 4)) = make_uint4(pl2[pc * 4], pl2[pc * 4 + 1], pl2[pc * 4 + 2], pl2[pc * 4 + 3]);
       }
+      fence_proxy_async_smem();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(p_full + pb);
     }
-    // ---- epilogue: the row's accumulator (lanes 2e and 2e+1 added), partial or finished
-    if (ok) {
-      int w_ok = 1;
-      if (lane == 0) w_ok = mbar_wait(o_done, (uint32_t)(n_groups - 1) & 1u) ? 1 : 0;
-      w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-      ok = w_ok != 0;
-    }
-    if (n_blk > 0 && !ok && lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);           // each lane of a pair summed half of the keys
+    // ---- epilogue: the row's accumulator (lanes 2e and 2e+1 added), partial or finished; each warp half of the columns
+    if (n_blk > 0) wait(p_empty + ((n_blk - 1) & 1), (uint32_t)((n_blk - 1) >> 1) & 1u);
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);           // each of a row's four threads summed a quarter of the keys
     u_run += __shfl_xor_sync(0xffffffffu, u_run, 1);
+    float *lx = mx_s + (n_blk & 1) * 128;
+    lx[half * 64 + (row >> 1)] = l_run;
+    bar_sync_pair(1 + q);
+    l_run += lx[(half ^ 1) * 64 + (row >> 1)];
+    if (want_ent) {
+      bar_sync_pair(1 + q);
+      lx[half * 64 + (row >> 1)] = u_run;
+      bar_sync_pair(1 + q);
+      u_run += lx[(half ^ 1) * 64 + (row >> 1)];
+    }
     pdl_trigger();                                            // the keys are done: the kernel that follows may take the SMs
-    if (n_blk == 0 || ok) {
+    if (ok) {
       tc_fence_after();
       const int Hkv = a.H / a.G;
       const long long pbase = ((((long long)slot * a.n_chunks + chunk) * Hkv + kvh) * a.n_rt + rt) * 64 + (row >> 1);
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
 #pragma unroll 1
-      for (int c0 = 0; c0 < HD; c0 += 32) {
+      for (int c0 = half * (HD / 2); c0 < (half + 1) * (HD / 2); c0 += 32) {
         uint32_t orr[32];
         if (n_blk > 0) { tmem_ld32(lane_addr + (uint32_t)c0, orr); tmem_ld_wait(); }
         else {
 #pragma unroll
           for (int c = 0; c < 32; ++c) orr[c] = 0u;
         }
-        // the even lane keeps columns 0..15 of the chunk, the odd lane 16..31 (as in the GEMM's epilogue)
+        // the even lane keeps columns 0..15 of the chunk, the odd lane 16..31
         float v[16];
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
@@ -519,9 +508,9 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4 *>(po + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
         }
       }
-      if (r >= 0 && part == 0) {
+      if (r >= 0 && part == 0 && half == 0) {
         if (a.n_chunks > 1) {
-          *reinterpret_cast<float2 *>(a.part_ml + pbase * 2) = make_float2(m_run, l_run);
+          *reinterpret_cast<float2 *>(a.part_ml + pbase * 2) = make_float2(m_ref, l_run);
           if (a.row_ent) a.part_u[pbase] = u_run;
         } else if (a.row_ent) {
           a.row_ent[(long long)r * a.H + h] = l_run > 0.f ? logf(l_run) - u_run * 0.6931471805599453f / l_run : 0.f;
@@ -530,7 +519,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           // natural-log units: lse = m ln 2 + ln l;  H = ln l - u ln 2 / l
           const int node = r - slot * a.rows_per_seq;
           const float ln2 = 0.6931471805599453f;
-          a.lse[(long long)h * a.n_keys + node] = m_run * ln2 + logf(l_run);
+          a.lse[(long long)h * a.n_keys + node] = m_ref * ln2 + logf(l_run);
           if (a.ent) a.ent[(long long)h * a.n_keys + node] = logf(l_run) - u_run * ln2 / l_run;
         }
       }

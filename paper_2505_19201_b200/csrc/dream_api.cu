@@ -755,7 +755,6 @@ template <typename T, int HD> struct AttnLaunch {
                  const int *row_vis = nullptr) {
     const dream_config &f = c->cfg;
     const bool flat_kv = cache != nullptr;
-    const int GROUP = flat_kv ? AtShape<HD, true>::GROUP : AtShape<HD, false>::GROUP;
     for (int b = 0; b < DREAM_MAX_BATCH; ++b) a.slot_seq[b] = b < B ? c->cur_seq[b] : 0;
     a.H = f.n_heads; a.G = f.n_heads / f.n_kv_heads; a.rows_per_seq = rows_per_seq; a.row_in = row_in; a.row_vis = row_vis;
     a.scale_log2 = 1.4426950408889634f / sqrtf((float)HD);
@@ -763,12 +762,10 @@ template <typename T, int HD> struct AttnLaunch {
     const int nb_ub = imax(1, (key_ub + AT_KBLK - 1) / AT_KBLK);
     const int tiles = f.n_kv_heads * a.n_rt * B;
     // as many key chunks as keep the grid in one wave of resident CTAs, the blocks dealt out evenly
-    // (a chunk walks its blocks GROUP at a time)
     const int per_sm = flat_kv ? AtShape<HD, true>::CTAS_PER_SM : AtShape<HD, false>::CTAS_PER_SM;
     const int want = imin(imin(AM_MAX_CHUNKS, nb_ub), imax(1, c->tc.n_sms * per_sm / tiles));
     a.blocks_per_chunk = (nb_ub + want - 1) / want;
     a.n_chunks = (nb_ub + a.blocks_per_chunk - 1) / a.blocks_per_chunk;
-    (void)GROUP;
     // a CTA walks every key its rows see: prefill, and row sets wider than the partials were sized for
     if (a.mode == AT_PREFILL || a.n_rt > c->am_rt_max) { a.n_chunks = 1; a.blocks_per_chunk = 1 << 24; }
     a.part_o = c->am_part_o; a.part_ml = c->am_part_ml; a.out = c->attn_out; a.status = c->status;
