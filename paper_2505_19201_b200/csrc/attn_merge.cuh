@@ -1,7 +1,7 @@
-// Merge of the split-K attention partials.
+// Merge of the split-K attention partials, where the chunks of a tile are too many for a cluster.
 //
 // The attention kernels (attn_tc.cuh) cut the keys of a sequence into chunks, one CTA each; a chunk
-// leaves, per query entry, the running maximum m, the sum l and the unnormalised output O of its
+// leaves, per query entry, the reference exponent m, the sum l and the unnormalised output O of its
 // keys (exp2 domain).  k_attn_combine merges them in chunk order, one thread per four output
 // values, and writes the finished rows as GEMM input rows (high and low bf16 parts).
 #pragma once
@@ -9,15 +9,6 @@
 #include "rows.cuh"
 
 #define AM_ROWS 64
-
-// Two floats -> packed bf16 pair (high parts) and the packed pair of the remainders.
-__device__ __forceinline__ void split_pair(float x, float y, uint32_t &hi, uint32_t &lo) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-  float2 f = __bfloat1622float2(h);
-  __nv_bfloat162 l = __floats2bfloat162_rn(x - f.x, y - f.y);
-  hi = *reinterpret_cast<uint32_t *>(&h);
-  lo = *reinterpret_cast<uint32_t *>(&l);
-}
 
 // What the merge kernel needs to know about the partials and the output rows.
 struct AttnMergeArgs {

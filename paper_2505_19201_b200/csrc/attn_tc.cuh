@@ -20,9 +20,11 @@
 //                        and B = V_b as stored ([key][head_dim]: an MN-major operand).
 // K/V blocks arrive through two TMA rings; during verification the blocks below the verified prefix
 // length are requested before the grid dependency resolves.  Flat draft caches carry a low plane
-// per key, which costs one more MMA per step.  A chunk leaves (m, l, O) partials for
-// k_attn_combine, or the finished rows (and, for the prefill, each row's log-sum-exp and entropy)
-// when it is the only chunk.  Warp roles: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..9 =
+// per key, which costs one more MMA per step.  The chunks of one tile are a thread-block cluster: each leaves
+// its (m, l, O) in its shared memory, and after a cluster barrier every CTA merges a share of the rows, reading
+// the others' through distributed shared memory (a merge kernel behind partials in global memory costs 4 us more
+// per launch, most of it the kernel boundary; it stays for tiles whose many chunks no cluster holds).  The
+// prefill has one chunk and also leaves each row's log-sum-exp and entropy.  Warp roles: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..9 =
 // softmax and epilogue.  What bounds it is the softmax's instruction latency: with four warps (one per
 // scheduler) and two passes over S a block of 64 keys took 2.0 us of a LLaVA-7B-shaped verify launch.
 // The loops are kept compact on purpose: this kernel's code is
@@ -46,7 +48,19 @@
 #define AT_KVTILE (64 * 64 * 2)        // one 64-column panel of a 64-key block
 #define AT_PTILE (128 * 64 * 2)        // probabilities of one block (128 rows x 64 keys)
 
+#define AT_MAX_CHUNKS 32               // most key chunks of a tile
+#define AT_MAX_CLUSTER 16              // ... that are a cluster
+
 enum { AT_VERIFY = 0, AT_DRAFT = 1, AT_PREFILL = 2 };
+
+// Two floats -> packed bf16 pair (high parts) and the packed pair of the remainders.
+__device__ __forceinline__ void split_pair(float x, float y, uint32_t &hi, uint32_t &lo) {
+  __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  float2 f = __bfloat1622float2(h);
+  __nv_bfloat162 l = __floats2bfloat162_rn(x - f.x, y - f.y);
+  hi = *reinterpret_cast<uint32_t *>(&h);
+  lo = *reinterpret_cast<uint32_t *>(&l);
+}
 
 // Ring depths: what shared memory (K and V blocks stay until their MMAs ran) and the TMEM columns
 // (head_dim for O, 64 per S_b) hold.
@@ -63,6 +77,7 @@ template <int HD, bool FLAT> struct AtShape {
   static constexpr int KP = HD / 64;                                 // 64-column panels per row
   static constexpr int KV_STAGE = PLANES * KP * AT_KVTILE;           // one block of K (or of V)
   static constexpr int Q_BYTES = KP * AT_QTILE;
+  static constexpr int O_LD = HD + 4;                                // floats per row of the merge's O tile (over the K/V rings)
   static constexpr size_t SMEM = 1024 + Q_BYTES + 2 * STAGES * KV_STAGE + 2 * AT_PTILE + 1024 + 384;
 };
 
@@ -79,14 +94,13 @@ struct AttnTcArgs {
   int n_keys;                       // prefill: keys in the sequence (row i sees keys 0..i)
   float scale_log2;
   int n_chunks, blocks_per_chunk, n_rt;
-  float *part_o, *part_ml;          // [slot][chunk][kvh][rt][64][hd], [..][64][2]
   void *out;                        // [R][H*hd] rows in GEMM-input layout
   XLayout lay;
   int out_chunk_rows;               // prefill: the output rows are laid out per chunk of this many rows ...
   long long out_chunk_stride;       // ... this many elements apart (0: one chunk)
   float *lse, *ent;                 // prefill: [H][n] row log-sum-exp and entropy, or null
   float *row_ent;                   // verify: [R][H] entropy of every tree row's attention distribution, or null
-  float *part_u;                    // ... and, with several chunks, the chunks' u = sum p (s - m) beside part_ml
+  float *part_o, *part_ml, *part_u; // null: the chunks are a cluster; else the partials [slot][chunk][kvh][rt][64][hd], [..][64][2], [..][64] (with row_ent)
   L2Prefetch next_w;
   // where the K/V blocks live, as rows of the K and V tensor maps
   const int *page_table;            // paged: [max_batch][pages_per_seq]
@@ -131,6 +145,13 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t saddr, uint32_t lbo_by
   return d;
 }
 
+// Reads from the shared memory of a CTA of this cluster (addresses from mapa).
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
 // 2^x for x <= 8 or so, subnormal results as zero.
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -148,6 +169,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   extern __shared__ uint8_t at_smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)at_smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *q_s = smem, *k_s = q_s + Sh::Q_BYTES, *v_s = k_s + STAGES * Sh::KV_STAGE, *p_s = v_s + STAGES * Sh::KV_STAGE;
+  float *o_s = (float *)k_s, *ml_s = o_s + 64 * Sh::O_LD;     // merge: O of the 64 entries, then (m, l, u, -) of each
   float *mx_s = (float *)(p_s + 2 * AT_PTILE);                // [2 buffers][2 halves][64 entries]: exchange between the two warps of a quarter
   uint64_t *bars = (uint64_t *)(mx_s + 256);
   uint64_t *q_full = bars, *k_full = q_full + 1, *k_empty = k_full + STAGES, *v_full = k_empty + STAGES, *v_empty = v_full + STAGES;
@@ -474,9 +496,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     pdl_trigger();                                            // the keys are done: the kernel that follows may take the SMs
     if (ok) {
       tc_fence_after();
-      const int Hkv = a.H / a.G;
-      const long long pbase = ((((long long)slot * a.n_chunks + chunk) * Hkv + kvh) * a.n_rt + rt) * 64 + (row >> 1);
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+      const long long pbase = ((((long long)slot * a.n_chunks + chunk) * a.hkv + kvh) * a.n_rt + rt) * 64 + (row >> 1);
 #pragma unroll 1
       for (int c0 = half * (HD / 2); c0 < (half + 1) * (HD / 2); c0 += 32) {
         uint32_t orr[32];
@@ -493,26 +514,28 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           const float mine = __uint_as_float(part ? orr[16 + c] : orr[c]);
           v[c] = mine + __shfl_xor_sync(0xffffffffu, send, 1);
         }
-        if (r < 0) continue;
         const int col = c0 + part * 16;
-        if (a.n_chunks == 1) {
+        if (a.n_chunks > 1) {
+          float *po = a.part_o ? a.part_o + pbase * HD + col : o_s + (row >> 1) * Sh::O_LD + col;
+#pragma unroll
+          for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4 *>(po + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+        } else if (r >= 0) {
           bf16 *out = reinterpret_cast<bf16 *>(a.out);
           long long o = a.out_chunk_stride ? (long long)(r / a.out_chunk_rows) * a.out_chunk_stride + (long long)(r % a.out_chunk_rows) * a.lay.row_stride
                                            : (long long)r * a.lay.row_stride;
 #pragma unroll
           for (int c = 0; c < 16; c += 4)
             store_split4<bf16>(out + o + h * HD + col + c, a.lay.lo_delta, make_float4(v[c] * inv, v[c + 1] * inv, v[c + 2] * inv, v[c + 3] * inv));
-        } else {
-          float *po = a.part_o + pbase * HD + col;
-#pragma unroll
-          for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4 *>(po + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
         }
       }
-      if (r >= 0 && part == 0 && half == 0) {
-        if (a.n_chunks > 1) {
+      if (a.n_chunks > 1 && part == 0 && half == 0) {
+        if (a.part_o) {
           *reinterpret_cast<float2 *>(a.part_ml + pbase * 2) = make_float2(m_ref, l_run);
           if (a.row_ent) a.part_u[pbase] = u_run;
-        } else if (a.row_ent) {
+        } else *reinterpret_cast<float4 *>(ml_s + (row >> 1) * 4) = make_float4(m_ref, l_run, u_run, 0.f);
+      }
+      if (r >= 0 && part == 0 && half == 0 && a.n_chunks == 1) {
+        if (a.row_ent) {
           a.row_ent[(long long)r * a.H + h] = l_run > 0.f ? logf(l_run) - u_run * 0.6931471805599453f / l_run : 0.f;
         }
         if (a.lse) {
@@ -526,7 +549,49 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     }
   }
   tc_fence_before();
-  __syncthreads();
+  if (a.n_chunks > 1 && !a.part_o) {
+    // ---- merge: out = sum_c w_c O_c / sum_c w_c l_c with w_c = 2^(m_c - max m), chunks in ascending order; this CTA's
+    // share of the (entry, four columns) items
+    __syncwarp();
+    cluster_sync_all();
+    const uint32_t o_addr = smem_u32(o_s), ml_addr = smem_u32(ml_s);
+    const int n = a.n_chunks;
+    bf16 *out = reinterpret_cast<bf16 *>(a.out);
+#pragma unroll 1
+    for (int i = chunk * AT_THREADS + (int)threadIdx.x; i < 64 * (HD / 4); i += n * AT_THREADS) {
+      const int en = i / (HD / 4), c4 = (i % (HD / 4)) * 4, e = e_base + en;
+      if (e >= rows_total) continue;
+      float M = -INFINITY, L = 0.f, U = 0.f;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+      for (int c = 0; c < n; c += 4) {
+        float4 ml[4], o[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t cc = (uint32_t)min(c + k, n - 1);
+          ml[k] = ld_cluster4(mapa(ml_addr + en * 16, cc));
+          o[k] = ld_cluster4(mapa(o_addr + (en * Sh::O_LD + c4) * 4, cc));
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (c + k >= n || ml[k].x == -INFINITY) continue;
+          const float Mn = fmaxf(M, ml[k].x), sc = ex2(M - Mn), w = ex2(ml[k].x - Mn);       // 2^-inf = 0 on the first live chunk
+          // u relative to the new reference: sum p' (s - Mn) with p' = p 2^(m - Mn)
+          U = (L > 0.f ? sc * (U + (M - Mn) * L) : 0.f) + w * (ml[k].z + (ml[k].x - Mn) * ml[k].y);
+          L = L * sc + ml[k].y * w;
+          acc.x = acc.x * sc + o[k].x * w; acc.y = acc.y * sc + o[k].y * w;
+          acc.z = acc.z * sc + o[k].z * w; acc.w = acc.w * sc + o[k].w * w;
+          M = Mn;
+        }
+      }
+      const float inv = L > 0.f ? 1.f / L : 0.f;
+      const int node = e / a.G, r = slot * a.rows_per_seq + node, h = kvh * a.G + (e - node * a.G);
+      if (a.row_ent && c4 == 0) a.row_ent[(long long)r * a.H + h] = L > 0.f ? logf(L) - U * 0.6931471805599453f * inv : 0.f;
+      store_split4<bf16>(out + (long long)r * a.lay.row_stride + h * HD + c4, a.lay.lo_delta, make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+    }
+    __syncwarp();
+    cluster_sync_relaxed();                     // no CTA leaves while another may still read its shared memory
+  } else __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)Sh::TMEM_COLS) : "memory");
@@ -562,22 +627,52 @@ static inline bool at_map(GemmTcPlan *pl, AtMapCache *cache, const void *ptr, in
 }
 
 template <int HD, bool FLAT>
-static inline const char *attn_tc_setup() {
-  if (cudaFuncSetAttribute(k_attn_tc<HD, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AtShape<HD, FLAT>::SMEM) != cudaSuccess)
-    return "cannot raise the attention kernel's shared memory limit";
+static inline void attn_tc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, cudaStream_t stream, int use_pdl, int n_chunks, int cluster, int tiles, int n_slots) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3(n_chunks, tiles, n_slots); cfg->blockDim = dim3(AT_THREADS);
+  cfg->dynamicSmemBytes = AtShape<HD, FLAT>::SMEM; cfg->stream = stream;
+  int n = 0;
+  if (cluster) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)n_chunks; attr[n].val.clusterDim.y = 1; attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (use_pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg->attrs = attr; cfg->numAttrs = n;
+}
+
+// max_tiles[n]: tiles of n chunks (clusters of n CTAs) that are resident at once.
+template <int HD, bool FLAT>
+static inline const char *attn_tc_setup(int *max_tiles, int n_sms) {
+  auto *kernel = k_attn_tc<HD, FLAT>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AtShape<HD, FLAT>::SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+    return "cannot raise the attention kernel's shared memory or cluster limit";
+  max_tiles[0] = 0;
+  max_tiles[1] = n_sms * AtShape<HD, FLAT>::CTAS_PER_SM;
+  for (int n = 2; n <= AT_MAX_CLUSTER; ++n) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    attn_tc_config<HD, FLAT>(&cfg, attr, nullptr, 0, n, 1, 1, 1);
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); clusters = 0; }
+    max_tiles[n] = clusters;
+  }
   return nullptr;
 }
 
-// Enqueue one attention launch: grid (a.n_chunks, H_kv * a.n_rt, n_slots).
+// Enqueue one attention launch: grid (a.n_chunks, H_kv * a.n_rt, n_slots), the chunks of a tile a cluster unless
+// there are partials.
 template <int HD, bool FLAT>
 static inline cudaError_t attn_tc_launch(cudaStream_t stream, int use_pdl, const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv,
                                          const AttnTcArgs &a, int n_slots) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.n_chunks, (a.H / a.G) * a.n_rt, n_slots); cfg.blockDim = dim3(AT_THREADS);
-  cfg.dynamicSmemBytes = AtShape<HD, FLAT>::SMEM; cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = use_pdl ? 1 : 0;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  attn_tc_config<HD, FLAT>(&cfg, attr, stream, use_pdl, a.n_chunks, a.n_chunks > 1 && !a.part_o, (a.H / a.G) * a.n_rt, n_slots);
   return cudaLaunchKernelEx(&cfg, k_attn_tc<HD, FLAT>, mq, mk, mv, a);
 }

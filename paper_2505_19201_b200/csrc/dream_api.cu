@@ -21,7 +21,6 @@
 #include "rows.cuh"
 #include "tree.cuh"
 
-#define AM_MAX_CHUNKS 32        // most key chunks the split-K attention cuts a sequence into
 #define ROW_CHUNK 256          // most rows a decode call holds (max_batch * tree nodes)
 // Most prompt rows per pass of the set-up.  The weights stream once per pass and a GEMM's output of this
 // many rows still stays in L2 for the row kernel behind it at the widths met (1152 x 16384 floats: 75 MB).
@@ -67,11 +66,12 @@ struct dream_ctx {
   void *xn, *raw, *act, *attn_out;
   float *top_val, *lse_rows, *margin_i;
   TopkScratch tks;
-  float *am_part_o, *am_part_ml;       // split-K attention partials
-  // track_entropy: the chunks' u beside am_part_ml, every tree row's entropy [layer][ROW_CHUNK][H] from
-  // the last verification, and the per-layer sums over the verified rows [seq][layer]
-  float *am_part_u, *row_ent, *ent_sum;
+  // track_entropy: every tree row's entropy [layer][ROW_CHUNK][H] from the last verification, and the
+  // per-layer sums over the verified rows [seq][layer]
+  float *row_ent, *ent_sum;
+  float *am_part_o, *am_part_ml, *am_part_u;   // split-K attention partials (where k_attn_combine merges)
   int am_rt_max;
+  int at_max_tiles[2][AT_MAX_CLUSTER + 1];   // attention tiles resident at once by chunks per tile: [paged | flat]
   int key_ub0[DREAM_MAX_BATCH];        // permanent rows of the draft caches right after compression
   // Verified lengths as the host knows them.  The device advances P by A + 1 per accept and the host
   // only knows A <= D, so p_ub grows by D + 1 per accept until a snapshot of the device's P arrives:
@@ -376,7 +376,7 @@ static size_t carve(dream_ctx *c, char *base) {
   c->lse_rows = a.take<float>(ROW_CHUNK);
   c->am_rt_max = (rows_per_seq_max(&c->ts) * (f.n_heads / f.n_kv_heads) + AM_ROWS - 1) / AM_ROWS;
   if (f.dtype == DREAM_BF16) {
-    size_t prow = (size_t)MB * AM_MAX_CHUNKS * f.n_kv_heads * c->am_rt_max * AM_ROWS;
+    size_t prow = (size_t)MB * AT_MAX_CHUNKS * f.n_kv_heads * c->am_rt_max * AM_ROWS;
     c->am_part_o = a.take<float>(prow * f.head_dim);
     c->am_part_ml = a.take<float>(prow * 2);
     c->am_part_u = f.track_entropy ? a.take<float>(prow) : nullptr;
@@ -511,9 +511,9 @@ static void refresh_bounds(dream_ctx *c) {
 // ------------------------------------------------------------------------------------- init / free
 
 template <int HD>
-static const char *attn_tc_setup_all() {
-  const char *w = attn_tc_setup<HD, false>();
-  if (!w) w = attn_tc_setup<HD, true>();
+static const char *attn_tc_setup_all(dream_ctx *c) {
+  const char *w = attn_tc_setup<HD, false>(c->at_max_tiles[0], c->tc.n_sms);
+  if (!w) w = attn_tc_setup<HD, true>(c->at_max_tiles[1], c->tc.n_sms);
   return w ? w : colsum_tc_setup<HD>();
 }
 
@@ -587,7 +587,7 @@ extern "C" dream_status dream_init(const dream_config *cfg, const dream_target_w
     if (why) { free_host_side(c); return fail(nullptr, DREAM_E_CUDA, "tensor-core GEMM set-up: %s", why); }
   }
   if (c->use_tc) {
-    const char *why = cfg->head_dim == 64 ? attn_tc_setup_all<64>() : cfg->head_dim == 128 ? attn_tc_setup_all<128>() : attn_tc_setup_all<256>();
+    const char *why = cfg->head_dim == 64 ? attn_tc_setup_all<64>(c) : cfg->head_dim == 128 ? attn_tc_setup_all<128>(c) : attn_tc_setup_all<256>(c);
     if (why) { free_host_side(c); return fail(nullptr, DREAM_E_CUDA, "%s", why); }
   }
   k_rope_table<<<(cfg->head_dim / 2 + 127) / 128, 128, 0, c->stream>>>(c->rope_inv, cfg->head_dim, cfg->rope_theta);
@@ -761,14 +761,21 @@ template <typename T, int HD> struct AttnLaunch {
     a.n_rt = (rows_per_seq * a.G + 63) / 64;
     const int nb_ub = imax(1, (key_ub + AT_KBLK - 1) / AT_KBLK);
     const int tiles = f.n_kv_heads * a.n_rt * B;
-    // as many key chunks as keep the grid in one wave of resident CTAs, the blocks dealt out evenly
-    const int per_sm = flat_kv ? AtShape<HD, true>::CTAS_PER_SM : AtShape<HD, false>::CTAS_PER_SM;
-    const int want = imin(imin(AM_MAX_CHUNKS, nb_ub), imax(1, c->tc.n_sms * per_sm / tiles));
-    a.blocks_per_chunk = (nb_ub + want - 1) / want;
+    // as many key chunks as keep the grid in one wave of resident CTAs, the blocks dealt out evenly; in a
+    // prefill a CTA walks every key its rows see
+    const int *max_tiles = c->at_max_tiles[flat_kv ? 1 : 0];
+    auto blocks_of = [&](int want) { return (nb_ub + want - 1) / want; };
+    int want = imin(AT_MAX_CLUSTER, nb_ub), many = imin(imin(AT_MAX_CHUNKS, nb_ub), imax(1, max_tiles[1] / tiles));
+    while (want > 1 && max_tiles[want] < tiles) --want;
+    // Clusters need free SMs of one GPC, so fewer chunks fit: partials and the merge kernel (4 us) where the longer
+    // chunks cost more than that (a block takes 1 us at head_dim 128 and in proportion): the Gemma-shaped
+    // round with 5 and 10 chunks per tile instead of 6 and 18 was 2 % slower, the others 1..2 % faster
+    const bool merge = a.mode != AT_PREFILL && a.n_rt <= c->am_rt_max && (blocks_of(want) - blocks_of(many)) * HD > 256;
+    if (merge) { want = many; a.part_o = c->am_part_o; a.part_ml = c->am_part_ml; a.part_u = c->am_part_u; }
+    a.blocks_per_chunk = blocks_of(want);
     a.n_chunks = (nb_ub + a.blocks_per_chunk - 1) / a.blocks_per_chunk;
-    // a CTA walks every key its rows see: prefill, and row sets wider than the partials were sized for
-    if (a.mode == AT_PREFILL || a.n_rt > c->am_rt_max) { a.n_chunks = 1; a.blocks_per_chunk = 1 << 24; }
-    a.part_o = c->am_part_o; a.part_ml = c->am_part_ml; a.out = c->attn_out; a.status = c->status;
+    if (a.mode == AT_PREFILL) { a.n_chunks = 1; a.blocks_per_chunk = 1 << 24; }
+    a.out = c->attn_out; a.status = c->status;
     a.hkv = f.n_kv_heads;
     CUtensorMap mq, mk, mv;
     bool ok;
@@ -799,7 +806,7 @@ template <typename T, int HD> struct AttnLaunch {
                             : attn_tc_launch<HD, false>(c->stream, c->use_pdl, mq, mk, mv, a, B);
     if (e != cudaSuccess && c->launch_err == cudaSuccess) { c->launch_err = e; c->launch_err_name = "k_attn_tc"; }
     c->launches++;
-    if (a.n_chunks > 1) {
+    if (a.n_chunks > 1 && a.part_o) {
       AttnMergeArgs m = {};
       m.row_in = row_in; m.row_vis = row_vis; m.rows_per_seq = rows_per_seq; m.H = a.H; m.G = a.G; m.n_chunks = a.n_chunks; m.n_rt = a.n_rt;
       m.part_o = a.part_o; m.part_ml = a.part_ml; m.out = a.out; m.lay = a.lay;
@@ -815,7 +822,7 @@ template <typename T, int HD> struct AttnLaunch {
       a.mode = AT_VERIFY;
       a.next_w.ptr = (const char *)c->wo[layer]; a.next_w.bytes = (unsigned long long)c->cfg.d_model * c->Hhd * 2;
       a.prefix_len = c->sd.P; a.mask = c->vmask; a.tail_len = c->T; a.lay = xlay(m, c->Hhd);
-      if (ent) { a.row_ent = ent; a.part_u = c->am_part_u; }
+      a.row_ent = ent;
       tc(c, a, layer, nullptr, B, c->T, key_ub, nullptr);
     } else {
       auto *kernel = ent ? k_attn_tree<HD, true> : k_attn_tree<HD, false>;
