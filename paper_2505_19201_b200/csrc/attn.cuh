@@ -114,35 +114,39 @@ k_attn_prefill(const float *__restrict__ qbuf, PagedKV kv, int seq, int n, int H
   }
 }
 
-// AE(l) = mean over rows and heads of the row entropies (Eq. 2).  One block, fixed order.
-// sum_out (may be null) receives the sum itself: the start of the running form of Eq. 2.
-__global__ void k_entropy_mean(const float *__restrict__ ent, int count, float *out, float *sum_out) {
+// AE(l) = mean over rows and heads of the row entropies (Eq. 2), all layers at once: a block per layer, fixed order.
+// sum_out (may be null) receives the sums themselves: the start of the running form of Eq. 2.
+__global__ void k_entropy_mean(const float *__restrict__ ent, long long layer_stride, int count, float *out, float *sum_out) {
   __shared__ float sh[33];
   kernel_entry(TR_k_entropy_mean);
+  const float *e = ent + blockIdx.x * layer_stride;
   float s = 0.f;
-  for (int i = threadIdx.x; i < count; i += blockDim.x) s += ent[i];
+  for (int i = threadIdx.x; i < count; i += blockDim.x) s += e[i];
   float t = block_sum(s, sh);
-  if (threadIdx.x == 0) { *out = t / (float)count; if (sum_out) *sum_out = t; }
+  if (threadIdx.x == 0) { out[blockIdx.x] = t / (float)count; if (sum_out) sum_out[blockIdx.x] = t; }
 }
 
-
-// Importance of visual token j at this layer (Section 3.3): the attention weight it receives,
+// Importance of visual token j at the tapped layer (Section 3.3): the attention weight it receives,
 // summed over the later query rows (and its own row when include_self) and over heads.
 // One warp per (visual column, head), grid (ceil(v / 8), H): rows ascending, four in flight at a
-// time, added in row order; k_colsum_heads then adds the heads in ascending order: a fixed order.
+// time, added in row order; k_colsum_heads then adds the heads in ascending order: a fixed order.  Queries and
+// log-sum-exps are kept for every candidate layer (q_stride, lse_stride apart), the layer is known on the device.
 template <int HD>
 __global__ void __launch_bounds__(ATT_WARPS * 32)
-k_colsum(const float *__restrict__ qbuf, PagedKV kv, int seq, int n, int H, float scale,
-         const float *__restrict__ lse, int vis_start, int v, int include_self, float *part /* [H][v] */) {
+k_colsum(const float *__restrict__ qbuf, long long q_stride, PagedKV kv, long long layer_stride, int seq, int n, int H, float scale,
+         const float *__restrict__ lse, long long lse_stride, const int *__restrict__ tap, int tap_lo, int vis_start, int v, int include_self,
+         float *part /* [H][v] */) {
   constexpr int EPL = HD / 32;
   kernel_entry(TR_k_colsum);
+  qbuf += (*tap - tap_lo) * q_stride; lse += (*tap - tap_lo) * lse_stride;
+  const float *K = (const float *)kv.base + (*tap - 1) * layer_stride;
   int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int jv = blockIdx.x * ATT_WARPS + w, h = blockIdx.y;
   if (jv >= v) return;
   int j = vis_start + jv;
   int kvh = h / (H / kv.hkv);
   float k[EPL];
-  RowLoad<EPL>::ld((const float *)kv.base + kv.off(seq, j, kvh), lane, k);
+  RowLoad<EPL>::ld(K + kv.off(seq, j, kvh), lane, k);
   const float *lse_h = lse + (long long)h * n;
   float hs = 0.f;
   int i = include_self ? j : j + 1;

@@ -30,7 +30,11 @@ struct ColsumTcArgs {
   int vis_start, v, include_self;   // the visual span; 1: a token's attention to itself counts
   int key0;                         // first key of tile 0 (vis_start rounded down to a multiple of 64)
   float scale_log2;
-  const float *lse;                 // [H][n] natural-log log-sum-exp of every row
+  const float *lse;                 // [candidate][..][H][n] natural-log log-sum-exp of every row
+  long long lse_stride;             // floats between candidate layers
+  const int *tap;                   // the tapped layer (1-based), known on the device only
+  int tap_lo, q_rows;               // first candidate layer, rows of a layer in the query map
+  int kv_rows;                      // rows of a layer (K and V) in the key map
   float *part;                      // [H][v] per-head sums
   const int *page_table;
   int pages_per_seq, page_tokens, page_shift, hkv;
@@ -69,7 +73,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   pdl_wait();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) trace_stamp(TR_k_colsum);
 
-  const int n = a.n;
+  const int n = a.n, cand = *a.tap - a.tap_lo, q_row0 = cand * a.q_rows, k_row0 = (*a.tap - 1) * a.kv_rows;
   const int j0 = a.key0 + tile * CS_KEYS;                   // first key of this tile; rows before it see none of its keys
   const int n_steps = n > j0 ? (n - j0 + NQ - 1) / NQ : 0;
 
@@ -88,7 +92,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       for (int sb = 0; sb < n_sub; ++sb) {
         const int j = min(j0 + sb * sub_rows, a.pages_per_seq * a.page_tokens - sub_rows);
         const int pg = a.page_table[a.seq * a.pages_per_seq + (j >> a.page_shift)];
-        const int row = (pg * a.hkv + kvh) * a.page_tokens + (j & (a.page_tokens - 1));
+        const int row = k_row0 + (pg * a.hkv + kvh) * a.page_tokens + (j & (a.page_tokens - 1));
         if (elect_one())
           for (int kp = 0; kp < KP; ++kp)
             tma_load_2d(k_s + kp * (CS_KEYS * 128) + sb * sub_rows * 128, &map_k, k_full, kp * 64, row, pol);
@@ -102,7 +106,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
           mbar_expect_tx(q_full + st, (uint32_t)Sh::Q_STAGE);
           for (int pl = 0; pl < 2; ++pl)
             for (int kp = 0; kp < KP; ++kp)
-              tma_load_4d(q_s + st * Sh::Q_STAGE + (pl * KP + kp) * (NQ * 128), &map_q, q_full + st, kp * 64, pl, h, j0 + t * NQ, pol);
+              tma_load_4d(q_s + st * Sh::Q_STAGE + (pl * KP + kp) * (NQ * 128), &map_q, q_full + st, kp * 64, pl, h, q_row0 + j0 + t * NQ, pol);
         }
         __syncwarp();
       }
@@ -141,7 +145,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     const int i_min = j + (a.include_self ? 0 : 1);          // first row whose attention to key j counts
     const float scale = a.scale_log2;
-    const float *lse_h = a.lse + (long long)h * n;
+    const float *lse_h = a.lse + cand * a.lse_stride + (long long)h * n;
     float hs = 0.f;
     bool ok = true;
 #pragma unroll 1

@@ -40,7 +40,8 @@ struct dream_ctx {
   int use_tc, use_pdl, gemm_failed;
   cudaError_t launch_err;              // first refused kernel launch of the call being enqueued
   const char *launch_err_name;
-  double *rope_inv;                    // [head_dim / 2] rotary inverse frequencies
+  float2 *rope_pos;                    // [n_pos][head_dim / 2] rotary (cos, sin) of every position
+  int n_pos;
   float2 *rope_tab;                    // [ROW_CHUNK][head_dim / 2] rotary (cos, sin) of the rows of the call being enqueued
   std::vector<const void *> ln1, wqkv, wo, ln2, wgu, wd;
   const void *embed, *ln_f, *lm_head;
@@ -61,8 +62,10 @@ struct dream_ctx {
   int *gather_idx, *ctx_pos, *flags;
   uint32_t *vmask;
   void *qbuf;                          // query rows, 4 bytes per element (see q_store4)
+  void *q_taps;                        // prompt queries of the candidate tap layers [n_cand][XR][Hhd], for the importance of the chosen one
+  void *q_cur;                         // where the call being enqueued keeps its queries
   float *ssq;                          // [PR][SSQ_LD] sums of squares of the rows in xn (k_resid)
-  float *x, *x0, *gout, *lse_pre, *ent_pre, *ae, *scores_all, *taps_store, *tapbuf;
+  float *x, *x0, *gout, *lse_taps, *lse_pre, *ent_pre, *ae, *scores, *col_part, *taps_store, *tapbuf;
   void *xn, *raw, *act, *attn_out;
   float *top_val, *lse_rows, *margin_i;
   TopkScratch tks;
@@ -288,6 +291,7 @@ static void derive(dream_ctx *c) {
   c->XR = c->RM;
   c->PR = imax(ROW_CHUNK, imin(PROMPT_ROWS, (f.max_prompt + 15) & ~15));   // rows of a GEMM input buffer
   c->three = f.draft_blocks == 3;
+  c->n_pos = f.max_seq + DREAM_MAX_DEPTH + 1;           // a draft runs up to its depth behind the verified rows
 }
 
 static size_t carve(dream_ctx *c, char *base) {
@@ -363,12 +367,15 @@ static size_t carve(dream_ctx *c, char *base) {
   }
   c->gout = a.take<float>(c->gout_floats);
   c->ssq = a.take<float>((size_t)c->PR * SSQ_LD);
-  c->rope_inv = a.take<double>(f.head_dim / 2);
+  c->rope_pos = a.take<float2>((size_t)c->n_pos * (f.head_dim / 2));
   c->rope_tab = a.take<float2>((size_t)ROW_CHUNK * (f.head_dim / 2));
+  c->q_taps = a.take<float>((size_t)c->n_cand * c->XR * c->Hhd);
+  c->lse_taps = a.take<float>((size_t)c->n_cand * f.n_heads * f.max_prompt);
   c->lse_pre = a.take<float>((size_t)f.n_heads * f.max_prompt);
-  c->ent_pre = a.take<float>((size_t)f.n_heads * f.max_prompt);
+  c->ent_pre = a.take<float>((size_t)f.n_layers * f.n_heads * f.max_prompt);
+  c->col_part = a.take<float>((size_t)f.n_heads * imax(f.max_visual, 1));
   c->ae = a.take<float>(f.n_layers);
-  c->scores_all = a.take<float>((size_t)c->n_cand * imax(f.max_visual, 1));
+  c->scores = a.take<float>(imax(f.max_visual, 1));
   c->taps_store = a.take<float>((size_t)c->n_cand * f.max_prompt * d);
   c->tapbuf = a.take<float>((size_t)ROW_CHUNK * d);
   c->top_val = a.take<float>((size_t)ROW_CHUNK * TOPK_MAX);
@@ -590,7 +597,8 @@ extern "C" dream_status dream_init(const dream_config *cfg, const dream_target_w
     const char *why = cfg->head_dim == 64 ? attn_tc_setup_all<64>(c) : cfg->head_dim == 128 ? attn_tc_setup_all<128>(c) : attn_tc_setup_all<256>(c);
     if (why) { free_host_side(c); return fail(nullptr, DREAM_E_CUDA, "%s", why); }
   }
-  k_rope_table<<<(cfg->head_dim / 2 + 127) / 128, 128, 0, c->stream>>>(c->rope_inv, cfg->head_dim, cfg->rope_theta);
+  c->q_cur = c->qbuf;
+  k_rope_table<<<c->n_pos, 128, 0, c->stream>>>(c->rope_pos, cfg->head_dim, cfg->rope_theta);
   if (cudaGetLastError() != cudaSuccess) { free_host_side(c); return fail(nullptr, DREAM_E_CUDA, "rotary table launch failed"); }
   *out = c;
   return DREAM_OK;
@@ -691,7 +699,7 @@ static long long prefill_chunk_stride(const dream_ctx *c, int pass_rows) {
 }
 template <typename T, int HD> struct AttnLaunch {
   // The output rows are laid out per pass over the prompt (the O projection's input).
-  static void prefill(dream_ctx *c, int layer, int seq, int n) {
+  static void prefill(dream_ctx *c, int layer, int seq, int n, float *lse, float *ent) {
     if constexpr (sizeof(T) == 2) {
       // causal attention of the n prompt rows on the tensor cores: one CTA per (KV head, 64 entries)
       // walks all keys up to its last row; row log-sum-exp and entropy (Eq. 2) come out of the same pass
@@ -699,19 +707,20 @@ template <typename T, int HD> struct AttnLaunch {
       a.mode = AT_PREFILL;
       a.n_keys = n; a.lay = xlay(xmode(c), c->Hhd);
       a.out_chunk_rows = prompt_pass_rows(c, n); a.out_chunk_stride = prefill_chunk_stride(c, a.out_chunk_rows);
-      a.lse = c->lse_pre; a.ent = c->ent_pre;
+      a.lse = lse; a.ent = ent;
       c->cur_seq[0] = seq;
       tc(c, a, layer, nullptr, 1, n, 0, nullptr);
     } else {
       dim3 grid((n + ATT_WARPS * ATT_PF_ROWS - 1) / (ATT_WARPS * ATT_PF_ROWS), c->cfg.n_heads);
-      LAUNCH(c, (k_attn_prefill<HD>), grid, ATT_WARPS * 32, 0, (const float *)c->qbuf, paged(c, layer), seq, n, c->cfg.n_heads,
-             1.f / sqrtf((float)HD), (float *)c->attn_out, c->lse_pre, c->ent_pre);
+      LAUNCH(c, (k_attn_prefill<HD>), grid, ATT_WARPS * 32, 0, (const float *)c->q_cur, paged(c, layer), seq, n, c->cfg.n_heads,
+             1.f / sqrtf((float)HD), (float *)c->attn_out, lse, ent);
     }
   }
-  static void colsum(dream_ctx *c, int layer, int seq, int n, int vis_start, int v, float *score) {
+  // Importance of the v visual tokens at the tapped layer, after the prefill: only the device knows which layer that is,
+  // so its queries and log-sum-exps are found among those kept for every candidate layer.
+  static void colsum(dream_ctx *c, int seq, int n, int vis_start, int v, float *score) {
     if (v == 0) return;
-    // the per-head sums land in the entropy buffer, which is idle between this layer's entropy mean
-    // and the next layer's attention ([H][n] floats, v <= n)
+    const long long lse_stride = (long long)c->cfg.n_heads * c->cfg.max_prompt;
     if constexpr (sizeof(T) == 2) {
       // tensor cores: 128 keys of one head per CTA, the query rows stream past (colsum_tc.cuh)
       const dream_config &f = c->cfg;
@@ -720,20 +729,23 @@ template <typename T, int HD> struct AttnLaunch {
       a.vis_start = vis_start; a.v = v; a.include_self = f.score_include_self;
       a.key0 = vis_start & ~63;
       a.scale_log2 = 1.4426950408889634f / sqrtf((float)HD);
-      a.lse = c->lse_pre; a.part = c->ent_pre; a.status = c->status;
-      const PagedKV kv = paged(c, layer);
+      a.lse = c->lse_taps; a.lse_stride = lse_stride; a.tap = c->sd.tap + seq; a.tap_lo = c->tap_lo_eff; a.q_rows = c->XR;
+      a.part = c->col_part; a.status = c->status;
+      const PagedKV kv = paged(c, 0);
+      const long long layer_rows = (long long)c->n_pages * f.n_kv_heads * f.page_tokens;
+      a.kv_rows = (int)(2 * layer_rows);
       a.page_table = kv.page_table; a.pages_per_seq = kv.pages_per_seq; a.page_tokens = kv.page_tokens; a.page_shift = kv.page_shift;
       a.hkv = f.n_kv_heads;
       CUtensorMap mq, mk;
       bool ok;
       {
-        const unsigned long long dims[4] = {(unsigned long long)HD, 2ull, (unsigned long long)f.n_heads, (unsigned long long)c->XR};
+        const unsigned long long dims[4] = {(unsigned long long)HD, 2ull, (unsigned long long)f.n_heads, (unsigned long long)c->n_cand * c->XR};
         const unsigned long long st[3] = {(unsigned long long)HD * 2, (unsigned long long)HD * 4, (unsigned long long)f.n_heads * HD * 4};
         const unsigned box[4] = {64u, 1u, 1u, (unsigned)CsShape<HD>::NQ};
-        ok = at_map(&c->tc, &c->at_maps, c->qbuf, 4, dims, st, box, &mq);
+        ok = at_map(&c->tc, &c->at_maps, c->q_taps, 4, dims, st, box, &mq);
       }
       {
-        const unsigned long long dims[2] = {(unsigned long long)HD, (unsigned long long)c->n_pages * f.n_kv_heads * f.page_tokens};
+        const unsigned long long dims[2] = {(unsigned long long)HD, 2ull * layer_rows * f.n_layers};
         const unsigned long long st[1] = {(unsigned long long)HD * 2};
         const unsigned box[2] = {64u, (unsigned)imin(64, f.page_tokens)};
         ok = ok && at_map(&c->tc, &c->at_maps, kv.base, 2, dims, st, box, &mk);
@@ -744,10 +756,11 @@ template <typename T, int HD> struct AttnLaunch {
       if (e != cudaSuccess && c->launch_err == cudaSuccess) { c->launch_err = e; c->launch_err_name = "k_colsum_tc"; }
       c->launches++;
     } else {
-      LAUNCH(c, (k_colsum<HD>), dim3((v + ATT_WARPS - 1) / ATT_WARPS, c->cfg.n_heads), ATT_WARPS * 32, 0, (const float *)c->qbuf, paged(c, layer), seq, n,
-             c->cfg.n_heads, 1.f / sqrtf((float)HD), c->lse_pre, vis_start, v, c->cfg.score_include_self, c->ent_pre);
+      LAUNCH(c, (k_colsum<HD>), dim3((v + ATT_WARPS - 1) / ATT_WARPS, c->cfg.n_heads), ATT_WARPS * 32, 0, (const float *)c->q_taps, (long long)c->XR * c->Hhd,
+             paged(c, 0), c->layer_stride, seq, n, c->cfg.n_heads, 1.f / sqrtf((float)HD), (const float *)c->lse_taps, lse_stride,
+             (const int *)(c->sd.tap + seq), c->tap_lo_eff, vis_start, v, c->cfg.score_include_self, c->col_part);
     }
-    LAUNCH(c, k_colsum_heads, (v + 255) / 256, 256, 0, (const float *)c->ent_pre, c->cfg.n_heads, v, score);
+    LAUNCH(c, k_colsum_heads, (v + 255) / 256, 256, 0, (const float *)c->col_part, c->cfg.n_heads, v, score);
   }
   // The tcgen05 attention (bf16 configurations): split-K plan, tensor maps, launch, merge of the chunks.
   // cache: null = the paged target cache of `layer`, else a flat draft cache.
@@ -783,7 +796,7 @@ template <typename T, int HD> struct AttnLaunch {
       const unsigned long long dims[4] = {(unsigned long long)HD, 2ull, (unsigned long long)f.n_heads, (unsigned long long)c->XR};
       const unsigned long long st[3] = {(unsigned long long)HD * 2, (unsigned long long)HD * 4, (unsigned long long)f.n_heads * HD * 4};
       const unsigned box[4] = {64u, 2u, (unsigned)a.G, (unsigned)(64 / a.G)};
-      ok = at_map(&c->tc, &c->at_maps, c->qbuf, 4, dims, st, box, &mq);
+      ok = at_map(&c->tc, &c->at_maps, c->q_cur, 4, dims, st, box, &mq);
     }
     if (flat_kv) {
       const unsigned long long dims[3] = {(unsigned long long)HD, 2ull, (unsigned long long)f.max_batch * 2 * f.n_kv_heads * c->cap_rows};
@@ -889,35 +902,39 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
          d, f.vocab, c->status);
   const XMode mp = xmode(c);
   const long long att_chunk = prefill_chunk_stride(c, CH);
+  // queries and row log-sum-exps of the candidate tap layers stay until the compression
+  auto cand_of = [&](int l) { const int k = l + 1 - c->tap_lo_eff; return k >= 0 && k < c->n_cand ? k : -1; };
+  auto q_of = [&](int l) { return cand_of(l) < 0 ? c->qbuf : (void *)((float *)c->q_taps + (size_t)cand_of(l) * c->XR * c->Hhd); };
   // projections of layer l for the rows of one pass, whose normalised input sits in c->xn
   auto qkv = [&](int l, int r0, int rows, const RowScale &norm) {
     GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].pos, c->rm[0].slot, r0, c->qbuf,
-           paged(c, l), f.n_heads, c->rope_inv, (const float2 *)nullptr);
+    LAUNCH(c, (k_qkv_post_target<T>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].slot, r0, q_of(l),
+           paged(c, l), f.n_heads, (const float2 *)c->rope_pos);
   };
   for (int r0 = 0; r0 < n; r0 += CH) {
     const int rows = imin(CH, n - r0);
     qkv(0, r0, rows, norm_rows<T>(c, c->x + (size_t)r0 * d, NO_GEMM, false, c->ln1[0], rows, mp));
   }
   for (int l = 0; l < L; ++l) {
-    HD_DISPATCH(c, T, prefill(c, l, seq, n));
-    LAUNCH(c, k_entropy_mean, 1, 1024, 0, c->ent_pre, f.n_heads * n, c->ae + l,
-           c->ent_sum ? c->ent_sum + (size_t)seq * L + l : (float *)nullptr);
-    int cand = l + 1 - c->tap_lo_eff;
-    bool is_cand = cand >= 0 && cand < c->n_cand;
-    if (is_cand) HD_DISPATCH(c, T, colsum(c, l, seq, n, vis_start, v, c->scores_all + (size_t)cand * imax(f.max_visual, 1)));
-    // the rest of the layer and the next layer's projections, pass by pass (the queries of layer l are done with)
+    const int cand = cand_of(l);
+    c->q_cur = q_of(l);
+    HD_DISPATCH(c, T, prefill(c, l, seq, n, cand < 0 ? c->lse_pre : c->lse_taps + (size_t)cand * f.n_heads * f.max_prompt,
+                              c->ent_pre + (size_t)l * f.n_heads * f.max_prompt));
+    c->q_cur = c->qbuf;
+    // the rest of the layer and the next layer's projections, pass by pass (the attention of layer l is done with its queries)
     for (int r0 = 0; r0 < n; r0 += CH) {
       int rows = imin(CH, n - r0);
       float *xr = c->x + (size_t)r0 * d;
       GemmOut g = gemm<T>(c, c->wo[l], (const T *)c->attn_out + (long long)(r0 / CH) * att_chunk, mp, rows, d, c->Hhd);
       RowScale norm = norm_rows<T>(c, xr, g, true, c->ln2[l], rows, mp);
       g = mlp_rows<T>(c, norm, c->wgu[l], c->wd[l], rows, mp);
-      float *copy = is_cand ? c->taps_store + ((size_t)cand * f.max_prompt + r0) * d : nullptr;
+      float *copy = cand >= 0 ? c->taps_store + ((size_t)cand * f.max_prompt + r0) * d : nullptr;
       norm = norm_rows<T>(c, xr, g, true, l + 1 < L ? c->ln1[l + 1] : c->ln_f, rows, mp, copy);
       if (l + 1 < L) qkv(l + 1, r0, rows, norm);
     }
   }
+  LAUNCH(c, k_entropy_mean, L, 1024, 0, (const float *)c->ent_pre, (long long)f.n_heads * f.max_prompt, f.n_heads * n, c->ae,
+         c->ent_sum ? c->ent_sum + (size_t)seq * L : (float *)nullptr);
   // first token: LM head on the last prompt row
   const RowScale last = norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
   GemmOut g = gemm<T>(c, c->lm_head, c->xn, mp, 1, f.vocab, d);
@@ -987,7 +1004,7 @@ static GemmOut draft_rows(dream_ctx *c, const RowMeta &rm, int R, XMode xm, int 
   GemmOut g;
   RowScale norm = norm_rows<T>(c, c->x, NO_GEMM, false, w.ln1, R, xm);
   g = gemm<T>(c, w.wqkv, c->xn, xm, R, c->qkvN, d);
-  LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself), f.n_heads, c->rope_inv, rope_tab);
+  LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself), f.n_heads, rope_tab, context ? 1 : 0);
   HD_DISPATCH(c, T, draft(c, rm, c->dself, c->sd.nperm_d, 0, R, xm, B, m, key_ub, vd, tail));
   g = gemm<T>(c, w.wo, c->attn_out, xm, R, d, c->Hhd);
   if (c->three) {
@@ -1004,7 +1021,7 @@ static GemmOut draft_rows(dream_ctx *c, const RowMeta &rm, int R, XMode xm, int 
   if (c->three) {
     norm = norm_rows<T>(c, c->x, g, true, w.f_ln1, R, xm);
     g = gemm<T>(c, w.f_wqkv, c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself2), f.n_heads, c->rope_inv, rope_tab);
+    LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself2), f.n_heads, rope_tab, context ? 1 : 0);
     if (context) return g;
     HD_DISPATCH(c, T, draft(c, rm, c->dself2, c->sd.nperm_d, 0, R, xm, B, m, key_ub, vd, tail));
     g = gemm<T>(c, w.f_wo, c->attn_out, xm, R, d, c->Hhd);
@@ -1018,8 +1035,8 @@ template <typename T>
 static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *forced, int *kept, float *scores) {
   const dream_config &f = c->cfg;
   int v = c->pf_v, q = c->pf_q, n = v + q, d = f.d_model, nc = q + k, CH = c->PR;
-  LAUNCH(c, k_select_visual, 1, 1024, 0, c->scores_all, (long long)imax(f.max_visual, 1), c->sd.tap + seq, c->tap_lo_eff,
-         v, k, c->pf_vis_start, n, forced, kept, scores, c->ctx_pos, c->flags);
+  HD_DISPATCH(c, T, colsum(c, seq, n, c->pf_vis_start, v, c->scores));
+  LAUNCH(c, k_select_visual, 1, 1024, 0, (const float *)c->scores, v, k, c->pf_vis_start, n, forced, kept, scores, c->ctx_pos, c->flags);
   // draft self-attention K/V of the compressed context, from the input embeddings
   const char *wkv = (const char *)c->dw.wqkv + (size_t)c->Hhd * d * c->esz;
   const XMode m1 = xmode(c);
@@ -1030,7 +1047,7 @@ static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *force
     const RowScale norm = norm_rows<T>(c, c->x, NO_GEMM, false, c->dw.ln1, rows, m1);
     GemmOut g = gemm<T>(c, wkv, c->xn, m1, rows, c->kvN, d);
     LAUNCH(c, k_qkv_post_draft, dim3(rows, (c->kvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].pos, c->rm[0].dst, 0, (float *)nullptr,
-           flat(c, c->dself), f.n_heads, c->rope_inv, (const float2 *)nullptr);
+           flat(c, c->dself), f.n_heads, (const float2 *)c->rope_pos, 1);
   }
   // cross-attention memory: tapped features at the context positions, projected (Eq. 1)
   int nm = f.xattn_full_memory ? n : nc;
@@ -1054,7 +1071,7 @@ static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *force
       const XMode xm = xmode(c);
       LAUNCH(c, k_ctx_rows, (rows + 255) / 256, 256, 0, c->ctx_pos + r0, rows, 0, seq, c->rm[0], c->gather_idx, r0, f.xattn_full_memory);
       LAUNCH(c, (k_gather_rows<float>), rows, 256, 0, c->x0, c->gather_idx, c->x, d, (const int *)nullptr, 0, 0LL, XLayout{d, 0});
-      draft_rows<T>(c, c->rm[0], rows, xm, 1, rows, imax(nc, nm), true, false, true, (const float2 *)nullptr);
+      draft_rows<T>(c, c->rm[0], rows, xm, 1, rows, imax(nc, nm), true, false, true, (const float2 *)c->rope_pos);
     }
   }
   return DREAM_OK;
@@ -1118,7 +1135,7 @@ static dream_status draft_impl(dream_ctx *c, const TreeBatch &tb, int B) {
     RowMeta &rm = c->rm[cur], &rn = c->rm[cur ^ 1];
     if (p == 1) LAUNCH(c, k_draft_begin, 1, 32, 0, tb, B, c->sd, c->dt, ts, rm, m, c->cap_rows, c->status);
     LAUNCH(c, (k_embed<T>), dim3(R, (d + 1023) / 1024), 256, 0, (const T *)c->embed, rm.tok, c->x, d, f.vocab, c->status,
-           (const int *)rm.pos, (const double *)c->rope_inv, c->rope_tab, f.head_dim / 2);
+           (const int *)rm.pos, (const float2 *)c->rope_pos, c->n_pos, c->rope_tab, f.head_dim / 2);
     // pass 1 of the three-block draft carries the catch-up rows through every block
     GemmOut g = draft_rows<T>(c, rm, R, xm, B, m, key_ub, c->three && p == 1, true, false, (const float2 *)c->rope_tab);
     // e^M = x: the raw copy feeds the memory projection, the normalised copy the LM head
@@ -1164,13 +1181,13 @@ static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *a
   for (int b = 0; b < B; ++b) { key_ub = imax(key_ub, c->p_ub[tb.seq[b]] + c->T); c->cur_seq[b] = tb.seq[b]; }
   LAUNCH(c, k_verify_setup, (R + 127) / 128, 128, 0, tb, B, c->T, c->sd, rm, c->vmask, f.max_seq, c->status);
   LAUNCH(c, (k_embed<T>), dim3(R, (d + 1023) / 1024), 256, 0, (const T *)c->embed, rm.tok, c->x, d, f.vocab, c->status,
-           (const int *)rm.pos, (const double *)c->rope_inv, c->rope_tab, f.head_dim / 2);
+           (const int *)rm.pos, (const float2 *)c->rope_pos, c->n_pos, c->rope_tab, f.head_dim / 2);
   GemmOut gd = NO_GEMM, g;
   for (int l = 0; l < L; ++l) {
     // the first norm completes S^l (for l >= 1) and captures it where a sequence taps layer l
     RowScale norm = norm_rows<T>(c, c->x, gd, l > 0, c->ln1[l], R, xm, l > 0 ? c->tapbuf : nullptr, rm.seq, c->sd.tap, l);
     g = gemm<T>(c, c->wqkv[l], c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.slot, 0, c->qbuf, paged(c, l), f.n_heads, c->rope_inv, (const float2 *)c->rope_tab);
+    LAUNCH(c, (k_qkv_post_target<T>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.slot, 0, c->qbuf, paged(c, l), f.n_heads, (const float2 *)c->rope_tab);
     HD_DISPATCH(c, T, tree(c, l, R, xm, B, key_ub));
     g = gemm<T>(c, c->wo[l], c->attn_out, xm, R, d, c->Hhd);
     norm = norm_rows<T>(c, c->x, g, true, c->ln2[l], R, xm);

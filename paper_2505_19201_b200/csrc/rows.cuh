@@ -6,23 +6,17 @@
 #include "common.cuh"
 
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ void rope_cs(int pos, double inv, float *c, float *s);
 // x[r] = embed[tok[r]] (fp32 residual stream).  tok < 0 leaves a zero row.  One thread per four
-// elements: grid (rows, ceil(d / 1024)).  With rope_tab the first block of a row also tabulates
-// the row's rotary factors for every layer of the call: rope_tab[r][i] = (cos, sin)(pos[r] *
-// inv_freq[i]), i < half.
+// elements: grid (rows, ceil(d / 1024)).  The first block of a row also copies the rotary factors of the
+// row's position for every layer of the call: rope_tab[r][i] = rope_pos[pos[r]][i], i < half.
 template <typename T>
 __global__ void k_embed(const T *__restrict__ embed, const int *__restrict__ tok, float *x, int d,
-                        int vocab, int *status, const int *__restrict__ pos, const double *__restrict__ inv_freq,
+                        int vocab, int *status, const int *__restrict__ pos, const float2 *__restrict__ rope_pos, int n_pos,
                         float2 *rope_tab, int half) {
   kernel_entry(TR_k_embed);
   int r = blockIdx.x, t = tok[r];
-  if (rope_tab && blockIdx.y == 0)
-    for (int i = threadIdx.x; i < half; i += blockDim.x) {
-      float c, s;
-      rope_cs(pos[r], inv_freq[i], &c, &s);
-      rope_tab[(long long)r * half + i] = make_float2(c, s);
-    }
+  if (blockIdx.y == 0)
+    for (int i = threadIdx.x; i < half; i += blockDim.x) rope_tab[(long long)r * half + i] = rope_pos[(long long)min(pos[r], n_pos - 1) * half + i];
   int i = (blockIdx.y * blockDim.x + threadIdx.x) * 4;
   if (t >= vocab) { if (threadIdx.x == 0 && blockIdx.y == 0) atomicMax(status, DREAM_DEV_BAD_INDEX); t = -1; }
   if (i >= d) return;
@@ -108,31 +102,26 @@ k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, int d, T 
 }
 
 // ---------------------------------------------------------------------------------------
-// Rotary angle of (position, pair index) = position * theta^(-2i/hd).  The inverse frequencies
-// are tabulated once in double; the product is taken in double and reduced to [-pi, pi] before
-// the single-precision sincos, so long prefixes lose no phase accuracy.
-__global__ void k_rope_table(double *inv_freq, int hd, float theta) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < hd / 2) inv_freq[i] = exp2(-2.0 * (double)i / (double)hd * log2((double)theta));
-}
-__device__ __forceinline__ void rope_cs(int pos, double inv, float *c, float *s) {
-  double a = (double)pos * inv;
-  const double two_pi = 6.283185307179586476925286766559;
-  a -= two_pi * rint(a / two_pi);
-  sincosf((float)a, s, c);
+// Rotary factors of every position a sequence can reach, made once: rope_pos[pos][i] = (cos, sin)(pos * theta^(-2i/hd)).
+// The inverse frequency and the product are taken in double and reduced to [-pi, pi] before
+// the single-precision sincos, so long prefixes lose no phase accuracy.  (Computed per row, head and layer, the
+// double arithmetic took a third of a prompt's k_qkv_post_target.)  grid (n_pos).
+__global__ void k_rope_table(float2 *rope_pos, int hd, float theta) {
+  const int pos = blockIdx.x, half = hd / 2;
+  for (int i = threadIdx.x; i < half; i += blockDim.x) {
+    double a = (double)pos * exp2(-2.0 * (double)i / (double)hd * log2((double)theta));
+    const double two_pi = 6.283185307179586476925286766559;
+    a -= two_pi * rint(a / two_pi);
+    float c, s;
+    sincosf((float)a, &s, &c);
+    rope_pos[(long long)pos * half + i] = make_float2(c, s);
+  }
 }
 
-// (cos, sin) of four neighbouring rotary indices i..i+3 (i a multiple of 4) of row r: from the
-// table k_embed made for the call's rows, or computed when there is none (prefill).
-__device__ __forceinline__ void rope_cs4(const float2 *tab, int r, int half, int pos, const double *inv_freq, int i,
-                                         float4 &cs01, float4 &cs23) {
-  if (tab) {
-    const float4 *t = reinterpret_cast<const float4 *>(tab + (long long)r * half + i);
-    cs01 = t[0]; cs23 = t[1];
-  } else {
-    rope_cs(pos, inv_freq[i], &cs01.x, &cs01.y); rope_cs(pos, inv_freq[i + 1], &cs01.z, &cs01.w);
-    rope_cs(pos, inv_freq[i + 2], &cs23.x, &cs23.y); rope_cs(pos, inv_freq[i + 3], &cs23.z, &cs23.w);
-  }
+// (cos, sin) of four neighbouring rotary indices i..i+3 (i a multiple of 4) of a row of a rotary table.
+__device__ __forceinline__ void rope_cs4(const float2 *tab, int row, int half, int i, float4 &cs01, float4 &cs23) {
+  const float4 *t = reinterpret_cast<const float4 *>(tab + (long long)row * half + i);
+  cs01 = t[0]; cs23 = t[1];
 }
 
 // Where a row's K/V go.  Target cache: pages [layer][2][page][H_kv][page_tokens][hd].
@@ -155,13 +144,13 @@ __device__ __forceinline__ void rotate4(float4 &a, float4 &b, const float4 &cs01
   a = ra;
 }
 
-// After the QKV GEMM of target rows: rotary on q and k at row_pos, q -> qbuf (fp32),
+// After the QKV GEMM of target rows: rotary on q and k (row r of rope_tab), q -> qbuf,
 // k, v -> the paged cache at (row_seq, row_slot).  grid (rows, ceil(items / 256)); a work item
 // is four neighbouring rotary pairs of one head, read and written as 128-bit words.
 template <typename T>
-__global__ void __launch_bounds__(256)
-k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_slot,
-                  int row0, void *qbuf, PagedKV kv, int H, const double *__restrict__ inv_freq, const float2 *__restrict__ rope_tab) {
+__global__ void __launch_bounds__(256, 5)
+k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_slot,
+                  int row0, void *qbuf, PagedKV kv, int H, const float2 *__restrict__ rope_tab) {
   pdl_trigger();
   const int r = blockIdx.x + row0, lr = blockIdx.x;
   const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv;     // hd / 8 items per head
@@ -170,10 +159,10 @@ k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, con
   for (int pass = warm_first(); pass < 2; ++pass) {
     const bool live = warm_pass(pass, TR_k_qkv_post_target);
     bool on = live && hh < H + 2 * Hkv;
-    const int seq = on ? row_seq[r] : 0, pos = on ? row_pos[r] : 0, slot = on ? row_slot[r] : 0;
+    const int seq = on ? row_seq[r] : 0, slot = on ? row_slot[r] : 0;
     if (hh >= H && slot < 0) on = false;               // an idle row (malformed tree node) stores no K/V
     float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
-    if (on && hh < H + Hkv) rope_cs4(rope_tab, r, half, pos, inv_freq, i, cs01, cs23);      // fetched along with the slots
+    if (on && hh < H + Hkv) rope_cs4(rope_tab, r, half, i, cs01, cs23);      // fetched along with the slots
     const float inv = row_inv_rms(norm, lr, live);
     float4 a = gemm_val4<3>(g, lr, hh * hd + i, on), b = gemm_val4<3>(g, lr, hh * hd + i + half, on);
     scale4(a, inv); scale4(b, inv);
@@ -208,10 +197,10 @@ struct FlatKV {
 
 // After a draft QKV GEMM (has_q: the GEMM produced q columns first, then K, then V; otherwise
 // K then V only): rotary, q -> qbuf (when has_q), k/v -> draft self-attention cache row
-// row_dst[r] (skipped when < 0).  Work items and grid as in k_qkv_post_target.
-__global__ void __launch_bounds__(256)
+// row_dst[r] (skipped when < 0).  The rotary table is by row, or by position.  Work items and grid as in k_qkv_post_target.
+__global__ void __launch_bounds__(256, 5)
 k_qkv_post_draft(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_dst,
-                 int has_q, void *qbuf, FlatKV kv, int H, const double *__restrict__ inv_freq, const float2 *__restrict__ rope_tab) {
+                 int has_q, void *qbuf, FlatKV kv, int H, const float2 *__restrict__ rope_tab, int by_pos) {
   pdl_trigger();
   const int r = blockIdx.x;
   const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv, Hq = has_q ? H : 0;
@@ -220,10 +209,10 @@ k_qkv_post_draft(GemmOut g, RowScale norm, const int *__restrict__ row_seq, cons
   for (int pass = warm_first(); pass < 2; ++pass) {
     const bool live = warm_pass(pass, TR_k_qkv_post_draft);
     bool on = live && hh < Hq + 2 * Hkv;
-    const int dst = on ? row_dst[r] : 0, seq = on ? row_seq[r] : 0, pos = on ? row_pos[r] : 0;
+    const int dst = on ? row_dst[r] : 0, seq = on ? row_seq[r] : 0, tab_row = on && by_pos ? row_pos[r] : r;
     if (hh >= Hq && dst < 0) on = false;
     float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
-    if (on && hh < Hq + Hkv) rope_cs4(rope_tab, r, half, pos, inv_freq, i, cs01, cs23);
+    if (on && hh < Hq + Hkv) rope_cs4(rope_tab, tab_row, half, i, cs01, cs23);
     const float inv = row_inv_rms(norm, r, live);
     float4 a = gemm_val4<3>(g, r, hh * hd + i, on), b = gemm_val4<3>(g, r, hh * hd + i + half, on);
     scale4(a, inv); scale4(b, inv);

@@ -501,12 +501,10 @@ __global__ void k_select_tap(const float *__restrict__ ae, int mode, int fixed, 
 // Visual-token selection (Section 3.3): the k visual tokens with the largest importance (ties
 // -> lower index), returned ascending; then the compressed context C = kept visual
 // positions plus all text positions, ascending.  One block.
-__global__ void k_select_visual(const float *__restrict__ scores_all, long long layer_stride,
-                                const int *__restrict__ tap, int tap_lo, int v, int k, int vis_start,
+__global__ void k_select_visual(const float *__restrict__ sc, int v, int k, int vis_start,
                                 int n, const int *__restrict__ forced, int *kept, float *scores_out,
                                 int *ctx_pos, int *flags /* [n] scratch */) {
   kernel_entry(TR_k_select_visual);
-  const float *sc = scores_all + (long long)(*tap - tap_lo) * layer_stride;
   for (int j = threadIdx.x; j < n; j += blockDim.x) flags[j] = (j < vis_start || j >= vis_start + v) ? 1 : 0;
   __syncthreads();
   if (forced) {
