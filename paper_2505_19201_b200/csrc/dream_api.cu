@@ -88,7 +88,7 @@ struct dream_ctx {
   long long accepts[DREAM_MAX_BATCH], epoch[DREAM_MAX_BATCH];
   int last_verify_n, last_verify_seq[DREAM_MAX_BATCH];   // the sequence list of the last dream_verify_tree
   int cur_seq[DREAM_MAX_BATCH];        // sequences of the call being enqueued, by slot
-  int tk_nsplit, tk_nv;                // vocabulary blocks of the top-k kernel, columns per thread (4 or 16)
+  int tk_nsplit;                       // most vocabulary blocks of the top-k kernel
   int *top_id, *argmax_i, *accept_len_i, *out_tokens_i, *comp_src_i;
   size_t gout_floats;
   // host side
@@ -153,10 +153,15 @@ static inline void launch_k(dream_ctx *c, const char *name, void (*kernel)(P...)
   c->launches++;
 }
 #define LAUNCH(c, kernel, grid, block, smem, ...) launch_k(c, #kernel, kernel, dim3(grid), dim3(block), (size_t)(smem), __VA_ARGS__)
-#define TOPK_LAUNCH(c, grid, ...)                                                        \
-  do {                                                                                   \
-    if ((c)->tk_nv == 4) LAUNCH(c, (k_topk_lse<4>), grid, TOPK_THREADS, 0, __VA_ARGS__); \
-    else LAUNCH(c, (k_topk_lse<16>), grid, TOPK_THREADS, 0, __VA_ARGS__);                \
+// Top-k of `rows` rows of logits: blocks of 1024 columns where they are few enough to be resident at once (a draft
+// pass: latency counts) and their lists few enough to merge, else of 4096.
+#define TOPK_LAUNCH(c, rows, g, norm, ktop, logits)                                                                                     \
+  do {                                                                                                                                  \
+    const int V_ = (c)->cfg.vocab, n4_ = (V_ + 1023) / 1024;                                                                            \
+    const bool small_ = n4_ * (ktop) <= 1024 && n4_ <= (c)->tk_nsplit && (rows) * n4_ <= 1184;                                          \
+    const int n_ = small_ ? n4_ : (V_ + TOPK_COLS - 1) / TOPK_COLS;                                                                     \
+    if (small_) LAUNCH(c, (k_topk_lse<4>), dim3(rows, n_), TOPK_THREADS, 0, g, norm, V_, ktop, n_, (c)->tks, (c)->top_val, (c)->top_id, (c)->lse_rows, logits); \
+    else LAUNCH(c, (k_topk_lse<16>), dim3(rows, n_), TOPK_THREADS, 0, g, norm, V_, ktop, n_, (c)->tks, (c)->top_val, (c)->top_id, (c)->lse_rows, logits);       \
   } while (0)
 
 // ------------------------------------------------------------------------------------- shapes
@@ -244,12 +249,9 @@ static dream_status check_config(const dream_config *c, TreeShape *ts) {
   if (tree_shape(c, ts)) return fail(nullptr, DREAM_E_UNSUPPORTED, "tree: depth<=15, topk<=16, beam*topk<=256, input nodes<=64, nodes<=128");
   if (c->max_batch * rows_per_seq_max(ts) > ROW_CHUNK)
     return fail(nullptr, DREAM_E_UNSUPPORTED, "max_batch * max(tree nodes, depth + 2, widest beam) must be <= 256");
-  {   // the top-k kernel's last block merges at most 1024 candidates (vocabulary blocks x list length)
-    int nv = (c->vocab + 1023) / 1024 * TOPK_MAX <= 1024 ? 4 : 16;
-    int nsplit = (c->vocab + nv * TOPK_THREADS - 1) / (nv * TOPK_THREADS);
-    if (nsplit * imax(ts->K, 2) > 1024)
-      return fail(nullptr, DREAM_E_UNSUPPORTED, "vocab / 4096 * max(tree_topk, 2) must be <= 1024");
-  }
+  // the top-k kernel's last block merges at most 1024 candidates (vocabulary blocks x list length)
+  if ((c->vocab + TOPK_COLS - 1) / TOPK_COLS * imax(ts->K, 2) > 1024)
+    return fail(nullptr, DREAM_E_UNSUPPORTED, "vocab / 4096 * max(tree_topk, 2) must be <= 1024");
   if (c->tap_mode == DREAM_TAP_FIXED) {
     if (c->tap_layer < 1 || c->tap_layer > c->n_layers) return fail(nullptr, DREAM_E_ARG, "tap_layer");
   } else if (c->tap_mode == DREAM_TAP_ENTROPY_MIN || c->tap_mode == DREAM_TAP_ENTROPY_MAX) {
@@ -390,9 +392,8 @@ static size_t carve(dream_ctx *c, char *base) {
   } else { c->am_part_o = nullptr; c->am_part_ml = nullptr; c->am_part_u = nullptr; }
   c->row_ent = f.track_entropy ? a.take<float>((size_t)f.n_layers * ROW_CHUNK * f.n_heads) : nullptr;
   c->ent_sum = f.track_entropy ? a.take<float>((size_t)MB * f.n_layers) : nullptr;
-  // small blocks (1024 columns) while the merge of the blocks' lists stays within 1024 candidates
-  c->tk_nv = (f.vocab + 1023) / 1024 * TOPK_MAX <= 1024 ? 4 : 16;
-  c->tk_nsplit = (f.vocab + c->tk_nv * TOPK_THREADS - 1) / (c->tk_nv * TOPK_THREADS);
+  c->tk_nsplit = imin(256, (f.vocab + 1023) / 1024);           // at least as many as blocks of 4096 columns
+  if (c->tk_nsplit < (f.vocab + TOPK_COLS - 1) / TOPK_COLS) c->tk_nsplit = (f.vocab + TOPK_COLS - 1) / TOPK_COLS;
   c->tks.pv = a.take<float>((size_t)ROW_CHUNK * c->tk_nsplit * TOPK_MAX);
   c->tks.pi = a.take<int>((size_t)ROW_CHUNK * c->tk_nsplit * TOPK_MAX);
   c->tks.pm = a.take<float>((size_t)ROW_CHUNK * c->tk_nsplit);
@@ -938,7 +939,7 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
   // first token: LM head on the last prompt row
   const RowScale last = norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
   GemmOut g = gemm<T>(c, c->lm_head, c->xn, mp, 1, f.vocab, d);
-  TOPK_LAUNCH(c, dim3(1, c->tk_nsplit), g, last, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
+  TOPK_LAUNCH(c, 1, g, last, 2, (float *)nullptr);
   LAUNCH(c, k_first_token, 1, 32, 0, c->top_id, c->top_val, first_token, first_margin);
   LAUNCH(c, k_set_seq, 1, 32, 0, c->sd, seq, n, c->top_id, -1, -1);
   LAUNCH(c, k_select_tap, 1, 32, 0, c->ae, f.tap_mode, f.tap_layer, f.tap_lo, f.tap_hi, c->sd.tap + seq, tap_layer);
@@ -1145,7 +1146,7 @@ static dream_status draft_impl(dream_ctx *c, const TreeBatch &tb, int B) {
       LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, rm.in, c->sd.nperm_m, flat(c, c->dmem));
     }
     g = gemm<T>(c, c->lm_head, c->xn, xm, R, f.vocab, d);
-    TOPK_LAUNCH(c, dim3(R, c->tk_nsplit), g, norm, f.vocab, ts.K, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, (float *)nullptr);
+    TOPK_LAUNCH(c, R, g, norm, ts.K, (float *)nullptr);
     int next_m = p < ts.D ? ts.beam[p] : 1;
     LAUNCH(c, k_tree_expand, B, 128, 0, tb, c->sd, c->dt, ts, p, m, c->top_val, c->top_id, c->lse_rows, rn, next_m);
     cur ^= 1;
@@ -1195,7 +1196,7 @@ static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *a
   }
   const RowScale norm = norm_rows<T>(c, c->x, gd, true, c->ln_f, R, xm, c->tapbuf, rm.seq, c->sd.tap, L);
   g = gemm<T>(c, c->lm_head, c->xn, xm, R, f.vocab, d);
-  TOPK_LAUNCH(c, dim3(R, c->tk_nsplit), g, norm, f.vocab, 2, c->tk_nsplit, c->tks, c->top_val, c->top_id, c->lse_rows, logits);
+  TOPK_LAUNCH(c, R, g, norm, 2, logits);
   LAUNCH(c, k_argmax_out, (R + 127) / 128, 128, 0, c->top_id, c->top_val, R, argmax, margin,
          argmax == c->argmax_i ? (int *)nullptr : c->argmax_i);
   return DREAM_OK;

@@ -305,7 +305,7 @@ __global__ void k_gather_rows(const float *__restrict__ src, const int *__restri
 // descending order, and the log-sum-exp of the row.  grid (rows, nsplit): block (r, sp) scans
 // columns [sp * NV * 256, (sp + 1) * NV * 256), NV (4 or 16) per thread held in registers, and leaves a
 // sorted partial list and an (m, z) pair; the block that finishes a row last merges the partials,
-// always in the same order.  Selection is KTOP rounds of a block-wide "best remaining" search.
+// always in the same order.  Selection is KTOP rounds of "best remaining" (topk_warp, topk_block).
 #define TOPK_MAX 16
 #define TOPK_THREADS 256
 #define TOPK_COLS 4096
@@ -317,59 +317,61 @@ struct TopkScratch {
   int *counter;    // [rows] blocks done; zero between launches
 };
 
-// The ktop best of a block's candidates (NV per thread, in registers), in order, to out_v/out_i.
-// Two levels, so that only one block-wide step is needed: every warp selects its own ktop best in
-// ktop rounds of "best remaining" (a scan of the thread's candidates and a warp reduction), then
-// warp 0 selects from the warps' lists the same way.  Ids are unique, so a winner has one owner.
-// sh_* hold TOPK_THREADS / 32 * TOPK_MAX entries.
-template <int NV>
-__device__ __forceinline__ void topk_round(const float (&v)[NV], const int (&id)[NV], unsigned &taken, float &wv, int &wi) {
-  float bv = -INFINITY;
-  int bi = 0x7fffffff, bj = -1;
-#pragma unroll
-  for (int j = 0; j < NV; ++j)
-    if (!((taken >> j) & 1u) && better(v[j], id[j], bv, bi)) { bv = v[j]; bi = id[j]; bj = j; }
-  wv = bv; wi = bi;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float ov = __shfl_xor_sync(0xffffffffu, wv, o);
-    int oi = __shfl_xor_sync(0xffffffffu, wi, o);
-    if (better(ov, oi, wv, wi)) { wv = ov; wi = oi; }
-  }
-  if (bj >= 0 && bi == wi && bv == wv) taken |= 1u << bj;
+// A float as an unsigned key of the same order (-0 = +0); 0 is below every number and stands for nothing (and NaN).
+__device__ __forceinline__ uint32_t topk_key(float v) {
+  const uint32_t u = __float_as_uint(v + 0.f);
+  return v == v ? u ^ (u & 0x80000000u ? 0xffffffffu : 0x80000000u) : 0u;
 }
-template <int NV>
-__device__ __forceinline__ void topk_rounds(const float (&v)[NV], const int (&id)[NV], int ktop, float *out_v, int *out_i,
-                                            float *sh_v, int *sh_i) {
-  constexpr int NW = TOPK_THREADS / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned taken = 0u;
+__device__ __forceinline__ float topk_value(uint32_t k) {
+  return k ? __uint_as_float(k ^ (k & 0x80000000u ? 0x80000000u : 0xffffffffu)) : -INFINITY;
+}
+// The ktop best of a warp's candidates (key[j] with id(j), NV per lane), larger key first, then lower id, to out_k, out_i.
+// A lane keeps its best at hand and looks for the next one only after it has won a round, and a round is two
+// warp reductions in hardware (five shuffle steps of a pair and a scan in every lane: three times as long).
+template <int NV, typename Id>
+__device__ __forceinline__ void topk_warp(uint32_t (&key)[NV], Id id, int ktop, uint32_t *out_k, int *out_i) {
+  uint32_t bk = 0u;
+  int bi = 0x7fffffff;
+  auto scan = [&]() {
+    bk = 0u; bi = 0x7fffffff;
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+      if (key[j] > bk || (key[j] == bk && bk && id(j) < bi)) { bk = key[j]; bi = id(j); }
+  };
+  scan();
+#pragma unroll 1
   for (int round = 0; round < ktop; ++round) {
-    float wv;
-    int wi;
-    topk_round<NV>(v, id, taken, wv, wi);
-    if (lane == 0) { sh_v[warp * TOPK_MAX + round] = wv; sh_i[warp * TOPK_MAX + round] = wi; }
+    const uint32_t wk = __reduce_max_sync(0xffffffffu, bk);
+    const int wi = __reduce_min_sync(0xffffffffu, bk == wk ? bi : 0x7fffffff);
+    if ((threadIdx.x & 31) == 0) { out_k[round] = wk; out_i[round] = wi; }
+    if (bk == wk && bi == wi && wk) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) if (id(j) == wi) key[j] = 0u;
+      scan();
+    }
+    __syncwarp();
   }
+}
+// ... of a block's candidates, to out_v, out_i: every warp selects its own ktop, then warp 0 selects from the warps' lists.
+// sh_* hold TOPK_THREADS / 32 * TOPK_MAX entries.
+template <int NV, typename Id>
+__device__ __forceinline__ void topk_block(uint32_t (&key)[NV], Id id, int ktop, float *out_v, int *out_i, uint32_t *sh_k, int *sh_i) {
+  constexpr int NW = TOPK_THREADS / 32, NC = NW * TOPK_MAX / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  topk_warp<NV>(key, id, ktop, sh_k + warp * TOPK_MAX, sh_i + warp * TOPK_MAX);
   __syncthreads();
   if (warp == 0) {
-    constexpr int NC = NW * TOPK_MAX / 32;           // candidates per lane
-    float cv[NC];
+    uint32_t ck[NC];
     int ci[NC];
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
-      int e = j * 32 + lane;
-      bool ok = e < NW * ktop;
-      int q = ok ? e / ktop : 0, w = ok ? e - q * ktop : 0;
-      cv[j] = ok ? sh_v[q * TOPK_MAX + w] : -INFINITY;
-      ci[j] = ok ? sh_i[q * TOPK_MAX + w] : 0x7fffffff;
+      const int e = j * 32 + lane, k = e % TOPK_MAX;          // entry k of list e / TOPK_MAX
+      ck[j] = k < ktop ? sh_k[e] : 0u;
+      ci[j] = k < ktop ? sh_i[e] : 0x7fffffff;
     }
-    unsigned tk = 0u;
-    for (int round = 0; round < ktop; ++round) {
-      float wv;
-      int wi;
-      topk_round<NC>(cv, ci, tk, wv, wi);
-      if (lane == 0) { out_v[round] = wv; out_i[round] = wi; }
-    }
+    __syncwarp();
+    topk_warp<NC>(ck, [&](int j) { return ci[j]; }, ktop, sh_k, sh_i);
+    if (lane < ktop) { out_v[lane] = topk_value(sh_k[lane]); out_i[lane] = sh_i[lane]; }
   }
   __syncthreads();
 }
@@ -379,16 +381,18 @@ __global__ void __launch_bounds__(TOPK_THREADS)
 k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts, float *top_val, int *top_id, float *lse,
            float *logits_out) {
   __shared__ float red[33];
-  __shared__ float sh_v[TOPK_THREADS / 32 * TOPK_MAX];
+  __shared__ uint32_t sh_k[TOPK_THREADS / 32 * TOPK_MAX];
   __shared__ int sh_i[TOPK_THREADS / 32 * TOPK_MAX];
   __shared__ int is_last;
   kernel_entry(TR_k_topk_lse);
   int r = blockIdx.x, sp = blockIdx.y, tid = threadIdx.x;
   int c0 = sp * (NV * TOPK_THREADS);
   float v[NV];
-  int id[NV];
+  const bool vec = (V & 3) == 0;
+  // column of a thread's candidate j (ascending in j)
+  auto id = [&](int j) { return vec ? c0 + ((j >> 2) * TOPK_THREADS + tid) * 4 + (j & 3) : c0 + j * TOPK_THREADS + tid; };
   const float inv = row_inv_rms(norm, r, true);
-  if ((V & 3) == 0) {
+  if (vec) {
     float4 q[NV / 4];
 #pragma unroll
     for (int j = 0; j < NV / 4; ++j) {
@@ -402,19 +406,15 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
       int c = c0 + (j * TOPK_THREADS + tid) * 4;
       if (logits_out && c < V) *reinterpret_cast<float4 *>(logits_out + (long long)r * V + c) = q[j];
       v[4 * j] = q[j].x; v[4 * j + 1] = q[j].y; v[4 * j + 2] = q[j].z; v[4 * j + 3] = q[j].w;
-      id[4 * j] = c; id[4 * j + 1] = c + 1; id[4 * j + 2] = c + 2; id[4 * j + 3] = c + 3;
     }
   } else {
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       int c = c0 + j * TOPK_THREADS + tid;
       v[j] = c < V ? gemm_val(g, r, c) * inv : -INFINITY;
-      id[j] = c;
       if (logits_out && c < V) logits_out[(long long)r * V + c] = v[j];
     }
   }
-#pragma unroll
-  for (int j = 0; j < NV; ++j) if (id[j] >= V) id[j] = 0x7fffffff;
   // (m, z) of this block's columns, combined in a fixed order
   float m = -INFINITY;
 #pragma unroll
@@ -431,7 +431,10 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
   float tot = block_sum(z, red);
   long long po = (long long)r * nsplit + sp;
   if (tid == 0) { ts.pm[po] = gm; ts.pz[po] = tot; }
-  topk_rounds<NV>(v, id, ktop, ts.pv + po * TOPK_MAX, ts.pi + po * TOPK_MAX, sh_v, sh_i);
+  uint32_t key[NV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) key[j] = id(j) < V ? topk_key(v[j]) : 0u;
+  topk_block<NV>(key, id, ktop, ts.pv + po * TOPK_MAX, ts.pi + po * TOPK_MAX, sh_k, sh_i);
   // the last block of the row merges
   __threadfence();
   __syncthreads();
@@ -444,7 +447,7 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
   if (!is_last) return;
   __threadfence();
   // candidates: nsplit lists of ktop entries, up to 4 per thread (nsplit * ktop <= 1024)
-  float cv[4];
+  uint32_t ck[4];
   int ci[4];
   int ncand = nsplit * ktop;
 #pragma unroll
@@ -452,8 +455,9 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
     int e = j * TOPK_THREADS + tid;
     bool ok = e < ncand;
     int q = ok ? e / ktop : 0, w = ok ? e - q * ktop : 0;
-    cv[j] = ok ? __ldcg(ts.pv + ((long long)r * nsplit + q) * TOPK_MAX + w) : -INFINITY;
     ci[j] = ok ? __ldcg(ts.pi + ((long long)r * nsplit + q) * TOPK_MAX + w) : 0x7fffffff;
+    const float cv = ok ? __ldcg(ts.pv + ((long long)r * nsplit + q) * TOPK_MAX + w) : 0.f;
+    ck[j] = ok && ci[j] != 0x7fffffff ? topk_key(cv) : 0u;
   }
   if (tid < 32) {                 // log-sum-exp of the row from the blocks' (max, sum) pairs, one warp, fixed order
     float pm[8], pz[8];           // up to 256 blocks
@@ -472,5 +476,5 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
     zz = warp_sum(zz);
     if (tid == 0) lse[r] = mm + logf(zz);
   }
-  topk_rounds<4>(cv, ci, ktop, top_val + (long long)r * ktop, top_id + (long long)r * ktop, sh_v, sh_i);
+  topk_block<4>(ck, [&](int j) { return ci[j]; }, ktop, top_val + (long long)r * ktop, top_id + (long long)r * ktop, sh_k, sh_i);
 }
