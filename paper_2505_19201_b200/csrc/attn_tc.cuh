@@ -178,7 +178,9 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
-  const int chunk = blockIdx.x, kvh = blockIdx.y / a.n_rt, rt = blockIdx.y - kvh * a.n_rt, slot = blockIdx.z;
+  // (prefill: the tiles with the most keys first, so that the last wave is short)
+  const int chunk = blockIdx.x, slot = blockIdx.z;
+  const int kvh = a.mode == AT_PREFILL ? blockIdx.y % a.hkv : blockIdx.y / a.n_rt, rt = a.mode == AT_PREFILL ? a.n_rt - 1 - blockIdx.y / a.hkv : blockIdx.y - kvh * a.n_rt;
   const int seq = a.slot_seq[slot];
   if (warp == 0) {      // a lane per ring stage: the set-up is a few instructions deep instead of a loop
     if (lane < STAGES) { mbar_init(k_full + lane, 1); mbar_init(k_empty + lane, 1); mbar_init(v_full + lane, 1); mbar_init(v_empty + lane, 1); }
