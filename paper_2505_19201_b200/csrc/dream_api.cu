@@ -353,14 +353,16 @@ static size_t carve(dream_ctx *c, char *base) {
   // GEMM output: the widest of every projection's footprint.  fp32: rows x N.  bf16: room for the
   // stream-K partial-sum slots (bound for <= 192 SMs).
   {
-    const int shapes[8][2] = {{c->qkvN, d}, {d, c->Hhd}, {2 * f.d_ff, d}, {d, f.d_ff}, {c->Hhd, d}, {c->kvN, d}, {f.vocab, d}, {0, 0}};
+    // (a fused epilogue's columns come in whole tiles of 256)
+    const int shapes[8][2] = {{(c->qkvN + 255) / 256 * 256, d}, {d, c->Hhd}, {(f.d_ff + 127) / 128 * 256, d}, {d, f.d_ff}, {c->Hhd, d}, {c->kvN, d}, {f.vocab, d}, {0, 0}};
     size_t need = 0;
     for (int i = 0; shapes[i][0]; ++i) {
       const int N = shapes[i][0], K = shapes[i][1], most = N == f.vocab && K == d ? ROW_CHUNK : c->PR;
       if (f.dtype == DREAM_BF16) {
-        // more workers mean more slots (never fewer than two); fewer rows mean fewer tiles, so more slots per tile
+        // more workers mean more slots, fewer rows fewer tiles and so more slots per tile; never fewer than two, and up to
+        // five behind full waves (a quarter of a wave shared by all)
         for (int rows = 16; rows <= most; rows += 16) {
-          const size_t fl = (size_t)imax(2, gemm_tc_split(192, rows, N, K).slots) * rows * N;
+          const size_t fl = (size_t)imax(rows > TC_TOKENS ? 5 : 2, gemm_tc_split(192, rows, N, K).slots) * rows * N;
           if (fl > need) need = fl;
         }
       } else if ((size_t)most * N > need) need = (size_t)most * N;
@@ -433,12 +435,12 @@ static XLayout xlay(XMode m, long long width) {
 // out[r][c] = sum_k X[r][k] W[c][k] for r < rows <= PR, c < N; X holds the rows in layout m.
 // Returns the descriptor consumers read the result through.
 template <typename T>
-static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int rows, int N, int K) {
+static GemmOut gemm(dream_ctx *c, const void *W, const void *X, XMode m, int rows, int N, int K, int epi = TC_EPI_STORE, const TcEpi *e = nullptr) {
   GemmOut g;
   if constexpr (sizeof(T) == 2) {
     bool timed = c->prof_on && 2 * (c->prof_n + 1) <= (int)c->prof_ev.size();
     if (timed) cudaEventRecord(c->prof_ev[2 * c->prof_n], c->stream);
-    if (!gemm_tc_launch(&c->tc, c->stream, W, X, m.mode, m.lo_rows, rows, N, K, c->gout, (long long)c->gout_floats, &g))
+    if (!gemm_tc_launch(&c->tc, c->stream, W, X, m.mode, m.lo_rows, rows, N, K, c->gout, (long long)c->gout_floats, &g, epi, e))
       c->gemm_failed = 1;
     if (timed) { cudaEventRecord(c->prof_ev[2 * c->prof_n + 1], c->stream); c->prof_n++; c->prof_bytes += 2.0 * N * K; }
     c->launches++;
@@ -884,8 +886,18 @@ static const RowScale NO_NORM = {nullptr, 0, 0.f, 0.f};
 template <typename T>
 static GemmOut mlp_rows(dream_ctx *c, const RowScale &norm, const void *wgu, const void *wd, int rows, XMode m) {
   const dream_config &f = c->cfg;
+  if constexpr (sizeof(T) == 2) {
+    if (rows > TC_TOKENS) {                    // a prompt: the GEMM's epilogue gates, the row kernel does the rest
+      TcEpi e = {};
+      e.norm = norm; e.dst = (bf16 *)c->act; e.lay = xlay(m, f.d_ff); e.ff = f.d_ff;
+      const GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model, TC_EPI_SILU, &e);
+      const int i0 = g.n_full / g.n_tt * 128;
+      if (i0 < f.d_ff) LAUNCH(c, (k_silu_mul<T, true>), dim3((f.d_ff - i0 + 1023) / 1024, rows), 256, 0, g, norm, (T *)c->act, f.d_ff, i0, xlay(m, f.d_ff));
+      return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
+    }
+  }
   GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model);
-  LAUNCH(c, (k_silu_mul<T>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, norm, (T *)c->act, f.d_ff, xlay(m, f.d_ff));
+  LAUNCH(c, (k_silu_mul<T, false>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, norm, (T *)c->act, f.d_ff, 0, xlay(m, f.d_ff));
   return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
 }
 
@@ -908,8 +920,20 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
   auto q_of = [&](int l) { return cand_of(l) < 0 ? c->qbuf : (void *)((float *)c->q_taps + (size_t)cand_of(l) * c->XR * c->Hhd); };
   // projections of layer l for the rows of one pass, whose normalised input sits in c->xn
   auto qkv = [&](int l, int r0, int rows, const RowScale &norm) {
+    if constexpr (sizeof(T) == 2) {
+      if (rows > TC_TOKENS) {                  // the GEMM's epilogue rotates and stores, the row kernel does the rest
+        TcEpi e = {};
+        e.norm = norm; e.dst = (bf16 *)q_of(l); e.H = f.n_heads; e.row0 = r0; e.seq = seq; e.rope_pos = c->rope_pos; e.kv = paged(c, l);
+        const GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d, TC_EPI_ROPE, &e);
+        const int hh0 = g.n_full / g.n_tt * (TC_BN / f.head_dim), left = c->qkvN - hh0 * f.head_dim;
+        if (left > 0)
+          LAUNCH(c, (k_qkv_post_target<T, true>), dim3(rows, (left / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].slot, r0, hh0, q_of(l),
+                 paged(c, l), f.n_heads, (const float2 *)c->rope_pos);
+        return;
+      }
+    }
     GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].slot, r0, q_of(l),
+    LAUNCH(c, (k_qkv_post_target<T, false>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].slot, r0, 0, q_of(l),
            paged(c, l), f.n_heads, (const float2 *)c->rope_pos);
   };
   for (int r0 = 0; r0 < n; r0 += CH) {
@@ -1188,7 +1212,7 @@ static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *a
     // the first norm completes S^l (for l >= 1) and captures it where a sequence taps layer l
     RowScale norm = norm_rows<T>(c, c->x, gd, l > 0, c->ln1[l], R, xm, l > 0 ? c->tapbuf : nullptr, rm.seq, c->sd.tap, l);
     g = gemm<T>(c, c->wqkv[l], c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.slot, 0, c->qbuf, paged(c, l), f.n_heads, (const float2 *)c->rope_tab);
+    LAUNCH(c, (k_qkv_post_target<T, false>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.slot, 0, 0, c->qbuf, paged(c, l), f.n_heads, (const float2 *)c->rope_tab);
     HD_DISPATCH(c, T, tree(c, l, R, xm, B, key_ub));
     g = gemm<T>(c, c->wo[l], c->attn_out, xm, R, d, c->Hhd);
     norm = norm_rows<T>(c, c->x, g, true, c->ln2[l], R, xm);

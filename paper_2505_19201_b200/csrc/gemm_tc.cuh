@@ -26,6 +26,11 @@
 //     (or all of them when there are fewer than two), is stream-K: its (tile, panel) units are dealt
 //     out in equal contiguous ranges; a pair that covers part of a tile writes a partial sum to its own
 //     slot and the consumer adds the slots in a fixed order;
+//   * a prompt's gate/up and QKV projections finish in the epilogue (TC_EPI_SILU, TC_EPI_ROPE): their weight rows
+//     are loaded in pairs (gate and up of a column; the two halves of a rotary pair), 16 rows of one kind and
+//     16 of the other per TMEM lane quarter, so that one shuffle brings a pair together, and the
+//     finished values go where the next kernel reads them.  Only the stream-K tiles still leave partial
+//     sums (in the same paired column order) for the row kernel;
 //   * programmatic dependent launch: W never changes, so its ring fills before the grid
 //     dependency resolves; only the X producer and the epilogue wait for the previous kernel;
 //   * the MMA issuer and the producers are whole warps that run their loops together and elect a lane for
@@ -45,6 +50,7 @@
 #include <tuple>
 
 #include "common.cuh"
+#include "rows.cuh"
 
 #define TC_BN 256               // weight rows per tile (MMA M, both CTAs)
 #define TC_BK 64                // k elements per panel (128 bytes: one swizzle row)
@@ -62,6 +68,20 @@ enum { TC_X_PLAIN = 0, TC_X_PLANAR = 1 };
 // code is fetched anew at every launch and each division in it shows (one kernel for all: rounds 4 % slower).
 enum { TC_X_ONE = 0, TC_X_CONCAT = 1, TC_X_TWO = 2, TC_X_TILES = 3 };
 
+enum { TC_EPI_STORE = 0, TC_EPI_SILU = 1, TC_EPI_ROPE = 2 };
+#define TC_MAX_ROWS 1280        // token rows of a launch with a fused epilogue
+
+// What a fused epilogue needs besides the sums.
+struct TcEpi {
+  RowScale norm;                // of the input rows
+  bf16 *dst;                    // SILU: act rows (row_stride, lo_delta apart).  ROPE: query rows [row][head][hi | lo][hd]
+  XLayout lay;
+  int ff;                       // SILU: real gate columns
+  int H, row0, seq;             // ROPE: query heads; the prompt row of token 0 (its position and cache slot)
+  const float2 *rope_pos;
+  PagedKV kv;
+};
+
 struct TcParams {
   float *out;
   long long slot_stride;        // floats between partial-sum slots
@@ -75,6 +95,7 @@ struct TcParams {
   int lo_rows;                  // row of the first low part in the X tensor map
   int wp, w_stages, x_stages;   // panels per stage, ring depths
   int *status;
+  TcEpi epi;
 };
 
 // ------------------------------------------------------------------------------------------ PTX wrappers
@@ -223,11 +244,47 @@ template <bool TILES> struct TcWalk {
   }
 };
 
+// Eight lanes hold one column each of eight rows (v[j]: row j): turned so that lane m of the eight stores 8 consecutive
+// columns of row m in one piece per part, high parts at d and (lo_delta != 0) low parts lo_delta behind.  (Stored one
+// by one as 2-byte words the epilogue outlasted the MMAs of the next tile: 6 % of a request.)
+__device__ __forceinline__ void tc_store8(const float (&v)[8], int lane, bool on, bf16 *d, long long lo_delta) {
+  uint32_t w[8];                               // high part | low part
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const bf16 h = __float2bfloat16_rn(v[j]), l = __float2bfloat16_rn(v[j] - __bfloat162float(h));
+    w[j] = (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
+  }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (!(j & o)) {
+        const bool up = (lane & o) != 0;
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? w[j] : w[j | o], o);
+        if (up) w[j] = got; else w[j | o] = got;
+      }
+  if (!on) return;
+  *reinterpret_cast<uint4 *>(d) = make_uint4(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410), __byte_perm(w[4], w[5], 0x5410), __byte_perm(w[6], w[7], 0x5410));
+  if (lo_delta)
+    *reinterpret_cast<uint4 *>(d + lo_delta) = make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632), __byte_perm(w[4], w[5], 0x7632), __byte_perm(w[6], w[7], 0x7632));
+}
+
+// Weight rows of pair `a` (0..127, a multiple of 16) of column tile ct.
+template <int EPI>
+__device__ __forceinline__ void tc_pair_rows(const TcEpi &e, int ct, int a, int &ya, int &yb) {
+  if (EPI == TC_EPI_SILU) { ya = ct * 128 + a; yb = e.ff + ya; }
+  else {
+    const int half_log2 = 30 - __clz(e.kv.hd), half = 1 << half_log2;
+    ya = ct * TC_BN + (a >> half_log2) * e.kv.hd + (a & (half - 1));
+    yb = ya + half;
+  }
+}
+
 // ------------------------------------------------------------------------------------------ kernel
 // Dynamic shared memory (1024-byte aligned): W ring [w_stages][wp][16 KB], X ring [x_stages][wp][panel], barriers.
 // Registers: the decode forms are held to 64, so that the row kernel that waits for this launch is resident beside
 // it as a whole (its blocks have started, hence the next GEMM's CTAs can start as soon as these leave).
-template <int FORM>
+template <int FORM, int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, FORM >= TC_X_TWO ? 1 : 2)
 k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const __grid_constant__ TcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -242,6 +299,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   uint64_t *acc_full = full_x + TC_MAX_STAGES, *acc_empty = acc_full + 2;
   uint32_t *tmem_base_p = (uint32_t *)(acc_empty + 2);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
+  float *inv_s = (float *)(bars + 64);         // EPI: 1 / rms of every token row, 512 bytes behind the barriers' start
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   const uint32_t rank = cluster_ctarank();
@@ -288,7 +346,17 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         if (elect_one()) {
           if (rank == 0) mbar_expect_tx(full_w + s, 2u * (uint32_t)np * TC_WPANEL);
           uint8_t *dst = wring + (size_t)s * wstage_bytes;
-          for (int i = 0; i < np; ++i) tma_load_2d_pair(dst + (size_t)i * TC_WPANEL, &map_w, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
+          if (EPI == TC_EPI_STORE) {
+            for (int i = 0; i < np; ++i) tma_load_2d_pair(dst + (size_t)i * TC_WPANEL, &map_w, bar0 + 8u * s, (kb + i) * TC_BK, y, pol);
+          } else {                               // pairs of 16 rows (one panel per stage)
+#pragma unroll 1
+            for (int g = 0; g < 4; ++g) {
+              int ya, yb;
+              tc_pair_rows<EPI>(p.epi, tile / p.n_tt, (int)rank * 64 + g * 16, ya, yb);
+              tma_load_2d_pair(dst + g * 4096, &map_w, bar0 + 8u * s, kb * TC_BK, ya, pol);
+              tma_load_2d_pair(dst + g * 4096 + 2048, &map_w, bar0 + 8u * s, kb * TC_BK, yb, pol);
+            }
+          }
         }
         __syncwarp();
         if (++s == p.w_stages) { s = 0; ph ^= 1; }
@@ -389,6 +457,27 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t done_bar = mapa(smem_u32(acc_empty), 0);
     pdl_wait();                               // the output buffer belongs to earlier kernels
+    if (EPI != TC_EPI_STORE) {                // the rows' factors, a thread per row, while the first tile is computed
+      const RowScale n = p.epi.norm;
+#pragma unroll 1
+      for (int t = threadIdx.x - 128; t < p.n_tok; t += 256) {
+        const float *row = n.ssq + (long long)t * SSQ_LD;
+        float sum = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < n.parts; i += 16) {
+          float4 v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] = ld_f4(row + i + 4 * k);     // (a row has room for SSQ_LD pieces, what lies behind `parts` is not used)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int left = n.parts - i - 4 * k;
+            sum += (left > 0 ? v[k].x : 0.f) + (left > 1 ? v[k].y : 0.f) + (left > 2 ? v[k].z : 0.f) + (left > 3 ? v[k].w : 0.f);
+          }
+        }
+        inv_s[t] = rsqrtf(sum * n.inv_d + n.eps);
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+    }
     uint32_t fill = 0;
     bool ok = true;
     auto wait_full = [&](uint32_t buf, uint32_t use) {
@@ -427,7 +516,58 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(done_bar + 8u * buf);
         }
-        if (ok && c < p.N) {
+        if (EPI != TC_EPI_STORE && sk_tile < 0) {
+          // lanes l and l + 16 hold the two columns of a pair; each takes 8 of a group's 16 tokens
+          const TcEpi &e = p.epi;
+          const int a0 = (int)rank * 64 + q * 16 + (lane & 15), hi16 = lane >> 4;       // pair index in the tile
+          int ya, yb;
+          tc_pair_rows<EPI>(e, ct, a0, ya, yb);
+          const int hd_log2 = EPI == TC_EPI_ROPE ? 31 - __clz(e.kv.hd) : 0, hh = ya >> hd_log2, i = ya - (hh << hd_log2), hkv = e.kv.hkv;
+          const bool col_ok = EPI == TC_EPI_SILU ? ya < e.ff : hh < e.H + 2 * hkv;
+#pragma unroll
+          for (int g = 0; g < 8; ++g) {
+            if ((2 * g + half) * 16 >= nt) continue;                                    // (warp-uniform)
+            // the 8 tokens from t0 on, in the column this lane holds
+            const int t0 = (2 * g + half) * 16 + hi16 * 8;
+            float va[8], vb[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float lo8 = run[g * 16 + j], hi8 = run[g * 16 + 8 + j];
+              const float other = __shfl_xor_sync(0xffffffffu, hi16 ? lo8 : hi8, 16);
+              va[j] = hi16 ? other : lo8; vb[j] = hi16 ? hi8 : other;
+            }
+            const float4 i0 = *reinterpret_cast<const float4 *>(inv_s + tok0 + t0), i1 = *reinterpret_cast<const float4 *>(inv_s + tok0 + t0 + 4);
+            const float inv[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
+            const int t = t0 + (lane & 7);                    // the token this lane stores
+            const bool st = ok && col_ok && t < nt;
+            if (EPI == TC_EPI_SILU) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float x = va[j] * inv[j];
+                va[j] = x / (1.f + __expf(-x)) * (vb[j] * inv[j]);
+              }
+              tc_store8(va, lane, st, e.dst + (long long)(tok0 + t) * e.lay.row_stride + (ya & ~7), e.lay.lo_delta);
+            } else {
+              const int r0 = e.row0 + tok0 + t0, r = e.row0 + tok0 + t;
+              const bool rot = hh < e.H + hkv, is_q = hh < e.H;
+              const int v = rot ? 0 : 1;
+              bf16 *d = !st ? e.dst
+                        : is_q ? e.dst + (((long long)r * e.H + hh) << (hd_log2 + 1)) + (i & ~7)
+                               : (bf16 *)e.kv.base + (v ? e.kv.kv_stride : 0) + e.kv.off(e.seq, r, hh - e.H - (v ? hkv : 0)) + (i & ~7);
+              float2 cs[8];
+#pragma unroll
+              for (int j = 0; j < 8; ++j) cs[j] = rot && t0 + j < nt ? e.rope_pos[(long long)(r0 + j) * (e.kv.hd >> 1) + i] : make_float2(1.f, 0.f);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float x = va[j] * inv[j], y = vb[j] * inv[j];
+                va[j] = x * cs[j].x - y * cs[j].y;
+                vb[j] = y * cs[j].x + x * cs[j].y;
+              }
+              tc_store8(va, lane, st, d, is_q ? e.kv.hd : 0);
+              tc_store8(vb, lane, st, d + (e.kv.hd >> 1), is_q ? e.kv.hd : 0);
+            }
+          }
+        } else if (ok && c < p.N) {
 #pragma unroll
           for (int g = 0; g < 8; ++g)
 #pragma unroll
@@ -502,10 +642,11 @@ static inline const char *gemm_tc_plan_init(GemmTcPlan *pl, int *status, int use
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&pl->n_sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&pl->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (cudaFuncSetAttribute(k_gemm_tc<TC_X_ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_gemm_tc<TC_X_CONCAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_gemm_tc<TC_X_TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_gemm_tc<TC_X_TILES>, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) != cudaSuccess)
+  bool ok = true;
+  auto raise = [&](auto *kernel) { ok = ok && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl->max_smem) == cudaSuccess; };
+  raise(k_gemm_tc<TC_X_ONE, TC_EPI_STORE>); raise(k_gemm_tc<TC_X_CONCAT, TC_EPI_STORE>); raise(k_gemm_tc<TC_X_TWO, TC_EPI_STORE>);
+  raise(k_gemm_tc<TC_X_TILES, TC_EPI_STORE>); raise(k_gemm_tc<TC_X_TILES, TC_EPI_SILU>); raise(k_gemm_tc<TC_X_TILES, TC_EPI_ROPE>);
+  if (!ok)
     return "cannot raise the dynamic shared memory limit";
   pl->status = status;
   pl->use_pdl = use_pdl;
@@ -540,6 +681,7 @@ static inline bool tc_map(GemmTcPlan *pl, const void *ptr, int rows, int K, int 
   return true;
 }
 
+static inline int imax_tc(int a, int b) { return a > b ? a : b; }
 // How a launch of `rows` token rows is cut (see the head of the file).
 struct TcSplit { int n_tt, tile_t, n_pairs, n_waves, sk_units, upc, slots; };
 static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
@@ -549,7 +691,9 @@ static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
   // tokens in 16s (the N of an MMA over both CTAs); up to 128 rows both planes share an MMA, so 8s do
   t.tile_t = t.n_tt > 1 || rows > 128 ? ((rows + t.n_tt - 1) / t.n_tt + 15) & ~15 : (rows + 7) & ~7;
   const int pairs = n_sms / 2 > 0 ? n_sms / 2 : 1, tiles = (N + TC_BN - 1) / TC_BN * t.n_tt;
-  t.n_waves = t.n_tt > 1 && tiles / pairs > 1 ? tiles / pairs - (tiles % pairs ? 1 : 0) : 0;
+  // full waves, less one when the rest alone is so small that a tile would be shared by many pairs
+  t.n_waves = t.n_tt > 1 ? tiles / pairs : 0;
+  if (t.n_waves && tiles % pairs && 4 * (tiles % pairs) < pairs) --t.n_waves;
   t.sk_units = (tiles - t.n_waves * pairs) * KB;
   t.upc = t.sk_units ? (t.sk_units + pairs - 1) / pairs : 1;
   t.n_pairs = t.n_waves ? pairs : (t.sk_units + t.upc - 1) / t.upc;
@@ -566,8 +710,14 @@ static inline long long gemm_tc_out_floats(int n_sms, int rows, int N, int K) {
 //   high part, row lo_rows + t = low part.
 // *g receives the descriptor consumers read the result through.  Returns false if the launch could
 // not be made.
+//   epi / e: a fused epilogue (launches of several token tiles only).  The sums of the stream-K tiles (n_full and up) then
+//   lie in pairs: N counts 256 columns per column tile of 128 pairs.
 static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const void *W, const void *X, int x_mode, int lo_rows,
-                                  int rows, int N, int K, float *out, long long out_floats, GemmOut *g) {
+                                  int rows, int N, int K, float *out, long long out_floats, GemmOut *g, int epi = TC_EPI_STORE, const TcEpi *e = nullptr) {
+  const int w_rows = N;
+  if (epi == TC_EPI_SILU) N = (e->ff + 127) / 128 * TC_BN;
+  if (epi == TC_EPI_ROPE) N = (N + TC_BN - 1) / TC_BN * TC_BN;
+  if (epi != TC_EPI_STORE && (rows > TC_MAX_ROWS || rows <= TC_TOKENS)) return false;
   if (rows < 1 || (x_mode == TC_X_PLAIN && rows > 128)) return false;
   const TcSplit t = gemm_tc_split(pl->n_sms, rows, N, K);
   if (t.sk_units + K / TC_BK >= 1 << 21) return false;          // div_small
@@ -589,7 +739,7 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   CUtensorMap mw, mx;
   const int x_rows = x_mode == TC_X_PLANAR ? lo_rows + rows : rows;
   const int x_box = form == TC_X_CONCAT ? p.tile_t : p.mma_n / 2;
-  if (!tc_map(pl, W, N, K, 128, &mw) || !tc_map(pl, X, x_rows, K, x_box, &mx)) return false;
+  if (!tc_map(pl, W, w_rows, K, epi == TC_EPI_STORE ? 128 : 16, &mw) || !tc_map(pl, X, x_rows, K, x_box, &mx)) return false;
   g->base = p.out; g->slot_stride = p.slot_stride; g->ld = N; g->kb = p.KB; g->n_full = p.n_full; g->n_tt = p.n_tt;
   g->inv_upc = p.inv_upc; g->inv_tile = p.n_tt > 1 ? 1.f / (float)p.tile_t : 0.f;
   // Stages of two panels halve the waits and commits per panel (61 rows, 12288 x 4096: 22.2 -> 20.9 us) as
@@ -597,21 +747,25 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   // rings are deeper with one
   const int xpanel = x_box * 128 * (form >= TC_X_TWO ? 2 : 1);
   p.wp = xpanel <= TC_WPANEL / 2 ? 2 : 1;
+  if (e) p.epi = *e;
+  const int epi_bytes = epi == TC_EPI_STORE ? 0 : TC_MAX_ROWS * 4;
+  if (epi != TC_EPI_STORE) p.wp = 1;
   const int xstage = p.wp * xpanel, wstage = p.wp * TC_WPANEL;
   // a few KB stay free for the blocks of the row kernel that waits beside this launch (1 KB each)
-  const int room = pl->max_smem - 2048 - 4096;
+  const int room = pl->max_smem - 2048 - imax_tc(4096, epi_bytes);
   p.x_stages = xpanel < TC_WPANEL ? 6 / p.wp : xpanel == TC_WPANEL ? 4 : room / (xstage + wstage);
   p.w_stages = (room - p.x_stages * xstage) / wstage;
   if (p.w_stages > TC_MAX_STAGES) p.w_stages = TC_MAX_STAGES;
   if (p.w_stages < 2 || p.x_stages < 2) return false;
   p.status = pl->status;
-  size_t smem = (size_t)p.w_stages * wstage + (size_t)p.x_stages * xstage + 2048;
+  size_t smem = (size_t)p.w_stages * wstage + (size_t)p.x_stages * xstage + 2048 + epi_bytes;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * p.n_pairs); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = pl->use_pdl ? 1 : 0;
-  auto *kernel = form == TC_X_CONCAT ? k_gemm_tc<TC_X_CONCAT> : form == TC_X_TWO ? k_gemm_tc<TC_X_TWO> : form == TC_X_TILES ? k_gemm_tc<TC_X_TILES> : k_gemm_tc<TC_X_ONE>;
+  auto *kernel = form == TC_X_CONCAT ? k_gemm_tc<TC_X_CONCAT, TC_EPI_STORE> : form == TC_X_TWO ? k_gemm_tc<TC_X_TWO, TC_EPI_STORE> : form == TC_X_ONE ? k_gemm_tc<TC_X_ONE, TC_EPI_STORE>
+               : epi == TC_EPI_SILU ? k_gemm_tc<TC_X_TILES, TC_EPI_SILU> : epi == TC_EPI_ROPE ? k_gemm_tc<TC_X_TILES, TC_EPI_ROPE> : k_gemm_tc<TC_X_TILES, TC_EPI_STORE>;
   return cudaLaunchKernelEx(&cfg, kernel, mw, mx, p) == cudaSuccess;
 }

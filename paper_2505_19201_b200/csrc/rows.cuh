@@ -144,27 +144,35 @@ __device__ __forceinline__ void rotate4(float4 &a, float4 &b, const float4 &cs01
   a = ra;
 }
 
+// Column of the first value of pair `a` of column tile ct in the paired order of a GEMM with a fused epilogue
+// (gemm_tc.cuh): 16 first and 16 second values alternate.
+__device__ __forceinline__ int paired_col(int ct, int a) { return ct * 256 + (a >> 6) * 128 + ((a & 63) >> 4) * 32 + (a & 15); }
+__device__ __forceinline__ int gemm_tile(const GemmOut &g, int r, int c) { return (c >> 8) * g.n_tt + div_small(r, g.inv_tile); }
+
 // After the QKV GEMM of target rows: rotary on q and k (row r of rope_tab), q -> qbuf,
 // k, v -> the paged cache at (row_seq, row_slot).  grid (rows, ceil(items / 256)); a work item
-// is four neighbouring rotary pairs of one head, read and written as 128-bit words.
-template <typename T>
+// is four neighbouring rotary pairs of one head, read and written as 128-bit words.  PAIRED: only what the GEMM's own
+// epilogue has left (its stream-K tiles, in paired columns), from head hh0 on.
+template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(256, 5)
 k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_slot,
-                  int row0, void *qbuf, PagedKV kv, int H, const float2 *__restrict__ rope_tab) {
+                  int row0, int hh0, void *qbuf, PagedKV kv, int H, const float2 *__restrict__ rope_tab) {
   pdl_trigger();
   const int r = blockIdx.x + row0, lr = blockIdx.x;
   const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv;     // hd / 8 items per head
-  const int w = blockIdx.y * 256 + threadIdx.x, hh = w >> q4_log2, i = (w - (hh << q4_log2)) * 4;
+  const int w = blockIdx.y * 256 + threadIdx.x, hw = w >> q4_log2, hh = hh0 + hw, i = (w - (hw << q4_log2)) * 4;
+  const int ca = PAIRED ? paired_col(hh * hd >> 8, ((hh * hd & 255) >> 1) + i) : hh * hd + i, cb = ca + (PAIRED ? 16 : half);
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
     const bool live = warm_pass(pass, TR_k_qkv_post_target);
     bool on = live && hh < H + 2 * Hkv;
+    if (PAIRED) on = on && gemm_tile(g, lr, ca) >= g.n_full;
     const int seq = on ? row_seq[r] : 0, slot = on ? row_slot[r] : 0;
     if (hh >= H && slot < 0) on = false;               // an idle row (malformed tree node) stores no K/V
     float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
     if (on && hh < H + Hkv) rope_cs4(rope_tab, r, half, i, cs01, cs23);      // fetched along with the slots
     const float inv = row_inv_rms(norm, lr, live);
-    float4 a = gemm_val4<3>(g, lr, hh * hd + i, on), b = gemm_val4<3>(g, lr, hh * hd + i + half, on);
+    float4 a = gemm_val4<3>(g, lr, ca, on), b = gemm_val4<3>(g, lr, cb, on);
     scale4(a, inv); scale4(b, inv);
     rotate4(a, b, cs01, cs23);
     if (!on) continue;
@@ -269,17 +277,18 @@ k_mem_append(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__
 }
 
 // act = silu(gate) * up, from a GEMM output whose columns are [gate(ff) | up(ff)].
-// grid (ceil(ff / 1024), rows).
-template <typename T>
+// grid (ceil(ff / 1024), rows).  PAIRED: only what the GEMM's own epilogue has left, from gate column i0 on.
+template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(256, 8)
-k_silu_mul(GemmOut g, RowScale norm, T *act, int ff, XLayout lay) {
+k_silu_mul(GemmOut g, RowScale norm, T *act, int ff, int i0, XLayout lay) {
   pdl_trigger();
-  const int r = blockIdx.y, i = (blockIdx.x * 256 + threadIdx.x) * 4;
+  const int r = blockIdx.y, i = i0 + (blockIdx.x * 256 + threadIdx.x) * 4;
+  const int ca = PAIRED ? paired_col(i >> 7, i & 127) : i, cb = ca + (PAIRED ? 16 : ff);
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool live = warm_pass(pass, TR_k_silu_mul), on = live && i < ff;
+    const bool live = warm_pass(pass, TR_k_silu_mul), on = live && i < ff && (!PAIRED || gemm_tile(g, r, ca) >= g.n_full);
     const float inv = row_inv_rms(norm, r, live);
-    float4 a = gemm_val4<2>(g, r, i, on), b = gemm_val4<2>(g, r, ff + i, on);
+    float4 a = gemm_val4<2>(g, r, ca, on), b = gemm_val4<2>(g, r, cb, on);
     scale4(a, inv); scale4(b, inv);
     const float4 o = make_float4(a.x / (1.f + __expf(-a.x)) * b.x, a.y / (1.f + __expf(-a.y)) * b.y,
                                  a.z / (1.f + __expf(-a.z)) * b.z, a.w / (1.f + __expf(-a.w)) * b.w);

@@ -21,12 +21,20 @@ def test_prompt(n, draft_blocks):
         pr.close()
 
 
-def test_wide_model_long_prompt():
-    """As many token tiles as give full waves of tiles and a stream-K rest, at a real model's widths."""
+# as many token tiles as give full waves of tiles (whose projections finish in the GEMM's epilogue) and a stream-K
+# rest, at real models' widths: head_dim 128 in two passes, 64, 128 with grouped queries, 256; an odd gate width
+@pytest.mark.parametrize("model,over", [
+    ("llava7b", dict(n_visual=700, k_visual=100, n_prompt=620)),
+    ("smolvlm2b", dict(n_visual=900, k_visual=100, n_prompt=252)),
+    ("smolvlm2b", dict(n_visual=300, k_visual=100, n_prompt=701, d_ff=8000)),
+    ("pixtral12b", dict(n_visual=500, k_visual=100, n_prompt=250)),
+    ("gemma3_12b", dict(n_visual=256, k_visual=64, n_prompt=901)),
+])
+def test_wide_models(model, over):
     from tests.parity import Pair
-    pr = Pair("llava7b", n_layers=1, n_visual=700, k_visual=100, n_prompt=620, decode_steps=2, tap_lo=1, tap_hi=1)
+    pr = Pair(model, n_layers=1, vocab=2048, decode_steps=2, tap_lo=1, tap_hi=1, **over)
     try:
-        pr.prefill()
+        pr.prefill(vis_start=over["n_prompt"] // 2)
         pr.step()
     finally:
         pr.close()
