@@ -145,13 +145,6 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t saddr, uint32_t lbo_by
   return d;
 }
 
-// Reads from the shared memory of a CTA of this cluster (addresses from mapa).
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
-}
-
 // 2^x for x <= 8 or so, subnormal results as zero.
 __device__ __forceinline__ float ex2(float x) {
   float y;

@@ -64,7 +64,6 @@ struct dream_ctx {
   void *qbuf;                          // query rows, 4 bytes per element (see q_store4)
   void *q_taps;                        // prompt queries of the candidate tap layers [n_cand][XR][Hhd], for the importance of the chosen one
   void *q_cur;                         // where the call being enqueued keeps its queries
-  float *ssq;                          // [PR][SSQ_LD] sums of squares of the rows in xn (k_resid)
   float *x, *x0, *gout, *lse_taps, *lse_pre, *ent_pre, *ae, *scores, *col_part, *taps_store, *tapbuf;
   void *xn, *raw, *act, *attn_out;
   float *top_val, *lse_rows, *margin_i;
@@ -141,27 +140,40 @@ static dream_status call_done(dream_ctx *c) {
 // A refused launch is remembered with the kernel's name (the first one of a call); the entry point
 // that enqueued it reports it through call_done().
 template <typename... P, typename... A>
-static inline void launch_k(dream_ctx *c, const char *name, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A... args) {
+static inline void launch_cluster(dream_ctx *c, const char *name, void (*kernel)(P...), int cluster, dim3 grid, dim3 block, size_t smem, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = c->stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = c->use_pdl ? 1 : 0;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (cluster > 1) {                         // blocks of a cluster, along x
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster; attr[n].val.clusterDim.y = 1; attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (c->use_pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
   if (e != cudaSuccess && c->launch_err == cudaSuccess) { c->launch_err = e; c->launch_err_name = name; }
   c->launches++;
 }
+template <typename... P, typename... A>
+static inline void launch_k(dream_ctx *c, const char *name, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A... args) {
+  launch_cluster(c, name, kernel, 1, grid, block, smem, args...);
+}
 #define LAUNCH(c, kernel, grid, block, smem, ...) launch_k(c, #kernel, kernel, dim3(grid), dim3(block), (size_t)(smem), __VA_ARGS__)
 // Top-k of `rows` rows of logits: blocks of 1024 columns where they are few enough to be resident at once (a draft
 // pass: latency counts) and their lists few enough to merge, else of 4096.
-#define TOPK_LAUNCH(c, rows, g, norm, ktop, logits)                                                                                     \
+#define TOPK_LAUNCH(c, rows, g, ktop, logits)                                                                                           \
   do {                                                                                                                                  \
     const int V_ = (c)->cfg.vocab, n4_ = (V_ + 1023) / 1024;                                                                            \
     const bool small_ = n4_ * (ktop) <= 1024 && n4_ <= (c)->tk_nsplit && (rows) * n4_ <= 1184;                                          \
     const int n_ = small_ ? n4_ : (V_ + TOPK_COLS - 1) / TOPK_COLS;                                                                     \
-    if (small_) LAUNCH(c, (k_topk_lse<4>), dim3(rows, n_), TOPK_THREADS, 0, g, norm, V_, ktop, n_, (c)->tks, (c)->top_val, (c)->top_id, (c)->lse_rows, logits); \
-    else LAUNCH(c, (k_topk_lse<16>), dim3(rows, n_), TOPK_THREADS, 0, g, norm, V_, ktop, n_, (c)->tks, (c)->top_val, (c)->top_id, (c)->lse_rows, logits);       \
+    if (small_) LAUNCH(c, (k_topk_lse<4>), dim3(rows, n_), TOPK_THREADS, 0, g, V_, ktop, n_, (c)->tks, (c)->top_val, (c)->top_id, (c)->lse_rows, logits); \
+    else LAUNCH(c, (k_topk_lse<16>), dim3(rows, n_), TOPK_THREADS, 0, g, V_, ktop, n_, (c)->tks, (c)->top_val, (c)->top_id, (c)->lse_rows, logits);       \
   } while (0)
 
 // ------------------------------------------------------------------------------------- shapes
@@ -370,7 +382,6 @@ static size_t carve(dream_ctx *c, char *base) {
     c->gout_floats = need;
   }
   c->gout = a.take<float>(c->gout_floats);
-  c->ssq = a.take<float>((size_t)c->PR * SSQ_LD);
   c->rope_pos = a.take<float2>((size_t)c->n_pos * (f.head_dim / 2));
   c->rope_tab = a.take<float2>((size_t)ROW_CHUNK * (f.head_dim / 2));
   c->q_taps = a.take<float>((size_t)c->n_cand * c->XR * c->Hhd);
@@ -870,34 +881,31 @@ template <typename T, int HD> struct AttnLaunch {
     else AttnLaunch<T, 256>::call;                                \
   } while (0)
 
-// x (+= GEMM output) -> x * gain, GEMM input rows in c->xn; see k_resid for the side outputs.  The consumer of the
-// GEMM that reads them scales its rows by what this returns.
+// x (+= GEMM output) -> RMSNorm -> GEMM input rows in c->xn; see k_resid for the side outputs.
 template <typename T>
-static RowScale norm_rows(dream_ctx *c, float *x, const GemmOut &gin, bool has_in, const void *gain, int rows, XMode m,
-                          float *copy = nullptr, const int *row_seq = nullptr, const int *tap = nullptr, int layer = 0,
-                          bool want_raw = false) {
-  const int d = c->cfg.d_model;
-  LAUNCH(c, (k_resid<T>), dim3((d + 1023) / 1024, rows), 256, 0, x, gin, has_in ? 1 : 0, (const T *)gain, d,
-         (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, d), c->ssq);
-  return RowScale{c->ssq, (d + 127) / 128, 1.f / (float)d, c->cfg.rms_eps};
+static void norm_rows(dream_ctx *c, float *x, const GemmOut &gin, bool has_in, const void *gain, int rows, XMode m,
+                      float *copy = nullptr, const int *row_seq = nullptr, const int *tap = nullptr, int layer = 0,
+                      bool want_raw = false) {
+  const int d = c->cfg.d_model, blocks = (d + 1023) / 1024, nv = blocks > RESID_MAX_CLUSTER ? 2 : 1, n = (blocks + nv - 1) / nv;   // d_model <= 16384
+  auto *kernel = nv == 1 ? k_resid<T, 1> : k_resid<T, 2>;
+  launch_cluster(c, "k_resid", kernel, n, dim3(n, rows), dim3(256), 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, d,
+                 (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, d));
 }
-static const RowScale NO_NORM = {nullptr, 0, 0.f, 0.f};
-// norm: of the rows in c->xn.
 template <typename T>
-static GemmOut mlp_rows(dream_ctx *c, const RowScale &norm, const void *wgu, const void *wd, int rows, XMode m) {
+static GemmOut mlp_rows(dream_ctx *c, const void *wgu, const void *wd, int rows, XMode m) {
   const dream_config &f = c->cfg;
   if constexpr (sizeof(T) == 2) {
     if (rows > TC_TOKENS) {                    // a prompt: the GEMM's epilogue gates, the row kernel does the rest
       TcEpi e = {};
-      e.norm = norm; e.dst = (bf16 *)c->act; e.lay = xlay(m, f.d_ff); e.ff = f.d_ff;
+      e.dst = (bf16 *)c->act; e.lay = xlay(m, f.d_ff); e.ff = f.d_ff;
       const GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model, TC_EPI_SILU, &e);
       const int i0 = g.n_full / g.n_tt * 128;
-      if (i0 < f.d_ff) LAUNCH(c, (k_silu_mul<T, true>), dim3((f.d_ff - i0 + 1023) / 1024, rows), 256, 0, g, norm, (T *)c->act, f.d_ff, i0, xlay(m, f.d_ff));
+      if (i0 < f.d_ff) LAUNCH(c, (k_silu_mul<T, true>), dim3((f.d_ff - i0 + 1023) / 1024, rows), 256, 0, g, (T *)c->act, f.d_ff, i0, xlay(m, f.d_ff));
       return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
     }
   }
   GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model);
-  LAUNCH(c, (k_silu_mul<T, false>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, norm, (T *)c->act, f.d_ff, 0, xlay(m, f.d_ff));
+  LAUNCH(c, (k_silu_mul<T, false>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, (T *)c->act, f.d_ff, 0, xlay(m, f.d_ff));
   return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
 }
 
@@ -919,26 +927,27 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
   auto cand_of = [&](int l) { const int k = l + 1 - c->tap_lo_eff; return k >= 0 && k < c->n_cand ? k : -1; };
   auto q_of = [&](int l) { return cand_of(l) < 0 ? c->qbuf : (void *)((float *)c->q_taps + (size_t)cand_of(l) * c->XR * c->Hhd); };
   // projections of layer l for the rows of one pass, whose normalised input sits in c->xn
-  auto qkv = [&](int l, int r0, int rows, const RowScale &norm) {
+  auto qkv = [&](int l, int r0, int rows) {
     if constexpr (sizeof(T) == 2) {
       if (rows > TC_TOKENS) {                  // the GEMM's epilogue rotates and stores, the row kernel does the rest
         TcEpi e = {};
-        e.norm = norm; e.dst = (bf16 *)q_of(l); e.H = f.n_heads; e.row0 = r0; e.seq = seq; e.rope_pos = c->rope_pos; e.kv = paged(c, l);
+        e.dst = (bf16 *)q_of(l); e.H = f.n_heads; e.row0 = r0; e.seq = seq; e.rope_pos = c->rope_pos; e.kv = paged(c, l);
         const GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d, TC_EPI_ROPE, &e);
         const int hh0 = g.n_full / g.n_tt * (TC_BN / f.head_dim), left = c->qkvN - hh0 * f.head_dim;
         if (left > 0)
-          LAUNCH(c, (k_qkv_post_target<T, true>), dim3(rows, (left / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].slot, r0, hh0, q_of(l),
+          LAUNCH(c, (k_qkv_post_target<T, true>), dim3(rows, (left / 8 + 255) / 256), 256, 0, g, c->rm[0].seq, c->rm[0].slot, r0, hh0, q_of(l),
                  paged(c, l), f.n_heads, (const float2 *)c->rope_pos);
         return;
       }
     }
     GemmOut g = gemm<T>(c, c->wqkv[l], c->xn, mp, rows, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T, false>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].slot, r0, 0, q_of(l),
+    LAUNCH(c, (k_qkv_post_target<T, false>), dim3(rows, (c->qkvN / 8 + 255) / 256), 256, 0, g, c->rm[0].seq, c->rm[0].slot, r0, 0, q_of(l),
            paged(c, l), f.n_heads, (const float2 *)c->rope_pos);
   };
   for (int r0 = 0; r0 < n; r0 += CH) {
     const int rows = imin(CH, n - r0);
-    qkv(0, r0, rows, norm_rows<T>(c, c->x + (size_t)r0 * d, NO_GEMM, false, c->ln1[0], rows, mp));
+    norm_rows<T>(c, c->x + (size_t)r0 * d, NO_GEMM, false, c->ln1[0], rows, mp);
+    qkv(0, r0, rows);
   }
   for (int l = 0; l < L; ++l) {
     const int cand = cand_of(l);
@@ -951,19 +960,19 @@ static dream_status prefill_impl(dream_ctx *c, int seq, const void *visual, int 
       int rows = imin(CH, n - r0);
       float *xr = c->x + (size_t)r0 * d;
       GemmOut g = gemm<T>(c, c->wo[l], (const T *)c->attn_out + (long long)(r0 / CH) * att_chunk, mp, rows, d, c->Hhd);
-      RowScale norm = norm_rows<T>(c, xr, g, true, c->ln2[l], rows, mp);
-      g = mlp_rows<T>(c, norm, c->wgu[l], c->wd[l], rows, mp);
+      norm_rows<T>(c, xr, g, true, c->ln2[l], rows, mp);
+      g = mlp_rows<T>(c, c->wgu[l], c->wd[l], rows, mp);
       float *copy = cand >= 0 ? c->taps_store + ((size_t)cand * f.max_prompt + r0) * d : nullptr;
-      norm = norm_rows<T>(c, xr, g, true, l + 1 < L ? c->ln1[l + 1] : c->ln_f, rows, mp, copy);
-      if (l + 1 < L) qkv(l + 1, r0, rows, norm);
+      norm_rows<T>(c, xr, g, true, l + 1 < L ? c->ln1[l + 1] : c->ln_f, rows, mp, copy);
+      if (l + 1 < L) qkv(l + 1, r0, rows);
     }
   }
   LAUNCH(c, k_entropy_mean, L, 1024, 0, (const float *)c->ent_pre, (long long)f.n_heads * f.max_prompt, f.n_heads * n, c->ae,
          c->ent_sum ? c->ent_sum + (size_t)seq * L : (float *)nullptr);
   // first token: LM head on the last prompt row
-  const RowScale last = norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
+  norm_rows<T>(c, c->x + (size_t)(n - 1) * d, NO_GEMM, false, c->ln_f, 1, mp);
   GemmOut g = gemm<T>(c, c->lm_head, c->xn, mp, 1, f.vocab, d);
-  TOPK_LAUNCH(c, 1, g, last, 2, (float *)nullptr);
+  TOPK_LAUNCH(c, 1, g, 2, (float *)nullptr);
   LAUNCH(c, k_first_token, 1, 32, 0, c->top_id, c->top_val, first_token, first_margin);
   LAUNCH(c, k_set_seq, 1, 32, 0, c->sd, seq, n, c->top_id, -1, -1);
   LAUNCH(c, k_select_tap, 1, 32, 0, c->ae, f.tap_mode, f.tap_layer, f.tap_lo, f.tap_hi, c->sd.tap + seq, tap_layer);
@@ -1027,31 +1036,31 @@ static GemmOut draft_rows(dream_ctx *c, const RowMeta &rm, int R, XMode xm, int 
   const dream_draft_weights &w = c->dw;
   const int *vd = vis ? rm.vis_d : nullptr, *vm = vis ? rm.vis_m : nullptr;
   GemmOut g;
-  RowScale norm = norm_rows<T>(c, c->x, NO_GEMM, false, w.ln1, R, xm);
+  norm_rows<T>(c, c->x, NO_GEMM, false, w.ln1, R, xm);
   g = gemm<T>(c, w.wqkv, c->xn, xm, R, c->qkvN, d);
-  LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself), f.n_heads, rope_tab, context ? 1 : 0);
+  LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself), f.n_heads, rope_tab, context ? 1 : 0);
   HD_DISPATCH(c, T, draft(c, rm, c->dself, c->sd.nperm_d, 0, R, xm, B, m, key_ub, vd, tail));
   g = gemm<T>(c, w.wo, c->attn_out, xm, R, d, c->Hhd);
   if (c->three) {
-    norm = norm_rows<T>(c, c->x, g, true, w.i_ln2, R, xm);
-    g = mlp_rows<T>(c, norm, w.i_wgu, w.i_wd, R, xm);
+    norm_rows<T>(c, c->x, g, true, w.i_ln2, R, xm);
+    g = mlp_rows<T>(c, w.i_wgu, w.i_wd, R, xm);
   }
-  norm = norm_rows<T>(c, c->x, g, true, w.lnx, R, xm);
+  norm_rows<T>(c, c->x, g, true, w.lnx, R, xm);
   g = gemm<T>(c, w.xq, c->xn, xm, R, c->Hhd, d);
-  LAUNCH(c, k_gemm_to_q, dim3(R, (c->Hhd + 1023) / 1024), 256, 0, g, norm, c->qbuf, f.n_heads, f.head_dim, sizeof(T) == 2 ? 1 : 0);
+  LAUNCH(c, k_gemm_to_q, dim3(R, (c->Hhd + 1023) / 1024), 256, 0, g, c->qbuf, f.n_heads, f.head_dim, sizeof(T) == 2 ? 1 : 0);
   HD_DISPATCH(c, T, draft(c, rm, c->dmem, c->sd.nperm_m, 1, R, xm, B, m, key_ub, vm, tail));
   g = gemm<T>(c, w.xo, c->attn_out, xm, R, d, c->Hhd);
-  norm = norm_rows<T>(c, c->x, g, true, w.ln2, R, xm);
-  g = mlp_rows<T>(c, norm, w.wgu, w.wd, R, xm);
+  norm_rows<T>(c, c->x, g, true, w.ln2, R, xm);
+  g = mlp_rows<T>(c, w.wgu, w.wd, R, xm);
   if (c->three) {
-    norm = norm_rows<T>(c, c->x, g, true, w.f_ln1, R, xm);
+    norm_rows<T>(c, c->x, g, true, w.f_ln1, R, xm);
     g = gemm<T>(c, w.f_wqkv, c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself2), f.n_heads, rope_tab, context ? 1 : 0);
+    LAUNCH(c, k_qkv_post_draft, dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, rm.seq, rm.pos, rm.dst, 1, c->qbuf, flat(c, c->dself2), f.n_heads, rope_tab, context ? 1 : 0);
     if (context) return g;
     HD_DISPATCH(c, T, draft(c, rm, c->dself2, c->sd.nperm_d, 0, R, xm, B, m, key_ub, vd, tail));
     g = gemm<T>(c, w.f_wo, c->attn_out, xm, R, d, c->Hhd);
-    norm = norm_rows<T>(c, c->x, g, true, w.f_ln2, R, xm);
-    g = mlp_rows<T>(c, norm, w.f_wgu, w.f_wd, R, xm);
+    norm_rows<T>(c, c->x, g, true, w.f_ln2, R, xm);
+    g = mlp_rows<T>(c, w.f_wgu, w.f_wd, R, xm);
   }
   return g;
 }
@@ -1069,9 +1078,9 @@ static dream_status compress_impl(dream_ctx *c, int seq, int k, const int *force
     int rows = imin(CH, nc - r0);
     LAUNCH(c, k_ctx_rows, (rows + 255) / 256, 256, 0, c->ctx_pos + r0, rows, 0, seq, c->rm[0], c->gather_idx, r0, 0);
     LAUNCH(c, (k_gather_rows<float>), rows, 256, 0, c->x0, c->gather_idx, c->x, d, (const int *)nullptr, 0, 0LL, XLayout{d, 0});
-    const RowScale norm = norm_rows<T>(c, c->x, NO_GEMM, false, c->dw.ln1, rows, m1);
+    norm_rows<T>(c, c->x, NO_GEMM, false, c->dw.ln1, rows, m1);
     GemmOut g = gemm<T>(c, wkv, c->xn, m1, rows, c->kvN, d);
-    LAUNCH(c, k_qkv_post_draft, dim3(rows, (c->kvN / 8 + 255) / 256), 256, 0, g, norm, c->rm[0].seq, c->rm[0].pos, c->rm[0].dst, 0, (float *)nullptr,
+    LAUNCH(c, k_qkv_post_draft, dim3(rows, (c->kvN / 8 + 255) / 256), 256, 0, g, c->rm[0].seq, c->rm[0].pos, c->rm[0].dst, 0, (float *)nullptr,
            flat(c, c->dself), f.n_heads, (const float2 *)c->rope_pos, 1);
   }
   // cross-attention memory: tapped features at the context positions, projected (Eq. 1)
@@ -1164,13 +1173,13 @@ static dream_status draft_impl(dream_ctx *c, const TreeBatch &tb, int B) {
     // pass 1 of the three-block draft carries the catch-up rows through every block
     GemmOut g = draft_rows<T>(c, rm, R, xm, B, m, key_ub, c->three && p == 1, true, false, (const float2 *)c->rope_tab);
     // e^M = x: the raw copy feeds the memory projection, the normalised copy the LM head
-    const RowScale norm = norm_rows<T>(c, c->x, g, true, c->ln_f, R, xm, nullptr, nullptr, nullptr, 0, true);
+    norm_rows<T>(c, c->x, g, true, c->ln_f, R, xm, nullptr, nullptr, nullptr, 0, true);
     if (p < ts.D) {     // the last pass's features have no descendants to attend to them
       g = gemm<T>(c, c->dw.xkv, c->raw, xm, R, c->kvN, d);
       LAUNCH(c, k_mem_append, dim3(R, (c->kvN + 1023) / 1024), 256, 0, g, rm.seq, rm.dst, rm.in, c->sd.nperm_m, flat(c, c->dmem));
     }
     g = gemm<T>(c, c->lm_head, c->xn, xm, R, f.vocab, d);
-    TOPK_LAUNCH(c, R, g, norm, ts.K, (float *)nullptr);
+    TOPK_LAUNCH(c, R, g, ts.K, (float *)nullptr);
     int next_m = p < ts.D ? ts.beam[p] : 1;
     LAUNCH(c, k_tree_expand, B, 128, 0, tb, c->sd, c->dt, ts, p, m, c->top_val, c->top_id, c->lse_rows, rn, next_m);
     cur ^= 1;
@@ -1210,17 +1219,17 @@ static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *a
   GemmOut gd = NO_GEMM, g;
   for (int l = 0; l < L; ++l) {
     // the first norm completes S^l (for l >= 1) and captures it where a sequence taps layer l
-    RowScale norm = norm_rows<T>(c, c->x, gd, l > 0, c->ln1[l], R, xm, l > 0 ? c->tapbuf : nullptr, rm.seq, c->sd.tap, l);
+    norm_rows<T>(c, c->x, gd, l > 0, c->ln1[l], R, xm, l > 0 ? c->tapbuf : nullptr, rm.seq, c->sd.tap, l);
     g = gemm<T>(c, c->wqkv[l], c->xn, xm, R, c->qkvN, d);
-    LAUNCH(c, (k_qkv_post_target<T, false>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, norm, rm.seq, rm.slot, 0, 0, c->qbuf, paged(c, l), f.n_heads, (const float2 *)c->rope_tab);
+    LAUNCH(c, (k_qkv_post_target<T, false>), dim3(R, (c->qkvN / 8 + 255) / 256), 256, 0, g, rm.seq, rm.slot, 0, 0, c->qbuf, paged(c, l), f.n_heads, (const float2 *)c->rope_tab);
     HD_DISPATCH(c, T, tree(c, l, R, xm, B, key_ub));
     g = gemm<T>(c, c->wo[l], c->attn_out, xm, R, d, c->Hhd);
-    norm = norm_rows<T>(c, c->x, g, true, c->ln2[l], R, xm);
-    gd = mlp_rows<T>(c, norm, c->wgu[l], c->wd[l], R, xm);
+    norm_rows<T>(c, c->x, g, true, c->ln2[l], R, xm);
+    gd = mlp_rows<T>(c, c->wgu[l], c->wd[l], R, xm);
   }
-  const RowScale norm = norm_rows<T>(c, c->x, gd, true, c->ln_f, R, xm, c->tapbuf, rm.seq, c->sd.tap, L);
+  norm_rows<T>(c, c->x, gd, true, c->ln_f, R, xm, c->tapbuf, rm.seq, c->sd.tap, L);
   g = gemm<T>(c, c->lm_head, c->xn, xm, R, f.vocab, d);
-  TOPK_LAUNCH(c, R, g, norm, 2, logits);
+  TOPK_LAUNCH(c, R, g, 2, logits);
   LAUNCH(c, k_argmax_out, (R + 127) / 128, 128, 0, c->top_id, c->top_val, R, argmax, margin,
          argmax == c->argmax_i ? (int *)nullptr : c->argmax_i);
   return DREAM_OK;
@@ -1510,7 +1519,7 @@ extern "C" dream_status dream_topk_lse_static(const float *logits, int32_t rows,
   GemmOut g;                                   // a plain [rows][vocab] matrix: one slot, one chunk
   g.base = logits; g.slot_stride = 0; g.ld = vocab; g.kb = 0; g.n_full = 0; g.n_tt = 1; g.inv_upc = g.inv_tile = 0.f;
   int nsplit = (vocab + TOPK_COLS - 1) / TOPK_COLS;
-  k_topk_lse<TOPK_COLS / TOPK_THREADS><<<dim3(rows, nsplit), TOPK_THREADS, 0, stream>>>(g, NO_NORM, vocab, ktop, nsplit, ts, top_val, top_id, lse, (float *)nullptr);
+  k_topk_lse<TOPK_COLS / TOPK_THREADS><<<dim3(rows, nsplit), TOPK_THREADS, 0, stream>>>(g, vocab, ktop, nsplit, ts, top_val, top_id, lse, (float *)nullptr);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(nullptr, DREAM_E_CUDA, "k_topk_lse launch: %s", cudaGetErrorString(e));
   return DREAM_OK;

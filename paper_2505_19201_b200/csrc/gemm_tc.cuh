@@ -69,11 +69,9 @@ enum { TC_X_PLAIN = 0, TC_X_PLANAR = 1 };
 enum { TC_X_ONE = 0, TC_X_CONCAT = 1, TC_X_TWO = 2, TC_X_TILES = 3 };
 
 enum { TC_EPI_STORE = 0, TC_EPI_SILU = 1, TC_EPI_ROPE = 2 };
-#define TC_MAX_ROWS 1280        // token rows of a launch with a fused epilogue
 
 // What a fused epilogue needs besides the sums.
 struct TcEpi {
-  RowScale norm;                // of the input rows
   bf16 *dst;                    // SILU: act rows (row_stride, lo_delta apart).  ROPE: query rows [row][head][hi | lo][hd]
   XLayout lay;
   int ff;                       // SILU: real gate columns
@@ -99,7 +97,6 @@ struct TcParams {
 };
 
 // ------------------------------------------------------------------------------------------ PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -195,23 +192,10 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
 }
 
 // ---- pairs of CTAs (cluster of two; the even rank leads)
-__device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r)); return r; }
-// Address of this shared-memory location in the CTA of the given rank.
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-}
 // Releases nothing: what it hands over is TMEM, ordered by the tcgen05 fences.  (An arrive with release at cluster
 // scope waits until the thread's stores to global memory have been performed, 1.5 us behind an epilogue.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed;\n barrier.cluster.wait;" ::: "memory");
 }
 // A load into this CTA's shared memory that completes on the pair leader's barrier.
 __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *map, uint32_t leader_bar, int x, int y, uint64_t policy) {
@@ -299,7 +283,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   uint64_t *acc_full = full_x + TC_MAX_STAGES, *acc_empty = acc_full + 2;
   uint32_t *tmem_base_p = (uint32_t *)(acc_empty + 2);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
-  float *inv_s = (float *)(bars + 64);         // EPI: 1 / rms of every token row, 512 bytes behind the barriers' start
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   const uint32_t rank = cluster_ctarank();
@@ -457,27 +440,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     const uint32_t done_bar = mapa(smem_u32(acc_empty), 0);
     pdl_wait();                               // the output buffer belongs to earlier kernels
-    if (EPI != TC_EPI_STORE) {                // the rows' factors, a thread per row, while the first tile is computed
-      const RowScale n = p.epi.norm;
-#pragma unroll 1
-      for (int t = threadIdx.x - 128; t < p.n_tok; t += 256) {
-        const float *row = n.ssq + (long long)t * SSQ_LD;
-        float sum = 0.f;
-#pragma unroll 1
-        for (int i = 0; i < n.parts; i += 16) {
-          float4 v[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) v[k] = ld_f4(row + i + 4 * k);     // (a row has room for SSQ_LD pieces, what lies behind `parts` is not used)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int left = n.parts - i - 4 * k;
-            sum += (left > 0 ? v[k].x : 0.f) + (left > 1 ? v[k].y : 0.f) + (left > 2 ? v[k].z : 0.f) + (left > 3 ? v[k].w : 0.f);
-          }
-        }
-        inv_s[t] = rsqrtf(sum * n.inv_d + n.eps);
-      }
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-    }
     uint32_t fill = 0;
     bool ok = true;
     auto wait_full = [&](uint32_t buf, uint32_t use) {
@@ -536,16 +498,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
               const float other = __shfl_xor_sync(0xffffffffu, hi16 ? lo8 : hi8, 16);
               va[j] = hi16 ? other : lo8; vb[j] = hi16 ? hi8 : other;
             }
-            const float4 i0 = *reinterpret_cast<const float4 *>(inv_s + tok0 + t0), i1 = *reinterpret_cast<const float4 *>(inv_s + tok0 + t0 + 4);
-            const float inv[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
             const int t = t0 + (lane & 7);                    // the token this lane stores
             const bool st = ok && col_ok && t < nt;
             if (EPI == TC_EPI_SILU) {
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float x = va[j] * inv[j];
-                va[j] = x / (1.f + __expf(-x)) * (vb[j] * inv[j]);
-              }
+              for (int j = 0; j < 8; ++j) va[j] = va[j] / (1.f + __expf(-va[j])) * vb[j];
               tc_store8(va, lane, st, e.dst + (long long)(tok0 + t) * e.lay.row_stride + (ya & ~7), e.lay.lo_delta);
             } else {
               const int r0 = e.row0 + tok0 + t0, r = e.row0 + tok0 + t;
@@ -559,7 +516,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
               for (int j = 0; j < 8; ++j) cs[j] = rot && t0 + j < nt ? e.rope_pos[(long long)(r0 + j) * (e.kv.hd >> 1) + i] : make_float2(1.f, 0.f);
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
-                const float x = va[j] * inv[j], y = vb[j] * inv[j];
+                const float x = va[j], y = vb[j];
                 va[j] = x * cs[j].x - y * cs[j].y;
                 vb[j] = y * cs[j].x + x * cs[j].y;
               }
@@ -681,7 +638,6 @@ static inline bool tc_map(GemmTcPlan *pl, const void *ptr, int rows, int K, int 
   return true;
 }
 
-static inline int imax_tc(int a, int b) { return a > b ? a : b; }
 // How a launch of `rows` token rows is cut (see the head of the file).
 struct TcSplit { int n_tt, tile_t, n_pairs, n_waves, sk_units, upc, slots; };
 static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
@@ -717,7 +673,7 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   const int w_rows = N;
   if (epi == TC_EPI_SILU) N = (e->ff + 127) / 128 * TC_BN;
   if (epi == TC_EPI_ROPE) N = (N + TC_BN - 1) / TC_BN * TC_BN;
-  if (epi != TC_EPI_STORE && (rows > TC_MAX_ROWS || rows <= TC_TOKENS)) return false;
+  if (epi != TC_EPI_STORE && rows <= TC_TOKENS) return false;
   if (rows < 1 || (x_mode == TC_X_PLAIN && rows > 128)) return false;
   const TcSplit t = gemm_tc_split(pl->n_sms, rows, N, K);
   if (t.sk_units + K / TC_BK >= 1 << 21) return false;          // div_small
@@ -748,17 +704,16 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   const int xpanel = x_box * 128 * (form >= TC_X_TWO ? 2 : 1);
   p.wp = xpanel <= TC_WPANEL / 2 ? 2 : 1;
   if (e) p.epi = *e;
-  const int epi_bytes = epi == TC_EPI_STORE ? 0 : TC_MAX_ROWS * 4;
   if (epi != TC_EPI_STORE) p.wp = 1;
   const int xstage = p.wp * xpanel, wstage = p.wp * TC_WPANEL;
   // a few KB stay free for the blocks of the row kernel that waits beside this launch (1 KB each)
-  const int room = pl->max_smem - 2048 - imax_tc(4096, epi_bytes);
+  const int room = pl->max_smem - 2048 - 4096;
   p.x_stages = xpanel < TC_WPANEL ? 6 / p.wp : xpanel == TC_WPANEL ? 4 : room / (xstage + wstage);
   p.w_stages = (room - p.x_stages * xstage) / wstage;
   if (p.w_stages > TC_MAX_STAGES) p.w_stages = TC_MAX_STAGES;
   if (p.w_stages < 2 || p.x_stages < 2) return false;
   p.status = pl->status;
-  size_t smem = (size_t)p.w_stages * wstage + (size_t)p.x_stages * xstage + 2048 + epi_bytes;
+  size_t smem = (size_t)p.w_stages * wstage + (size_t)p.x_stages * xstage + 2048;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * p.n_pairs); cfg.blockDim = dim3(TC_THREADS); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
   cudaLaunchAttribute attr[1];

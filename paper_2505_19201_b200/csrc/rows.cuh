@@ -46,59 +46,68 @@ __global__ void k_build_prompt(const T *__restrict__ embed, const T *__restrict_
 }
 
 // ---------------------------------------------------------------------------------------
-// RMSNorm in two halves.  k_resid writes x * gain as the next GEMM's input and leaves, per row, the sums
-// of squares of its 128-column pieces; the factor 1 / rms is common to a row, so it commutes with the
-// projection and the GEMM's consumer applies it (row_inv_rms).  No kernel has to wait for a whole row.
-#define SSQ_LD 128                       // pieces per row, d_model <= 16384
-struct RowScale {
-  const float *ssq;                      // [rows][SSQ_LD], or null: the rows are not normalised
-  int parts;
-  float inv_d, eps;
-};
-// Every lane of the warp must take part; the pieces are added in a fixed order.
-__device__ __forceinline__ float row_inv_rms(const RowScale &n, int r, bool on) {
-  float s = 0.f;
-  int i = threadIdx.x & 31;
-  do {
-    s += on && n.ssq && i < n.parts ? n.ssq[(long long)r * SSQ_LD + i] : 0.f;
-    i += 32;
-  } while (i < n.parts);
-  s = warp_sum(s);
-  return n.ssq ? rsqrtf(s * n.inv_d + n.eps) : 1.f;
-}
-
-// Per row: x += (GEMM output, if any); xn = x * gain as the next GEMM's input, ssq as above.
+// Per row: x += (GEMM output, if any); xn = RMSNorm(x) * gain as the next GEMM's input.
 // Optional side outputs of the updated residual: `copy` (fp32; when tap_state is given the
 // row is copied only if its sequence's tap layer equals `layer`) and `raw` (element type,
 // unnormalised: the memory side of Eq. 1 takes features without a norm).
-// grid (ceil(d / 1024), rows), a thread per four columns.  Blocks of 256 threads and 56 registers without
-// shared memory, so that they are resident beside a GEMM's CTA before it ends and the next GEMM's CTAs start
-// filling their rings when it does; a block of 1024 threads per row kept those out until the norm was done.
-template <typename T>
-__global__ void __launch_bounds__(256, 5)
-k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, int d, T *xn, float *copy, const int *row_seq,
-        const int *tap_state, int layer, T *raw, XLayout lay, float *ssq) {
+// A row is a cluster of blocks, 1024 NV columns each (NV groups of four per thread), grid (blocks of a row, rows); they
+// exchange their sums of squares through distributed shared memory, before anything is stored (a cluster barrier
+// behind stores to global memory waits for them).  Blocks of 256 threads and 48 registers, so that they are
+// resident beside a GEMM's CTA before it ends and the next GEMM's CTAs start filling their rings when it
+// does; a block of 1024 threads per row kept those out until the norm was done.
+#define RESID_MAX_CLUSTER 8
+template <typename T, int NV>
+__global__ void __launch_bounds__(256, NV == 1 ? 5 : 3)
+k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps, int d, T *xn, float *copy, const int *row_seq,
+        const int *tap_state, int layer, T *raw, XLayout lay) {
+  __shared__ float warp_ss[8], block_ss[2];
   pdl_trigger();
-  const int r = blockIdx.y, i = (blockIdx.x * 256 + threadIdx.x) * 4;
+  const int r = blockIdx.y, i0 = (blockIdx.x * NV * 256 + threadIdx.x) * 4, n = gridDim.x;
   // the gains are weights: they can be fetched before the predecessor has finished
-  const float4 g = xn && i < d ? ld_f4(gain + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-  float4 *xr = reinterpret_cast<float4 *>(x + (long long)r * d + i);
+  float4 g[NV];
+#pragma unroll
+  for (int j = 0; j < NV; ++j) g[j] = xn && i0 + j * 1024 < d ? ld_f4(gain + i0 + j * 1024) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float *xr = x + (long long)r * d;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool on = warm_pass(pass, TR_k_resid) && i < d;
-    float4 v = on ? *xr : make_float4(0.f, 0.f, 0.f, 0.f);
-    bool do_copy = copy != nullptr && on;
-    if (tap_state && do_copy) do_copy = tap_state[row_seq[r]] == layer;
-    if (has_in) {
-      add4(v, gemm_val4<5>(gin, r, i, on));
-      if (on) *xr = v;
+    const bool live = warm_pass(pass, TR_k_resid);
+    float4 v[NV];
+    float ss = 0.f;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int i = i0 + j * 1024;
+      const bool on = live && i < d;
+      v[j] = on ? *reinterpret_cast<const float4 *>(xr + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (has_in) add4(v[j], gemm_val4<5>(gin, r, i, on));
+      ss += v[j].x * v[j].x + v[j].y * v[j].y + v[j].z * v[j].z + v[j].w * v[j].w;
     }
-    const float ss = warp_sum(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
-    if (on && (threadIdx.x & 31) == 0) ssq[(long long)r * SSQ_LD + (i >> 7)] = ss;
-    if (do_copy) *reinterpret_cast<float4 *>(copy + (long long)r * d + i) = v;
-    if (on && raw) store_split4<T>(raw + r * lay.row_stride + i, lay.lo_delta, v);
-    if (on && xn) store_split4<T>(xn + r * lay.row_stride + i, lay.lo_delta, make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
+    bool do_copy = copy != nullptr && live;
+    if (tap_state && do_copy) do_copy = tap_state[row_seq[r]] == layer;
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) warp_ss[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = warp_ss[0];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) tot += warp_ss[k];
+    if (n > 1) {                                             // the row's blocks in ascending order
+      if (threadIdx.x == 0) block_ss[pass] = tot;
+      cluster_sync_all();
+      tot = 0.f;
+      for (int k = 0; k < n; ++k) tot += ld_cluster(mapa(smem_u32(block_ss + pass), k));
+    } else __syncthreads();
+    const float inv = 1.f / sqrtf(tot / (float)d + eps);
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      const int i = i0 + j * 1024;
+      if (!live || i >= d) continue;
+      if (has_in) *reinterpret_cast<float4 *>(xr + i) = v[j];
+      if (do_copy) *reinterpret_cast<float4 *>(copy + (long long)r * d + i) = v[j];
+      if (raw) store_split4<T>(raw + r * lay.row_stride + i, lay.lo_delta, v[j]);
+      if (xn) store_split4<T>(xn + r * lay.row_stride + i, lay.lo_delta,
+                              make_float4(v[j].x * inv * g[j].x, v[j].y * inv * g[j].y, v[j].z * inv * g[j].z, v[j].w * inv * g[j].w));
+    }
   }
+  if (n > 1) cluster_sync_relaxed();                         // no block leaves while another may still read its sum
 }
 
 // ---------------------------------------------------------------------------------------
@@ -155,7 +164,7 @@ __device__ __forceinline__ int gemm_tile(const GemmOut &g, int r, int c) { retur
 // epilogue has left (its stream-K tiles, in paired columns), from head hh0 on.
 template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(256, 5)
-k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_slot,
+k_qkv_post_target(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__ row_slot,
                   int row0, int hh0, void *qbuf, PagedKV kv, int H, const float2 *__restrict__ rope_tab) {
   pdl_trigger();
   const int r = blockIdx.x + row0, lr = blockIdx.x;
@@ -171,9 +180,7 @@ k_qkv_post_target(GemmOut g, RowScale norm, const int *__restrict__ row_seq, con
     if (hh >= H && slot < 0) on = false;               // an idle row (malformed tree node) stores no K/V
     float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
     if (on && hh < H + Hkv) rope_cs4(rope_tab, r, half, i, cs01, cs23);      // fetched along with the slots
-    const float inv = row_inv_rms(norm, lr, live);
     float4 a = gemm_val4<3>(g, lr, ca, on), b = gemm_val4<3>(g, lr, cb, on);
-    scale4(a, inv); scale4(b, inv);
     rotate4(a, b, cs01, cs23);
     if (!on) continue;
     if (hh < H) {
@@ -207,7 +214,7 @@ struct FlatKV {
 // K then V only): rotary, q -> qbuf (when has_q), k/v -> draft self-attention cache row
 // row_dst[r] (skipped when < 0).  The rotary table is by row, or by position.  Work items and grid as in k_qkv_post_target.
 __global__ void __launch_bounds__(256, 5)
-k_qkv_post_draft(GemmOut g, RowScale norm, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_dst,
+k_qkv_post_draft(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_dst,
                  int has_q, void *qbuf, FlatKV kv, int H, const float2 *__restrict__ rope_tab, int by_pos) {
   pdl_trigger();
   const int r = blockIdx.x;
@@ -221,9 +228,7 @@ k_qkv_post_draft(GemmOut g, RowScale norm, const int *__restrict__ row_seq, cons
     if (hh >= Hq && dst < 0) on = false;
     float4 cs01 = make_float4(1.f, 0.f, 1.f, 0.f), cs23 = cs01;
     if (on && hh < Hq + Hkv) rope_cs4(rope_tab, tab_row, half, i, cs01, cs23);
-    const float inv = row_inv_rms(norm, r, live);
     float4 a = gemm_val4<3>(g, r, hh * hd + i, on), b = gemm_val4<3>(g, r, hh * hd + i + half, on);
-    scale4(a, inv); scale4(b, inv);
     rotate4(a, b, cs01, cs23);
     if (!on) continue;
     if (hh < Hq) {
@@ -241,15 +246,13 @@ k_qkv_post_draft(GemmOut g, RowScale norm, const int *__restrict__ row_seq, cons
 // A GEMM output [rows][H * hd] becomes the query rows of the cross-attention (no rotary).
 // grid (rows, ceil(H * hd / 1024)).
 __global__ void __launch_bounds__(256)
-k_gemm_to_q(GemmOut g, RowScale norm, void *qbuf, int H, int hd, int split) {
+k_gemm_to_q(GemmOut g, void *qbuf, int H, int hd, int split) {
   pdl_trigger();
   const int r = blockIdx.x, i = (blockIdx.y * 256 + threadIdx.x) * 4, hd_log2 = 31 - __clz(hd), h = i >> hd_log2;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
     const bool live = warm_pass(pass, TR_k_gemm_to_q), on = live && h < H;
-    const float inv = row_inv_rms(norm, r, live);
     float4 v = gemm_val4<6>(g, r, i, on);
-    scale4(v, inv);
     if (on) q_store4(qbuf, split, (long long)r * H + h, hd, i - (h << hd_log2), v);
   }
 }
@@ -280,16 +283,14 @@ k_mem_append(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__
 // grid (ceil(ff / 1024), rows).  PAIRED: only what the GEMM's own epilogue has left, from gate column i0 on.
 template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(256, 8)
-k_silu_mul(GemmOut g, RowScale norm, T *act, int ff, int i0, XLayout lay) {
+k_silu_mul(GemmOut g, T *act, int ff, int i0, XLayout lay) {
   pdl_trigger();
   const int r = blockIdx.y, i = i0 + (blockIdx.x * 256 + threadIdx.x) * 4;
   const int ca = PAIRED ? paired_col(i >> 7, i & 127) : i, cb = ca + (PAIRED ? 16 : ff);
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
     const bool live = warm_pass(pass, TR_k_silu_mul), on = live && i < ff && (!PAIRED || gemm_tile(g, r, ca) >= g.n_full);
-    const float inv = row_inv_rms(norm, r, live);
     float4 a = gemm_val4<2>(g, r, ca, on), b = gemm_val4<2>(g, r, cb, on);
-    scale4(a, inv); scale4(b, inv);
     const float4 o = make_float4(a.x / (1.f + __expf(-a.x)) * b.x, a.y / (1.f + __expf(-a.y)) * b.y,
                                  a.z / (1.f + __expf(-a.z)) * b.z, a.w / (1.f + __expf(-a.w)) * b.w);
     if (on) store_split4<T>(act + r * lay.row_stride + i, lay.lo_delta, o);
@@ -387,7 +388,7 @@ __device__ __forceinline__ void topk_block(uint32_t (&key)[NV], Id id, int ktop,
 
 template <int NV>
 __global__ void __launch_bounds__(TOPK_THREADS)
-k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts, float *top_val, int *top_id, float *lse,
+k_topk_lse(GemmOut g, int V, int ktop, int nsplit, TopkScratch ts, float *top_val, int *top_id, float *lse,
            float *logits_out) {
   __shared__ float red[33];
   __shared__ uint32_t sh_k[TOPK_THREADS / 32 * TOPK_MAX];
@@ -400,14 +401,12 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
   const bool vec = (V & 3) == 0;
   // column of a thread's candidate j (ascending in j)
   auto id = [&](int j) { return vec ? c0 + ((j >> 2) * TOPK_THREADS + tid) * 4 + (j & 3) : c0 + j * TOPK_THREADS + tid; };
-  const float inv = row_inv_rms(norm, r, true);
   if (vec) {
     float4 q[NV / 4];
 #pragma unroll
     for (int j = 0; j < NV / 4; ++j) {
       int c = c0 + (j * TOPK_THREADS + tid) * 4;
       q[j] = gemm_val4<2>(g, r, c, c < V);
-      scale4(q[j], inv);
       if (c >= V) q[j] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
     }
 #pragma unroll
@@ -420,7 +419,7 @@ k_topk_lse(GemmOut g, RowScale norm, int V, int ktop, int nsplit, TopkScratch ts
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       int c = c0 + j * TOPK_THREADS + tid;
-      v[j] = c < V ? gemm_val(g, r, c) * inv : -INFINITY;
+      v[j] = c < V ? gemm_val(g, r, c) : -INFINITY;
       if (logits_out && c < V) logits_out[(long long)r * V + c] = v[j];
     }
   }
