@@ -369,7 +369,7 @@ static size_t carve(dream_ctx *c, char *base) {
     const int shapes[8][2] = {{(c->qkvN + 255) / 256 * 256, d}, {d, c->Hhd}, {(f.d_ff + 127) / 128 * 256, d}, {d, f.d_ff}, {c->Hhd, d}, {c->kvN, d}, {f.vocab, d}, {0, 0}};
     size_t need = 0;
     for (int i = 0; shapes[i][0]; ++i) {
-      const int N = shapes[i][0], K = shapes[i][1], most = N == f.vocab && K == d ? ROW_CHUNK : c->PR;
+      const int N = shapes[i][0], K = shapes[i][1], most = i == 6 ? ROW_CHUNK : c->PR;   // the LM head never sees a whole prompt pass
       if (f.dtype == DREAM_BF16) {
         // more workers mean more slots, fewer rows fewer tiles and so more slots per tile; never fewer than two, and up to
         // five behind full waves (a quarter of a wave shared by all)
