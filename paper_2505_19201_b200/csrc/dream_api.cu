@@ -886,9 +886,10 @@ template <typename T>
 static void norm_rows(dream_ctx *c, float *x, const GemmOut &gin, bool has_in, const void *gain, int rows, XMode m,
                       float *copy = nullptr, const int *row_seq = nullptr, const int *tap = nullptr, int layer = 0,
                       bool want_raw = false) {
-  const int d = c->cfg.d_model, blocks = (d + 1023) / 1024, nv = blocks > RESID_MAX_CLUSTER ? 2 : 1, n = (blocks + nv - 1) / nv;   // d_model <= 16384
-  auto *kernel = nv == 1 ? k_resid<T, 1> : k_resid<T, 2>;
-  launch_cluster(c, "k_resid", kernel, n, dim3(n, rows), dim3(256), 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, d,
+  const int d = c->cfg.d_model, n = (d + 2047) / 2048;      // both forms take 2048 columns per block; d_model <= 16384: at most 8
+  const bool many = rows > ROW_CHUNK;
+  auto *kernel = many ? k_resid<T, 256, 2> : k_resid<T, 512, 1>;
+  launch_cluster(c, "k_resid", kernel, n, dim3(n, rows), dim3(many ? 256 : 512), 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, d,
                  (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, d));
 }
 template <typename T>

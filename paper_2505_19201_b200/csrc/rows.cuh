@@ -50,23 +50,26 @@ __global__ void k_build_prompt(const T *__restrict__ embed, const T *__restrict_
 // Optional side outputs of the updated residual: `copy` (fp32; when tap_state is given the
 // row is copied only if its sequence's tap layer equals `layer`) and `raw` (element type,
 // unnormalised: the memory side of Eq. 1 takes features without a norm).
-// A row is a cluster of blocks, 1024 NV columns each (NV groups of four per thread), grid (blocks of a row, rows); they
-// exchange their sums of squares through distributed shared memory, before anything is stored (a cluster barrier
-// behind stores to global memory waits for them).  Blocks of 256 threads and 48 registers, so that they are
-// resident beside a GEMM's CTA before it ends and the next GEMM's CTAs start filling their rings when it
-// does; a block of 1024 threads per row kept those out until the norm was done.
-#define RESID_MAX_CLUSTER 8
-template <typename T, int NV>
-__global__ void __launch_bounds__(256, NV == 1 ? 5 : 3)
+// A row is a cluster of blocks, 4 TH NV columns each, grid (blocks of a row, rows); they exchange their sums of
+// squares through distributed shared memory, before anything is stored (a cluster barrier behind stores to
+// global memory waits for them).  Bound by latency in a decode round, by memory in a prompt.
+// Decode rows: 512 threads with one group of four columns each and at most 64 registers, so that a block is
+// resident beside a GEMM's CTA before that ends and the next GEMM's CTAs start filling their rings when it does
+// (a block of 1024 threads per row kept those out until the norm was done).  Round, SmolVLM-shaped / LLaVA-7B-shaped:
+// 2339 / 4878 us; with 256 threads, twice the cluster, 2392 / 4923; with 256 threads of two groups 2371 / 4946.
+// Prompt rows, many waves of blocks: 256 threads with two groups, half the barriers per row: SmolVLM-shaped request
+// 11137 us, against 11205 with the decode form.
+template <typename T, int TH, int NV>
+__global__ void __launch_bounds__(TH, NV == 1 ? 1024 / TH : 768 / TH)
 k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps, int d, T *xn, float *copy, const int *row_seq,
         const int *tap_state, int layer, T *raw, XLayout lay) {
-  __shared__ float warp_ss[8], block_ss[2];
+  __shared__ float warp_ss[TH / 32], block_ss[2];
   pdl_trigger();
-  const int r = blockIdx.y, i0 = (blockIdx.x * NV * 256 + threadIdx.x) * 4, n = gridDim.x;
+  const int r = blockIdx.y, i0 = (blockIdx.x * NV * TH + threadIdx.x) * 4, n = gridDim.x;
   // the gains are weights: they can be fetched before the predecessor has finished
   float4 g[NV];
 #pragma unroll
-  for (int j = 0; j < NV; ++j) g[j] = xn && i0 + j * 1024 < d ? ld_f4(gain + i0 + j * 1024) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int j = 0; j < NV; ++j) g[j] = xn && i0 + j * 4 * TH < d ? ld_f4(gain + i0 + j * 4 * TH) : make_float4(0.f, 0.f, 0.f, 0.f);
   float *xr = x + (long long)r * d;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
@@ -75,7 +78,7 @@ k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps
     float ss = 0.f;
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
-      const int i = i0 + j * 1024;
+      const int i = i0 + j * 4 * TH;
       const bool on = live && i < d;
       v[j] = on ? *reinterpret_cast<const float4 *>(xr + i) : make_float4(0.f, 0.f, 0.f, 0.f);
       if (has_in) add4(v[j], gemm_val4<5>(gin, r, i, on));
@@ -88,7 +91,7 @@ k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps
     __syncthreads();
     float tot = warp_ss[0];
 #pragma unroll
-    for (int k = 1; k < 8; ++k) tot += warp_ss[k];
+    for (int k = 1; k < TH / 32; ++k) tot += warp_ss[k];
     if (n > 1) {                                             // the row's blocks in ascending order
       if (threadIdx.x == 0) block_ss[pass] = tot;
       cluster_sync_all();
@@ -98,7 +101,7 @@ k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps
     const float inv = 1.f / sqrtf(tot / (float)d + eps);
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
-      const int i = i0 + j * 1024;
+      const int i = i0 + j * 4 * TH;
       if (!live || i >= d) continue;
       if (has_in) *reinterpret_cast<float4 *>(xr + i) = v[j];
       if (do_copy) *reinterpret_cast<float4 *>(copy + (long long)r * d + i) = v[j];
