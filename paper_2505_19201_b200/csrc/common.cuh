@@ -145,7 +145,7 @@ template <> __device__ __forceinline__ void store_split<bf16>(bf16 *p, long long
 }
 
 // Output of a GEMM: [rows][ld].  The stream-K part of the tensor-core kernel (tiles n_full and up) leaves
-// up to ceil(kb / units per worker) + 1 partial sums per tile, stacked in slots of slot_stride floats; its full waves and
+// up to ceil(kb / units per worker) + 1 partial sums per tile, slot_stride floats apart; its full waves and
 // the SIMT kernel leave one.
 struct GemmOut {
   const float *base;

@@ -371,12 +371,8 @@ static size_t carve(dream_ctx *c, char *base) {
     for (int i = 0; shapes[i][0]; ++i) {
       const int N = shapes[i][0], K = shapes[i][1], most = i == 6 ? ROW_CHUNK : c->PR;   // the LM head never sees a whole prompt pass
       if (f.dtype == DREAM_BF16) {
-        // more workers mean more slots, fewer rows fewer tiles and so more slots per tile; never fewer than two, and up to
-        // five behind full waves (a quarter of a wave shared by all)
-        for (int rows = 16; rows <= most; rows += 16) {
-          const size_t fl = (size_t)imax(rows > TC_TOKENS ? 5 : 2, gemm_tc_split(192, rows, N, K).slots) * rows * N;
-          if (fl > need) need = fl;
-        }
+        const size_t fl = (size_t)gemm_tc_room(192, most, N, K);
+        if (fl > need) need = fl;
       } else if ((size_t)most * N > need) need = (size_t)most * N;
     }
     c->gout_floats = need;

@@ -83,7 +83,7 @@ struct TcEpi {
 struct TcParams {
   float *out;
   long long slot_stride;        // floats between partial-sum slots
-  int N, KB;                    // output columns, k panels
+  int N, KB, ld;                // output columns, k panels, floats between token rows
   int n_pairs, n_waves, n_full; // pairs, full waves, tiles in them (n_pairs * n_waves)
   int sk_units, upc;            // stream-K part: units = tiles x panels, units per pair
   float inv_kb, inv_upc;        // their reciprocals, for div_small
@@ -453,7 +453,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       const int sk_tile = TILES ? tile - p.n_full : tile, slot = TILES && sk_tile < 0 ? 0 : pair - div_small(sk_tile * p.KB, p.inv_upc);
       const int ct = TILES ? tile / p.n_tt : tile, tok0 = TILES ? (tile - ct * p.n_tt) * p.tile_t : 0, nt = min(p.tile_t, p.n_tok - tok0);
       const int c = ct * TC_BN + (int)rank * 128 + q * 32 + lane;
-      float *dst = p.out + (long long)slot * p.slot_stride + (long long)tok0 * p.N + c;
+      float *dst = p.out + (long long)slot * p.slot_stride + (long long)tok0 * p.ld + c;
       if (FORM >= TC_X_TWO) {
         // token groups of 16: half 0 takes groups 0, 2, .., half 1 groups 1, 3, ..
         float run[128];
@@ -530,7 +530,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int t = (2 * g + half) * 16 + j;
-              if (t < nt) dst[(long long)t * p.N] = run[g * 16 + j];
+              if (t < nt) dst[(long long)t * p.ld] = run[g * 16 + j];
             }
         }
       } else {
@@ -555,11 +555,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
             for (int j = 0; j < 16; ++j) v[j] += __uint_as_float(r[j]);
           }
           if (c < p.N) {
-            float *d = dst + (long long)t0 * p.N;
+            float *d = dst + (long long)t0 * p.ld;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               if (t0 + j < nt) *d = v[j];
-              d += p.N;
+              d += p.ld;
             }
           }
         }
@@ -656,9 +656,30 @@ static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
   t.slots = t.sk_units ? (KB + t.upc - 1) / t.upc + 1 : 1;      // a tile is shared by at most as many pairs
   return t;
 }
-// Floats one launch may write.
-static inline long long gemm_tc_out_floats(int n_sms, int rows, int N, int K) {
-  return gemm_tc_split(n_sms, rows, N, K).slots * (long long)rows * N;
+// Where the partial sums lie.  One token tile or no full wave: slots of rows x N.  Behind full waves only the columns
+// from c0 on have further slots, and a row holds them behind its N columns: five slots of everything were
+// 0.8 GB at 1280 rows of a gate/up projection of 30720 columns, this is 0.2.
+struct TcOut { long long slot_stride, floats; int ld; };
+static inline TcOut gemm_tc_out(const TcSplit &t, int rows, int N) {
+  TcOut o;
+  o.ld = N; o.slot_stride = (long long)rows * N;
+  if (t.n_waves) {
+    const int left = N - t.n_pairs * t.n_waves / t.n_tt * TC_BN;
+    o.ld = N + (t.slots - 1) * left; o.slot_stride = left;
+  }
+  o.floats = t.n_waves ? (long long)rows * o.ld : t.slots * o.slot_stride;
+  return o;
+}
+// Floats a launch of up to `rows` rows may write on a device of up to n_sms SMs (the split follows the SMs, not monotonically).
+static inline long long gemm_tc_room(int n_sms, int rows, int N, int K) {
+  long long most = 0;
+  for (int r = TC_TOKENS; r < rows + TC_TOKENS; r += TC_TOKENS)
+    for (int sms = 2; sms <= n_sms; sms += 2) {
+      const int n = r < rows ? r : rows;
+      const long long f = gemm_tc_out(gemm_tc_split(sms, n, N, K), n, N).floats;
+      if (f > most) most = f;
+    }
+  return most;
 }
 
 // Enqueue one GEMM of `rows` token rows.
@@ -690,13 +711,14 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   else { form = p.n_tt > 1 ? TC_X_TILES : TC_X_TWO; p.mma_n = p.tile_t; }
   p.n_sub = p.mma_n <= 64 ? 4 : p.mma_n <= 128 ? 2 : 1;
   p.out = out;
-  p.slot_stride = (long long)rows * N;
-  if (t.slots * p.slot_stride > out_floats) return false;
+  const TcOut o = gemm_tc_out(t, rows, N);
+  p.slot_stride = o.slot_stride; p.ld = o.ld;
+  if (o.floats > out_floats) return false;
   CUtensorMap mw, mx;
   const int x_rows = x_mode == TC_X_PLANAR ? lo_rows + rows : rows;
   const int x_box = form == TC_X_CONCAT ? p.tile_t : p.mma_n / 2;
   if (!tc_map(pl, W, w_rows, K, epi == TC_EPI_STORE ? 128 : 16, &mw) || !tc_map(pl, X, x_rows, K, x_box, &mx)) return false;
-  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = N; g->kb = p.KB; g->n_full = p.n_full; g->n_tt = p.n_tt;
+  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = o.ld; g->kb = p.KB; g->n_full = p.n_full; g->n_tt = p.n_tt;
   g->inv_upc = p.inv_upc; g->inv_tile = p.n_tt > 1 ? 1.f / (float)p.tile_t : 0.f;
   // Stages of two panels halve the waits and commits per panel (61 rows, 12288 x 4096: 22.2 -> 20.9 us) as
   // long as five fit; where a token panel is larger than a weight panel (244 rows: 38.3 against 39.4 us) the
