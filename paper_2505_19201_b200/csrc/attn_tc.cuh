@@ -101,7 +101,6 @@ struct AttnTcArgs {
   float *lse, *ent;                 // prefill: [H][n] row log-sum-exp and entropy, or null
   float *row_ent;                   // verify: [R][H] entropy of every tree row's attention distribution, or null
   float *part_o, *part_ml, *part_u; // null: the chunks are a cluster; else the partials [slot][chunk][kvh][rt][64][hd], [..][64][2], [..][64] (with row_ent)
-  L2Prefetch next_w;
   // where the K/V blocks live, as rows of the K and V tensor maps
   const int *page_table;            // paged: [max_batch][pages_per_seq]
   int pages_per_seq, page_tokens, page_shift, hkv;
@@ -186,7 +185,6 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_p)), "r"((uint32_t)Sh::TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  l2_prefetch_slice(a.next_w, blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z), gridDim.x * gridDim.y * gridDim.z);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();

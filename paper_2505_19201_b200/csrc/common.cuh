@@ -111,23 +111,6 @@ __device__ __forceinline__ bool warm_pass(int pass, int id) {
   return live != 0;
 }
 
-// Weights never change, so a kernel that leaves HBM idle can pull the next GEMM's weights into the
-// 126 MB L2 ahead of time, before its own grid dependency resolves.  Every CTA requests an equal
-// slice with bulk L2 prefetches issued by one thread.
-struct L2Prefetch {
-  const char *ptr;               // 128-byte aligned; null = nothing to fetch
-  unsigned long long bytes;
-};
-__device__ __forceinline__ void l2_prefetch_slice(const L2Prefetch &pf, unsigned cta, unsigned n_cta) {
-  if (!pf.ptr || threadIdx.x != 0) return;
-  unsigned long long per = ((pf.bytes + n_cta - 1) / n_cta + 127ull) & ~127ull;
-  unsigned long long lo = per * cta, hi = lo + per < pf.bytes ? lo + per : pf.bytes;
-  for (unsigned long long o = lo; o < hi; o += 32768ull) {
-    unsigned sz = (unsigned)((hi - o < 32768ull ? hi - o : 32768ull) & ~15ull);
-    if (sz) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(pf.ptr + o), "r"(sz) : "memory");
-  }
-}
-
 // A bf16 GEMM input row is stored as two bf16 rows, hi = bf16(v) and lo = bf16(v - hi), so the
 // tensor cores see the activation to ~16 mantissa bits while the weights stream once.  fp32
 // inputs have no lo part.  XLayout says where the rows of such a buffer live: token t starts at

@@ -842,8 +842,9 @@ template <typename T, int HD> struct AttnLaunch {
     float *ent = c->row_ent ? c->row_ent + (size_t)layer * ROW_CHUNK * c->cfg.n_heads : nullptr;
     if constexpr (sizeof(T) == 2) {
       AttnTcArgs a = {};
+      // (Fetching wo into L2 meanwhile, 30 to 40 MB, only delayed this kernel's and its predecessor's own loads: the next
+      // GEMM's rings hold as much already.  Without it 4858 instead of 4894 us for a LLaVA-7B-shaped round, 9711 / 9864 of four.)
       a.mode = AT_VERIFY;
-      a.next_w.ptr = (const char *)c->wo[layer]; a.next_w.bytes = (unsigned long long)c->cfg.d_model * c->Hhd * 2;
       a.prefix_len = c->sd.P; a.mask = c->vmask; a.tail_len = c->T; a.lay = xlay(m, c->Hhd);
       a.row_ent = ent;
       tc(c, a, layer, nullptr, B, c->T, key_ub, nullptr);
