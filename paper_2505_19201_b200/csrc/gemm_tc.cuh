@@ -58,6 +58,7 @@
 #define TC_SPIN_LIMIT (1u << 24)
 #define TC_WPANEL (128 * TC_BK * 2)          // one CTA's half of a weight panel
 #define TC_MAX_STAGES 12
+#define TC_EVEN 4               // units a pair may walk further for a share that lies in one tile
 #define TC_CHAIN 8              // panels per accumulator in the two-MMA form (64 MMAs)
 
 // How the token rows lie in the X buffer.  PLAIN: one bf16 row per token.  PLANAR: high parts, then
@@ -84,9 +85,10 @@ struct TcParams {
   float *out;
   long long slot_stride;        // floats between partial-sum slots
   int N, KB, ld;                // output columns, k panels, floats between token rows
+  int kbu;                      // work units per tile: KB, or more so that every pair's share lies in one tile
   int n_pairs, n_waves, n_full; // pairs, full waves, tiles in them (n_pairs * n_waves)
   int sk_units, upc;            // stream-K part: units = tiles x panels, units per pair
-  float inv_kb, inv_upc;        // their reciprocals, for div_small
+  float inv_kbu, inv_upc;       // reciprocals, for div_small
   int n_tt, tile_t, mma_n;      // token tiles, tokens per tile, N of an MMA
   int n_sub;                    // CONCAT / ONE: accumulators the k-steps of a segment are dealt out to (1, 2 or 4)
   int n_tok;                    // real token rows
@@ -221,8 +223,9 @@ template <bool TILES> struct TcWalk {
   __device__ __forceinline__ bool next(const TcParams &p, int &tile, int &k0, int &k1) {
     if (TILES && w < p.n_waves) { tile = w * p.n_pairs + pair; k0 = 0; k1 = p.KB; ++w; return true; }
     if (u >= u_end) return false;
-    tile = div_small(u, p.inv_kb); k0 = u - tile * p.KB; k1 = min(p.KB, k0 + u_end - u);
+    tile = div_small(u, p.inv_kbu); k0 = u - tile * p.kbu; k1 = min(p.kbu, k0 + u_end - u);
     u += k1 - k0;
+    k1 = min(k1, p.KB);
     if (TILES) tile += p.n_full;
     return true;
   }
@@ -450,7 +453,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       tc_fence_after();
     };
     while (ok && walk.next(p, tile, k0, k1)) {
-      const int sk_tile = TILES ? tile - p.n_full : tile, slot = TILES && sk_tile < 0 ? 0 : pair - div_small(sk_tile * p.KB, p.inv_upc);
+      const int sk_tile = TILES ? tile - p.n_full : tile, slot = TILES && sk_tile < 0 ? 0 : pair - div_small(sk_tile * p.kbu, p.inv_upc);
       const int ct = TILES ? tile / p.n_tt : tile, tok0 = TILES ? (tile - ct * p.n_tt) * p.tile_t : 0, nt = min(p.tile_t, p.n_tok - tok0);
       const int c = ct * TC_BN + (int)rank * 128 + q * 32 + lane;
       float *dst = p.out + (long long)slot * p.slot_stride + (long long)tok0 * p.ld + c;
@@ -639,7 +642,7 @@ static inline bool tc_map(GemmTcPlan *pl, const void *ptr, int rows, int K, int 
 }
 
 // How a launch of `rows` token rows is cut (see the head of the file).
-struct TcSplit { int n_tt, tile_t, n_pairs, n_waves, sk_units, upc, slots; };
+struct TcSplit { int n_tt, tile_t, n_pairs, n_waves, kbu, sk_units, upc, slots; };
 static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
   TcSplit t;
   const int KB = K / TC_BK;
@@ -650,10 +653,18 @@ static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
   // full waves, less one when the rest alone is so small that a tile would be shared by many pairs
   t.n_waves = t.n_tt > 1 ? tiles / pairs : 0;
   if (t.n_waves && tiles % pairs && 4 * (tiles % pairs) < pairs) --t.n_waves;
-  t.sk_units = (tiles - t.n_waves * pairs) * KB;
-  t.upc = t.sk_units ? (t.sk_units + pairs - 1) / pairs : 1;
+  // Few tiles: every pair a share of one tile, where that is at most TC_EVEN units longer than dealing all units out evenly.
+  // A share that crosses a tile's end empties two accumulators, and its tiles have one or two more slots for
+  // the next kernel to read.  Rounds, spread -> whole: SmolVLM-shaped 2321 -> 2222 us, LLaVA-7B-shaped 4719 -> 4701, four of it
+  // 9458 -> 9370, Pixtral- 7992 -> 7924, Gemma-shaped 10984 -> 10860; five units (172 panels: 43 instead of 38) lose 7 us.
+  const int left = tiles - t.n_waves * pairs, share = left > 0 ? pairs / left : 0;      // whole pairs per tile
+  const int spread = (left * KB + pairs - 1) / pairs, even = share > 1 ? (KB + share - 1) / share : 0;
+  const bool whole = even && even <= spread + TC_EVEN;
+  t.upc = whole ? even : left ? spread : 1;
+  t.kbu = whole ? (KB + even - 1) / even * even : KB;
+  t.sk_units = left * t.kbu;
   t.n_pairs = t.n_waves ? pairs : (t.sk_units + t.upc - 1) / t.upc;
-  t.slots = t.sk_units ? (KB + t.upc - 1) / t.upc + 1 : 1;      // a tile is shared by at most as many pairs
+  t.slots = whole ? t.kbu / t.upc : left ? (KB + t.upc - 1) / t.upc + 1 : 1;      // a tile is shared by at most as many pairs
   return t;
 }
 // Where the partial sums lie.  One token tile or no full wave: slots of rows x N.  Behind full waves only the columns
@@ -697,13 +708,13 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   if (epi != TC_EPI_STORE && rows <= TC_TOKENS) return false;
   if (rows < 1 || (x_mode == TC_X_PLAIN && rows > 128)) return false;
   const TcSplit t = gemm_tc_split(pl->n_sms, rows, N, K);
-  if (t.sk_units + K / TC_BK >= 1 << 21) return false;          // div_small
+  if (t.sk_units + t.kbu >= 1 << 21) return false;          // div_small
   TcParams p;
   p.n_tok = rows; p.lo_rows = lo_rows;
   p.N = N; p.KB = K / TC_BK;
   p.n_pairs = t.n_pairs; p.n_waves = t.n_waves; p.n_full = t.n_pairs * t.n_waves; p.sk_units = t.sk_units; p.upc = t.upc;
   p.n_tt = t.n_tt; p.tile_t = t.tile_t;
-  p.inv_kb = 1.f / (float)p.KB; p.inv_upc = 1.f / (float)p.upc;
+  p.kbu = t.kbu; p.inv_kbu = 1.f / (float)t.kbu; p.inv_upc = 1.f / (float)p.upc;
   // N of an MMA is a multiple of 16 and each CTA stages half of it (8-row groups)
   int form;
   if (x_mode == TC_X_PLAIN) { form = TC_X_ONE; p.tile_t = p.mma_n = (rows + 15) & ~15; }
@@ -718,7 +729,7 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   const int x_rows = x_mode == TC_X_PLANAR ? lo_rows + rows : rows;
   const int x_box = form == TC_X_CONCAT ? p.tile_t : p.mma_n / 2;
   if (!tc_map(pl, W, w_rows, K, epi == TC_EPI_STORE ? 128 : 16, &mw) || !tc_map(pl, X, x_rows, K, x_box, &mx)) return false;
-  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = o.ld; g->kb = p.KB; g->n_full = p.n_full; g->n_tt = p.n_tt;
+  g->base = p.out; g->slot_stride = p.slot_stride; g->ld = o.ld; g->kb = t.kbu; g->n_full = p.n_full; g->n_tt = p.n_tt;
   g->inv_upc = p.inv_upc; g->inv_tile = p.n_tt > 1 ? 1.f / (float)p.tile_t : 0.f;
   // Stages of two panels halve the waits and commits per panel (61 rows, 12288 x 4096: 22.2 -> 20.9 us) as
   // long as five fit; where a token panel is larger than a weight panel (244 rows: 38.3 against 39.4 us) the

@@ -49,3 +49,11 @@ def test_panels(ctx, rows, K):
 @pytest.mark.parametrize("rows", [61, 244])
 def test_columns(ctx, rows, N):
     check(ctx, rows, N, 320, N + rows)
+
+
+# shares of whole pairs per tile: two per tile exactly and not quite, as long as allowed and one unit longer, a last
+# share shorter than the others, more pairs per tile than panels
+@pytest.mark.parametrize("N,K", [(9472, 576), (9728, 576), (8192, 3840), (4096, 11008), (6144, 5120), (2048, 2048), (256, 128)])
+@pytest.mark.parametrize("rows", [9, 61, 244])
+def test_shares(ctx, rows, N, K):
+    check(ctx, rows, N, K, N + K)
