@@ -24,7 +24,7 @@
 //     With several token tiles, full waves of tiles come first, one tile per pair, so that neighbouring pairs read the same weight
 //     panels at the same time (one HBM read serves them all).  The rest, between one and two waves of tiles
 //     (or all of them when there are fewer than two), is stream-K: its (tile, panel) units are dealt
-//     out in equal contiguous ranges; a pair that covers part of a tile writes a partial sum to its own
+//     out in equal contiguous ranges, each inside one tile where tiles are few; a pair that covers part of a tile writes a partial sum to its own
 //     slot and the consumer adds the slots in a fixed order;
 //   * a prompt's gate/up and QKV projections finish in the epilogue (TC_EPI_SILU, TC_EPI_ROPE): their weight rows
 //     are loaded in pairs (gate and up of a column; the two halves of a rotary pair), 16 rows of one kind and
@@ -348,6 +348,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         if (++s == p.w_stages) { s = 0; ph ^= 1; }
       }
     }
+    // Until the last releases have arrived, which the pair's first CTA signals across: an arrival that comes in after this
+    // CTA has left would land in the shared memory of the CTA that follows it on the SM.
+    for (int i = 0; ok && i < p.w_stages; ++i) {
+      if (!mbar_wait_warp(empty_w + s, ph)) { give_up(); ok = false; }
+      if (++s == p.w_stages) { s = 0; ph ^= 1; }
+    }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ X producer: waits until the
     // input exists (previous kernel), then feeds one X stage per W stage
@@ -434,6 +440,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         if (ok && elect_one()) mma_commit_pair(acc_full + buf);       // accumulator complete
         __syncwarp();
       }
+      // as above for the second CTA's arrivals: both accumulators emptied (they are relaxed, and the barrier at the end
+      // does not wait for them; one that came late left a later launch waiting for good, once in some million)
+      for (uint32_t buf = 0; ok && buf < 2u; ++buf)
+        if (!mbar_wait_warp(acc_empty + buf, (((fill + 1u - buf) >> 1) & 1u) ^ 1u)) ok = false;
       if (!ok) give_up();
     }
   } else if (warp >= 4) {
