@@ -667,14 +667,17 @@ static inline TcSplit gemm_tc_split(int n_sms, int rows, int N, int K) {
   // A share that crosses a tile's end empties two accumulators, and its tiles have one or two more slots for
   // the next kernel to read.  Rounds, spread -> whole: SmolVLM-shaped 2321 -> 2222 us, LLaVA-7B-shaped 4719 -> 4701, four of it
   // 9458 -> 9370, Pixtral- 7992 -> 7924, Gemma-shaped 10984 -> 10860; five units (172 panels: 43 instead of 38) lose 7 us.
+  // Between a half and two thirds as many tiles as pairs, three pairs per two tiles in the same way (LLaVA-7B-shaped QKV, 48 tiles: the
+  // rotary kernel adds two slots instead of three): round 4711 -> 4669 us, chain 4318 -> 4279, four sequences 9435 -> 9324.
   const int left = tiles - t.n_waves * pairs, share = left > 0 ? pairs / left : 0;      // whole pairs per tile
-  const int spread = (left * KB + pairs - 1) / pairs, even = share > 1 ? (KB + share - 1) / share : 0;
+  const bool three = share == 1 && 3 * left <= 2 * pairs && KB > (KB + 2) / 3 * 2;        // three pairs per two tiles, no share empty
+  const int spread = (left * KB + pairs - 1) / pairs, even = share > 1 ? (KB + share - 1) / share : three ? (KB + 2) / 3 * 2 : 0;
   const bool whole = even && even <= spread + TC_EVEN;
   t.upc = whole ? even : left ? spread : 1;
-  t.kbu = whole ? (KB + even - 1) / even * even : KB;
+  t.kbu = !whole ? KB : three ? even / 2 * 3 : (KB + even - 1) / even * even;
   t.sk_units = left * t.kbu;
   t.n_pairs = t.n_waves ? pairs : (t.sk_units + t.upc - 1) / t.upc;
-  t.slots = whole ? t.kbu / t.upc : left ? (KB + t.upc - 1) / t.upc + 1 : 1;      // a tile is shared by at most as many pairs
+  t.slots = whole ? (t.kbu + t.upc - 1) / t.upc : left ? (KB + t.upc - 1) / t.upc + 1 : 1;      // a tile is shared by at most as many pairs
   return t;
 }
 // Where the partial sums lie.  One token tile or no full wave: slots of rows x N.  Behind full waves only the columns

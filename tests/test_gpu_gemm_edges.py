@@ -57,3 +57,10 @@ def test_columns(ctx, rows, N):
 @pytest.mark.parametrize("rows", [9, 61, 244])
 def test_shares(ctx, rows, N, K):
     check(ctx, rows, N, K, N + K)
+
+
+# three pairs per two tiles: an even and an odd number of tiles, the most and the fewest, too few panels for it
+@pytest.mark.parametrize("N,K", [(12288, 4096), (12032, 4096), (12544, 576), (9728, 320), (12800, 576), (12288, 256), (12288, 128)])
+@pytest.mark.parametrize("rows", [9, 61, 244])
+def test_three_pairs(ctx, rows, N, K):
+    check(ctx, rows, N, K, N + K)
