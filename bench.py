@@ -27,13 +27,11 @@ sys.path.insert(0, ROOT)
 
 from paper_2505_19201_b200 import configs, synth  # noqa: E402
 
-# DRAM traffic of the dominant kernel from an ncu capture of the current k_gemm_tc
-# (profiles/k_gemm_tc_llava7b_4layers_ncu_full.md): dram__bytes_read.sum + dram__bytes_write.sum
-# over the four projections of one verify layer (wqkv, wo, wgu, wd), and their weight bytes.  The
-# capture ran on the 4-layer cut of the workload (same layer shapes); traffic grows in proportion
-# to the weight bytes, so a step's mean launch is scaled by this ratio.  None for workloads without
-# a capture, and to be reset to None whenever the kernel changes.
-TRAFFIC_RATIO = {"llava7b": (105.94 + 34.63 + 187.11 + 96.19) / (100.66 + 33.55 + 180.36 + 90.18)}
+# DRAM traffic of the dominant kernel over its weight bytes, from an ncu capture of the current k_gemm_tc
+# (dram__bytes_read.sum + dram__bytes_write.sum over the four projections of one verify layer; traffic grows in
+# proportion to the weight bytes, so a step's mean launch is scaled by this ratio).  Empty for workloads without a
+# capture, and to be emptied whenever the kernel changes.
+TRAFFIC_RATIO = {}
 
 METRIC = "verified_tree_tokens_per_s"
 UNIT = "tokens/s"
