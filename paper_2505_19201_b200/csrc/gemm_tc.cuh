@@ -441,8 +441,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         __syncwarp();
       }
       // as above for the second CTA's arrivals: both accumulators emptied (they are relaxed, and the barrier at the end
-      // does not wait for them; one that came late left a later launch waiting for good, once in some million)
-      for (uint32_t buf = 0; ok && buf < 2u; ++buf)
+      // does not wait for them; one that came late left a later launch waiting for good, once in some million).  The
+      // decode forms send only the arrivals that the loop above has waited for.
+      for (uint32_t buf = 0; FORM >= TC_X_TWO && ok && buf < 2u; ++buf)
         if (!mbar_wait_warp(acc_empty + buf, (((fill + 1u - buf) >> 1) & 1u) ^ 1u)) ok = false;
       if (!ok) give_up();
     }
@@ -454,6 +455,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const uint32_t done_bar = mapa(smem_u32(acc_empty), 0);
     pdl_wait();                               // the output buffer belongs to earlier kernels
     uint32_t fill = 0;
+    const uint32_t n_seg = FORM >= TC_X_TWO || walk.u >= walk.u_end ? 0u : (uint32_t)(div_small(walk.u_end - 1, p.inv_kbu) - div_small(walk.u, p.inv_kbu) + 1);
     bool ok = true;
     auto wait_full = [&](uint32_t buf, uint32_t use) {
       int w = 1;
@@ -578,7 +580,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(done_bar + 8u * buf);
+        if (lane == 0 && fill + 1u < n_seg) mbar_arrive_cluster(done_bar + 8u * buf);      // the accumulator is filled again
       }
     }
   }
