@@ -407,10 +407,10 @@ def main():
     # distance to the next stamp, overlap with its neighbours included
     if gemm:
         n_tr = 4
-        ctx.dream_trace(n_tr * (int(launches) // args.steps + 64))
+        ctx.dream_trace(2 * n_tr * (int(launches) // args.steps + 64))
         for _ in range(n_tr):
             one_step()
-        tl = ctx.dream_trace(0)
+        tl = sorted((x for x in ctx.dream_trace(0) if x[0] != "none"), key=lambda x: x[1])   # "none": a CTA's start, before its dependency
         first = [i for i, (k, _) in enumerate(tl) if k == "k_draft_begin"]
         if len(first) >= 2:
             tl = tl[first[0]:first[-1] + 1]                      # whole steps only
