@@ -96,7 +96,7 @@ struct dream_ctx {
   int pf_v, pf_vis_start, pf_q;
   std::vector<int> free_pages;
   std::vector<int> seq_pages[DREAM_MAX_BATCH];
-  int *h_stage;                        // pinned: page-table staging + step_host results
+  int *h_stage;                        // pinned: step_host results
   long long launches, tc_launches, simt_launches;
   GemmTcPlan tc;
   AtMapCache at_maps;
@@ -575,7 +575,7 @@ extern "C" dream_status dream_init(const dream_config *cfg, const dream_target_w
   }
   cudaError_t e = cudaMemsetAsync(c->arena, 0, need, c->stream);
   if (e != cudaSuccess) { delete c; return fail(nullptr, DREAM_E_CUDA, "memset arena: %s", cudaGetErrorString(e)); }
-  e = cudaHostAlloc((void **)&c->h_stage, sizeof(int) * ((size_t)cfg->max_batch * c->pps + 64 + cfg->max_batch * (DREAM_MAX_DEPTH + 2)), cudaHostAllocDefault);
+  e = cudaHostAlloc((void **)&c->h_stage, sizeof(int) * (DREAM_MAX_BATCH + cfg->max_batch * (DREAM_MAX_DEPTH + 1)), cudaHostAllocDefault);
   if (e != cudaSuccess) { delete c; return fail(nullptr, DREAM_E_CUDA, "pinned staging: %s", cudaGetErrorString(e)); }
   e = cudaHostAlloc((void **)&c->h_snap, sizeof(int) * SNAP_SLOTS * DREAM_MAX_BATCH, cudaHostAllocDefault);
   if (e != cudaSuccess) { cudaFreeHost(c->h_stage); delete c; return fail(nullptr, DREAM_E_CUDA, "pinned snapshots: %s", cudaGetErrorString(e)); }
@@ -668,6 +668,15 @@ __global__ void k_set_seq(SeqDev s, int seq, int P, const int *pending_src, int 
 __global__ void k_set_int(int *p, int v) {
   kernel_entry(TR_k_set_int);
   if (!threadIdx.x) *p = v;
+}
+// A sequence's pages travel as a kernel argument.  (Copied from a staging buffer they were read when the stream got
+// there, and a host that ran ahead had by then filled the buffer for the sequence's next request: two sequences wrote one page.)
+#define PAGE_LIST 896
+struct PageList { int page[PAGE_LIST]; };
+__global__ void k_set_pages(const __grid_constant__ PageList l, int n, int *page_table) {
+  kernel_entry(TR_k_set_pages);
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) page_table[i] = l.page[i];
 }
 __global__ void k_first_token(const int *top_id, const float *top_val, int *tok, float *margin) {
   kernel_entry(TR_k_first_token);
@@ -990,14 +999,17 @@ extern "C" dream_status dream_prefill(dream_ctx *c, int32_t seq, const void *vis
   if (v > f.max_visual || v + q > f.max_prompt) return fail(c, DREAM_E_CAPACITY, "prompt of %d (+%d visual) exceeds max_prompt/max_visual", v + q, v);
   if (c->phase[seq] != PH_EMPTY) return fail(c, DREAM_E_STATE, "sequence %d is live; dream_seq_reset it first", seq);
   if ((int)c->free_pages.size() < c->pps) return fail(c, DREAM_E_CAPACITY, "page pool exhausted");
-  int *stage = c->h_stage + (size_t)seq * c->pps;
   for (int i = 0; i < c->pps; ++i) {
     int p = c->free_pages.back();
     c->free_pages.pop_back();
     c->seq_pages[seq].push_back(p);
-    stage[i] = p;
   }
-  CUDA_OK(c, cudaMemcpyAsync(c->page_table + (size_t)seq * c->pps, stage, sizeof(int) * c->pps, cudaMemcpyHostToDevice, c->stream));
+  for (int i0 = 0; i0 < c->pps; i0 += PAGE_LIST) {
+    PageList l;
+    const int m = imin(PAGE_LIST, c->pps - i0);
+    memcpy(l.page, c->seq_pages[seq].data() + i0, sizeof(int) * m);
+    LAUNCH(c, k_set_pages, (m + 255) / 256, 256, 0, l, m, c->page_table + (size_t)seq * c->pps + i0);
+  }
   if (f.dtype == DREAM_BF16) s = prefill_impl<bf16>(c, seq, visual, v, vis_start, ids, q, first_token, first_margin, layer_entropy, tap_layer);
   else s = prefill_impl<float>(c, seq, visual, v, vis_start, ids, q, first_token, first_margin, layer_entropy, tap_layer);
   if (s) return s;
@@ -1339,7 +1351,7 @@ extern "C" dream_status dream_step_host(dream_ctx *c, const int32_t *seqs, int32
   s = dream_accept(c, seqs, n_seqs, nullptr, c->argmax_i, c->accept_len_i, c->out_tokens_i, c->comp_src_i);
   if (s) return s;
   int D1 = c->ts.D + 1;
-  int *stage = c->h_stage + (size_t)c->cfg.max_batch * c->pps;
+  int *stage = c->h_stage;
   CUDA_OK(c, cudaMemcpyAsync(stage, c->accept_len_i, sizeof(int) * n_seqs, cudaMemcpyDeviceToHost, c->stream));
   CUDA_OK(c, cudaMemcpyAsync(stage + DREAM_MAX_BATCH, c->out_tokens_i, sizeof(int) * n_seqs * D1, cudaMemcpyDeviceToHost, c->stream));
   CUDA_OK(c, cudaStreamSynchronize(c->stream));
