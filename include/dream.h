@@ -255,6 +255,11 @@ dream_status dream_debug_read(dream_ctx *ctx, int32_t seq, int32_t what, int32_t
 dream_status dream_debug_gemm(dream_ctx *ctx, const void *W, const float *X, int32_t rows,
                               int32_t N, int32_t K, int32_t split, float *out);
 
+/* Test hook: a device-side wait that nothing ends, in a pair of CTAs.  The first gives up after limit_ms (1..1000)
+ * and raises the status word, the second because the first did.  seconds: device buffer of two floats, how long
+ * each waited.  dream_poll then reports DREAM_E_DEVICE_TIMEOUT on this context. */
+dream_status dream_debug_wait(dream_ctx *ctx, int32_t limit_ms, float *seconds);
+
 /* How many GEMM launches so far went to the tensor-core kernel and to the CUDA-core kernel. */
 dream_status dream_gemm_counts(const dream_ctx *ctx, int64_t *tensor_core, int64_t *cuda_core);
 
@@ -305,7 +310,7 @@ const char *dream_trace_name(int32_t id);
 dream_status dream_seq_reset(dream_ctx *ctx, int32_t seq);
 
 /* Wait for the stream and report the device status word: DREAM_OK, DREAM_E_DEVICE_TIMEOUT (a
- * bounded wait inside a kernel ran out) or DREAM_E_STATE (a kernel met a malformed tree, an index
+ * bounded wait inside a kernel ran out, after a second; the message names the kernel and the wait) or DREAM_E_STATE (a kernel met a malformed tree, an index
  * or a capacity out of range, or a logits row without mass; the offending rows were skipped).
  * The word is sticky: it is not cleared by reading it. */
 dream_status dream_poll(dream_ctx *ctx);

@@ -83,6 +83,7 @@ def lib():
             "dream_debug_read": [vp, i32, i32, i32, i32, vp],
             "dream_seq_reset": [vp, i32],
             "dream_debug_gemm": [vp, vp, vp, i32, i32, i32, i32, vp],
+            "dream_debug_wait": [vp, i32, vp],
             "dream_gemm_counts": [vp, C.POINTER(C.c_int64), C.POINTER(C.c_int64)],
             "dream_gemm_timing": [vp, i32, C.POINTER(C.c_int64), C.POINTER(C.c_double), C.POINTER(C.c_double)],
             "dream_poll": [vp],
@@ -305,6 +306,9 @@ class Context:
         out = torch.empty(rows, N, dtype=torch.float32, device=self.device)
         _check(self.h, lib().dream_debug_gemm(self.h, _ptr(W), _ptr(X), rows, N, K, split, _ptr(out)))
         return out
+
+    def dream_debug_wait(self, limit_ms, seconds):
+        _check(self.h, lib().dream_debug_wait(self.h, limit_ms, _ptr(seconds)))
 
     def dream_gemm_counts(self):
         a, b = C.c_int64(), C.c_int64()

@@ -30,8 +30,8 @@
 // The loops are kept compact on purpose: this kernel's code is
 // fetched anew at almost every launch (the weight stream between two launches pushes it out of the
 // caches), and straight-line code then costs its own fetch (a fully unrolled version of the same
-// loops ran four times slower).  Every mbarrier wait is bounded; on expiry the kernel raises the
-// status word and leaves.
+// loops ran four times slower).  Every mbarrier wait is bounded (mbar_wait, gemm_tc.cuh); a CTA of a cluster that gives
+// up still meets the others at the merge, and they finish with what it left.
 #pragma once
 #include <map>
 #include <vector>
@@ -189,7 +189,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_p;
-  auto give_up = [&]() { if (lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } };
+  int gave_up = WAIT_none;                                  // the wait of this warp that ran out
   // Verification reads the verified prefix and its length, which were written rounds ago (hundreds
   // of kernels back in the stream): its K/V blocks below the prefix length are fetched before the
   // grid dependency resolves.  Everything else is an output of the immediate predecessors.
@@ -269,14 +269,12 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       uint32_t kph = n_pre >= STAGES ? 0u : 1u, vph = kph;    // parity of the stage's last release (1: none needed yet)
       for (int it = n_pre; it <= n_blk; ++it) {
         if (it < n_blk) {
-          if (!mbar_wait_warp(k_empty + ks, kph)) { give_up(); break; }
-          if (__any_sync(0xffffffffu, *abort_flag)) break;
+          if (!mbar_wait_warp(k_empty + ks, kph, abort_flag)) { gave_up = WAIT_attn_k_ring; break; }
           issue(0, it, ks);
           if (++ks == STAGES) { ks = 0; kph ^= 1u; }
         }
         if (it > n_pre) {
-          if (!mbar_wait_warp(v_empty + vs, vph)) { give_up(); break; }
-          if (__any_sync(0xffffffffu, *abort_flag)) break;
+          if (!mbar_wait_warp(v_empty + vs, vph, abort_flag)) { gave_up = WAIT_attn_v_ring; break; }
           issue(1, it - 1, vs);
           if (++vs == STAGES) { vs = 0; vph ^= 1u; }
         }
@@ -291,16 +289,16 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t o_addr = tmem_base, s_addr0 = tmem_base + HD;
       const uint64_t qd = smem_desc(smem_u32(q_s)), kd = smem_desc(smem_u32(k_s)), pd = smem_desc(smem_u32(p_s)), vd = smem_desc_mn(smem_u32(v_s), AT_KVTILE);
-      bool ok = mbar_wait_warp(q_full, 0);
+      if (!mbar_wait_warp(q_full, 0, abort_flag)) gave_up = WAIT_attn_q;
       int ks = 0, sb = 0, vs = 0;                            // ring positions of K, S and V
       uint32_t kph = 0, sph = 1, vph = 0;
       // step i issues S of block i and O of block i - AHEAD
 #pragma unroll 1
-      for (int i = 0; i < n_blk + AHEAD && ok; ++i) {
+      for (int i = 0; i < n_blk + AHEAD && !gave_up; ++i) {
         const int it = i - AHEAD;
         if (it >= 0) {
           const int pb = it & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u) && mbar_wait(v_full + vs, vph))) { ok = false; break; }
+          if (!__all_sync(0xffffffffu, mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u, abort_flag) && mbar_wait(v_full + vs, vph, abort_flag))) { gave_up = WAIT_attn_p_v; break; }
           tc_fence_after();
           const uint64_t ad = pd + (uint64_t)(pb * (AT_PTILE >> 4));
           if (elect_one()) {
@@ -318,7 +316,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           if (++vs == STAGES) { vs = 0; vph ^= 1u; }
         }
         if (i < n_blk) {
-          if (!__all_sync(0xffffffffu, mbar_wait(k_full + ks, kph) && mbar_wait(s_free + sb, sph))) { ok = false; break; }
+          if (!__all_sync(0xffffffffu, mbar_wait(k_full + ks, kph, abort_flag) && mbar_wait(s_free + sb, sph, abort_flag))) { gave_up = WAIT_attn_k_s; break; }
           tc_fence_after();
           if (elect_one()) {
 #pragma unroll 1
@@ -335,7 +333,6 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           if (++sb == S_BUFS) { sb = 0; sph ^= 1u; }
         }
       }
-      if (!ok) give_up();
     }
   } else {
     // ------------------------------------------------------------------ softmax and epilogue: one row per thread,
@@ -393,8 +390,11 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     bool ok = true;
     auto wait = [&](uint64_t *bar, uint32_t parity) {            // one lane polls for the warp
       int w = 1;
-      if (lane == 0 && (*abort_flag || !mbar_wait(bar, parity))) w = 0;
-      if (!__shfl_sync(0xffffffffu, w, 0)) { if (ok) give_up(); ok = false; }
+      if (lane == 0 && (!ok || !mbar_wait(bar, parity, abort_flag))) w = 0;
+      if (!__shfl_sync(0xffffffffu, w, 0) && ok) {
+        ok = false;
+        if (lane == 0) wait_expired(a.status, WAIT_attn_softmax, abort_flag, -1);
+      }
     };
     float m_ref = -INFINITY, l_run = 0.f, u_run = 0.f;       // exp2 domain; u = sum p (s - m) for the entropy
     const bool want_ent = a.ent != nullptr || a.row_ent != nullptr;
@@ -541,6 +541,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       }
     }
   }
+  if (gave_up && lane == 0) wait_expired(a.status, gave_up, abort_flag, -1);
+  drain_if_aborted(abort_flag);
   tc_fence_before();
   if (a.n_chunks > 1 && !a.part_o) {
     // ---- merge: out = sum_c w_c O_c / sum_c w_c l_c with w_c = 2^(m_c - max m), chunks in ascending order; this CTA's

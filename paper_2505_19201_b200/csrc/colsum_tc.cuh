@@ -9,8 +9,8 @@
 // key per lane.  Each softmax thread then owns one column of the attention matrix and adds up
 // exp2(s * scale - lse) over the rows that may see it, in registers: no reduction across threads.
 // Warp roles: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..5 = one key per thread.  Two
-// accumulators and two query stages alternate.  Every mbarrier wait is bounded; on expiry the
-// kernel raises the status word and leaves.
+// accumulators and two query stages alternate.  Every mbarrier wait is bounded
+// (mbar_wait, gemm_tc.cuh).
 #pragma once
 #include "attn_tc.cuh"
 
@@ -70,6 +70,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_p;
+  int gave_up = WAIT_none;                                  // the wait of this warp that ran out
   pdl_wait();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) trace_stamp(TR_k_colsum);
 
@@ -100,8 +101,7 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       }
       for (int t = 0; t < n_steps; ++t) {
         const int st = t & 1, use = t >> 1;
-        if (use >= 1 && !mbar_wait_warp(q_empty + st, (uint32_t)(use - 1) & 1u)) { if (lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } break; }
-        if (__any_sync(0xffffffffu, *abort_flag)) break;
+        if (use >= 1 && !mbar_wait_warp(q_empty + st, (uint32_t)(use - 1) & 1u, abort_flag)) { gave_up = WAIT_colsum_q_ring; break; }
         if (elect_one()) {
           mbar_expect_tx(q_full + st, (uint32_t)Sh::Q_STAGE);
           for (int pl = 0; pl < 2; ++pl)
@@ -117,10 +117,10 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     if (n_steps > 0) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NQ >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint64_t kd = smem_desc(smem_u32(k_s)), qd = smem_desc(smem_u32(q_s));
-      bool ok = mbar_wait_warp(k_full, 0);
-      for (int t = 0; t < n_steps && ok; ++t) {
+      if (!mbar_wait_warp(k_full, 0, abort_flag)) gave_up = WAIT_colsum_k;
+      for (int t = 0; t < n_steps && !gave_up; ++t) {
         const int st = t & 1, use = t >> 1;
-        if (!__all_sync(0xffffffffu, mbar_wait(q_full + st, (uint32_t)use & 1u) && (use < 1 || mbar_wait(s_free + st, (uint32_t)(use - 1) & 1u)))) { ok = false; break; }
+        if (!__all_sync(0xffffffffu, mbar_wait(q_full + st, (uint32_t)use & 1u, abort_flag) && (use < 1 || mbar_wait(s_free + st, (uint32_t)(use - 1) & 1u, abort_flag)))) { gave_up = WAIT_colsum_operands; break; }
         tc_fence_after();
         uint32_t acc = 0u;
         for (int pl = 0; pl < 2; ++pl)
@@ -136,7 +136,6 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         if (elect_one()) { mma_commit(q_empty + st); mma_commit(s_full + st); }
         __syncwarp();
       }
-      if (!ok && lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
     }
   } else {
     // ------------------------------------------------------------------ one key (column of the attention matrix) per thread
@@ -147,14 +146,12 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
     const float scale = a.scale_log2;
     const float *lse_h = a.lse + cand * a.lse_stride + (long long)h * n;
     float hs = 0.f;
-    bool ok = true;
 #pragma unroll 1
-    for (int t = 0; t < n_steps && ok; ++t) {
+    for (int t = 0; t < n_steps; ++t) {
       const int st = t & 1, i0 = j0 + t * NQ;
       int w_ok = 1;
-      if (lane == 0) w_ok = mbar_wait(s_full + st, (uint32_t)(t >> 1) & 1u) ? 1 : 0;
-      w_ok = __shfl_sync(0xffffffffu, w_ok, 0);
-      if (!w_ok || *abort_flag) { ok = false; break; }
+      if (lane == 0) w_ok = mbar_wait(s_full + st, (uint32_t)(t >> 1) & 1u, abort_flag) ? 1 : 0;
+      if (!__shfl_sync(0xffffffffu, w_ok, 0)) { gave_up = WAIT_colsum_scores; break; }
       tc_fence_after();
 #pragma unroll 1
       for (int c0 = 0; c0 < NQ; c0 += 32) {
@@ -175,9 +172,10 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
       __syncwarp();
       if (lane == 0) mbar_arrive(s_free + st);
     }
-    if (n_steps > 0 && !ok && lane == 0) { atomicMax(a.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; }
-    if (ok && jv >= 0 && jv < a.v) a.part[(long long)h * a.v + jv] = hs;
+    if (!gave_up && jv >= 0 && jv < a.v) a.part[(long long)h * a.v + jv] = hs;
   }
+  if (gave_up && lane == 0) wait_expired(a.status, gave_up, abort_flag, -1);
+  drain_if_aborted(abort_flag);
   pdl_trigger();
   tc_fence_before();
   __syncthreads();

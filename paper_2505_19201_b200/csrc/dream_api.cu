@@ -626,10 +626,12 @@ extern "C" int64_t dream_launch_count(const dream_ctx *c) { return c ? c->launch
 extern "C" dream_status dream_poll(dream_ctx *c) {
   if (!c) return DREAM_E_ARG;
   CUDA_OK(c, cudaStreamSynchronize(c->stream));
-  int st = 0;
-  CUDA_OK(c, cudaMemcpy(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost));
-  if (st == DREAM_DEV_TIMEOUT) return fail(c, DREAM_E_DEVICE_TIMEOUT, "a bounded device-side wait expired");
-  if (st == DREAM_DEV_BAD_INDEX) return fail(c, DREAM_E_STATE, "a kernel met an index or capacity out of range");
+  int st[2] = {0, 0};                    // the code; which wait ran out first
+  CUDA_OK(c, cudaMemcpy(st, c->status, sizeof(st), cudaMemcpyDeviceToHost));
+  static const char *names[] = DREAM_WAIT_NAMES;
+  static_assert(sizeof(names) / sizeof(names[0]) == WAIT_probe + 1, "a name per wait");
+  if (st[1]) return fail(c, DREAM_E_DEVICE_TIMEOUT, "a bounded device-side wait expired (%s)", names[st[1] < 0 || st[1] > WAIT_probe ? 0 : st[1]]);
+  if (st[0] == DREAM_DEV_BAD_INDEX) return fail(c, DREAM_E_STATE, "a kernel met an index or capacity out of range");
   return DREAM_OK;
 }
 
@@ -647,6 +649,28 @@ extern "C" dream_status dream_seq_reset(dream_ctx *c, int32_t seq) {
   c->phase[seq] = PH_EMPTY;
   c->epoch[seq]++;
   if (c->prefill_seq == seq) c->prefill_seq = -1;
+  return DREAM_OK;
+}
+
+// A wait that nothing ends, in a pair of CTAs as the GEMM has them: the first gives up after limit_ns, the second (whose own
+// limit is the usual one) because the first did.  seconds[r]: how long CTA r waited.
+__global__ void __cluster_dims__(2, 1, 1) k_wait_probe(int *status, unsigned long long limit_ns, float *seconds) {
+  __shared__ uint64_t bar;
+  __shared__ int flag;
+  if (threadIdx.x == 0) { mbar_init(&bar, 1); flag = 0; }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  cluster_sync_all();
+  const uint32_t rank = cluster_ctarank();
+  const unsigned long long t0 = global_ns();
+  if (!mbar_wait_warp(&bar, 0, &flag, rank ? WAIT_LIMIT_NS : limit_ns) && threadIdx.x == 0) wait_expired(status, WAIT_probe, &flag, (int)(rank ^ 1u));
+  if (threadIdx.x == 0) seconds[rank] = (float)(global_ns() - t0) * 1e-9f;
+  drain_if_aborted(&flag);
+  cluster_sync_relaxed();
+}
+extern "C" dream_status dream_debug_wait(dream_ctx *c, int32_t limit_ms, float *seconds) {
+  if (!c || !seconds || limit_ms < 1 || limit_ms > 1000) return fail(c, DREAM_E_ARG, "limit_ms in 1..1000 and a device buffer of two floats");
+  k_wait_probe<<<2, 32, 0, c->stream>>>(c->status, (unsigned long long)limit_ms * 1000000ull, seconds);
+  CUDA_OK(c, cudaGetLastError());
   return DREAM_OK;
 }
 

@@ -40,7 +40,7 @@
 //     4..11 = epilogue.  A TMEM lane is an output column c, so a warp's store of one token covers 128
 //     contiguous bytes without a transpose; two TMEM accumulators alternate so that the epilogue of
 //     one segment overlaps the MMAs of the next;
-//   * every mbarrier wait is bounded: on expiry the kernel raises the status word and leaves.
+//   * every mbarrier wait is bounded, see mbar_wait.
 #pragma once
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -55,7 +55,6 @@
 #define TC_BN 256               // weight rows per tile (MMA M, both CTAs)
 #define TC_BK 64                // k elements per panel (128 bytes: one swizzle row)
 #define TC_THREADS 384          // 12 warps, see the roles above
-#define TC_SPIN_LIMIT (1u << 24)
 #define TC_WPANEL (128 * TC_BK * 2)          // one CTA's half of a weight panel
 #define TC_MAX_STAGES 12
 #define TC_EVEN 4               // units a pair may walk further for a share that lies in one tile
@@ -109,17 +108,55 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// Bounded wait on a phase parity; false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
-  uint32_t addr = smem_u32(bar);
-  for (uint32_t it = 0; it < TC_SPIN_LIMIT; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-    if (done) return true;
-  }
+// ---- bounded waits.  A wait gives up WAIT_LIMIT_NS after it first found its phase incomplete, or as soon as the CTA's abort
+// flag is set; the warp that gives up first names the wait in the status words and sets the flag in every CTA that depends on
+// its own (wait_expired), and all leave within a millisecond or so.  (A limit that counts attempts is no limit: each may
+// suspend the thread for as long as the hardware likes.)  No wait starts before the kernel's grid dependency has
+// resolved, so that the limit covers this kernel's own work, milliseconds at most, however long its predecessors take.
+// What has no limit: griddepcontrol.wait, whose predecessors end by the same rule; cluster and named barriers, which every
+// thread of the CTAs concerned reaches whatever its waits said; the TMEM allocation, which waits for CTAs on the same SM that
+// are past theirs and wait for nothing behind it.
+#define WAIT_LIMIT_NS 1000000000ull
+#define WAIT_SUSPEND_NS 1000000u         // an attempt suspends the thread no longer than this
+#define WAIT_DRAIN_NS 1000000ull
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(done) : "r"(addr), "r"(parity), "r"(WAIT_SUSPEND_NS) : "memory");
+  return done != 0;
+}
+// Waits for a phase parity; false when the limit ran out or the abort flag is set.
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const volatile int *abort_flag, unsigned long long limit_ns = WAIT_LIMIT_NS) {
+  const uint32_t addr = smem_u32(bar);
+  if (mbar_try(addr, parity)) return true;
+  const unsigned long long t0 = global_ns();
+  do {
+    if (mbar_try(addr, parity)) return true;
+    if (*abort_flag) return false;
+  } while (global_ns() - t0 < limit_ns);
   return false;
+}
+// One thread of a warp whose wait gave up.  peer: the CTA of the cluster that depends on this one (none: -1); it cannot
+// have left, the closing barrier needs this thread too.
+__device__ __forceinline__ void wait_expired(int *status, int where, volatile int *abort_flag, int peer) {
+  if (*abort_flag) return;                     // somebody else's wait was the first
+  *abort_flag = 1;
+  atomicCAS(status + 1, 0, where);
+  atomicMax(status, DREAM_DEV_TIMEOUT);
+  if (peer >= 0)
+    asm volatile("{\n .reg .b32 a;\n mapa.shared::cluster.u32 a, %0, %1;\n st.relaxed.cluster.shared::cluster.u32 [a], 1;\n fence.acq_rel.cluster;\n}"
+                 ::"r"((uint32_t)__cvta_generic_to_shared((const void *)abort_flag)), "r"(peer) : "memory");
+}
+// Before a CTA that gave up leaves: its copies and matrix instructions under way land within microseconds.
+__device__ __forceinline__ void drain_if_aborted(const volatile int *abort_flag) {
+  if (!*abort_flag) return;
+  for (const unsigned long long t0 = global_ns(); global_ns() - t0 < WAIT_DRAIN_NS;) {}
 }
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, uint64_t policy) {
   asm volatile(
@@ -189,8 +226,8 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 // The bounded wait made by a whole warp, which stays together whatever its lanes see.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, const volatile int *abort_flag, unsigned long long limit_ns = WAIT_LIMIT_NS) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit_ns));
 }
 
 // ---- pairs of CTAs (cluster of two; the even rank leads)
@@ -311,7 +348,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   int tile, k0, k1;
   constexpr bool TILES = FORM == TC_X_TILES;
   TcWalk<TILES> walk(p, pair);
-  auto give_up = [&]() { if (lane == 0) { atomicMax(p.status, DREAM_DEV_TIMEOUT); *abort_flag = 1; } };
+  int gave_up = WAIT_none;                       // the wait of this warp that ran out
 
   if (warp == 0) {
     // ------------------------------------------------------------------ W producer: weights are
@@ -322,13 +359,11 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const uint32_t bar0 = mapa(smem_u32(full_w), 0);
     int s = 0;
     uint32_t ph = 1;
-    bool ok = true;
-    while (ok && walk.next(p, tile, k0, k1)) {
+    while (!gave_up && walk.next(p, tile, k0, k1)) {
       const int y = (TILES ? tile / p.n_tt : tile) * TC_BN + (int)rank * 128;
       for (int kb = k0; kb < k1; kb += p.wp) {
         const int np = min(p.wp, k1 - kb);
-        if (!mbar_wait_warp(empty_w + s, ph)) { give_up(); ok = false; break; }
-        if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(empty_w + s, ph, abort_flag)) { gave_up = WAIT_gemm_w_ring; break; }
         if (elect_one()) {
           if (rank == 0) mbar_expect_tx(full_w + s, 2u * (uint32_t)np * TC_WPANEL);
           uint8_t *dst = wring + (size_t)s * wstage_bytes;
@@ -345,13 +380,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
           }
         }
         __syncwarp();
-        if (++s == p.w_stages) { s = 0; ph ^= 1; }
+        if (++s == p.w_stages) { s = 0; ph ^= 1; pdl_wait(); }      // (a stage is released only behind the dependency)
       }
     }
+    pdl_wait();
     // Until the last releases have arrived, which the pair's first CTA signals across: an arrival that comes in after this
     // CTA has left would land in the shared memory of the CTA that follows it on the SM.
-    for (int i = 0; ok && i < p.w_stages; ++i) {
-      if (!mbar_wait_warp(empty_w + s, ph)) { give_up(); ok = false; }
+    for (int i = 0; !gave_up && i < p.w_stages; ++i) {
+      if (!mbar_wait_warp(empty_w + s, ph, abort_flag)) gave_up = WAIT_gemm_w_last;
       if (++s == p.w_stages) { s = 0; ph ^= 1; }
     }
   } else if (warp == 2) {
@@ -368,17 +404,15 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     const int y_off = FORM == TC_X_CONCAT ? (int)rank * p.lo_rows : (int)rank * (p.mma_n >> 1);   // first token row this CTA stages, from the tile's
     int s = 0, n_free = p.x_stages, ws = 0;      // unused X stages left; W stage that went with the X stage to reuse
     uint32_t wph = 0;
-    bool ok = true;
-    for (; ok && more; more = walk.next(p, tile, k0, k1)) {
+    for (; !gave_up && more; more = walk.next(p, tile, k0, k1)) {
       const int y = (TILES ? tile % p.n_tt * p.tile_t : 0) + y_off;
       for (int kb = k0; kb < k1; kb += p.wp) {
         const int np = min(p.wp, k1 - kb);
         if (n_free > 0) --n_free;
         else {
-          if (!mbar_wait_warp(empty_w + ws, wph)) { give_up(); ok = false; break; }
+          if (!mbar_wait_warp(empty_w + ws, wph, abort_flag)) { gave_up = WAIT_gemm_x_ring; break; }
           if (++ws == p.w_stages) { ws = 0; wph ^= 1; }
         }
-        if (__any_sync(0xffffffffu, *abort_flag)) { ok = false; break; }
         if (elect_one()) {
           if (rank == 0) mbar_expect_tx(full_x + s, 2u * (uint32_t)np * xpanel_bytes);
           for (int i = 0; i < np; ++i) {
@@ -401,19 +435,19 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       const uint32_t sub_n = (uint32_t)p.mma_n, sub_mask = (uint32_t)p.n_sub - 1u;
       int ws = 0, xs = 0;
       uint32_t wph = 0, xph = 0, fill = 0;                            // fill counts accumulator fills
-      bool ok = true;
       k0 = k1 = 0;
-      while (ok && (k0 < k1 || walk.next(p, tile, k0, k1))) {
+      pdl_wait();
+      while (!gave_up && (k0 < k1 || walk.next(p, tile, k0, k1))) {
         const int fill_end = FORM >= TC_X_TWO ? min(k1, k0 + TC_CHAIN) : k1;
         const uint32_t buf = fill & 1u, use = fill >> 1;              // use: earlier fills of this accumulator
         ++fill;
-        if (!mbar_wait_warp(acc_empty + buf, (use & 1u) ^ 1u)) { ok = false; break; }
+        if (!mbar_wait_warp(acc_empty + buf, (use & 1u) ^ 1u, abort_flag)) { gave_up = WAIT_gemm_acc_empty; break; }
         tc_fence_after();
         const uint32_t d_addr = tmem_base + buf * 256u;
         uint32_t begun = 0u;                                          // 0: the first MMA of an accumulator overwrites it
         while (k0 < fill_end) {
           const int np = min(wp, fill_end - k0);
-          if (!__all_sync(0xffffffffu, mbar_wait(full_w + ws, wph) && mbar_wait(full_x + xs, xph))) { ok = false; break; }
+          if (!__all_sync(0xffffffffu, mbar_wait(full_w + ws, wph, abort_flag) && mbar_wait(full_x + xs, xph, abort_flag))) { gave_up = WAIT_gemm_operands; break; }
           tc_fence_after();
           for (int i = 0; i < np; ++i) {
             const uint64_t ad = wdesc + (uint64_t)((ws * wp + i) * (TC_WPANEL >> 4));
@@ -437,15 +471,14 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
           if (++ws == w_stages) { ws = 0; wph ^= 1; }
           if (++xs == x_stages) { xs = 0; xph ^= 1; }
         }
-        if (ok && elect_one()) mma_commit_pair(acc_full + buf);       // accumulator complete
+        if (!gave_up && elect_one()) mma_commit_pair(acc_full + buf);       // accumulator complete
         __syncwarp();
       }
       // as above for the second CTA's arrivals: both accumulators emptied (they are relaxed, and the barrier at the end
       // does not wait for them; one that came late left a later launch waiting for good, once in some million).  The
       // decode forms send only the arrivals that the loop above has waited for.
-      for (uint32_t buf = 0; FORM >= TC_X_TWO && ok && buf < 2u; ++buf)
-        if (!mbar_wait_warp(acc_empty + buf, (((fill + 1u - buf) >> 1) & 1u) ^ 1u)) ok = false;
-      if (!ok) give_up();
+      for (uint32_t buf = 0; FORM >= TC_X_TWO && !gave_up && buf < 2u; ++buf)
+        if (!mbar_wait_warp(acc_empty + buf, (((fill + 1u - buf) >> 1) & 1u) ^ 1u, abort_flag)) gave_up = WAIT_gemm_acc_last;
     }
   } else if (warp >= 4) {
     // ------------------------------------------------------------------ epilogue: this CTA's 128 output
@@ -459,9 +492,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     bool ok = true;
     auto wait_full = [&](uint32_t buf, uint32_t use) {
       int w = 1;
-      if (lane == 0) w = mbar_wait(acc_full + buf, use & 1u) ? 1 : 0;
-      w = __shfl_sync(0xffffffffu, w, 0);
-      if (!w || __any_sync(0xffffffffu, *abort_flag)) { give_up(); ok = false; }
+      if (lane == 0) w = mbar_wait(acc_full + buf, use & 1u, abort_flag) ? 1 : 0;
+      ok = __shfl_sync(0xffffffffu, w, 0) != 0;
+      if (!ok) gave_up = WAIT_gemm_acc_full;
       tc_fence_after();
     };
     while (ok && walk.next(p, tile, k0, k1)) {
@@ -584,6 +617,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       }
     }
   }
+  if (gave_up && lane == 0) wait_expired(p.status, gave_up, abort_flag, (int)(rank ^ 1u));
+  drain_if_aborted(abort_flag);
   tc_fence_before();
   __syncthreads();
   cluster_sync_relaxed();                      // neither CTA leaves while its peer may still signal it or read its operands
