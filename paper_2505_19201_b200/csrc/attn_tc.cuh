@@ -279,6 +279,17 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
           if (++vs == STAGES) { vs = 0; vph ^= 1u; }
         }
       }
+      // Until the last releases have arrived (the commits that nothing else waits for): one that came in after this CTA has
+      // left would land in the shared memory of the CTA that follows it on the SM.
+#pragma unroll 1
+      for (int i = 0; i < STAGES && !gave_up; ++i) {
+        if (!mbar_wait_warp(k_empty + ks, kph, abort_flag) || !mbar_wait_warp(v_empty + vs, vph, abort_flag)) gave_up = WAIT_attn_last;
+        if (++ks == STAGES) { ks = 0; kph ^= 1u; }
+        if (++vs == STAGES) { vs = 0; vph ^= 1u; }
+      }
+      // (parity of the last phase of a barrier used n times: n - 1; never used: 1)
+      for (int b = 0; b < 2 && !gave_up; ++b)
+        if (!mbar_wait_warp(p_empty + b, (uint32_t)(((n_blk + 1 - b) >> 1) + 1) & 1u, abort_flag)) gave_up = WAIT_attn_last;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: the whole warp, an elected

@@ -110,6 +110,9 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
         }
         __syncwarp();
       }
+      // until the last two releases have arrived, as in the attention kernel
+      for (int st = 0; st < 2 && !gave_up; ++st)
+        if (!mbar_wait_warp(q_empty + st, (uint32_t)(((n_steps + 1 - st) >> 1) + 1) & 1u, abort_flag)) gave_up = WAIT_colsum_last;
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer: S^T = K Q_hi^T + K Q_lo^T

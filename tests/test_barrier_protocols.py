@@ -1,0 +1,258 @@
+"""Models of the barrier traffic of k_gemm_tc (a pair of CTAs) and k_attn_tc (a CTA), run in random order on the CPU: every
+agent ends, and when the last one has, no asynchronous arrival is under way any more.  An arrival that came in later would
+land in the shared memory of the CTA that follows on the SM.  Without the closing waits the models show such arrivals."""
+import heapq
+import random
+
+import pytest
+
+
+class Clock:
+    """Asynchronous completions, each after a delay of its own."""
+
+    def __init__(self, rng):
+        self.rng, self.now, self.queue, self.n = rng, 0.0, [], 0
+
+    def at(self, when, f):
+        self.n += 1
+        heapq.heappush(self.queue, (when, self.n, f))
+
+    def later(self, f, lo=0.1, hi=4.0):
+        self.at(self.now + self.rng.uniform(lo, hi), f)
+
+
+class Barrier:
+    def __init__(self, count):
+        self.count = self.pending = count
+        self.tx = self.phase = 0
+
+    def arrive(self):
+        assert self.pending > 0
+        self.pending -= 1
+        self.add(0)
+
+    def add(self, tx):
+        self.tx += tx
+        if self.pending == 0 and self.tx == 0:
+            self.phase, self.pending = self.phase + 1, self.count
+
+    def load(self, clock, boxes):            # expect_tx by one thread, the boxes land one by one
+        self.add(boxes)
+        self.arrive()
+        for _ in range(boxes):
+            clock.later(lambda: self.add(-1))
+
+    def done(self, parity):
+        return (self.phase & 1) != parity
+
+
+class Committer:
+    """tcgen05.commit: arrives behind the MMAs issued before it, barriers of one commit point at times of their own."""
+
+    def __init__(self, clock):
+        self.clock, self.last = clock, 0.0
+
+    def __call__(self, *barriers):
+        self.last = max(self.last, self.clock.now) + self.clock.rng.uniform(0.05, 0.6)
+        for b in barriers:
+            self.clock.at(self.last + self.clock.rng.uniform(0, 1.5), b.arrive)
+
+
+def play(clock, agents):
+    """Arrivals under way when the last agent has ended."""
+    idle = 0
+    while agents:
+        clock.rng.shuffle(agents)
+        alive = []
+        for g in agents:
+            try:
+                next(g)
+                alive.append(g)
+            except StopIteration:
+                pass
+        agents = alive
+        clock.now += 0.1
+        while clock.queue and clock.queue[0][0] <= clock.now:
+            heapq.heappop(clock.queue)[2]()
+        idle = 0 if clock.queue else idle + 1
+        assert idle < 500, "nothing under way and nobody moves"
+    return len(clock.queue)
+
+
+def until(cond):
+    while not cond():
+        yield
+
+
+def some(rng, most):
+    for _ in range(rng.randint(0, most)):
+        yield
+
+
+# ring depths of K and V blocks and of score buffers, by (head_dim, flat cache)
+ATTN = {(64, False): (3, 3), (64, True): (4, 3), (128, False): (5, 4), (128, True): (2, 4), (256, False): (2, 4), (256, True): (1, 4)}
+
+
+def attention(shape, n_blk, early, seed, closing=True):
+    rng = random.Random(seed)
+    stages, s_bufs = ATTN[shape]
+    ahead = min(stages, s_bufs)
+    clock = Clock(rng)
+    bars = lambda n, count=1: [Barrier(count) for _ in range(n)]
+    k_full, k_empty, v_full, v_empty = bars(stages), bars(stages), bars(stages), bars(stages)
+    s_full, s_free, p_full, p_empty = bars(s_bufs), bars(s_bufs, 8), bars(2, 8), bars(2)
+    n_pre = min(early, n_blk, stages)
+
+    def producer():
+        for i in range(n_pre):
+            k_full[i].load(clock, 2)
+            v_full[i].load(clock, 2)
+        ks = vs = n_pre % stages
+        kph = vph = 0 if n_pre >= stages else 1
+        for it in range(n_pre, n_blk + 1):
+            if it < n_blk:
+                yield from until(lambda: k_empty[ks].done(kph))
+                k_full[ks].load(clock, 2)
+                ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
+            if it > n_pre:
+                yield from until(lambda: v_empty[vs].done(vph))
+                v_full[vs].load(clock, 2)
+                vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
+        if not closing:
+            return
+        for _ in range(stages):
+            yield from until(lambda: k_empty[ks].done(kph) and v_empty[vs].done(vph))
+            ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
+            vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
+        for b in (0, 1):
+            yield from until(lambda: p_empty[b].done((((n_blk + 1 - b) >> 1) + 1) & 1))
+
+    def issuer():
+        commit = Committer(clock)
+        ks = sb = vs = kph = vph = 0
+        sph = 1
+        for i in range(n_blk + ahead):
+            it = i - ahead
+            if it >= 0:
+                yield from until(lambda: p_full[it & 1].done((it >> 1) & 1) and v_full[vs].done(vph))
+                commit(p_empty[it & 1], v_empty[vs])
+                vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
+            if i < n_blk:
+                yield from until(lambda: k_full[ks].done(kph) and s_free[sb].done(sph))
+                commit(k_empty[ks], s_full[sb])
+                ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
+                sb, sph = (sb + 1, sph) if sb + 1 < s_bufs else (0, sph ^ 1)
+
+    met = {}
+
+    def softmax(quarter, half):
+        sb = sph = 0
+        for it in range(n_blk):
+            pb = it & 1
+            yield from until(lambda: s_full[sb].done(sph))
+            yield from some(rng, 3)
+            s_free[sb].arrive()
+            sb, sph = (sb + 1, sph) if sb + 1 < s_bufs else (0, sph ^ 1)
+            met[quarter, half] = it
+            yield from until(lambda: met.get((quarter, half ^ 1), -1) >= it)
+            if it and rng.random() < 0.3:                     # the row's reference moves
+                yield from until(lambda: p_empty[pb ^ 1].done(((it - 1) >> 1) & 1))
+            if it >= 2:
+                yield from until(lambda: p_empty[pb].done(((it >> 1) - 1) & 1))
+            yield from some(rng, 3)
+            p_full[pb].arrive()
+        yield from until(lambda: p_empty[(n_blk - 1) & 1].done(((n_blk - 1) >> 1) & 1))
+
+    return play(clock, [producer(), issuer()] + [softmax(q, h) for q in range(4) for h in range(2)])
+
+
+@pytest.mark.parametrize("shape", list(ATTN))
+def test_attention(shape):
+    for n_blk in (1, 2, 3, 4, 5, 6, 7, 11, 33):
+        for early in ((0,) if shape[1] else (0, 1, n_blk)):
+            for seed in range(3):
+                assert attention(shape, n_blk, early, seed) == 0
+
+
+def test_attention_without_closing_waits():
+    assert any(attention((128, False), 5, 0, seed, closing=False) for seed in range(20))
+
+
+def gemm(panels, w_stages, x_stages, wp, chain, seed, closing=True):
+    """panels: k panels of the pair's segments.  chain: panels per accumulator fill (0: a segment is one fill and only an arrival
+    that the issuer waits for is sent, the forms of up to 128 rows)."""
+    rng = random.Random(seed)
+    clock = Clock(rng)
+    bars = lambda n, count=1: [Barrier(count) for _ in range(n)]
+    empty_w, full_w, full_x = [bars(w_stages), bars(w_stages)], bars(w_stages), bars(x_stages)
+    acc_full, acc_empty = [bars(2), bars(2)], bars(2, 16)
+
+    def w_producer(rank):
+        s, ph = 0, 1
+        for k in panels:
+            for kb in range(0, k, wp):
+                yield from until(lambda: empty_w[rank][s].done(ph))
+                if rank == 0:
+                    full_w[s].load(clock, 2 * min(wp, k - kb))      # its own boxes and the second CTA's
+                s, ph = (s + 1, ph) if s + 1 < w_stages else (0, ph ^ 1)
+        for _ in range(w_stages if closing else 0):
+            yield from until(lambda: empty_w[rank][s].done(ph))
+            s, ph = (s + 1, ph) if s + 1 < w_stages else (0, ph ^ 1)
+
+    def x_producer(rank):
+        yield from some(rng, 30)
+        s = ws = wph = 0
+        free = x_stages
+        for k in panels:
+            for kb in range(0, k, wp):
+                if free:
+                    free -= 1
+                else:
+                    yield from until(lambda: empty_w[rank][ws].done(wph))
+                    ws, wph = (ws + 1, wph) if ws + 1 < w_stages else (0, wph ^ 1)
+                if rank == 0:
+                    full_x[s].load(clock, 2 * min(wp, k - kb))
+                s = (s + 1) % x_stages
+
+    fills = [[min(chain, k - a) for a in range(0, k, chain)] if chain else [k] for k in panels]
+
+    def issuer():
+        commit = Committer(clock)
+        ws = xs = wph = xph = fill = 0
+        for segment in fills:
+            for k in segment:
+                buf, use = fill & 1, fill >> 1
+                fill += 1
+                yield from until(lambda: acc_empty[buf].done((use & 1) ^ 1))
+                for _ in range(0, k, wp):
+                    yield from until(lambda: full_w[ws].done(wph) and full_x[xs].done(xph))
+                    commit(empty_w[0][ws], empty_w[1][ws])
+                    ws, wph = (ws + 1, wph) if ws + 1 < w_stages else (0, wph ^ 1)
+                    xs, xph = (xs + 1, xph) if xs + 1 < x_stages else (0, xph ^ 1)
+                commit(acc_full[0][buf], acc_full[1][buf])
+        for buf in (0, 1) if chain and closing else ():
+            yield from until(lambda: acc_empty[buf].done((((fill + 1 - buf) >> 1) & 1) ^ 1))
+
+    def epilogue(rank):
+        fill = 0
+        for segment in fills:
+            for _ in segment:
+                buf = fill & 1
+                yield from until(lambda: acc_full[rank][buf].done((fill >> 1) & 1))
+                fill += 1
+                yield from some(rng, 4)
+                if chain or fill + 1 < len(panels):
+                    clock.later(acc_empty[buf].arrive, 0, 3)         # relaxed and remote: it lands when it lands
+
+    return play(clock, [w_producer(0), w_producer(1), x_producer(0), x_producer(1), issuer()] + [epilogue(r) for r in (0, 1) for _ in range(8)])
+
+
+@pytest.mark.parametrize("panels", [[1], [3], [32], [25, 39], [7, 64, 46], [64, 64, 64, 20], [1, 1, 1]])
+@pytest.mark.parametrize("w_stages,x_stages,wp,chain", [(6, 3, 2, 0), (10, 6, 1, 0), (9, 4, 1, 0), (7, 6, 1, 8), (5, 4, 1, 8), (5, 5, 1, 8)])
+def test_gemm_pair(panels, w_stages, x_stages, wp, chain):
+    for seed in range(2):
+        assert gemm(panels, w_stages, x_stages, wp, chain, seed) == 0
+
+
+def test_gemm_pair_without_closing_waits():
+    assert any(gemm([25, 39], 5, 4, 1, 8, seed, closing=False) for seed in range(20))
