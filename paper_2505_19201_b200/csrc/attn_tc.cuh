@@ -574,19 +574,21 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         float4 ml[4], o[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const uint32_t cc = (uint32_t)min(c + k, n - 1);
-          ml[k] = ld_cluster4(mapa(ml_addr + en * 16, cc));
-          o[k] = ld_cluster4(mapa(o_addr + (en * Sh::O_LD + c4) * 4, cc));
+          ml[k] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+          o[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (c + k < n) { ml[k] = ld_cluster4(mapa(ml_addr + en * 16, c + k)); o[k] = ld_cluster4(mapa(o_addr + (en * Sh::O_LD + c4) * 4, c + k)); }
         }
+        // A chunk without a visible key has no weight, but what was read of it enters the sums all the same: the closing
+        // barrier does not wait for a read whose value nobody uses, and its CTA might leave before the read gets there.
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          if (c + k >= n || ml[k].x == -INFINITY) continue;
-          const float Mn = fmaxf(M, ml[k].x), sc = ex2(M - Mn), w = ex2(ml[k].x - Mn);       // 2^-inf = 0 on the first live chunk
+          const bool on = ml[k].x != -INFINITY;
+          const float Mn = fmaxf(M, ml[k].x), sc = on ? ex2(M - Mn) : 1.f, w = on ? ex2(ml[k].x - Mn) : 0.f;       // 2^-inf = 0 on the first live chunk
           // u relative to the new reference: sum p' (s - Mn) with p' = p 2^(m - Mn)
-          U = (L > 0.f ? sc * (U + (M - Mn) * L) : 0.f) + w * (ml[k].z + (ml[k].x - Mn) * ml[k].y);
+          U = on ? (L > 0.f ? sc * (U + (M - Mn) * L) : 0.f) + w * (ml[k].z + (ml[k].x - Mn) * ml[k].y) : U;
           L = L * sc + ml[k].y * w;
-          acc.x = acc.x * sc + o[k].x * w; acc.y = acc.y * sc + o[k].y * w;
-          acc.z = acc.z * sc + o[k].z * w; acc.w = acc.w * sc + o[k].w * w;
+          acc.x = acc.x * sc + (on ? o[k].x : 0.f) * w; acc.y = acc.y * sc + (on ? o[k].y : 0.f) * w;
+          acc.z = acc.z * sc + (on ? o[k].z : 0.f) * w; acc.w = acc.w * sc + (on ? o[k].w : 0.f) * w;
           M = Mn;
         }
       }
