@@ -15,12 +15,12 @@ typedef __nv_bfloat16 bf16;
 // The waits that can expire, as the second status word names the first one that did.
 enum {
   WAIT_none = 0,
-  WAIT_gemm_w_ring, WAIT_gemm_w_last, WAIT_gemm_x_ring, WAIT_gemm_operands, WAIT_gemm_acc_empty, WAIT_gemm_acc_last, WAIT_gemm_acc_full,
+  WAIT_gemm_peer, WAIT_gemm_w_ring, WAIT_gemm_w_last, WAIT_gemm_x_ring, WAIT_gemm_operands, WAIT_gemm_acc_empty, WAIT_gemm_acc_last, WAIT_gemm_acc_full,
   WAIT_attn_k_ring, WAIT_attn_v_ring, WAIT_attn_q, WAIT_attn_p_v, WAIT_attn_k_s, WAIT_attn_softmax, WAIT_attn_last,
   WAIT_colsum_q_ring, WAIT_colsum_k, WAIT_colsum_operands, WAIT_colsum_scores, WAIT_colsum_last,
   WAIT_probe
 };
-#define DREAM_WAIT_NAMES {"none", "k_gemm_tc: weight ring", "k_gemm_tc: last weight stages", "k_gemm_tc: token ring", "k_gemm_tc: operands", "k_gemm_tc: accumulator emptied", "k_gemm_tc: last accumulators emptied", "k_gemm_tc: accumulator complete", "k_attn_tc: key ring", "k_attn_tc: value ring", "k_attn_tc: queries", "k_attn_tc: probabilities and values", "k_attn_tc: keys and score buffer", "k_attn_tc: softmax", "k_attn_tc: last releases", "k_colsum_tc: query ring", "k_colsum_tc: keys", "k_colsum_tc: queries and accumulator", "k_colsum_tc: scores", "k_colsum_tc: last releases", "k_wait_probe"}
+#define DREAM_WAIT_NAMES {"none", "k_gemm_tc: partner's TMEM", "k_gemm_tc: weight ring", "k_gemm_tc: last weight stages", "k_gemm_tc: token ring", "k_gemm_tc: operands", "k_gemm_tc: accumulator emptied", "k_gemm_tc: last accumulators emptied", "k_gemm_tc: accumulator complete", "k_attn_tc: key ring", "k_attn_tc: value ring", "k_attn_tc: queries", "k_attn_tc: probabilities and values", "k_attn_tc: keys and score buffer", "k_attn_tc: softmax", "k_attn_tc: last releases", "k_colsum_tc: query ring", "k_colsum_tc: keys", "k_colsum_tc: queries and accumulator", "k_colsum_tc: scores", "k_colsum_tc: last releases", "k_wait_probe"}
 
 __device__ __forceinline__ float to_f(float v) { return v; }
 __device__ __forceinline__ float to_f(bf16 v) { return __bfloat162float(v); }

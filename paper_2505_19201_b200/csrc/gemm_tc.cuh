@@ -114,8 +114,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // suspend the thread for as long as the hardware likes.)  No wait starts before the kernel's grid dependency has
 // resolved, so that the limit covers this kernel's own work, milliseconds at most, however long its predecessors take.
 // What has no limit: griddepcontrol.wait, whose predecessors end by the same rule; cluster and named barriers, which every
-// thread of the CTAs concerned reaches whatever its waits said; the TMEM allocation, which waits for CTAs on the same SM that
-// are past theirs and wait for nothing behind it.
+// thread of the CTAs concerned reaches whatever its waits said; the TMEM allocation, which waits for CTAs that
+// hold some on the same SM, and these wait for no allocation any more.
 #define WAIT_LIMIT_NS 1000000000ull
 #define WAIT_SUSPEND_NS 1000000u         // an attempt suspends the thread no longer than this
 #define WAIT_DRAIN_NS 1000000ull
@@ -321,7 +321,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   uint64_t *bars = (uint64_t *)(xring + (size_t)p.x_stages * xstage_bytes);
   uint64_t *full_w = bars, *empty_w = full_w + TC_MAX_STAGES, *full_x = empty_w + TC_MAX_STAGES;
   uint64_t *acc_full = full_x + TC_MAX_STAGES, *acc_empty = acc_full + 2;
-  uint32_t *tmem_base_p = (uint32_t *)(acc_empty + 2);
+  uint64_t *peer_tmem = acc_empty + 2;            // first CTA: the second one has its TMEM
+  uint32_t *tmem_base_p = (uint32_t *)(peer_tmem + 1);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
@@ -332,19 +333,24 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     if (lane < TC_MAX_STAGES) { mbar_init(full_w + lane, 1); mbar_init(empty_w + lane, 1); }
     else if (lane < 2 * TC_MAX_STAGES) mbar_init(full_x + lane - TC_MAX_STAGES, 1);
     else if (lane < 2 * TC_MAX_STAGES + 2) { mbar_init(acc_full + lane - 2 * TC_MAX_STAGES, 1); mbar_init(acc_empty + lane - 2 * TC_MAX_STAGES, 16); }
-    else if (lane == 31) *abort_flag = 0;
+    else if (lane == 31) { mbar_init(peer_tmem, 1); *abort_flag = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // Both CTAs run from here on, and their barriers are initialised.  The allocation is an act of the pair: issued before its
+  // partner was known to run it hung, once in some ten million launches (the first CTA's had come back, the second's never did).
+  cluster_sync_all();
   if (warp == 1) {      // all 512 TMEM columns (two accumulators of 256), allocated by one full warp of each CTA
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_base_p)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    tc_fence_before();
+    if (rank == 1 && lane == 0) mbar_arrive_cluster(mapa(smem_u32(peer_tmem), 0));
   }
-  tc_fence_before();
-  __syncthreads();
-  cluster_sync_all();                            // the peer's barriers are initialised
-  tc_fence_after();
   pdl_trigger();
-  const uint32_t tmem_base = *tmem_base_p;
+  uint32_t tmem_base = 0;
+  if (warp == 1 || warp >= 4) {                  // the warps that use them
+    asm volatile("bar.sync 1, 288;" ::: "memory");
+    tc_fence_after();
+    tmem_base = *tmem_base_p;
+  }
   int tile, k0, k1;
   constexpr bool TILES = FORM == TC_X_TILES;
   TcWalk<TILES> walk(p, pair);
@@ -437,6 +443,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       uint32_t wph = 0, xph = 0, fill = 0;                            // fill counts accumulator fills
       k0 = k1 = 0;
       pdl_wait();
+      if (!mbar_wait_warp(peer_tmem, 0, abort_flag)) gave_up = WAIT_gemm_peer;
       while (!gave_up && (k0 < k1 || walk.next(p, tile, k0, k1))) {
         const int fill_end = FORM >= TC_X_TWO ? min(k1, k0 + TC_CHAIN) : k1;
         const uint32_t buf = fill & 1u, use = fill >> 1;              // use: earlier fills of this accumulator
@@ -619,6 +626,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   }
   if (gave_up && lane == 0) wait_expired(p.status, gave_up, abort_flag, (int)(rank ^ 1u));
   drain_if_aborted(abort_flag);
+  __syncwarp();
+  if (warp == 1) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");     // the pair's too: both have allocated
   tc_fence_before();
   __syncthreads();
   cluster_sync_relaxed();                      // neither CTA leaves while its peer may still signal it or read its operands

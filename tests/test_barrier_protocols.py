@@ -256,3 +256,13 @@ def test_gemm_pair(panels, w_stages, x_stages, wp, chain):
 
 def test_gemm_pair_without_closing_waits():
     assert any(gemm([25, 39], 5, 4, 1, 8, seed, closing=False) for seed in range(20))
+
+
+def test_pair_allocates_tmem_behind_the_barrier_that_shows_its_partner_running():
+    """tcgen05.alloc of a pair is an act of both CTAs; issued before the start barrier it hung once in some ten million launches."""
+    import os
+    src = open(os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2505_19201_b200", "csrc", "gemm_tc.cuh")).read()
+    body = src[src.index("k_gemm_tc(const __grid_constant__"):]
+    alloc, release, free = (body.index("tcgen05." + op + ".cta_group::2") for op in ("alloc", "relinquish_alloc_permit", "dealloc"))
+    assert body.index("cluster_sync_all();") < alloc
+    assert alloc < release < body.index("cluster_sync_relaxed();") < free
