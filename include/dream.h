@@ -249,11 +249,18 @@ dream_status dream_debug_read(dream_ctx *ctx, int32_t seq, int32_t what, int32_t
 
 /* Test hook: out[r][c] = sum_k X[r][k] W[c][k] through the context's GEMM path (the same
  * kernels every projection of the model uses).  W: device [N][K] in config.dtype; X: device
- * float [rows][K]; out: device float [rows][N]; rows <= 256 (128 for bf16 with split == 0);
+ * float [rows][K]; out: device float [rows][N]; rows <= 256 (128 for bf16 with split == 0), or as many as the
+ * context puts through a projection at a time;
  * K <= max(d_model, d_ff); bf16: K a multiple of 64, N of 8.  split != 0 feeds bf16 inputs as a
- * high and a low bf16 row per token. */
+ * high and a low bf16 row per token.  split == 2: W holds N / 2 gate rows, then N / 2 up rows, and out is
+ * silu(gate) * up [rows][N / 2] as the MLP's next projection reads it (bf16; K <= d_model, N / 2 a multiple of 64 up to d_ff). */
 dream_status dream_debug_gemm(dream_ctx *ctx, const void *W, const float *X, int32_t rows,
                               int32_t N, int32_t K, int32_t split, float *out);
+
+/* Test hook: top-k and log-sum-exp of device logits [rows][config.vocab] as the draft and verify calls compute them.
+ * rows <= 256, ktop <= 16; top_val, top_id: device [rows][ktop]; lse: device [rows]. */
+dream_status dream_debug_topk(dream_ctx *ctx, const float *logits, int32_t rows, int32_t ktop, float *top_val,
+                              int32_t *top_id, float *lse);
 
 /* Test hook: a device-side wait that nothing ends, in a pair of CTAs.  The first gives up after limit_ms (1..1000)
  * and raises the status word, the second because the first did.  seconds: device buffer of two floats, how long

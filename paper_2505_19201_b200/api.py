@@ -83,6 +83,7 @@ def lib():
             "dream_debug_read": [vp, i32, i32, i32, i32, vp],
             "dream_seq_reset": [vp, i32],
             "dream_debug_gemm": [vp, vp, vp, i32, i32, i32, i32, vp],
+            "dream_debug_topk": [vp, vp, i32, i32, vp, vp, vp],
             "dream_debug_wait": [vp, i32, vp],
             "dream_gemm_counts": [vp, C.POINTER(C.c_int64), C.POINTER(C.c_int64)],
             "dream_gemm_timing": [vp, i32, C.POINTER(C.c_int64), C.POINTER(C.c_double), C.POINTER(C.c_double)],
@@ -303,9 +304,12 @@ class Context:
     def dream_debug_gemm(self, W, X, split=1):
         rows, K = X.shape
         N = W.shape[0]
-        out = torch.empty(rows, N, dtype=torch.float32, device=self.device)
+        out = torch.empty(rows, N // 2 if split == 2 else N, dtype=torch.float32, device=self.device)
         _check(self.h, lib().dream_debug_gemm(self.h, _ptr(W), _ptr(X), rows, N, K, split, _ptr(out)))
         return out
+
+    def dream_debug_topk(self, logits, ktop, top_val, top_id, lse):
+        _check(self.h, lib().dream_debug_topk(self.h, _ptr(logits), logits.shape[0], ktop, _ptr(top_val), _ptr(top_id), _ptr(lse)))
 
     def dream_debug_wait(self, limit_ms, seconds):
         _check(self.h, lib().dream_debug_wait(self.h, limit_ms, _ptr(seconds)))

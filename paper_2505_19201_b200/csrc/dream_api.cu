@@ -36,7 +36,7 @@ struct dream_ctx {
   dream_config cfg;
   cudaStream_t stream;
   TreeShape ts;
-  int T, esz, qkvN, Hhd, kvN, n_cand, tap_lo_eff, cap_rows, pps, n_pages, RM, XR, PR, gemm_rows_lm;
+  int T, esz, qkvN, Hhd, kvN, n_cand, tap_lo_eff, cap_rows, pps, n_pages, RM, XR, PR;
   int use_tc, use_pdl, gemm_failed;
   cudaError_t launch_err;              // first refused kernel launch of the call being enqueued
   const char *launch_err_name;
@@ -360,8 +360,6 @@ static size_t carve(dream_ctx *c, char *base) {
   c->xn = a.take_bytes((size_t)planes * c->PR * d * e);
   c->raw = a.take_bytes((size_t)planes * c->PR * d * e);
   c->act = a.take_bytes((size_t)planes * c->PR * f.d_ff * e);
-  int lm_rows = ((imax(MB * T, MB * imax(c->ts.D + 2, f.tree_beam)) + 15) / 16) * 16;
-  c->gemm_rows_lm = lm_rows;
   // GEMM output: the widest of every projection's footprint.  fp32: rows x N.  bf16: room for the
   // stream-K partial-sum slots (bound for <= 192 SMs).
   {
@@ -922,22 +920,26 @@ static void norm_rows(dream_ctx *c, float *x, const GemmOut &gin, bool has_in, c
   launch_cluster(c, "k_resid", kernel, n, dim3(n, rows), dim3(many ? 256 : 512), 0, x, gin, has_in ? 1 : 0, (const T *)gain, c->cfg.rms_eps, d,
                  (T *)c->xn, copy, row_seq, tap, layer, want_raw ? (T *)c->raw : (T *)nullptr, xlay(m, d));
 }
+// act = silu(gate) * up of `rows` normalised rows in c->xn: wgu holds ff gate rows, then ff up rows, of d columns.
 template <typename T>
-static GemmOut mlp_rows(dream_ctx *c, const void *wgu, const void *wd, int rows, XMode m) {
-  const dream_config &f = c->cfg;
+static void gate_rows(dream_ctx *c, const void *wgu, int ff, int d, int rows, XMode m) {
   if constexpr (sizeof(T) == 2) {
     if (rows > TC_TOKENS) {                    // a prompt: the GEMM's epilogue gates, the row kernel does the rest
       TcEpi e = {};
-      e.dst = (bf16 *)c->act; e.lay = xlay(m, f.d_ff); e.ff = f.d_ff;
-      const GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model, TC_EPI_SILU, &e);
+      e.dst = (bf16 *)c->act; e.lay = xlay(m, ff); e.ff = ff;
+      const GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * ff, d, TC_EPI_SILU, &e);
       const int i0 = g.n_full / g.n_tt * 128;
-      if (i0 < f.d_ff) LAUNCH(c, (k_silu_mul<T, true>), dim3((f.d_ff - i0 + 1023) / 1024, rows), 256, 0, g, (T *)c->act, f.d_ff, i0, xlay(m, f.d_ff));
-      return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
+      if (i0 < ff) LAUNCH(c, (k_silu_mul<T, true>), dim3((ff - i0 + 1023) / 1024, rows), 256, 0, g, (T *)c->act, ff, i0, xlay(m, ff));
+      return;
     }
   }
-  GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * f.d_ff, f.d_model);
-  LAUNCH(c, (k_silu_mul<T, false>), dim3((f.d_ff + 1023) / 1024, rows), 256, 0, g, (T *)c->act, f.d_ff, 0, xlay(m, f.d_ff));
-  return gemm<T>(c, wd, c->act, m, rows, f.d_model, f.d_ff);
+  GemmOut g = gemm<T>(c, wgu, c->xn, m, rows, 2 * ff, d);
+  LAUNCH(c, (k_silu_mul<T, false>), dim3((ff + 1023) / 1024, rows), 256, 0, g, (T *)c->act, ff, 0, xlay(m, ff));
+}
+template <typename T>
+static GemmOut mlp_rows(dream_ctx *c, const void *wgu, const void *wd, int rows, XMode m) {
+  gate_rows<T>(c, wgu, c->cfg.d_ff, c->cfg.d_model, rows, m);
+  return gemm<T>(c, wd, c->act, m, rows, c->cfg.d_model, c->cfg.d_ff);
 }
 
 // ------------------------------------------------------------------------------------- prefill
@@ -1165,7 +1167,7 @@ extern "C" dream_status dream_compress_visual(dream_ctx *c, int32_t seq, int32_t
 
 // ------------------------------------------------------------------------------------- batch helpers
 
-static dream_status make_batch(dream_ctx *c, const int *seqs, int n_seqs, const dream_tree *trees, bool need_cum,
+static dream_status make_batch(dream_ctx *c, const int *seqs, int n_seqs, const dream_tree *trees,
                                TreeBatch *tb) {
   if (!c) return DREAM_E_ARG;
   if (!seqs || n_seqs < 1 || n_seqs > c->cfg.max_batch) return fail(c, DREAM_E_ARG, "n_seqs outside 1..max_batch");
@@ -1181,7 +1183,6 @@ static dream_status make_batch(dream_ctx *c, const int *seqs, int n_seqs, const 
       tb->t[b].tokens = t.tokens; tb->t[b].parent = t.parent; tb->t[b].depth = t.depth;
       tb->t[b].mask = t.mask; tb->t[b].cum = t.cum_logp;
     } else tb->t[b] = c->itree[seqs[b]];
-    (void)need_cum;
   }
   return DREAM_OK;
 }
@@ -1224,7 +1225,7 @@ static dream_status draft_impl(dream_ctx *c, const TreeBatch &tb, int B) {
 
 extern "C" dream_status dream_draft_tree(dream_ctx *c, const int32_t *seqs, int32_t n_seqs, const dream_tree *trees) {
   TreeBatch tb;
-  dream_status s = make_batch(c, seqs, n_seqs, trees, true, &tb);
+  dream_status s = make_batch(c, seqs, n_seqs, trees, &tb);
   if (s) return s;
   for (int b = 0; b < n_seqs; ++b)
     if (c->phase[seqs[b]] != PH_READY) return fail(c, DREAM_E_STATE, "sequence %d: dream_draft_tree follows dream_compress_visual or dream_accept", seqs[b]);
@@ -1272,7 +1273,7 @@ static dream_status verify_impl(dream_ctx *c, const TreeBatch &tb, int B, int *a
 extern "C" dream_status dream_verify_tree(dream_ctx *c, const int32_t *seqs, int32_t n_seqs, const dream_tree *trees,
                                           int32_t *node_argmax, float *node_margin, float *logits) {
   TreeBatch tb;
-  dream_status s = make_batch(c, seqs, n_seqs, trees, false, &tb);
+  dream_status s = make_batch(c, seqs, n_seqs, trees, &tb);
   if (s) return s;
   if (!node_argmax) return fail(c, DREAM_E_ARG, "node_argmax is required");
   refresh_bounds(c);
@@ -1326,7 +1327,7 @@ extern "C" dream_status dream_accept(dream_ctx *c, const int32_t *seqs, int32_t 
                                      const int32_t *node_argmax, int32_t *accept_len, int32_t *out_tokens,
                                      int32_t *comp_src) {
   TreeBatch tb;
-  dream_status s = make_batch(c, seqs, n_seqs, trees, false, &tb);
+  dream_status s = make_batch(c, seqs, n_seqs, trees, &tb);
   if (s) return s;
   if (!node_argmax || !accept_len || !out_tokens) return fail(c, DREAM_E_ARG, "node_argmax, accept_len, out_tokens are required");
   for (int b = 0; b < n_seqs; ++b)
@@ -1346,7 +1347,7 @@ extern "C" dream_status dream_accept_sample(dream_ctx *c, const int32_t *seqs, i
                                             const float *logits, float temperature, const float *uniforms,
                                             int32_t *accept_len, int32_t *out_tokens, int32_t *comp_src) {
   TreeBatch tb;
-  dream_status s = make_batch(c, seqs, n_seqs, trees, false, &tb);
+  dream_status s = make_batch(c, seqs, n_seqs, trees, &tb);
   if (s) return s;
   if (!logits || !uniforms || !accept_len || !out_tokens) return fail(c, DREAM_E_ARG, "logits, uniforms, accept_len, out_tokens are required");
   if (!(temperature > 0.f)) return fail(c, DREAM_E_ARG, "temperature must be above zero (dream_accept is the greedy form)");
@@ -1479,6 +1480,11 @@ __global__ void k_gemm_collect(GemmOut g, float *dst, int N) {
   if (c < N) dst[(long long)r * N + c] = gemm_val(g, r, c);
 }
 
+__global__ void k_join_rows(const bf16 *src, XLayout lay, float *dst, int n) {
+  kernel_entry(TR_k_copy_f32);
+  const bf16 *s = src + blockIdx.x * lay.row_stride;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[(long long)blockIdx.x * n + i] = to_f(s[i]) + to_f(s[lay.lo_delta + i]);
+}
 extern "C" dream_status dream_debug_gemm(dream_ctx *c, const void *W, const float *X, int32_t rows, int32_t N,
                                          int32_t K, int32_t split, float *out) {
   if (!c || !W || !X || !out) return fail(c, DREAM_E_ARG, "null argument");
@@ -1488,12 +1494,19 @@ extern "C" dream_status dream_debug_gemm(dream_ctx *c, const void *W, const floa
   if (K <= f.d_model) buf = c->xn;
   else if (K <= f.d_ff) buf = c->act;
   else return fail(c, DREAM_E_ARG, "K exceeds the context's widest GEMM input");
-  if (rows < 1 || rows > ROW_CHUNK) return fail(c, DREAM_E_ARG, "rows out of range");
+  if (rows < 1 || rows > c->PR) return fail(c, DREAM_E_ARG, "rows out of range");
   if (bf && (K % 64 || N % 8)) return fail(c, DREAM_E_ARG, "K must be a multiple of 64 and N of 8");
   XMode xm = xmode(c);
   if (bf && !split) {                     // single bf16 row per token
     if (rows > 128) return fail(c, DREAM_E_ARG, "unsplit inputs take at most 128 rows");
     xm = XMode{TC_X_PLAIN, 0};
+  }
+  if (split == 2) {                       // gated: W holds N / 2 gate rows, then as many up rows
+    if (!bf || buf != c->xn || N % 128 || N / 2 > f.d_ff) return fail(c, DREAM_E_ARG, "gated form: bf16, K <= d_model, N / 2 a multiple of 64 up to d_ff");
+    LAUNCH(c, k_split_rows, rows, 256, 0, X, buf, K, xlay(xm, K), 1);
+    gate_rows<bf16>(c, W, N / 2, K, rows, xm);
+    LAUNCH(c, k_join_rows, rows, 256, 0, (const bf16 *)c->act, xlay(xm, N / 2), out, N / 2);
+    return call_done(c);
   }
   LAUNCH(c, k_split_rows, rows, 256, 0, X, buf, K, xlay(xm, K), bf ? 1 : 0);
   GemmOut g = bf ? gemm<bf16>(c, W, buf, xm, rows, N, K) : gemm<float>(c, W, buf, xm, rows, N, K);
@@ -1501,6 +1514,20 @@ extern "C" dream_status dream_debug_gemm(dream_ctx *c, const void *W, const floa
   CUDA_OK(c, cudaGetLastError());
   if (c->gemm_failed) { c->gemm_failed = 0; return fail(c, DREAM_E_UNSUPPORTED, "the GEMM launch was refused (shape or output room)"); }
   return DREAM_OK;
+}
+
+// Top-k and log-sum-exp through the context's own choice of blocks (test hook).
+extern "C" dream_status dream_debug_topk(dream_ctx *c, const float *logits, int32_t rows, int32_t ktop, float *top_val, int32_t *top_id, float *lse) {
+  if (!c || !logits || !top_val || !top_id || !lse) return fail(c, DREAM_E_ARG, "null argument");
+  const int V = c->cfg.vocab;
+  if (rows < 1 || rows > ROW_CHUNK || ktop < 1 || ktop > imin(TOPK_MAX, V) || (V + TOPK_COLS - 1) / TOPK_COLS * ktop > 1024) return fail(c, DREAM_E_ARG, "rows or ktop out of range");
+  GemmOut g = NO_GEMM;                         // a plain [rows][vocab] matrix
+  g.base = logits; g.ld = V;
+  TOPK_LAUNCH(c, rows, g, ktop, (float *)nullptr);
+  LAUNCH(c, k_copy_f32, (rows * ktop + 255) / 256, 256, 0, (const float *)c->top_val, top_val, rows * ktop);
+  LAUNCH(c, k_copy_f32, (rows * ktop + 255) / 256, 256, 0, (const float *)c->top_id, (float *)top_id, rows * ktop);
+  LAUNCH(c, k_copy_f32, 1, 256, 0, (const float *)c->lse_rows, lse, rows);
+  return call_done(c);
 }
 
 // ------------------------------------------------------------------------------------- top-k without an arena
