@@ -634,7 +634,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    __syncwarp();
   }
+  // Freeing is an act of the pair too: both have freed before either leaves.  (0.2 to 0.5 % of a round.)
+  cluster_sync_relaxed();
 }
 
 // ------------------------------------------------------------------------------------------ host side

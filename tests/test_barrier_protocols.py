@@ -258,11 +258,13 @@ def test_gemm_pair_without_closing_waits():
     assert any(gemm([25, 39], 5, 4, 1, 8, seed, closing=False) for seed in range(20))
 
 
-def test_pair_allocates_tmem_behind_the_barrier_that_shows_its_partner_running():
-    """tcgen05.alloc of a pair is an act of both CTAs; issued before the start barrier it hung once in some ten million launches."""
+def test_pair_holds_tmem_between_barriers_that_show_its_partner_running():
+    """tcgen05.alloc and .dealloc of a pair are acts of both CTAs; with the first issued before the start barrier (and the second with
+    nothing behind it) a launch hung once in some ten million."""
     import os
     src = open(os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2505_19201_b200", "csrc", "gemm_tc.cuh")).read()
     body = src[src.index("k_gemm_tc(const __grid_constant__"):]
     alloc, release, free = (body.index("tcgen05." + op + ".cta_group::2") for op in ("alloc", "relinquish_alloc_permit", "dealloc"))
     assert body.index("cluster_sync_all();") < alloc
-    assert alloc < release < body.index("cluster_sync_relaxed();") < free
+    closing = body.index("cluster_sync_relaxed();")
+    assert alloc < release < closing < free < body.index("cluster_sync_relaxed();", closing + 1)
