@@ -14,7 +14,7 @@
 //       - more tokens (TC_X_TWO): two MMAs per k-step, high then low, into the same columns;
 //   * the tensor core adds into its accumulator with truncation, about half a unit in the last place
 //     per MMA and always towards zero, so chains of MMAs into one accumulator are kept short: CONCAT deals
-//     its k-steps out to as many accumulators as fit, TWO changes the accumulator every TC_CHAIN panels
+//     its k-steps out to as many accumulators as fit, TWO changes the accumulator every few panels (TcParams::chain)
 //     and the epilogue warps carry the sums in registers;
 //   * two shared-memory rings fed by TMA (cp.async.bulk.tensor.2d, 128-byte swizzle, no multicast), wp
 //     panels of 64 k per stage: W (128 rows, 16 KB a panel) and X.  W gets all the room X leaves: it is
@@ -58,7 +58,6 @@
 #define TC_WPANEL (128 * TC_BK * 2)          // one CTA's half of a weight panel
 #define TC_MAX_STAGES 12
 #define TC_EVEN 4               // units a pair may walk further for a share that lies in one tile
-#define TC_CHAIN 8              // panels per accumulator in the two-MMA form (64 MMAs)
 
 // How the token rows lie in the X buffer.  PLAIN: one bf16 row per token.  PLANAR: high parts, then
 // the low parts lo_rows rows further on.
@@ -89,6 +88,7 @@ struct TcParams {
   int sk_units, upc;            // stream-K part: units = tiles x panels, units per pair
   float inv_kbu, inv_upc;       // reciprocals, for div_small
   int n_tt, tile_t, mma_n;      // token tiles, tokens per tile, N of an MMA
+  int chain;                    // TWO / TILES: panels per accumulator
   int n_sub;                    // CONCAT / ONE: accumulators the k-steps of a segment are dealt out to (1, 2 or 4)
   int n_tok;                    // real token rows
   int lo_rows;                  // row of the first low part in the X tensor map
@@ -445,7 +445,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       pdl_wait();
       if (!mbar_wait_warp(peer_tmem, 0, abort_flag)) gave_up = WAIT_gemm_peer;
       while (!gave_up && (k0 < k1 || walk.next(p, tile, k0, k1))) {
-        const int fill_end = FORM >= TC_X_TWO ? min(k1, k0 + TC_CHAIN) : k1;
+        const int fill_end = FORM >= TC_X_TWO ? min(k1, k0 + p.chain) : k1;
         const uint32_t buf = fill & 1u, use = fill >> 1;              // use: earlier fills of this accumulator
         ++fill;
         if (!mbar_wait_warp(acc_empty + buf, (use & 1u) ^ 1u, abort_flag)) { gave_up = WAIT_gemm_acc_empty; break; }
@@ -514,7 +514,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         float run[128];
 #pragma unroll
         for (int j = 0; j < 128; ++j) run[j] = 0.f;
-        for (; k0 < k1; k0 += TC_CHAIN) {
+        for (; k0 < k1; k0 += p.chain) {
           const uint32_t buf = fill & 1u;
           wait_full(buf, fill >> 1);
           ++fill;
@@ -782,6 +782,10 @@ static inline bool gemm_tc_launch(GemmTcPlan *pl, cudaStream_t stream, const voi
   if (x_mode == TC_X_PLAIN) { form = TC_X_ONE; p.tile_t = p.mma_n = (rows + 15) & ~15; }
   else if (rows <= 128) { form = TC_X_CONCAT; p.mma_n = 2 * p.tile_t; }
   else { form = p.n_tt > 1 ? TC_X_TILES : TC_X_TWO; p.mma_n = p.tile_t; }
+  // Every eight MMAs of a chain (a panel) add 1.7e-7 of bias to sums of one sign, and emptying an accumulator costs time: at most
+  // eight panels, fewer where K is small, so that no width is less exact than when 148 CTAs shared the panels.  K 2048, 200
+  // rows, relative L2 against float64: eight panels 2.68e-6, four 2.51e-6 (as before); four everywhere: prompts 3 % slower.
+  p.chain = p.KB / 8 < 4 ? 4 : p.KB / 8 > 8 ? 8 : p.KB / 8;
   p.n_sub = p.mma_n <= 64 ? 4 : p.mma_n <= 128 ? 2 : 1;
   p.out = out;
   const TcOut o = gemm_tc_out(t, rows, N);

@@ -89,3 +89,16 @@ def test_rotary_and_append(model, v, q):
                 assert bool(((got - want).abs() <= want.abs() * 2.0 ** -8 + err).all()), (model, r, what)      # the cache is bf16
     finally:
         c.close()
+
+
+# the tensor core truncates when it accumulates: a chain of n MMAs loses half an ulp of its running sum, on average half the
+# chain's, per MMA, n * 2^-25 of a sum of one sign; chains are KB / 8 panels of eight MMAs, four to eight
+@pytest.mark.parametrize("K", [512, 2048, 3840, 4096])
+@pytest.mark.parametrize("rows", [129, 256, 257, 1280])
+def test_bias_of_same_sign_sums(ctx, rows, K):
+    W, X = operands(rows, 2048, K)
+    W, X = W.abs(), X.abs()
+    out = ctx.dream_debug_gemm(W, X, 1)
+    ctx.dream_poll()
+    ref = X.double() @ W.double().t()
+    assert abs(float(((out.double() - ref) / ref).mean())) <= 8 * min(8, max(4, K // 64 // 8)) * 2.0 ** -25
