@@ -29,9 +29,9 @@ from paper_2505_19201_b200 import configs, synth  # noqa: E402
 
 # DRAM traffic of the dominant kernel over its weight bytes, from an ncu capture of the current k_gemm_tc
 # (dram__bytes_read.sum + dram__bytes_write.sum over the four projections of one verify layer; traffic grows in
-# proportion to the weight bytes, so a step's mean launch is scaled by this ratio).  Empty for workloads without a
+# proportion to the weight bytes, so a step's mean launch is scaled by this ratio).  Absent for workloads without a
 # capture, and to be emptied whenever the kernel changes.
-TRAFFIC_RATIO = {}
+TRAFFIC_RATIO = {"llava7b": (106.03 + 34.61 + 187.11 + 95.99) / (100.66 + 33.55 + 180.36 + 90.18)}
 
 METRIC = "verified_tree_tokens_per_s"
 UNIT = "tokens/s"

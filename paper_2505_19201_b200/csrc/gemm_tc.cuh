@@ -482,8 +482,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
         __syncwarp();
       }
       // as above for the second CTA's arrivals: both accumulators emptied (they are relaxed, and the barrier at the end
-      // does not wait for them; one that came late left a later launch waiting for good, once in some million).  The
-      // decode forms send only the arrivals that the loop above has waited for.
+      // does not wait for them).  The decode forms send only the arrivals that the loop above has waited for.
       for (uint32_t buf = 0; FORM >= TC_X_TWO && !gave_up && buf < 2u; ++buf)
         if (!mbar_wait_warp(acc_empty + buf, (((fill + 1u - buf) >> 1) & 1u) ^ 1u, abort_flag)) gave_up = WAIT_gemm_acc_last;
     }
