@@ -174,6 +174,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   const int chunk = blockIdx.x, slot = blockIdx.z;
   const int kvh = a.mode == AT_PREFILL ? blockIdx.y % a.hkv : blockIdx.y / a.n_rt, rt = a.mode == AT_PREFILL ? a.n_rt - 1 - blockIdx.y / a.hkv : blockIdx.y - kvh * a.n_rt;
   const int seq = a.slot_seq[slot];
+  unsigned long long *tr = trace_open();
   if (warp == 0) {      // a lane per ring stage: the set-up is a few instructions deep instead of a loop
     if (lane < STAGES) { mbar_init(k_full + lane, 1); mbar_init(k_empty + lane, 1); mbar_init(v_full + lane, 1); mbar_init(v_empty + lane, 1); }
     else if (lane >= 8 && lane < 8 + S_BUFS) { mbar_init(s_full + lane - 8, 1); mbar_init(s_free + lane - 8, 8); }
@@ -249,7 +250,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     }
     pdl_wait();
   }
-  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) trace_stamp(TR_k_attn_tc);
+  trace_stamp(tr, TR_k_attn_tc);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer

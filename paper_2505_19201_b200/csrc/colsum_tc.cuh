@@ -71,8 +71,9 @@ k_colsum_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_p;
   int gave_up = WAIT_none;                                  // the wait of this warp that ran out
+  unsigned long long *tr = trace_open();
   pdl_wait();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) trace_stamp(TR_k_colsum);
+  trace_stamp(tr, TR_k_colsum);
 
   const int n = a.n, cand = *a.tap - a.tap_lo, q_row0 = cand * a.q_rows, k_row0 = (*a.tap - 1) * a.kv_rows;
   const int j0 = a.key0 + tile * CS_KEYS;                   // first key of this tile; rows before it see none of its keys

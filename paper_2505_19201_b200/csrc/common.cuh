@@ -85,36 +85,48 @@ enum {
   TR_count
 };
 #define DREAM_TRACE_NAMES {"none", "k_embed", "k_build_prompt", "k_resid", "k_qkv_post_target", "k_qkv_post_draft", "k_gemm_to_q", "k_mem_append", "k_silu_mul", "k_gather_rows", "k_topk_lse", "k_attn_prefill", "k_entropy_mean", "k_colsum", "k_attn_tree", "k_attn_draft", "k_attn_tc", "k_attn_combine", "k_draft_begin", "k_tree_expand", "k_tree_finalize", "k_verify_setup", "k_accept", "k_compact_kv", "k_accept_rows", "k_select_tap", "k_select_visual", "k_ctx_rows", "k_gemm_simt", "k_iota_rows", "k_set_seq", "k_set_int", "k_set_pages", "k_first_token", "k_argmax_out", "k_copy_f32", "k_split_rows", "k_gemm_collect", "k_gemm_tc"}
-__device__ __forceinline__ void trace_stamp(int id) {
-  unsigned long long *tr = g_dream_trace;
-  if (tr) {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    unsigned long long i = atomicAdd(tr, 1ull);
-    if (i < tr[1]) { tr[2 + 2 * i] = (unsigned long long)id; tr[3 + 2 * i] = t; }
-  }
+// The buffer's address is asked for at a kernel's entry, by the one thread that will use it (trace_open), and looked at behind the grid
+// dependency.  Asked for behind the dependency, as it first was, every kernel began with a round trip to L2 or, behind a GEMM's weight
+// stream, to HBM, in the block that the others then waited for (SmolVLM-shaped round 2315 -> 2290 us, fp32 toy request 4900 -> 4856).
+__device__ __forceinline__ unsigned long long *trace_open(bool me) { return me ? g_dream_trace : nullptr; }
+__device__ __forceinline__ unsigned long long *trace_open() {
+  return trace_open(blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
+}
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+__device__ __forceinline__ void trace_stamp(unsigned long long *tr, int id, unsigned long long t) {
+  unsigned long long i = atomicAdd(tr, 1ull);
+  if (i < tr[1]) { tr[2 + 2 * i] = (unsigned long long)id; tr[3 + 2 * i] = t; }
+}
+__device__ __forceinline__ void trace_stamp(unsigned long long *tr, int id) {
+  if (tr) trace_stamp(tr, id, global_ns());
 }
 // Entry of every kernel of the library: let the successor start, wait for the predecessor.
 __device__ __forceinline__ void kernel_entry(int id) {
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   pdl_wait();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) trace_stamp(id);
+  trace_stamp(tr, id);
 }
 
 // A kernel whose code has left the instruction caches fetches it line by line, a few hundred nanoseconds each,
 // and the short kernels between two GEMMs are then mostly that.  So they run their body twice: a first time
 // with every load and store switched off, while they wait for their predecessor anyway, and then for real:
 //   pdl_trigger();
-//   for (int pass = warm_first(); pass < 2; ++pass) { const bool live = warm_pass(pass, id); ... }
+//   unsigned long long *tr = trace_open();
+//   for (int pass = warm_first(); pass < 2; ++pass) { const bool live = warm_pass(pass, tr, id); ... }
 // live is false the first time; the compiler does not know.  LLaVA-7B-shaped round 5.22 -> 5.07 ms, SmolVLM-shaped
 // 2.64 -> 2.56 ms.  A grid of many waves skips it: its later blocks find the code there, and would run it
 // twice for nothing (LLaVA-7B-shaped request 29.4 -> 30.0 ms).
 #define WARM_BLOCKS 740
 __device__ __forceinline__ int warm_first() { return gridDim.x * gridDim.y * gridDim.z <= WARM_BLOCKS ? 0 : 1; }
-__device__ __forceinline__ bool warm_pass(int pass, int id) {
+__device__ __forceinline__ bool warm_pass(int pass, unsigned long long *tr, int id) {
   if (pass) {
     pdl_wait();
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) trace_stamp(id);
+    trace_stamp(tr, id);
   }
   int live = pass;
   asm volatile("" : "+r"(live));

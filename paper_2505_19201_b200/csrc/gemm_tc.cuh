@@ -119,11 +119,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 #define WAIT_LIMIT_NS 1000000000ull
 #define WAIT_SUSPEND_NS 1000000u         // an attempt suspends the thread no longer than this
 #define WAIT_DRAIN_NS 1000000ull
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
 __device__ __forceinline__ bool mbar_try(uint32_t addr, uint32_t parity) {
   uint32_t done;
   asm volatile(
@@ -328,7 +323,8 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1;
-  if (blockIdx.x == 0 && threadIdx.x == 0) trace_stamp(TR_none);     // CTA start, before any dependency
+  unsigned long long *tr = trace_open(blockIdx.x == 0 && lane == 0 && (warp == 0 || warp == 2));
+  const unsigned long long t_start = global_ns();
   if (warp == 0) {      // a lane per barrier: the set-up is a few instructions deep instead of a loop
     if (lane < TC_MAX_STAGES) { mbar_init(full_w + lane, 1); mbar_init(empty_w + lane, 1); }
     else if (lane < 2 * TC_MAX_STAGES) mbar_init(full_x + lane - TC_MAX_STAGES, 1);
@@ -390,6 +386,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
       }
     }
     pdl_wait();
+    if (tr) trace_stamp(tr, TR_none, t_start);                    // CTA start, before any dependency
     // Until the last releases have arrived, which the pair's first CTA signals across: an arrival that comes in after this
     // CTA has left would land in the shared memory of the CTA that follows it on the SM.
     for (int i = 0; !gave_up && i < p.w_stages; ++i) {
@@ -404,7 +401,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
     __syncwarp();
     bool more = walk.next(p, tile, k0, k1);
     pdl_wait();
-    if (blockIdx.x == 0 && lane == 0) trace_stamp(TR_k_gemm_tc);
+    trace_stamp(tr, TR_k_gemm_tc);
     __syncwarp();
     const uint32_t bar0 = mapa(smem_u32(full_x), 0);
     const int y_off = FORM == TC_X_CONCAT ? (int)rank * p.lo_rows : (int)rank * (p.mma_n >> 1);   // first token row this CTA stages, from the tile's

@@ -65,6 +65,7 @@ k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps
         const int *tap_state, int layer, T *raw, XLayout lay) {
   __shared__ float warp_ss[TH / 32], block_ss[2];
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   const int r = blockIdx.y, i0 = (blockIdx.x * NV * TH + threadIdx.x) * 4, n = gridDim.x;
   // the gains are weights: they can be fetched before the predecessor has finished
   float4 g[NV];
@@ -73,7 +74,7 @@ k_resid(float *x, GemmOut gin, int has_in, const T *__restrict__ gain, float eps
   float *xr = x + (long long)r * d;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool live = warm_pass(pass, TR_k_resid);
+    const bool live = warm_pass(pass, tr, TR_k_resid);
     float4 v[NV];
     float ss = 0.f;
 #pragma unroll
@@ -170,13 +171,14 @@ __global__ void __launch_bounds__(256, 5)
 k_qkv_post_target(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__ row_slot,
                   int row0, int hh0, void *qbuf, PagedKV kv, int H, const float2 *__restrict__ rope_tab) {
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   const int r = blockIdx.x + row0, lr = blockIdx.x;
   const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv;     // hd / 8 items per head
   const int w = blockIdx.y * 256 + threadIdx.x, hw = w >> q4_log2, hh = hh0 + hw, i = (w - (hw << q4_log2)) * 4;
   const int ca = PAIRED ? paired_col(hh * hd >> 8, ((hh * hd & 255) >> 1) + i) : hh * hd + i, cb = ca + (PAIRED ? 16 : half);
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool live = warm_pass(pass, TR_k_qkv_post_target);
+    const bool live = warm_pass(pass, tr, TR_k_qkv_post_target);
     bool on = live && hh < H + 2 * Hkv;
     if (PAIRED) on = on && gemm_tile(g, lr, ca) >= g.n_full;
     const int seq = on ? row_seq[r] : 0, slot = on ? row_slot[r] : 0;
@@ -220,12 +222,13 @@ __global__ void __launch_bounds__(256, 5)
 k_qkv_post_draft(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__ row_pos, const int *__restrict__ row_dst,
                  int has_q, void *qbuf, FlatKV kv, int H, const float2 *__restrict__ rope_tab, int by_pos) {
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   const int r = blockIdx.x;
   const int hd = kv.hd, half = hd >> 1, q4_log2 = 28 - __clz(hd), Hkv = kv.hkv, Hq = has_q ? H : 0;
   const int w = blockIdx.y * 256 + threadIdx.x, hh = w >> q4_log2, i = (w - (hh << q4_log2)) * 4;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool live = warm_pass(pass, TR_k_qkv_post_draft);
+    const bool live = warm_pass(pass, tr, TR_k_qkv_post_draft);
     bool on = live && hh < Hq + 2 * Hkv;
     const int dst = on ? row_dst[r] : 0, seq = on ? row_seq[r] : 0, tab_row = on && by_pos ? row_pos[r] : r;
     if (hh >= Hq && dst < 0) on = false;
@@ -251,10 +254,11 @@ k_qkv_post_draft(GemmOut g, const int *__restrict__ row_seq, const int *__restri
 __global__ void __launch_bounds__(256)
 k_gemm_to_q(GemmOut g, void *qbuf, int H, int hd, int split) {
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   const int r = blockIdx.x, i = (blockIdx.y * 256 + threadIdx.x) * 4, hd_log2 = 31 - __clz(hd), h = i >> hd_log2;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool live = warm_pass(pass, TR_k_gemm_to_q), on = live && h < H;
+    const bool live = warm_pass(pass, tr, TR_k_gemm_to_q), on = live && h < H;
     float4 v = gemm_val4<6>(g, r, i, on);
     if (on) q_store4(qbuf, split, (long long)r * H + h, hd, i - (h << hd_log2), v);
   }
@@ -268,10 +272,11 @@ __global__ void __launch_bounds__(256)
 k_mem_append(GemmOut g, const int *__restrict__ row_seq, const int *__restrict__ row_dst, const int *__restrict__ row_in,
              const int *__restrict__ nperm, FlatKV kv) {
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   const int r = blockIdx.x, i = (blockIdx.y * 256 + threadIdx.x) * 4, hd_log2 = 31 - __clz(kv.hd), hh = i >> hd_log2;
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    bool on = warm_pass(pass, TR_k_mem_append) && hh < 2 * kv.hkv;
+    bool on = warm_pass(pass, tr, TR_k_mem_append) && hh < 2 * kv.hkv;
     const int seq = on ? row_seq[r] : 0;
     int dst = on ? (nperm ? row_in : row_dst)[r] : 0;
     if (dst < 0) on = false;
@@ -288,11 +293,12 @@ template <typename T, bool PAIRED>
 __global__ void __launch_bounds__(256, 8)
 k_silu_mul(GemmOut g, T *act, int ff, int i0, XLayout lay) {
   pdl_trigger();
+  unsigned long long *tr = trace_open();
   const int r = blockIdx.y, i = i0 + (blockIdx.x * 256 + threadIdx.x) * 4;
   const int ca = PAIRED ? paired_col(i >> 7, i & 127) : i, cb = ca + (PAIRED ? 16 : ff);
 #pragma unroll 1
   for (int pass = warm_first(); pass < 2; ++pass) {
-    const bool live = warm_pass(pass, TR_k_silu_mul), on = live && i < ff && (!PAIRED || gemm_tile(g, r, ca) >= g.n_full);
+    const bool live = warm_pass(pass, tr, TR_k_silu_mul), on = live && i < ff && (!PAIRED || gemm_tile(g, r, ca) >= g.n_full);
     float4 a = gemm_val4<2>(g, r, ca, on), b = gemm_val4<2>(g, r, cb, on);
     const float4 o = make_float4(a.x / (1.f + __expf(-a.x)) * b.x, a.y / (1.f + __expf(-a.y)) * b.y,
                                  a.z / (1.f + __expf(-a.z)) * b.z, a.w / (1.f + __expf(-a.w)) * b.w);
