@@ -4,29 +4,32 @@
 //
 // A CTA owns one tile of 64 query entries (entry = (row, query head of one KV-head group)), one KV
 // head and one chunk of keys.  Queries carry ~16 mantissa bits as a high and a low bf16 row, so
-// the tile is the MMA's M = 128: row 2e = high part of entry e, row 2e + 1 = its low part; the two
-// accumulator lanes of an entry are added with one shuffle.  Keys are walked in blocks of 64:
+// the tile is the MMA's M = 128: eight entries' high parts, then their low parts, then the next eight entries.  A warp reads its
+// accumulators as 16 lanes x 8 columns fragments (tcgen05.ld.16x256b), in which lanes i and i + 8 come to the same thread: the two
+// products of an entry are added without a shuffle.  (High and low part in neighbouring lanes, two shuffles and four selects per pair of
+// keys, was half of the softmax's instructions.)  Keys are walked in blocks of 64:
 //   S_b = Q K_b^T        tcgen05.mma 128 x 64 x 16 over head_dim, A = Q and B = K_b from shared memory
-//                        (K-major, 128-byte swizzle, TMA-fed), fp32 accumulators in a TMEM ring, up to
-//                        AHEAD blocks ahead of the softmax;
-//   softmax              eight warps, one TMEM lane per thread: two warps share a lane quarter and take 32 of
-//                        the block's keys each, the two lanes of an entry 16 each.  One pass: the block's row
-//                        maximum (the two warps exchange theirs through shared memory), then
-//                        P = 2^(s - m), its row sum, and P's high bf16 part to the entry's even row and its low
-//                        part to the odd row of a shared-memory tile in the operand layout.  m is any reference
-//                        near the maximum: it follows the maximum only when that has outgrown it by 2^8, so
+//                        (K-major, 128-byte swizzle, TMA-fed), fp32 accumulators in a TMEM ring, as far
+//                        ahead of the softmax as the rings allow;
+//   softmax              eight warps, each eight entries: the four lanes of a quad take 16 of the block's keys each for one entry, so
+//                        a row's maximum and sums are two shuffles and nothing is exchanged between warps.  One pass: the block's row
+//                        maximum, then P = 2^(s - m), its row sum, and P's high and low bf16 parts to the entry's two rows
+//                        of a shared-memory tile in the operand layout; adds and multiply-adds take two values per instruction.  m is any
+//                        reference near the maximum: it follows the maximum only when that has outgrown it by 2^8, so
 //                        the O accumulator is hardly ever rescaled (in TMEM, tcgen05.ld / tcgen05.st);
 //   O += P_b V_b         tcgen05.mma 128 x head_dim x 16 steps over the block's keys, A = P_b (K-major)
 //                        and B = V_b as stored ([key][head_dim]: an MN-major operand).
 // K/V blocks arrive through two TMA rings; during verification the blocks below the verified prefix
-// length are requested before the grid dependency resolves.  Flat draft caches carry a low plane
-// per key, which costs one more MMA per step.  The chunks of one tile are a thread-block cluster: each leaves
+// are requested before the grid dependency resolves.  Each CTA of a split tile keeps
 // its (m, l, O) in its shared memory, and after a cluster barrier every CTA merges a share of the rows, reading
 // the others' through distributed shared memory (a merge kernel behind partials in global memory costs 4 us more
 // per launch, most of it the kernel boundary; it stays for tiles whose many chunks no cluster holds).  The
-// prefill has one chunk and also leaves each row's log-sum-exp and entropy.  Warp roles: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..9 =
-// softmax and epilogue.  What bounds it is the softmax's instruction latency: with four warps (one per
-// scheduler) and two passes over S a block of 64 keys took 2.0 us of a LLaVA-7B-shaped verify launch.
+// prefill has one chunk and also leaves each row's log-sum-exp and entropy.  Warp roles: 0 = TMA producer, 1 = S issuer and TMEM owner,
+// 2..9 = softmax and epilogue, 10 = O issuer.  One warp issuing both products spent 2.1k cycles per block at head_dim 256, 1.3k of them the
+// matrix instructions' own time and the rest its waits in turn for P, V, K and a free S; of the 2.3k cycles of a block the softmax waited 0.9k.
+// Prompt attention per layer, before -> now: 832 rows, 32 heads of 128 60 -> 34 us (two CTAs per SM: half of a CTA's 25k cycles is start,
+// first fetch and end), 1152 rows, 32 heads of 64 47 -> 42, 4352 rows, 16 heads of 256 on 8 KV heads 509 -> 415; what bounds
+// the last is the MMA of N = 64, whose A operand's shared-memory reads take half again its own time.
 // The loops are kept compact on purpose: this kernel's code is
 // fetched anew at almost every launch (the weight stream between two launches pushes it out of the
 // caches), and straight-line code then costs its own fetch (a fully unrolled version of the same
@@ -41,7 +44,7 @@
 #include "gemm_tc.cuh"
 #include "rows.cuh"
 
-#define AT_THREADS 320
+#define AT_THREADS 352
 #define AT_RESCALE 8.f                 // the maximum may outgrow its reference by this power of two
 #define AT_KBLK 64
 #define AT_QTILE (128 * 64 * 2)        // one 64-column panel of the query tile (128 rows)
@@ -63,22 +66,23 @@ __device__ __forceinline__ void split_pair(float x, float y, uint32_t &hi, uint3
 }
 
 // Ring depths: what shared memory (K and V blocks stay until their MMAs ran) and the TMEM columns
-// (head_dim for O, 64 per S_b) hold.
-template <int HD, bool FLAT> struct AtShape {
+// (head_dim for O, 64 per S_b) hold.  PF: the prefill's form.
+template <int HD, bool FLAT, bool PF = false> struct AtShape {
   static constexpr int PLANES = FLAT ? 2 : 1;
-  // head_dim 64 over the paged cache takes three blocks, so that O and S fit 256 TMEM columns and two
-  // CTAs share an SM (98 KB of shared memory each): twice the key chunks in flight per layer
-  static constexpr int STAGES = HD == 64 ? (FLAT ? 4 : 3) : (HD == 128 ? (FLAT ? 2 : 5) : (FLAT ? 1 : 2));   // K (and V) blocks
-  static constexpr int S_BUFS = HD == 64 ? 3 : 4;                    // S blocks in TMEM
-  // S blocks issued before the first O: with more than STAGES the K ring would wait for V blocks to be freed, which wait for O
-  static constexpr int AHEAD = S_BUFS < STAGES ? S_BUFS : STAGES;
+  // head_dim 64 over the paged cache, and a prompt's head_dim 128, take fewer blocks, so that O and S fit 256 TMEM columns and two
+  // CTAs (98 and 113 KB of shared memory each) share an SM: twice the key chunks in flight per layer; in a prompt, one walks its keys while the
+  // other starts or ends
+  static constexpr bool SMALL = PF && HD == 128;
+  static constexpr int STAGES = SMALL ? 2 : HD == 64 ? (FLAT ? 4 : 3) : (HD == 128 ? (FLAT ? 2 : 5) : (FLAT ? 1 : 2));   // K (and V) blocks
+  static constexpr int S_BUFS = SMALL ? 2 : HD == 64 ? 3 : 4;        // S blocks in TMEM
+  static constexpr int P_BUFS = SMALL ? 1 : 2;                       // blocks of probabilities
   static constexpr int TMEM_COLS = HD + S_BUFS * 64 <= 256 ? 256 : 512;
-  static constexpr int CTAS_PER_SM = HD == 64 && !FLAT ? 2 : 1;
+  static constexpr int CTAS_PER_SM = (HD == 64 && !FLAT) || SMALL ? 2 : 1;
   static constexpr int KP = HD / 64;                                 // 64-column panels per row
   static constexpr int KV_STAGE = PLANES * KP * AT_KVTILE;           // one block of K (or of V)
   static constexpr int Q_BYTES = KP * AT_QTILE;
-  static constexpr int O_LD = HD + 4;                                // floats per row of the merge's O tile (over the K/V rings)
-  static constexpr size_t SMEM = 1024 + Q_BYTES + 2 * STAGES * KV_STAGE + 2 * AT_PTILE + 1024 + 384;
+  static constexpr int O_LD = HD + 8;                                // floats per row of the merge's O tile (over the K/V rings)
+  static constexpr size_t SMEM = (SMALL ? 0 : 1024) + Q_BYTES + 2 * STAGES * KV_STAGE + P_BUFS * AT_PTILE + 384;
 };
 
 struct AttnTcArgs {
@@ -118,9 +122,26 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, u
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
       ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w), "l"(policy) : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tma_load_5d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z, int w, int v, uint64_t policy) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(v), "l"(policy) : "memory");
+}
+// 16 TMEM lanes x 64 columns, as the accumulator fragment of a warp-level MMA: lane 4 i + j of the warp gets columns 8 c + 2 j and 8 c + 2 j + 1
+// of TMEM lane i in r[4 c] and r[4 c + 1], of TMEM lane i + 8 in r[4 c + 2] and r[4 c + 3].
+__device__ __forceinline__ void tmem_ld16x64(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st16x64(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
       "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
         "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
@@ -150,35 +171,62 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ void bar_sync_pair(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+// Two single-precision operations in one instruction, each rounded as the single one.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 c;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;\n}"
+      : "=f"(c.x), "=f"(c.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return c;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 d) {
+  float2 c;
+  asm("{\n .reg .b64 x, y, w, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 w, {%6, %7};\n fma.rn.f32x2 z, x, y, w;\n mov.b64 {%0, %1}, z;\n}"
+      : "=f"(c.x), "=f"(c.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(d.x), "f"(d.y));
+  return c;
+}
+// w[i] of the four lanes of a quad: lane j ends up with the quad's words j, in lane order.
+__device__ __forceinline__ void quad_transpose(uint32_t (&w)[4], int lane) {
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (!(j & o)) {
+        const bool up = (lane & o) != 0;
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? w[j] : w[j | o], o);
+        if (up) w[j] = got; else w[j | o] = got;
+      }
+}
 
-template <int HD, bool FLAT>
-__global__ void __launch_bounds__(AT_THREADS, (AtShape<HD, FLAT>::CTAS_PER_SM))
+template <int HD, bool FLAT, bool PF>
+__global__ void __launch_bounds__(AT_THREADS, (AtShape<HD, FLAT, PF>::CTAS_PER_SM))
 k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
           const __grid_constant__ AttnTcArgs a) {
-  using Sh = AtShape<HD, FLAT>;
-  constexpr int STAGES = Sh::STAGES, S_BUFS = Sh::S_BUFS, AHEAD = Sh::AHEAD, KP = Sh::KP, PLANES = Sh::PLANES;
-  extern __shared__ uint8_t at_smem_raw[];
+  using Sh = AtShape<HD, FLAT, PF>;
+  constexpr int STAGES = Sh::STAGES, S_BUFS = Sh::S_BUFS, P_BUFS = Sh::P_BUFS, KP = Sh::KP, PLANES = Sh::PLANES;
+  extern __shared__ __align__(1024) uint8_t at_smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)at_smem_raw + 1023) & ~(uintptr_t)1023);
+  if (Sh::SMALL && smem != at_smem_raw) {                   // no room to align by hand: two CTAs fill an SM's shared memory
+    if (threadIdx.x == 0) atomicMax(a.status, DREAM_DEV_TIMEOUT);
+    return;
+  }
   uint8_t *q_s = smem, *k_s = q_s + Sh::Q_BYTES, *v_s = k_s + STAGES * Sh::KV_STAGE, *p_s = v_s + STAGES * Sh::KV_STAGE;
   float *o_s = (float *)k_s, *ml_s = o_s + 64 * Sh::O_LD;     // merge: O of the 64 entries, then (m, l, u, -) of each
-  float *mx_s = (float *)(p_s + 2 * AT_PTILE);                // [2 buffers][2 halves][64 entries]: exchange between the two warps of a quarter
-  uint64_t *bars = (uint64_t *)(mx_s + 256);
+  uint64_t *bars = (uint64_t *)(p_s + P_BUFS * AT_PTILE);
   uint64_t *q_full = bars, *k_full = q_full + 1, *k_empty = k_full + STAGES, *v_full = k_empty + STAGES, *v_empty = v_full + STAGES;
-  uint64_t *s_full = v_empty + STAGES, *s_free = s_full + S_BUFS, *p_full = s_free + S_BUFS, *p_empty = p_full + 2;
-  uint32_t *tmem_base_p = (uint32_t *)(p_empty + 2);
+  uint64_t *s_full = v_empty + STAGES, *s_free = s_full + S_BUFS, *p_full = s_free + S_BUFS, *p_empty = p_full + P_BUFS;
+  uint32_t *tmem_base_p = (uint32_t *)(p_empty + P_BUFS);
   volatile int *abort_flag = (volatile int *)(tmem_base_p + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   // (prefill: the tiles with the most keys first, so that the last wave is short)
   const int chunk = blockIdx.x, slot = blockIdx.z;
-  const int kvh = a.mode == AT_PREFILL ? blockIdx.y % a.hkv : blockIdx.y / a.n_rt, rt = a.mode == AT_PREFILL ? a.n_rt - 1 - blockIdx.y / a.hkv : blockIdx.y - kvh * a.n_rt;
+  const int kvh = PF ? blockIdx.y % a.hkv : blockIdx.y / a.n_rt, rt = PF ? a.n_rt - 1 - blockIdx.y / a.hkv : blockIdx.y - kvh * a.n_rt;
   const int seq = a.slot_seq[slot];
   unsigned long long *tr = trace_open();
   if (warp == 0) {      // a lane per ring stage: the set-up is a few instructions deep instead of a loop
     if (lane < STAGES) { mbar_init(k_full + lane, 1); mbar_init(k_empty + lane, 1); mbar_init(v_full + lane, 1); mbar_init(v_empty + lane, 1); }
     else if (lane >= 8 && lane < 8 + S_BUFS) { mbar_init(s_full + lane - 8, 1); mbar_init(s_free + lane - 8, 8); }
-    else if (lane >= 16 && lane < 18) { mbar_init(p_full + lane - 16, 8); mbar_init(p_empty + lane - 16, 1); }
+    else if (lane >= 16 && lane < 16 + P_BUFS) { mbar_init(p_full + lane - 16, 8); mbar_init(p_empty + lane - 16, 1); }
     else if (lane == 24) { mbar_init(q_full, 1); *abort_flag = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -201,7 +249,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   const int rows_total = a.rows_per_seq * a.G;              // entries of this sequence slot
   const int e_base = rt * 64;                               // first entry of the tile
   int total_keys, P = 0;
-  if (a.mode == AT_PREFILL) {
+  if (PF) {
     // causal: nothing beyond the tile's last row is visible to any of its rows
     int last_node = min(rows_total - 1, e_base + 63) / a.G;
     total_keys = min(a.n_keys, last_node + 1);
@@ -258,11 +306,11 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       const uint64_t pol_q = policy_evict_last();
       if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
       __syncwarp();
-      // queries: box (64 columns, high | low, G heads, 64 / G rows) -> row 2 e + part of the tile
-      const int node0 = slot * a.rows_per_seq + e_base / a.G;
+      // queries: boxes of 64 columns, whose rows come as the tile has them (see attn_q_map)
+      const int node0 = slot * a.rows_per_seq + e_base / a.G, c2 = a.G > 8 ? 0 : node0, c4 = a.G > 8 ? node0 : 0;
       if (elect_one()) {
         mbar_expect_tx(q_full, (uint32_t)Sh::Q_BYTES);
-        for (int kp = 0; kp < KP; ++kp) tma_load_4d(q_s + kp * AT_QTILE, &map_q, q_full, kp * 64, 0, kvh * a.G, node0, pol_q);
+        for (int kp = 0; kp < KP; ++kp) tma_load_5d(q_s + kp * AT_QTILE, &map_q, q_full, kp * 64, kvh * a.G, c2, 0, c4, pol_q);
       }
       __syncwarp();
       // K runs one block ahead of V: its stage is free as soon as S was computed, V's only after O
@@ -289,76 +337,81 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         if (++vs == STAGES) { vs = 0; vph ^= 1u; }
       }
       // (parity of the last phase of a barrier used n times: n - 1; never used: 1)
-      for (int b = 0; b < 2 && !gave_up; ++b)
-        if (!mbar_wait_warp(p_empty + b, (uint32_t)(((n_blk + 1 - b) >> 1) + 1) & 1u, abort_flag)) gave_up = WAIT_attn_last;
+      for (int b = 0; b < P_BUFS && !gave_up; ++b)
+        if (!mbar_wait_warp(p_empty + b, (uint32_t)((n_blk + P_BUFS - 1 - b) / P_BUFS + 1) & 1u, abort_flag)) gave_up = WAIT_attn_last;
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer: the whole warp, an elected
-    // lane for the tcgen05 instructions (as in the GEMM)
+    // ------------------------------------------------------------------ S issuer: the whole warp, an elected
+    // lane for the tcgen05 instructions (as in the GEMM).  fp32 accumulate, bf16 operands, M = 128, N = 64, both K-major
     if (n_blk > 0) {
-      // fp32 accumulate, bf16 operands, M = 128; S: N = 64, both K-major; O: N = head_dim, B MN-major
-      const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-      const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-      const uint32_t o_addr = tmem_base, s_addr0 = tmem_base + HD;
-      const uint64_t qd = smem_desc(smem_u32(q_s)), kd = smem_desc(smem_u32(k_s)), pd = smem_desc(smem_u32(p_s)), vd = smem_desc_mn(smem_u32(v_s), AT_KVTILE);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(64 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+      const uint32_t s_addr0 = tmem_base + HD;
+      const uint64_t qd = smem_desc(smem_u32(q_s)), kd = smem_desc(smem_u32(k_s));
       if (!mbar_wait_warp(q_full, 0, abort_flag)) gave_up = WAIT_attn_q;
-      int ks = 0, sb = 0, vs = 0;                            // ring positions of K, S and V
-      uint32_t kph = 0, sph = 1, vph = 0;
-      // step i issues S of block i and O of block i - AHEAD
+      int ks = 0, sb = 0;                                    // ring positions of K and S
+      uint32_t kph = 0, sph = 1;
 #pragma unroll 1
-      for (int i = 0; i < n_blk + AHEAD && !gave_up; ++i) {
-        const int it = i - AHEAD;
-        if (it >= 0) {
-          const int pb = it & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(p_full + pb, (uint32_t)(it >> 1) & 1u, abort_flag) && mbar_wait(v_full + vs, vph, abort_flag))) { gave_up = WAIT_attn_p_v; break; }
-          tc_fence_after();
-          const uint64_t ad = pd + (uint64_t)(pb * (AT_PTILE >> 4));
-          if (elect_one()) {
-#pragma unroll
-            for (int pl = 0; pl < PLANES; ++pl) {
-              const uint64_t bd = vd + (uint64_t)((vs * Sh::KV_STAGE + pl * KP * AT_KVTILE) >> 4);
-#pragma unroll
-              for (int k = 0; k < 4; ++k)                                 // 16 keys = two groups of 8 K-rows = 2048 bytes
-                mma_bf16(o_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc_o, (it > 0 || pl > 0 || k > 0) ? 1u : 0u);
-            }
-            mma_commit(p_empty + pb);
-            mma_commit(v_empty + vs);
-          }
-          __syncwarp();
-          if (++vs == STAGES) { vs = 0; vph ^= 1u; }
-        }
-        if (i < n_blk) {
-          if (!__all_sync(0xffffffffu, mbar_wait(k_full + ks, kph, abort_flag) && mbar_wait(s_free + sb, sph, abort_flag))) { gave_up = WAIT_attn_k_s; break; }
-          tc_fence_after();
-          if (elect_one()) {
+      for (int it = 0; it < n_blk && !gave_up; ++it) {
+        if (!__all_sync(0xffffffffu, mbar_wait(s_free + sb, sph, abort_flag) && mbar_wait(k_full + ks, kph, abort_flag))) { gave_up = WAIT_attn_k_s; break; }
+        tc_fence_after();
+        if (elect_one()) {
 #pragma unroll 1
-            for (int pp = 0; pp < PLANES * KP; ++pp) {
-              const uint64_t ad = qd + (uint64_t)((pp % KP) * (AT_QTILE >> 4)), bd = kd + (uint64_t)((ks * Sh::KV_STAGE + pp * AT_KVTILE) >> 4);
+          for (int pp = 0; pp < PLANES * KP; ++pp) {
+            const uint64_t ad = qd + (uint64_t)((pp % KP) * (AT_QTILE >> 4)), bd = kd + (uint64_t)((ks * Sh::KV_STAGE + pp * AT_KVTILE) >> 4);
 #pragma unroll
-              for (int k = 0; k < 4; ++k) mma_bf16(s_addr0 + (uint32_t)(sb * 64), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc_s, (pp > 0 || k > 0) ? 1u : 0u);
-            }
-            mma_commit(k_empty + ks);
-            mma_commit(s_full + sb);
+            for (int k = 0; k < 4; ++k) mma_bf16(s_addr0 + (uint32_t)(sb * 64), ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), idesc, (pp > 0 || k > 0) ? 1u : 0u);
           }
-          __syncwarp();
-          if (++ks == STAGES) { ks = 0; kph ^= 1u; }
-          if (++sb == S_BUFS) { sb = 0; sph ^= 1u; }
+          mma_commit(k_empty + ks);
+          mma_commit(s_full + sb);
         }
+        __syncwarp();
+        if (++ks == STAGES) { ks = 0; kph ^= 1u; }
+        if (++sb == S_BUFS) { sb = 0; sph ^= 1u; }
+      }
+    }
+  } else if (warp == 10) {
+    // ------------------------------------------------------------------ O issuer: N = head_dim, B MN-major
+    if (n_blk > 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(HD >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+      const uint32_t o_addr = tmem_base;
+      const uint64_t pd = smem_desc(smem_u32(p_s)), vd = smem_desc_mn(smem_u32(v_s), AT_KVTILE);
+      int vs = 0;
+      uint32_t vph = 0;
+#pragma unroll 1
+      for (int it = 0; it < n_blk; ++it) {
+        const int pb = it % P_BUFS;
+        if (!__all_sync(0xffffffffu, mbar_wait(v_full + vs, vph, abort_flag) && mbar_wait(p_full + pb, (uint32_t)(it / P_BUFS) & 1u, abort_flag))) { gave_up = WAIT_attn_p_v; break; }
+        tc_fence_after();
+        const uint64_t ad = pd + (uint64_t)(pb * (AT_PTILE >> 4));
+        if (elect_one()) {
+#pragma unroll
+          for (int pl = 0; pl < PLANES; ++pl) {
+            const uint64_t bd = vd + (uint64_t)((vs * Sh::KV_STAGE + pl * KP * AT_KVTILE) >> 4);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)                                 // 16 keys = two groups of 8 K-rows = 2048 bytes
+              mma_bf16(o_addr, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 128), idesc, (it > 0 || pl > 0 || k > 0) ? 1u : 0u);
+          }
+          mma_commit(p_empty + pb);
+          mma_commit(v_empty + vs);
+        }
+        __syncwarp();
+        if (++vs == STAGES) { vs = 0; vph ^= 1u; }
       }
     }
   } else {
-    // ------------------------------------------------------------------ softmax and epilogue: one row per thread,
-    // warps 2..5 and 6..9 each cover the 128 rows; `half` is the half of every block's keys this warp takes
-    const int q = warp & 3, half = warp >= 6 ? 1 : 0;          // TMEM lane quarter this warp may access
-    const int row = q * 32 + lane, e = e_base + (row >> 1), part = row & 1;
-    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    // ------------------------------------------------------------------ softmax and epilogue: warps 2..5 and 6..9 each take 16
+    // lanes of a quarter, that is eight entries; the four lanes of a quad share an entry
+    const int q = warp & 3, half = warp >= 6 ? 1 : 0;          // TMEM lane quarter this warp may access, its half of it
+    const int quad = lane >> 2, ql = lane & 3;
+    const int ei = q * 16 + half * 8 + quad, row = q * 32 + half * 16 + quad, e = e_base + ei;      // entry of the tile; its high parts' row (low parts: + 8)
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32 + half * 16) << 16);
     // what this row sees: keys below `vis_end`, plus tail key j (key index tail0 + j) for the bits of mw
     int r = -1, h = 0, vis_end = 0, tail0 = 0;
     uint32_t mw[4] = {0u, 0u, 0u, 0u};
     if (e < rows_total) {
       const int node = e / a.G;
       r = slot * a.rows_per_seq + node; h = kvh * a.G + (e - node * a.G);
-      if (a.mode == AT_PREFILL) vis_end = node + 1;
+      if (PF) vis_end = node + 1;
       else {
         vis_end = P; tail0 = P;
         if (a.mode == AT_VERIFY) {
@@ -380,25 +433,22 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
     // and the loops are kept small on purpose: the kernel's code is fetched anew at every launch
     // (the weight stream has pushed it out of L2 by then), so straight-line code costs its fetch.
     const float scale = a.scale_log2;
-    const int tail_len = a.mode == AT_PREFILL ? 0 : a.tail_len;
+    const int tail_len = PF ? 0 : a.tail_len;
     const unsigned long long mlo = (unsigned long long)mw[0] | ((unsigned long long)mw[1] << 32),
                              mhi = (unsigned long long)mw[2] | ((unsigned long long)mw[3] << 32);
-    // visibility of the 32 keys j32 .. j32 + 31 as a bit mask
-    auto vis32 = [=](int j32) -> uint32_t {
-      const int npre = min(32, max(0, vis_end - j32));
-      uint32_t m = npre >= 32 ? 0xffffffffu : (1u << npre) - 1u;
-      if (npre < 32 && tail_len > 0) {
-        const int sh = j32 - tail0;                            // tail key index of bit 0
-        unsigned long long t;
-        if (sh < 0) t = sh > -32 ? mlo << (-sh) : 0ull;
-        else if (sh < 64) t = (mlo >> sh) | (sh ? mhi << (64 - sh) : 0ull);
-        else t = sh < 128 ? mhi >> (sh - 64) : 0ull;
-        m |= (uint32_t)t;
+    // visibility of the 64 keys j0 .. j0 + 63 as a bit mask
+    auto vis64 = [=](int j0) -> unsigned long long {
+      const int npre = min(64, max(0, vis_end - j0));
+      unsigned long long m = npre >= 64 ? ~0ull : (1ull << npre) - 1ull;
+      if (npre < 64 && tail_len > 0) {
+        const int sh = j0 - tail0;                             // tail key index of bit 0
+        if (sh < 0) m |= sh > -64 ? mlo << (-sh) : 0ull;
+        else if (sh < 64) m |= (mlo >> sh) | (sh ? mhi << (64 - sh) : 0ull);
+        else m |= sh < 128 ? mhi >> (sh - 64) : 0ull;
       }
       return m;
     };
-    // A wait that runs out (or finds that another warp's did) clears ok.  The warp then walks on to the end, its waits
-    // skipped, because its partner meets it at a barrier in every block.
+    // A wait that runs out (or finds that another warp's did) clears ok.  The warp then walks on to the end, its waits skipped.
     bool ok = true;
     auto wait = [&](uint64_t *bar, uint32_t parity) {            // one lane polls for the warp
       int w = 1;
@@ -408,138 +458,150 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
         if (lane == 0) wait_expired(a.status, WAIT_attn_softmax, abort_flag, -1);
       }
     };
-    float m_ref = -INFINITY, l_run = 0.f, u_run = 0.f;       // exp2 domain; u = sum p (s - m) for the entropy
+    float m_ref = -INFINITY;                                   // exp2 domain
+    float2 l2 = make_float2(0.f, 0.f), u2 = l2;                // this lane's share of l = sum p and of u = sum p (s - m) for the entropy
     const bool want_ent = a.ent != nullptr || a.row_ent != nullptr;
+    const float2 scale2 = make_float2(scale, scale);
+    // where the lane's pairs of probabilities go: rows of 128 bytes, 16-byte pieces swizzled like the MMA expects a K-major operand
+    // (piece ^ (row & 7)); low parts eight rows further on
+    const uint32_t p_off = (uint32_t)(row * 128 + (quad << 4) + ql * 4);
     int sb = 0;
     uint32_t sph = 0;
 #pragma unroll 1
     for (int it = 0; it < n_blk; ++it) {
-      const int pb = it & 1;
+      const int pb = it % P_BUFS, j0 = (b0 + it) * AT_KBLK;
+      const bool all = __all_sync(0xffffffffu, vis_end >= j0 + AT_KBLK);
       wait(s_full + sb, sph);
       tc_fence_after();
       uint32_t sr[32];
-      tmem_ld32(lane_addr + (uint32_t)(HD + sb * 64 + half * 32), sr);
-      const uint32_t vm = vis32((b0 + it) * AT_KBLK + half * 32) >> (part * 16);
+      tmem_ld16x64(lane_addr + (uint32_t)(HD + sb * 64), sr);
       tmem_ld_wait();
       tc_fence_before();
       if (lane == 0) mbar_arrive(s_free + sb);
       if (++sb == S_BUFS) { sb = 0; sph ^= 1u; }
-      // lanes 2e and 2e+1 hold the products of entry e's high and low query parts: the even lane
-      // keeps keys 0..15 of the 32 and the odd lane 16..31, each sends the partner what it needs
-      float t[16], bm = -INFINITY;
+      // the products of the entry's high and low query parts; this lane's keys are 8 c + 2 ql and the next one
+      float2 t[8];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        const float send = __uint_as_float(part ? sr[c] : sr[16 + c]), mine = __uint_as_float(part ? sr[16 + c] : sr[c]);
-        t[c] = mine + __shfl_xor_sync(0xffffffffu, send, 1);
-        t[c] = ((vm >> c) & 1u) ? t[c] : -INFINITY;
-        bm = fmaxf(bm, t[c]);
+      for (int c = 0; c < 8; ++c)
+        t[c] = add2(make_float2(__uint_as_float(sr[4 * c]), __uint_as_float(sr[4 * c + 1])), make_float2(__uint_as_float(sr[4 * c + 2]), __uint_as_float(sr[4 * c + 3])));
+      if (!all) {
+        const unsigned long long vm = vis64(j0) >> (2 * ql);
+        const uint32_t v0 = (uint32_t)vm, v1 = (uint32_t)(vm >> 32);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const uint32_t v = c < 4 ? v0 >> (8 * c) : v1 >> (8 * c - 32);
+          t[c].x = v & 1u ? t[c].x : -INFINITY;
+          t[c].y = v & 2u ? t[c].y : -INFINITY;
+        }
       }
+      float bm = fmaxf(t[0].x, t[0].y), bn = fmaxf(t[1].x, t[1].y);
+#pragma unroll
+      for (int c = 2; c < 8; c += 2) { bm = fmaxf(bm, fmaxf(t[c].x, t[c].y)); bn = fmaxf(bn, fmaxf(t[c + 1].x, t[c + 1].y)); }
+      bm = fmaxf(bm, bn);
       bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
-      float *mx = mx_s + pb * 128;
-      mx[half * 64 + (row >> 1)] = bm;
-      bar_sync_pair(1 + q);
-      bm = fmaxf(bm, mx[(half ^ 1) * 64 + (row >> 1)]) * scale;     // the block's row maximum, the same in all four threads of the row
+      bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2)) * scale;        // the block's row maximum, the same in the four lanes of the quad
       const bool grow = bm > m_ref + AT_RESCALE && m_ref != -INFINITY;
       if (__any_sync(0xffffffffu, grow)) {
         // ---- the accumulator takes the new reference (behind the O of every earlier block)
-        wait(p_empty + (pb ^ 1), (uint32_t)((it - 1) >> 1) & 1u);
+        wait(p_empty + (it - 1) % P_BUFS, (uint32_t)((it - 1) / P_BUFS) & 1u);
         tc_fence_after();
         const float corr = grow ? ex2(m_ref - bm) : 1.f;
 #pragma unroll 1
-        for (int c0 = half * (HD / 2); c0 < (half + 1) * (HD / 2); c0 += 32) {
+        for (int c0 = 0; c0 < HD; c0 += 64) {
           uint32_t orr[32];
-          tmem_ld32(lane_addr + (uint32_t)c0, orr);
+          tmem_ld16x64(lane_addr + (uint32_t)c0, orr);
           tmem_ld_wait();
 #pragma unroll
           for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * corr);
-          tmem_st32(lane_addr + (uint32_t)c0, orr);
+          tmem_st16x64(lane_addr + (uint32_t)c0, orr);
         }
         tmem_st_wait();
-        if (grow) { u_run = corr * (u_run - (bm - m_ref) * l_run); l_run *= corr; m_ref = bm; }
+        if (grow) {
+          const float dm = bm - m_ref;
+          u2 = make_float2(corr * (u2.x - dm * l2.x), corr * (u2.y - dm * l2.y));
+          l2 = make_float2(l2.x * corr, l2.y * corr);
+          m_ref = bm;
+        }
       }
       if (m_ref == -INFINITY) m_ref = bm;
       const float base = m_ref == -INFINITY ? 0.f : m_ref;
-      if (it >= 2) wait(p_empty + pb, (uint32_t)((it >> 1) - 1) & 1u);
+      const float2 nbase2 = make_float2(-base, -base);
+      if (it >= P_BUFS) wait(p_empty + pb, (uint32_t)(it / P_BUFS - 1) & 1u);
       // ---- probabilities, row sum, P's high and low parts into shared memory
-      uint32_t ph[8], pl2[8];
+      uint8_t *p_buf = p_s + pb * AT_PTILE;
 #pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const float d0 = fmaf(t[c], scale, -base), d1 = fmaf(t[c + 1], scale, -base);
-        const float p0 = ex2(d0), p1 = ex2(d1);               // a masked key: 2^-inf = 0
-        l_run += p0 + p1;
-        if (want_ent) u_run += (p0 > 0.f ? p0 * d0 : 0.f) + (p1 > 0.f ? p1 * d1 : 0.f);
-        split_pair(p0, p1, ph[c >> 1], pl2[c >> 1]);
-      }
-      // this lane's 16 keys: high parts into the entry's even row, low parts into its odd row; 16-byte
-      // pieces swizzled like the MMA expects a K-major operand (piece ^ (row & 7))
-      uint8_t *row_hi = p_s + pb * AT_PTILE + (row & ~1) * 128, *row_lo = row_hi + 128;
-#pragma unroll
-      for (int pc = 0; pc < 2; ++pc) {
-        const int piece = half * 4 + part * 2 + pc;
-        *reinterpret_cast<uint4 *>(row_hi + ((piece ^ (row & 6)) << 4)) = make_uint4(ph[pc * 4], ph[pc * 4 + 1], ph[pc * 4 + 2], ph[pc * 4 + 3]);
-        *reinterpret_cast<uint4 *>(row_lo + ((piece ^ ((row & 6) | 1)) << 4)) = make_uint4(pl2[pc * 4], pl2[pc * 4 + 1], pl2[pc * 4 + 2], pl2[pc * 4 + 3]);
+      for (int c = 0; c < 8; ++c) {
+        const float2 d = fma2(t[c], scale2, nbase2);
+        const float2 p = make_float2(ex2(d.x), ex2(d.y));      // a masked key: 2^-inf = 0
+        l2 = add2(l2, p);
+        if (want_ent) u2 = fma2(p, make_float2(fmaxf(d.x, -1024.f), fmaxf(d.y, -1024.f)), u2);      // (p is 0 far above that)
+        uint32_t hi, lo;
+        split_pair(p.x, p.y, hi, lo);
+        uint8_t *w = p_buf + (p_off ^ (uint32_t)(c << 4));
+        *reinterpret_cast<uint32_t *>(w) = hi;
+        *reinterpret_cast<uint32_t *>(w + 1024) = lo;
       }
       fence_proxy_async_smem();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(p_full + pb);
     }
-    // ---- epilogue: the row's accumulator (lanes 2e and 2e+1 added), partial or finished; each warp half of the columns
-    if (n_blk > 0) wait(p_empty + ((n_blk - 1) & 1), (uint32_t)((n_blk - 1) >> 1) & 1u);
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);           // each of a row's four threads summed a quarter of the keys
+    // ---- epilogue: the entry's accumulator (TMEM lanes i and i + 8 added), partial or finished
+    if (n_blk > 0) wait(p_empty + (n_blk - 1) % P_BUFS, (uint32_t)((n_blk - 1) / P_BUFS) & 1u);
+    float l_run = l2.x + l2.y, u_run = u2.x + u2.y;            // each of the quad's lanes summed a quarter of the keys
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
     u_run += __shfl_xor_sync(0xffffffffu, u_run, 1);
-    float *lx = mx_s + (n_blk & 1) * 128;
-    lx[half * 64 + (row >> 1)] = l_run;
-    bar_sync_pair(1 + q);
-    l_run += lx[(half ^ 1) * 64 + (row >> 1)];
-    if (want_ent) {
-      bar_sync_pair(1 + q);
-      lx[half * 64 + (row >> 1)] = u_run;
-      bar_sync_pair(1 + q);
-      u_run += lx[(half ^ 1) * 64 + (row >> 1)];
-    }
+    u_run += __shfl_xor_sync(0xffffffffu, u_run, 2);
     pdl_trigger();                                            // the keys are done: the kernel that follows may take the SMs
     if (ok) {
       tc_fence_after();
       const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-      const long long pbase = ((((long long)slot * a.n_chunks + chunk) * a.hkv + kvh) * a.n_rt + rt) * 64 + (row >> 1);
+      const long long pbase = ((((long long)slot * a.n_chunks + chunk) * a.hkv + kvh) * a.n_rt + rt) * 64 + ei;
+      float *po = PF || a.n_chunks == 1 ? nullptr : a.part_o ? a.part_o + pbase * HD : o_s + ei * Sh::O_LD;
+      bf16 *out = reinterpret_cast<bf16 *>(a.out) + h * HD;
+      if (a.out_chunk_stride) out += (long long)(r / a.out_chunk_rows) * a.out_chunk_stride + (long long)(r % a.out_chunk_rows) * a.lay.row_stride;
+      else out += (long long)r * a.lay.row_stride;
 #pragma unroll 1
-      for (int c0 = half * (HD / 2); c0 < (half + 1) * (HD / 2); c0 += 32) {
+      for (int c0 = 0; c0 < HD; c0 += 64) {
         uint32_t orr[32];
-        if (n_blk > 0) { tmem_ld32(lane_addr + (uint32_t)c0, orr); tmem_ld_wait(); }
+        if (n_blk > 0) { tmem_ld16x64(lane_addr + (uint32_t)c0, orr); tmem_ld_wait(); }
         else {
 #pragma unroll
           for (int c = 0; c < 32; ++c) orr[c] = 0u;
         }
-        // the even lane keeps columns 0..15 of the chunk, the odd lane 16..31
-        float v[16];
+        // columns c0 + 8 c + 2 ql and the next one
+        float2 v[8];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const float send = __uint_as_float(part ? orr[c] : orr[16 + c]);
-          const float mine = __uint_as_float(part ? orr[16 + c] : orr[c]);
-          v[c] = mine + __shfl_xor_sync(0xffffffffu, send, 1);
-        }
-        const int col = c0 + part * 16;
-        if (a.n_chunks > 1) {
-          float *po = a.part_o ? a.part_o + pbase * HD + col : o_s + (row >> 1) * Sh::O_LD + col;
+        for (int c = 0; c < 8; ++c)
+          v[c] = add2(make_float2(__uint_as_float(orr[4 * c]), __uint_as_float(orr[4 * c + 1])), make_float2(__uint_as_float(orr[4 * c + 2]), __uint_as_float(orr[4 * c + 3])));
+        if (!PF && a.n_chunks > 1) {
 #pragma unroll
-          for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4 *>(po + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
-        } else if (r >= 0) {
-          bf16 *out = reinterpret_cast<bf16 *>(a.out);
-          long long o = a.out_chunk_stride ? (long long)(r / a.out_chunk_rows) * a.out_chunk_stride + (long long)(r % a.out_chunk_rows) * a.lay.row_stride
-                                           : (long long)r * a.lay.row_stride;
+          for (int c = 0; c < 8; ++c) *reinterpret_cast<float2 *>(po + c0 + 8 * c + 2 * ql) = v[c];
+        } else {
+          // turned within the quad: a lane stores eight consecutive columns
 #pragma unroll
-          for (int c = 0; c < 16; c += 4)
-            store_split4<bf16>(out + o + h * HD + col + c, a.lay.lo_delta, make_float4(v[c] * inv, v[c + 1] * inv, v[c + 2] * inv, v[c + 3] * inv));
+          for (int g = 0; g < 2; ++g) {
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) split_pair(v[4 * g + c].x * inv, v[4 * g + c].y * inv, hi[c], lo[c]);
+            quad_transpose(hi, lane);
+            quad_transpose(lo, lane);
+            if (r >= 0) {
+              bf16 *o = out + c0 + 32 * g + 8 * ql;
+              *reinterpret_cast<uint4 *>(o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+              if (a.lay.lo_delta) *reinterpret_cast<uint4 *>(o + a.lay.lo_delta) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            }
+          }
         }
       }
-      if (a.n_chunks > 1 && part == 0 && half == 0) {
+      if (!PF && a.n_chunks > 1 && ql == 0) {
         if (a.part_o) {
           *reinterpret_cast<float2 *>(a.part_ml + pbase * 2) = make_float2(m_ref, l_run);
           if (a.row_ent) a.part_u[pbase] = u_run;
-        } else *reinterpret_cast<float4 *>(ml_s + (row >> 1) * 4) = make_float4(m_ref, l_run, u_run, 0.f);
+        } else *reinterpret_cast<float4 *>(ml_s + ei * 4) = make_float4(m_ref, l_run, u_run, 0.f);
       }
-      if (r >= 0 && part == 0 && half == 0 && a.n_chunks == 1) {
+      if (r >= 0 && ql == 0 && (PF || a.n_chunks == 1)) {
         if (a.row_ent) {
           a.row_ent[(long long)r * a.H + h] = l_run > 0.f ? logf(l_run) - u_run * 0.6931471805599453f / l_run : 0.f;
         }
@@ -556,7 +618,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   if (gave_up && lane == 0) wait_expired(a.status, gave_up, abort_flag, -1);
   drain_if_aborted(abort_flag);
   tc_fence_before();
-  if (a.n_chunks > 1 && !a.part_o) {
+  if (!PF && a.n_chunks > 1 && !a.part_o) {
     // ---- merge: out = sum_c w_c O_c / sum_c w_c l_c with w_c = 2^(m_c - max m), chunks in ascending order; this CTA's
     // share of the (entry, four columns) items
     __syncwarp();
@@ -635,11 +697,29 @@ static inline bool at_map(GemmTcPlan *pl, AtMapCache *cache, const void *ptr, in
   return true;
 }
 
-template <int HD, bool FLAT>
+// The query rows [rows][H][high | low][hd] as k_attn_tc's tiles take them: eight entries' high parts, then their low parts, then the next
+// eight entries.  With G heads per KV head an eight is 8 / G rows of G heads, or eight heads of one row; the box is the whole
+// 128-row tile either way, from coordinates (column, first head, row, 0, 0) or (column, first head, 0, 0, row).  In the first form the
+// row enters through two dimensions, so rows behind the last of a tile are not cut off: up to 63 rows of what
+// follows the buffer are read, and belong to no entry.
+static inline bool attn_q_map(GemmTcPlan *pl, AtMapCache *cache, const void *q, int rows, int H, int G, int hd, CUtensorMap *out) {
+  const unsigned long long part = (unsigned long long)hd * 2, head = part * 2, row = head * H;
+  if (G <= 8) {
+    const unsigned rpg = 8u / (unsigned)G;
+    const unsigned long long dims[5] = {(unsigned long long)hd, (unsigned long long)H, (unsigned long long)rows, 2ull, 8ull}, st[4] = {head, row, part, row * rpg};
+    const unsigned box[5] = {64u, (unsigned)G, rpg, 2u, 8u};
+    return at_map(pl, cache, q, 5, dims, st, box, out);
+  }
+  const unsigned long long dims[5] = {(unsigned long long)hd, (unsigned long long)H, 2ull, (unsigned long long)(G / 8), (unsigned long long)rows}, st[4] = {head, part, head * 8, row};
+  const unsigned box[5] = {64u, 8u, 2u, (unsigned)(G / 8), (unsigned)(64 / G)};
+  return at_map(pl, cache, q, 5, dims, st, box, out);
+}
+
+template <int HD, bool FLAT, bool PF>
 static inline void attn_tc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, cudaStream_t stream, int use_pdl, int n_chunks, int cluster, int tiles, int n_slots) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3(n_chunks, tiles, n_slots); cfg->blockDim = dim3(AT_THREADS);
-  cfg->dynamicSmemBytes = AtShape<HD, FLAT>::SMEM; cfg->stream = stream;
+  cfg->dynamicSmemBytes = AtShape<HD, FLAT, PF>::SMEM; cfg->stream = stream;
   int n = 0;
   if (cluster) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
@@ -655,19 +735,20 @@ static inline void attn_tc_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *
 }
 
 // max_tiles[n]: tiles of n chunks (clusters of n CTAs) that are resident at once.
-template <int HD, bool FLAT>
+template <int HD, bool FLAT, bool PF>
 static inline const char *attn_tc_setup(int *max_tiles, int n_sms) {
-  auto *kernel = k_attn_tc<HD, FLAT>;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AtShape<HD, FLAT>::SMEM) != cudaSuccess ||
+  auto *kernel = k_attn_tc<HD, FLAT, PF>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AtShape<HD, FLAT, PF>::SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
       cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return "cannot raise the attention kernel's shared memory or cluster limit";
+  if (PF) return nullptr;                      // one chunk, no clusters
   max_tiles[0] = 0;
-  max_tiles[1] = n_sms * AtShape<HD, FLAT>::CTAS_PER_SM;
+  max_tiles[1] = n_sms * AtShape<HD, FLAT, PF>::CTAS_PER_SM;
   for (int n = 2; n <= AT_MAX_CLUSTER; ++n) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
-    attn_tc_config<HD, FLAT>(&cfg, attr, nullptr, 0, n, 1, 1, 1);
+    attn_tc_config<HD, FLAT, PF>(&cfg, attr, nullptr, 0, n, 1, 1, 1);
     int clusters = 0;
     if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); clusters = 0; }
     max_tiles[n] = clusters;
@@ -677,11 +758,11 @@ static inline const char *attn_tc_setup(int *max_tiles, int n_sms) {
 
 // Enqueue one attention launch: grid (a.n_chunks, H_kv * a.n_rt, n_slots), the chunks of a tile a cluster unless
 // there are partials.
-template <int HD, bool FLAT>
+template <int HD, bool FLAT, bool PF>
 static inline cudaError_t attn_tc_launch(cudaStream_t stream, int use_pdl, const CUtensorMap &mq, const CUtensorMap &mk, const CUtensorMap &mv,
                                          const AttnTcArgs &a, int n_slots) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  attn_tc_config<HD, FLAT>(&cfg, attr, stream, use_pdl, a.n_chunks, a.n_chunks > 1 && !a.part_o, (a.H / a.G) * a.n_rt, n_slots);
-  return cudaLaunchKernelEx(&cfg, k_attn_tc<HD, FLAT>, mq, mk, mv, a);
+  attn_tc_config<HD, FLAT, PF>(&cfg, attr, stream, use_pdl, a.n_chunks, a.n_chunks > 1 && !a.part_o, (a.H / a.G) * a.n_rt, n_slots);
+  return cudaLaunchKernelEx(&cfg, k_attn_tc<HD, FLAT, PF>, mq, mk, mv, a);
 }

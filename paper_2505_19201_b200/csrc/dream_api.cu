@@ -527,8 +527,9 @@ static void refresh_bounds(dream_ctx *c) {
 
 template <int HD>
 static const char *attn_tc_setup_all(dream_ctx *c) {
-  const char *w = attn_tc_setup<HD, false>(c->at_max_tiles[0], c->tc.n_sms);
-  if (!w) w = attn_tc_setup<HD, true>(c->at_max_tiles[1], c->tc.n_sms);
+  const char *w = attn_tc_setup<HD, false, false>(c->at_max_tiles[0], c->tc.n_sms);
+  if (!w) w = attn_tc_setup<HD, true, false>(c->at_max_tiles[1], c->tc.n_sms);
+  if (!w) w = attn_tc_setup<HD, false, true>(nullptr, c->tc.n_sms);
   return w ? w : colsum_tc_setup<HD>();
 }
 
@@ -832,13 +833,7 @@ template <typename T, int HD> struct AttnLaunch {
     a.out = c->attn_out; a.status = c->status;
     a.hkv = f.n_kv_heads;
     CUtensorMap mq, mk, mv;
-    bool ok;
-    {
-      const unsigned long long dims[4] = {(unsigned long long)HD, 2ull, (unsigned long long)f.n_heads, (unsigned long long)c->XR};
-      const unsigned long long st[3] = {(unsigned long long)HD * 2, (unsigned long long)HD * 4, (unsigned long long)f.n_heads * HD * 4};
-      const unsigned box[4] = {64u, 2u, (unsigned)a.G, (unsigned)(64 / a.G)};
-      ok = at_map(&c->tc, &c->at_maps, c->q_cur, 4, dims, st, box, &mq);
-    }
+    bool ok = attn_q_map(&c->tc, &c->at_maps, c->q_cur, c->XR, f.n_heads, a.G, HD, &mq);
     if (flat_kv) {
       const unsigned long long dims[3] = {(unsigned long long)HD, 2ull, (unsigned long long)f.max_batch * 2 * f.n_kv_heads * c->cap_rows};
       const unsigned long long st[2] = {(unsigned long long)HD * 2, (unsigned long long)HD * 4};
@@ -856,8 +851,9 @@ template <typename T, int HD> struct AttnLaunch {
       a.page_table = kv.page_table; a.pages_per_seq = kv.pages_per_seq; a.page_tokens = kv.page_tokens; a.page_shift = kv.page_shift;
     }
     if (!ok) { c->gemm_failed = 1; return; }
-    cudaError_t e = flat_kv ? attn_tc_launch<HD, true>(c->stream, c->use_pdl, mq, mk, mv, a, B)
-                            : attn_tc_launch<HD, false>(c->stream, c->use_pdl, mq, mk, mv, a, B);
+    cudaError_t e = flat_kv                ? attn_tc_launch<HD, true, false>(c->stream, c->use_pdl, mq, mk, mv, a, B)
+                    : a.mode == AT_PREFILL ? attn_tc_launch<HD, false, true>(c->stream, c->use_pdl, mq, mk, mv, a, B)
+                                           : attn_tc_launch<HD, false, false>(c->stream, c->use_pdl, mq, mk, mv, a, B);
     if (e != cudaSuccess && c->launch_err == cudaSuccess) { c->launch_err = e; c->launch_err_name = "k_attn_tc"; }
     c->launches++;
     if (a.n_chunks > 1 && a.part_o) {
