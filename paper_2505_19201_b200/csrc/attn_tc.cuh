@@ -14,7 +14,7 @@
 //   softmax              eight warps, each eight entries: the four lanes of a quad take 16 of the block's keys each for one entry, so
 //                        a row's maximum and sums are two shuffles and nothing is exchanged between warps.  One pass: the block's row
 //                        maximum, then P = 2^(s - m), its row sum, and P's high and low bf16 parts to the entry's two rows
-//                        of a shared-memory tile in the operand layout; adds and multiply-adds take two values per instruction.  m is any
+//                        of a shared-memory tile in the operand layout.   m is any
 //                        reference near the maximum: it follows the maximum only when that has outgrown it by 2^8, so
 //                        the O accumulator is hardly ever rescaled (in TMEM, tcgen05.ld / tcgen05.st);
 //   O += P_b V_b         tcgen05.mma 128 x head_dim x 16 steps over the block's keys, A = P_b (K-major)
@@ -171,19 +171,10 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// Two single-precision operations in one instruction, each rounded as the single one.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  float2 c;
-  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 z, x, y;\n mov.b64 {%0, %1}, z;\n}"
-      : "=f"(c.x), "=f"(c.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return c;
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 d) {
-  float2 c;
-  asm("{\n .reg .b64 x, y, w, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 w, {%6, %7};\n fma.rn.f32x2 z, x, y, w;\n mov.b64 {%0, %1}, z;\n}"
-      : "=f"(c.x), "=f"(c.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(d.x), "f"(d.y));
-  return c;
-}
+// (As packed instructions, add.rn.f32x2 and fma.rn.f32x2, the same values: LLaVA-7B-shaped request 24.0 -> 24.3 ms, Gemma-shaped round 11.39 ->
+// 11.45; the packing costs more than it saves.)
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 d) { return make_float2(fmaf(a.x, b.x, d.x), fmaf(a.y, b.y, d.y)); }
 // w[i] of the four lanes of a quad: lane j ends up with the quad's words j, in lane order.
 __device__ __forceinline__ void quad_transpose(uint32_t (&w)[4], int lane) {
 #pragma unroll
