@@ -42,6 +42,7 @@
 #include "attn_merge.cuh"
 #include "common.cuh"
 #include "gemm_tc.cuh"
+#include "q_tile.cuh"
 #include "rows.cuh"
 
 #define AT_THREADS 352
@@ -297,8 +298,9 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       const uint64_t pol_q = policy_evict_last();
       if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_q) : "memory");
       __syncwarp();
-      // queries: boxes of 64 columns, whose rows come as the tile has them (see attn_q_map)
-      const int node0 = slot * a.rows_per_seq + e_base / a.G, c2 = a.G > 8 ? 0 : node0, c4 = a.G > 8 ? node0 : 0;
+      // queries: boxes of 64 columns, whose rows come as the tile has them
+      int c2, c4;
+      q_tile_start(a.G, slot * a.rows_per_seq + e_base / a.G, c2, c4);
       if (elect_one()) {
         mbar_expect_tx(q_full, (uint32_t)Sh::Q_BYTES);
         for (int kp = 0; kp < KP; ++kp) tma_load_5d(q_s + kp * AT_QTILE, &map_q, q_full, kp * 64, kvh * a.G, c2, 0, c4, pol_q);
@@ -688,22 +690,10 @@ static inline bool at_map(GemmTcPlan *pl, AtMapCache *cache, const void *ptr, in
   return true;
 }
 
-// The query rows [rows][H][high | low][hd] as k_attn_tc's tiles take them: eight entries' high parts, then their low parts, then the next
-// eight entries.  With G heads per KV head an eight is 8 / G rows of G heads, or eight heads of one row; the box is the whole
-// 128-row tile either way, from coordinates (column, first head, row, 0, 0) or (column, first head, 0, 0, row).  In the first form the
-// row enters through two dimensions, so rows behind the last of a tile are not cut off: up to 63 rows of what
-// follows the buffer are read, and belong to no entry.
+// The query rows as the tiles take them (q_tile.cuh).
 static inline bool attn_q_map(GemmTcPlan *pl, AtMapCache *cache, const void *q, int rows, int H, int G, int hd, CUtensorMap *out) {
-  const unsigned long long part = (unsigned long long)hd * 2, head = part * 2, row = head * H;
-  if (G <= 8) {
-    const unsigned rpg = 8u / (unsigned)G;
-    const unsigned long long dims[5] = {(unsigned long long)hd, (unsigned long long)H, (unsigned long long)rows, 2ull, 8ull}, st[4] = {head, row, part, row * rpg};
-    const unsigned box[5] = {64u, (unsigned)G, rpg, 2u, 8u};
-    return at_map(pl, cache, q, 5, dims, st, box, out);
-  }
-  const unsigned long long dims[5] = {(unsigned long long)hd, (unsigned long long)H, 2ull, (unsigned long long)(G / 8), (unsigned long long)rows}, st[4] = {head, part, head * 8, row};
-  const unsigned box[5] = {64u, 8u, 2u, (unsigned)(G / 8), (unsigned)(64 / G)};
-  return at_map(pl, cache, q, 5, dims, st, box, out);
+  const QTileMap m = q_tile_map(rows, H, G, hd);
+  return at_map(pl, cache, q, 5, m.dims, m.strides, m.box, out);
 }
 
 template <int HD, bool FLAT, bool PF>

@@ -353,7 +353,9 @@ static size_t carve(dream_ctx *c, char *base) {
   c->vmask = a.take<uint32_t>((size_t)ROW_CHUNK * 4);
   c->x = a.take<float>((size_t)c->XR * d);
   c->x0 = a.take<float>((size_t)f.max_prompt * d);
-  c->qbuf = a.take<float>((size_t)c->XR * c->Hhd);
+  // query rows and, behind them, what the tensor-core attention's tiles read past the last one (in a decode round; a prompt's do not,
+  // so q_taps has no such room)
+  c->qbuf = a.take<float>((size_t)(f.dtype == DREAM_BF16 ? q_tile_room(c->XR) : c->XR) * c->Hhd);
   int planes = f.dtype == DREAM_BF16 ? 2 : 1;      // bf16 GEMM inputs: a high and a low row per token
   // attention outputs: whole passes over the prompt of PR rows
   c->attn_out = a.take_bytes((size_t)planes * ((c->XR + c->PR - 1) / c->PR * c->PR) * c->Hhd * e);
