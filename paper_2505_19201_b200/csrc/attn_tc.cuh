@@ -539,22 +539,25 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
       __syncwarp();
       if (lane == 0) mbar_arrive(p_full + pb);
     }
-    // ---- epilogue: the entry's accumulator (TMEM lanes i and i + 8 added), partial or finished
-    if (n_blk > 0) wait(p_empty + (n_blk - 1) % P_BUFS, (uint32_t)((n_blk - 1) / P_BUFS) & 1u);
+    // ---- epilogue: the entry's accumulator (TMEM lanes i and i + 8 added), partial or finished.  What does not need the accumulator stands before
+    // the wait for it: this code too is fetched at every launch, and as long as it stood behind, the CTA waited for O first and
+    // then for the code.  From the last P to the end a draft launch at head_dim 128 took 7.2k cycles of 16.0k, now 5.4k of 14.0k (two blocks of keys);
+    // LLaVA-7B-shaped round with all options 5160 -> 5115 us, SmolVLM-shaped 2290 -> 2260, LLaVA-7B-shaped 4897 -> 4857.
     float l_run = l2.x + l2.y, u_run = u2.x + u2.y;            // each of the quad's lanes summed a quarter of the keys
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
     l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
     u_run += __shfl_xor_sync(0xffffffffu, u_run, 1);
     u_run += __shfl_xor_sync(0xffffffffu, u_run, 2);
+    const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+    const long long pbase = ((((long long)slot * a.n_chunks + chunk) * a.hkv + kvh) * a.n_rt + rt) * 64 + ei;
+    float *po = PF || a.n_chunks == 1 ? nullptr : a.part_o ? a.part_o + pbase * HD : o_s + ei * Sh::O_LD;
+    bf16 *out = reinterpret_cast<bf16 *>(a.out) + h * HD;
+    if (a.out_chunk_stride) out += (long long)(r / a.out_chunk_rows) * a.out_chunk_stride + (long long)(r % a.out_chunk_rows) * a.lay.row_stride;
+    else out += (long long)r * a.lay.row_stride;
+    if (n_blk > 0) wait(p_empty + (n_blk - 1) % P_BUFS, (uint32_t)((n_blk - 1) / P_BUFS) & 1u);
     pdl_trigger();                                            // the keys are done: the kernel that follows may take the SMs
     if (ok) {
       tc_fence_after();
-      const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-      const long long pbase = ((((long long)slot * a.n_chunks + chunk) * a.hkv + kvh) * a.n_rt + rt) * 64 + ei;
-      float *po = PF || a.n_chunks == 1 ? nullptr : a.part_o ? a.part_o + pbase * HD : o_s + ei * Sh::O_LD;
-      bf16 *out = reinterpret_cast<bf16 *>(a.out) + h * HD;
-      if (a.out_chunk_stride) out += (long long)(r / a.out_chunk_rows) * a.out_chunk_stride + (long long)(r % a.out_chunk_rows) * a.lay.row_stride;
-      else out += (long long)r * a.lay.row_stride;
 #pragma unroll 1
       for (int c0 = 0; c0 < HD; c0 += 64) {
         uint32_t orr[32];
