@@ -318,7 +318,8 @@ dream_status dream_seq_reset(dream_ctx *ctx, int32_t seq);
 
 /* Wait for the stream and report the device status word: DREAM_OK, DREAM_E_DEVICE_TIMEOUT (a
  * bounded wait inside a kernel ran out, after a second; the message names the kernel and the wait) or DREAM_E_STATE (a kernel met a malformed tree, an index
- * or a capacity out of range, or a logits row without mass; the offending rows were skipped).
+ * or a capacity out of range, or a logits row without mass; the offending rows were skipped), or DREAM_E_CUDA (a kernel could not
+ * lay out its shared memory and did nothing; dream_init checks what this depends on).
  * The word is sticky: it is not cleared by reading it. */
 dream_status dream_poll(dream_ctx *ctx);
 

@@ -197,8 +197,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUt
   constexpr int STAGES = Sh::STAGES, S_BUFS = Sh::S_BUFS, P_BUFS = Sh::P_BUFS, KP = Sh::KP, PLANES = Sh::PLANES;
   extern __shared__ __align__(1024) uint8_t at_smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)at_smem_raw + 1023) & ~(uintptr_t)1023);
-  if (Sh::SMALL && smem != at_smem_raw) {                   // no room to align by hand: two CTAs fill an SM's shared memory
-    if (threadIdx.x == 0) atomicMax(a.status, DREAM_DEV_TIMEOUT);
+  if (Sh::SMALL && smem != at_smem_raw) {                   // no room to align by hand: two CTAs fill an SM's shared memory (attn_tc_setup checks too)
+    if (threadIdx.x == 0) atomicMax(a.status, DREAM_DEV_LAYOUT);
     return;
   }
   uint8_t *q_s = smem, *k_s = q_s + Sh::Q_BYTES, *v_s = k_s + STAGES * Sh::KV_STAGE, *p_s = v_s + STAGES * Sh::KV_STAGE;
@@ -726,6 +726,14 @@ static inline const char *attn_tc_setup(int *max_tiles, int n_sms) {
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
       cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
     return "cannot raise the attention kernel's shared memory or cluster limit";
+  if (AtShape<HD, FLAT, PF>::SMALL) {          // dynamic shared memory lies behind the system's and the kernel's own
+    int dev = 0, reserved = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, kernel) != cudaSuccess)
+      return "cannot read the attention kernel's shared memory layout";
+    if (reserved % 1024 || fa.sharedSizeBytes % 1024) return "the prompt's attention needs shared memory that starts on a multiple of 1024 bytes";
+  }
   if (PF) return nullptr;                      // one chunk, no clusters
   max_tiles[0] = 0;
   max_tiles[1] = n_sms * AtShape<HD, FLAT, PF>::CTAS_PER_SM;

@@ -12,6 +12,7 @@ typedef __nv_bfloat16 bf16;
 #define DREAM_DEV_OK 0
 #define DREAM_DEV_TIMEOUT 1
 #define DREAM_DEV_BAD_INDEX 2
+#define DREAM_DEV_LAYOUT 3             // a block's shared memory does not start where its kernel needs it (dream_init checks; see attn_tc.cuh)
 // The waits that can expire, as the second status word names the first one that did.
 enum {
   WAIT_none = 0,

@@ -633,6 +633,7 @@ extern "C" dream_status dream_poll(dream_ctx *c) {
   static_assert(sizeof(names) / sizeof(names[0]) == WAIT_probe + 1, "a name per wait");
   if (st[1]) return fail(c, DREAM_E_DEVICE_TIMEOUT, "a bounded device-side wait expired (%s)", names[st[1] < 0 || st[1] > WAIT_probe ? 0 : st[1]]);
   if (st[0] == DREAM_DEV_BAD_INDEX) return fail(c, DREAM_E_STATE, "a kernel met an index or capacity out of range");
+  if (st[0] == DREAM_DEV_LAYOUT) return fail(c, DREAM_E_CUDA, "k_attn_tc: shared memory does not start on a multiple of 1024 bytes");
   return DREAM_OK;
 }
 

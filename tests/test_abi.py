@@ -73,6 +73,23 @@ def test_draft_shape_and_entropy_switch_are_validated_and_sized():
             raise AssertionError(f"{bad} was accepted")
 
 
+def test_every_status_code_a_kernel_stores_is_reported():
+    """DREAM_DEV_TIMEOUT counts only beside the wait that ran out (wait_expired stores both words); every other code is answered by
+    dream_poll itself, so that a launch that did nothing is never reported as fine."""
+    csrc = os.path.join(ROOT, "paper_2505_19201_b200", "csrc")
+    stores = {}
+    for name in os.listdir(csrc):
+        text = open(os.path.join(csrc, name)).read()
+        for m in re.finditer(r"atomicMax\([^;]*?(DREAM_DEV_\w+)\)", text):
+            stores.setdefault(m.group(1), []).append((name, text.rfind("\n__", 0, m.start()), text.rfind("void wait_expired(", 0, m.start())))
+    assert len(stores) >= 2
+    for name, kernel, expired in stores.pop("DREAM_DEV_TIMEOUT"):
+        assert name == "gemm_tc.cuh" and expired > kernel >= 0, f"{name}: a time-out without the name of a wait"
+    api_cu = open(os.path.join(csrc, "dream_api.cu")).read()
+    poll = api_cu[api_cu.index("dream_status dream_poll("):api_cu.index("static dream_status check_seq(")]
+    assert not [code for code in stores if code not in poll]
+
+
 def test_tree_from_parents_checks_its_input():
     import ctypes as C
     import torch
