@@ -307,7 +307,8 @@ dream_status dream_topk_lse_static(const float *logits, int32_t rows, int32_t vo
  * installed, every kernel of the library appends (kernel id, nanosecond timer) at the moment its
  * predecessor in the stream has completed; word 0 counts the entries.  Differences between
  * consecutive entries give each kernel's time on the critical path, overlap included.  The
- * buffer is process-wide (one traced context at a time).  Synchronises the stream. */
+ * buffer is process-wide (one traced context at a time).  Waits for all work on the device, so that no kernel
+ * of any context still holds the buffer that was installed before. */
 dream_status dream_trace(dream_ctx *ctx, unsigned long long *buffer, int64_t capacity_entries);
 
 /* Name of a kernel id found in a trace buffer.  Host-only. */

@@ -1598,6 +1598,9 @@ extern "C" dream_status dream_trace(dream_ctx *c, unsigned long long *buffer, in
     ptr = buffer;
   }
   CUDA_OK(c, cudaMemcpyToSymbol(g_dream_trace, &ptr, sizeof(ptr)));
+  // A kernel asks for the buffer's address when it starts and uses it when its predecessor has ended (trace_open, trace_stamp), and the address
+  // is every context's: those of the other streams may still hold the old one, whose memory the caller is free to give up.
+  CUDA_OK(c, cudaDeviceSynchronize());
   return DREAM_OK;
 }
 
