@@ -2,9 +2,14 @@
 agent ends, and when the last one has, no asynchronous arrival is under way any more.  An arrival that came in later would
 land in the shared memory of the CTA that follows on the SM.  Without the closing waits the models show such arrivals."""
 import heapq
+import os
 import random
+import re
+import subprocess
 
 import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2505_19201_b200", "csrc")
 
 
 class Clock:
@@ -89,93 +94,130 @@ def some(rng, most):
         yield
 
 
-# ring depths of K and V blocks and of score buffers, by (head_dim, flat cache)
-ATTN = {(64, False): (3, 3), (64, True): (4, 3), (128, False): (5, 4), (128, True): (2, 4), (256, False): (2, 4), (256, True): (1, 4)}
+# ring depths by (head_dim, form): blocks of K and of V, score buffers, buffers of probabilities (AtShape in attn_tc.cuh)
+ATTN = {(64, "paged"): (3, 3, 2), (64, "flat"): (4, 3, 2), (64, "prompt"): (3, 3, 2), (128, "paged"): (5, 4, 2), (128, "flat"): (2, 4, 2),
+        (128, "prompt"): (2, 2, 1), (256, "paged"): (2, 4, 2), (256, "flat"): (1, 4, 2), (256, "prompt"): (2, 4, 2)}
 
 
 def attention(shape, n_blk, early, seed, closing=True):
     rng = random.Random(seed)
-    stages, s_bufs = ATTN[shape]
-    ahead = min(stages, s_bufs)
+    stages, s_bufs, p_bufs = ATTN[shape]
     clock = Clock(rng)
     bars = lambda n, count=1: [Barrier(count) for _ in range(n)]
-    k_full, k_empty, v_full, v_empty = bars(stages), bars(stages), bars(stages), bars(stages)
-    s_full, s_free, p_full, p_empty = bars(s_bufs), bars(s_bufs, 8), bars(2, 8), bars(2)
+    q_full, k_full, k_empty, v_full, v_empty = bars(1)[0], bars(stages), bars(stages), bars(stages), bars(stages)
+    s_full, s_free, p_full, p_empty = bars(s_bufs), bars(s_bufs, 8), bars(p_bufs, 8), bars(p_bufs)
     n_pre = min(early, n_blk, stages)
+    # what the buffers hold, to see that nobody reads or overwrites the wrong block
+    held = dict(k=[None] * stages, v=[None] * stages, s=[None] * s_bufs, p=[[None] * 8 for _ in range(p_bufs)], o=-1)
+
+    def load(what, full, st, it):
+        held[what][st] = it
+        full[st].load(clock, 2)
 
     def producer():
         for i in range(n_pre):
-            k_full[i].load(clock, 2)
-            v_full[i].load(clock, 2)
+            load("k", k_full, i, i)
+            load("v", v_full, i, i)
+        q_full.load(clock, 2)
         ks = vs = n_pre % stages
         kph = vph = 0 if n_pre >= stages else 1
         for it in range(n_pre, n_blk + 1):
             if it < n_blk:
                 yield from until(lambda: k_empty[ks].done(kph))
-                k_full[ks].load(clock, 2)
+                load("k", k_full, ks, it)
                 ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
             if it > n_pre:
                 yield from until(lambda: v_empty[vs].done(vph))
-                v_full[vs].load(clock, 2)
+                load("v", v_full, vs, it - 1)
                 vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
         if not closing:
             return
         for _ in range(stages):
-            yield from until(lambda: k_empty[ks].done(kph) and v_empty[vs].done(vph))
+            yield from until(lambda: k_empty[ks].done(kph))
+            yield from until(lambda: v_empty[vs].done(vph))
             ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
             vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
-        for b in (0, 1):
-            yield from until(lambda: p_empty[b].done((((n_blk + 1 - b) >> 1) + 1) & 1))
+        for b in range(p_bufs):
+            yield from until(lambda: p_empty[b].done(((n_blk + p_bufs - 1 - b) // p_bufs + 1) & 1))
 
-    def issuer():
+    def s_issuer():
         commit = Committer(clock)
-        ks = sb = vs = kph = vph = 0
+        yield from until(lambda: q_full.done(0))
+        ks = sb = kph = 0
         sph = 1
-        for i in range(n_blk + ahead):
-            it = i - ahead
-            if it >= 0:
-                yield from until(lambda: p_full[it & 1].done((it >> 1) & 1) and v_full[vs].done(vph))
-                commit(p_empty[it & 1], v_empty[vs])
-                vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
-            if i < n_blk:
-                yield from until(lambda: k_full[ks].done(kph) and s_free[sb].done(sph))
-                commit(k_empty[ks], s_full[sb])
-                ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
-                sb, sph = (sb + 1, sph) if sb + 1 < s_bufs else (0, sph ^ 1)
+        for it in range(n_blk):
+            yield from until(lambda: s_free[sb].done(sph))
+            yield from until(lambda: k_full[ks].done(kph))
+            assert held["k"][ks] == it
+            held["s"][sb] = it
+            commit(k_empty[ks], s_full[sb])
+            ks, kph = (ks + 1, kph) if ks + 1 < stages else (0, kph ^ 1)
+            sb, sph = (sb + 1, sph) if sb + 1 < s_bufs else (0, sph ^ 1)
 
-    met = {}
+    def o_issuer():
+        commit = Committer(clock)
+        vs = vph = 0
+        for it in range(n_blk):
+            pb = it % p_bufs
+            yield from until(lambda: v_full[vs].done(vph))
+            yield from until(lambda: p_full[pb].done((it // p_bufs) & 1))
+            assert held["v"][vs] == it and held["p"][pb] == [it] * 8
+            commit(p_empty[pb], v_empty[vs])
+            held["o"] = it
+            vs, vph = (vs + 1, vph) if vs + 1 < stages else (0, vph ^ 1)
 
-    def softmax(quarter, half):
+    def softmax(w):
         sb = sph = 0
         for it in range(n_blk):
-            pb = it & 1
+            pb = it % p_bufs
             yield from until(lambda: s_full[sb].done(sph))
+            assert held["s"][sb] == it
             yield from some(rng, 3)
             s_free[sb].arrive()
             sb, sph = (sb + 1, sph) if sb + 1 < s_bufs else (0, sph ^ 1)
-            met[quarter, half] = it
-            yield from until(lambda: met.get((quarter, half ^ 1), -1) >= it)
-            if it and rng.random() < 0.3:                     # the row's reference moves
-                yield from until(lambda: p_empty[pb ^ 1].done(((it - 1) >> 1) & 1))
-            if it >= 2:
-                yield from until(lambda: p_empty[pb].done(((it >> 1) - 1) & 1))
+            if it and rng.random() < 0.3:                     # the row's reference moves: behind the O of every earlier block, before this block's
+                yield from until(lambda: p_empty[(it - 1) % p_bufs].done(((it - 1) // p_bufs) & 1))
+                assert held["o"] == it - 1
+                yield from some(rng, 2)
+                assert held["o"] == it - 1
+            if it >= p_bufs:
+                yield from until(lambda: p_empty[pb].done((it // p_bufs - 1) & 1))
+                assert held["o"] >= it - p_bufs
+            held["p"][pb][w] = it
             yield from some(rng, 3)
             p_full[pb].arrive()
-        yield from until(lambda: p_empty[(n_blk - 1) & 1].done(((n_blk - 1) >> 1) & 1))
+        yield from until(lambda: p_empty[(n_blk - 1) % p_bufs].done(((n_blk - 1) // p_bufs) & 1))
+        assert held["o"] == n_blk - 1
 
-    return play(clock, [producer(), issuer()] + [softmax(q, h) for q in range(4) for h in range(2)])
+    return play(clock, [producer(), s_issuer(), o_issuer()] + [softmax(w) for w in range(8)])
 
 
 @pytest.mark.parametrize("shape", list(ATTN))
 def test_attention(shape):
     for n_blk in (1, 2, 3, 4, 5, 6, 7, 11, 33):
-        for early in ((0,) if shape[1] else (0, 1, n_blk)):
+        for early in ((0, 1, n_blk) if shape[1] == "paged" else (0,)):
             for seed in range(3):
                 assert attention(shape, n_blk, early, seed) == 0
 
 
-def test_attention_without_closing_waits():
-    assert any(attention((128, False), 5, 0, seed, closing=False) for seed in range(20))
+@pytest.mark.parametrize("shape", [(128, "paged"), (128, "prompt"), (256, "flat")])
+def test_attention_without_closing_waits(shape):
+    assert any(attention(shape, 5, 0, seed, closing=False) for seed in range(40))
+
+
+def test_attention_shapes(tmp_path):
+    """The depths above are those that AtShape gives to the forms that are launched."""
+    src = open(os.path.join(CSRC, "attn_tc.cuh")).read()
+    shape = src[src.index("template <int HD, bool FLAT, bool PF = false> struct AtShape"):]
+    shape = shape[:shape.index("\n};") + 3]
+    lines = ["#include <cstddef>", "#include <cstdio>"] + re.findall(r"^#define AT_[A-Z]+ .*$", src, re.M) + [shape, "int main() {"]
+    for hd, form in ATTN:
+        lines.append("  { using S = AtShape<%d, %s, %s>; printf(\"%%d %%d %%d\\n\", S::STAGES, S::S_BUFS, S::P_BUFS); }"
+                     % (hd, str(form == "flat").lower(), str(form == "prompt").lower()))
+    (tmp_path / "shape.cpp").write_text("\n".join(lines + ["}"]))
+    subprocess.run(["g++", "-std=c++17", "-o", str(tmp_path / "shape"), str(tmp_path / "shape.cpp")], check=True)
+    out = subprocess.run([str(tmp_path / "shape")], check=True, capture_output=True, text=True).stdout.split("\n")
+    assert [tuple(map(int, line.split())) for line in out if line] == list(ATTN.values())
 
 
 def gemm(panels, w_stages, x_stages, wp, chain, seed, closing=True):
@@ -261,8 +303,7 @@ def test_gemm_pair_without_closing_waits():
 def test_pair_holds_tmem_between_barriers_that_show_its_partner_running():
     """tcgen05.alloc and .dealloc of a pair are acts of both CTAs; with the first issued before the start barrier (and the second with
     nothing behind it) a launch hung once in some ten million."""
-    import os
-    src = open(os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2505_19201_b200", "csrc", "gemm_tc.cuh")).read()
+    src = open(os.path.join(CSRC, "gemm_tc.cuh")).read()
     body = src[src.index("k_gemm_tc(const __grid_constant__"):]
     alloc, release, free = (body.index("tcgen05." + op + ".cta_group::2") for op in ("alloc", "relinquish_alloc_permit", "dealloc"))
     assert body.index("cluster_sync_all();") < alloc
