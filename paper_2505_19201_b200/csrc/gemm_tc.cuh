@@ -324,7 +324,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUt
   const uint32_t rank = cluster_ctarank();
   const int pair = blockIdx.x >> 1;
   unsigned long long *tr = trace_open(blockIdx.x == 0 && lane == 0 && (warp == 0 || warp == 2));
-  const unsigned long long t_start = global_ns();
+  const unsigned long long t_start = blockIdx.x == 0 && threadIdx.x == 0 ? global_ns() : 0ull;
   if (warp == 0) {      // a lane per barrier: the set-up is a few instructions deep instead of a loop
     if (lane < TC_MAX_STAGES) { mbar_init(full_w + lane, 1); mbar_init(empty_w + lane, 1); }
     else if (lane < 2 * TC_MAX_STAGES) mbar_init(full_x + lane - TC_MAX_STAGES, 1);
