@@ -27,9 +27,10 @@
 // prefill has one chunk and also leaves each row's log-sum-exp and entropy.  Warp roles: 0 = TMA producer, 1 = S issuer and TMEM owner,
 // 2..9 = softmax and epilogue, 10 = O issuer.  One warp issuing both products spent 2.1k cycles per block at head_dim 256, 1.3k of them the
 // matrix instructions' own time and the rest its waits in turn for P, V, K and a free S; of the 2.3k cycles of a block the softmax waited 0.9k.
-// Prompt attention per layer, before -> now: 832 rows, 32 heads of 128 60 -> 34 us (two CTAs per SM: half of a CTA's 25k cycles is start,
-// first fetch and end), 1152 rows, 32 heads of 64 47 -> 42, 4352 rows, 16 heads of 256 on 8 KV heads 509 -> 415; what bounds
-// the last is the MMA of N = 64, whose A operand's shared-memory reads take half again its own time.
+// In-stream time per layer, one issuer and rows in pairs -> now, us: prompts of 832 rows, 32 heads of 128 52 -> 29 (two CTAs per SM: half of a
+// CTA's 25k cycles is start, first fetch and end), 1152 rows, 32 heads of 64 45 -> 34, 4352 rows, 16 heads of 256 on 8 KV heads 502 -> 405 (bound by
+// the MMA of N = 64, whose A operand's shared-memory reads take half again its own time); verification of 61 rows behind 832, 32 heads of
+// 128 13.6 -> 12.7, of 81 rows behind 4352 at head_dim 256 22.5 -> 19.8 and its merge; draft, 32 heads of 128 10.2 -> 9.9.
 // The loops are kept compact on purpose: this kernel's code is
 // fetched anew at almost every launch (the weight stream between two launches pushes it out of the
 // caches), and straight-line code then costs its own fetch (a fully unrolled version of the same
@@ -172,8 +173,7 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// (As packed instructions, add.rn.f32x2 and fma.rn.f32x2, the same values: LLaVA-7B-shaped request 24.0 -> 24.3 ms, Gemma-shaped round 11.39 ->
-// 11.45; the packing costs more than it saves.)
+// Pairs of keys, added and scaled one by one (the packed instructions give the same values and cost more in packing than they save).
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 d) { return make_float2(fmaf(a.x, b.x, d.x), fmaf(a.y, b.y, d.y)); }
 // w[i] of the four lanes of a quad: lane j ends up with the quad's words j, in lane order.

@@ -825,9 +825,12 @@ template <typename T, int HD> struct AttnLaunch {
     auto blocks_of = [&](int want) { return (nb_ub + want - 1) / want; };
     int want = imin(AT_MAX_CLUSTER, nb_ub), many = imin(imin(AT_MAX_CHUNKS, nb_ub), imax(1, max_tiles[1] / tiles));
     while (want > 1 && max_tiles[want] < tiles) --want;
-    // Clusters need free SMs of one GPC, so fewer chunks fit: partials and the merge kernel (4 us) where the longer
-    // chunks cost more than that (a block takes 1 us at head_dim 128 and in proportion): the Gemma-shaped
-    // round with 5 and 10 chunks per tile instead of 6 and 18 was 2 % slower, the others 1..2 % faster
+    // Clusters need free SMs of one GPC, so fewer chunks fit: partials and the merge kernel (4 to 8 us, of which a launch saves 3 to 6 by not
+    // merging itself) where the longer chunks cost more than that.  A block takes 0.9, 1.0 and 1.2 us at head_dim 64, 128 and 256.  Time from the
+    // attention's start to the end of the projection behind it, cluster / merge kernel, us: head_dim 256 with 24 tiles 14 blocks a chunk instead
+    // of 12 39.1 / 36.2, 5 instead of 4 27.9 / 26.8; with 8 tiles 7 instead of 4 36.2 / 34.4 (draft) and 25.7 / 26.2, 4 instead of 2 29.1 / 29.0, 3 instead of 2
+    // 19.7 / 20.5, 2 instead of 1 21.7 / 24.1; head_dim 128 9 instead of 6 31.7 / 30.2, 6 instead of 3 24.9 / 25.5, 2 instead of 1 19.1 / 21.6; head_dim 64 17
+    // instead of 8 28.6 / 26.6, 5 instead of 3 17.2 / 18.7.  The line costs at most 1.1 us of these 37 to 20 on its wrong side.
     const bool merge = a.mode != AT_PREFILL && a.n_rt <= c->am_rt_max && (blocks_of(want) - blocks_of(many)) * HD > 256;
     if (merge) { want = many; a.part_o = c->am_part_o; a.part_ml = c->am_part_ml; a.part_u = c->am_part_u; }
     a.blocks_per_chunk = blocks_of(want);
